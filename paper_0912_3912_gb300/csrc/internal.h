@@ -169,7 +169,10 @@ struct ising_handle {
   int32_t tiles_R = -1;
   int32_t n_tiles = 0;
   unsigned long long *h_stats_pinned = nullptr;
-  // energy work list (per replica count) and partial sums
+  // energy form, work list (per replica count), partial sums, replica words
+  int32_t en_form = 0, en_part = 0;
+  uint32_t *d_en_words = nullptr;
+  unsigned long long *d_en_acc = nullptr;
   int32_t en_R = -1, en_nwork = 0;
   int4 *d_en_work = nullptr;
   int32_t *d_en_first = nullptr;
