@@ -54,6 +54,7 @@ DevGraph ising_handle::graph() const {
   g.runit = d_runit;
   g.nsp = total_spins;
   g.dtype = dtype;
+  g.hyper = has_hyper ? 1 : 0;
   return g;
 }
 
@@ -132,6 +133,62 @@ int32_t fp64_exact(const HostInst &I, bool fl, int32_t ebase) {
   for (float v : I.hf) rest += units(v);
   for (float v : I.hJf) rest += units(v);
   return pairs2 / 2 + rest < ((unsigned __int128)1 << 53) ? 1 : 0;
+}
+
+// InstDesc::fm_ent, fbits and funit (see there); inc: hyper-edges per spin.
+// Returns the most entries of one spin with the same target.
+int32_t fm_entries(const HostInst &I, const std::vector<std::vector<int32_t>> &inc, bool fl, InstDesc &D) {
+  D.fm_ent = D.fbits = D.funit = -1;
+  if (I.n > fm_max_spins()) return 1;
+  const int32_t n_hyper = (int32_t)I.hptr.size() - 1;
+  for (int32_t e = 0; e < n_hyper; ++e)
+    if (I.hptr[e + 1] - I.hptr[e] > 3) return 1;
+  int64_t most = 0;
+  int32_t rounds = 1, t[32];
+  for (int32_t i = 0; i < I.n; ++i) {
+    int64_t ent = I.row[i + 1] - I.row[i];
+    for (int32_t e : inc[i]) ent += I.hptr[e + 1] - I.hptr[e] - 1;
+    most = std::max(most, ent);
+    if (most > 31) return 1;
+    if (inc[i].empty()) continue;  // the row's columns are distinct
+    int32_t k = 0;
+    for (int64_t q = I.row[i]; q < I.row[i + 1]; ++q) t[k++] = I.col[q];
+    for (int32_t e : inc[i])
+      for (int64_t q = I.hptr[e]; q < I.hptr[e + 1]; ++q)
+        if (I.hmem[q] != i) {
+          int32_t same = 1;
+          for (int32_t a = 0; a < k; ++a) same += t[a] == I.hmem[q];
+          rounds = std::max(rounds, same);
+          t[k++] = I.hmem[q];
+        }
+    if (rounds > 15) return 1;
+  }
+  D.fm_ent = (int32_t)most;
+  if (fl && D.ebase < 0) return rounds;
+  // (the FP64 sums of at most 32 magnitudes round up by far less than the factor)
+  double top = 0.0;
+  int32_t unit = 256;
+  auto see = [&](float v) -> double {
+    uint32_t b;
+    std::memcpy(&b, &v, 4);
+    b &= 0x7fffffffu;
+    if (b) unit = std::min(unit, (int32_t)(b >> 23) + __builtin_ctz((b & 0x7fffffu) | 0x800000u));
+    return std::fabs((double)v);
+  };
+  for (int32_t i = 0; i < I.n; ++i) {
+    double a = fl ? see(I.hf[i]) : std::abs((int)I.hi[i]);
+    for (int64_t k = I.row[i]; k < I.row[i + 1]; ++k) a += fl ? see(I.Jf[k]) : std::abs((int)I.Ji[k]);
+    for (int32_t e : inc[i]) a += fl ? see(I.hJf[e]) : std::abs((int)I.hJi[e]);
+    top = std::max(top, a);
+  }
+  D.funit = fl ? (unit < 256 ? unit : D.ebase) : -1;
+  D.fbits = 0;
+  if (top > 0.0) {
+    int ex = 0;
+    std::frexp(top * (1.0 + 1e-12), &ex);  // top < 2^ex
+    D.fbits = std::max(0, ex - (fl ? D.funit - 150 : 0));
+  }
+  return rounds;
 }
 
 // Recognise a periodic hypercubic lattice (side L >= 3, d = 2 or 3, spin index
@@ -774,6 +831,8 @@ ising_status ising_create(const ising_instance_desc *descs, int32_t n_instances,
         inc_oth.push_back(o);
       }
     }
+    D.fm_ent = D.fbits = D.funit = -1;
+    if (!f64) h->fm_rounds = std::max(h->fm_rounds, fm_entries(I, inc, fl, D));
     for (int32_t e = 0; e < D.n_hyper; ++e) hptr.push_back((uint32_t)(mem_off + I.hptr[e]));
     hmem.insert(hmem.end(), I.hmem.begin(), I.hmem.end());
     // colour classes: spins sorted by (colour, index)

@@ -21,10 +21,12 @@
 // results and no FP64 on the per-move path.
 //
 // One warp per search.  The paper keeps the gains in a heap (Fig. 4);
-// fm_kernel keeps per-warp maxima of 32-spin blocks in shared memory and takes
-// the move's spin by warp reductions over them (gains compared as
-// order-preserving integers); fm_reg_kernel holds a small instance's fields in
-// the lanes' registers.  Both select the heap's spin.
+// fm_key_kernel keeps one key per spin in shared memory (gain, index and spin
+// in one integer) under a tree of maxima, and each spin's changes in one
+// fixed-stride record; it serves the integer forms with hyper-edges of at most
+// three members and at most 31 changes a move.  fm_kernel serves the others:
+// per-warp maxima of 32-spin blocks and the CSR rows.  fm_reg_kernel holds a
+// small instance's fields in the lanes' registers.  All select the heap's spin.
 #include <algorithm>
 #include <cfloat>
 #include <cmath>
@@ -45,6 +47,8 @@ constexpr int kFmMaxSpins = 4096;
 // arithmetic of a search (InstDesc::fx53): FP64 as defined; int64 in one unit
 // per instance; int64 fields in per-spin units with FP64 energies
 constexpr int kFp64 = 0, kFx = 1, kFxSpin = 2;
+// ... with gain keys: the word alone, with 32 and with 64 low bits beside it
+constexpr int kKeyExact = 3, kKeyWide = 4, kKeyWide64 = 5;
 // a move that changes more fields than this recomputes every block maximum
 constexpr int kTouched = 64;
 
@@ -556,6 +560,408 @@ __global__ void __launch_bounds__(kFT, 3) fm_kernel(FmArgs A, int nmax) {
   }
 }
 
+// ---- gain keys ---------------------------------------------------------------
+// The tree of maxima works on one 32-bit word per spin,
+//   gq << 13 | (4095 - index) << 1 | x,   gq = g >> sh,
+// with g = -s f (half the gain) in the instance's unit and sh the bits of g that
+// do not fit (0 for int8 instances, whose words hold g itself): a larger word is
+// a larger gain, or an equal one of a lower index, as long as the gq differ.
+//   exact form (sh = 0): x = the spin is +1; the largest word is the move.
+//   wide forms: a second word (32 or 64 bits) per spin holds the low sh bits of g
+//     and the spin, (g & mask) << 1 | (spin is +1); x is 0.  When a second word has the largest
+//     gq (few moves for Gaussian couplings) the tied spins' low bits decide.
+// A spin moved in this pass keeps MIN | step << 1 | x, below every unlocked word
+// (gq >= -2^17): the step tells at the pass's end whether the best prefix holds it.
+constexpr int kGq = 17;  // |g| < 2^(kGq + sh)
+// largest InstDesc::fbits of the wide forms: sums and differences of low parts fit
+// a signed word
+constexpr int kWideBits = kGq + 30, kWide64Bits = 60;
+constexpr int kLocked = INT32_MIN;
+constexpr int kLeaf = 8;       // words of one leaf
+constexpr int kFlatMax = 512;  // up to this size the lanes scan all words, without leaves
+
+// 16-byte reads of a lane over n words spread on 32 lanes: 1, 2 or 4
+__host__ __device__ constexpr int lane_reads(int words) {
+  const int r = ((words + 31) / 32 + 3) / 4;
+  return r <= 1 ? 1 : (r <= 2 ? 2 : 4);
+}
+// Lane-major words (word q of lane l at l * stride + q): the stride is an odd
+// number of 16-byte units, so the 32 lanes' reads do not collide on banks.
+__host__ __device__ constexpr int lane_stride(int words) { return (lane_reads(words) | 1) * 4; }
+__host__ __device__ constexpr int leaves_of(int n) { return (n + kLeaf - 1) / kLeaf; }
+// a warp's shared memory in words: keys (and the leaves' maxima), low words
+__host__ __device__ constexpr int key_words(int n) {
+  return n <= kFlatMax ? 32 * lane_stride(n) : leaves_of(n) * kLeaf + 32 * lane_stride(leaves_of(n));
+}
+// (low: words of 4 bytes beside a spin's first)
+__host__ __device__ constexpr size_t key_warp_bytes(int n, int low) {
+  return ((size_t)key_words(n) + low * ((n + 3) / 4 * 4)) * 4;
+}
+__device__ __forceinline__ int max4(const int4 &v) { return max(max(v.x, v.y), max(v.z, v.w)); }
+
+// A move's changes: `stride` entries per spin, {x, hi, low}: x = target |
+// round << 12 | other << 16, 2 J = hi << sh | low (64 bits) in units.  The target's half gain
+// changes by -+2 J with the product of the spins of i, the target and, for a
+// 3-member hyper-edge, the third member (other; kNone: no third).  Entries of one
+// spin with the same target lie in different rounds.  kPad: no entry.
+constexpr uint32_t kNone = 0xffffu, kPad = 0xfffeu;
+constexpr size_t kStageMax = 188 * 1024;  // bytes of records in shared memory at most
+
+// coupling or field k of array p in units of 2^(I.funit - 150) (int8: 1)
+__device__ __forceinline__ long long key_term(const void *p, bool fl, int64_t k, const InstDesc &I) {
+  return fl ? fx_of(p, true, k, I.ebase) >> (I.funit - I.ebase) : fx_of(p, false, k, 0);
+}
+// low bits kept apart from the words of instance I
+__host__ __device__ inline int key_shift(const InstDesc &I) { return I.fbits > kGq ? I.fbits - kGq : 0; }
+
+__global__ void fm_entries_kernel(DevGraph G, int4 *ent, int stride) {
+  const InstDesc &I = G.inst[blockIdx.x];
+  if (I.fm_ent < 0 || I.fbits < 0 || I.fbits > kWide64Bits) return;
+  const bool fl = G.dtype == ISING_F32;
+  const int sh = key_shift(I);
+  for (int i = threadIdx.x; i < I.n; i += blockDim.x) {
+    const int64_t gi = I.spin_off + i;
+    int4 *e = ent + gi * stride;
+    int cnt = 0;
+    auto put = [&](int target, uint32_t other, const void *arr, int64_t at) {
+      int round = 0;
+      for (int q = 0; q < cnt; ++q) round += (e[q].x & 0xfff) == target;
+      const long long d = 2 * key_term(arr, fl, at, I);
+      const unsigned long long low = (unsigned long long)d & ((1ull << sh) - 1ull);
+      e[cnt++] = make_int4((int)((uint32_t)target | (uint32_t)round << 12 | other << 16), (int)(d >> sh),
+                           (int)(uint32_t)low, (int)(uint32_t)(low >> 32));
+    };
+    for (uint32_t k = G.row[gi]; k < G.row[gi + 1]; ++k) put(G.col[k], kNone, G.J, k);
+    for (uint32_t u = G.inc_ptr[gi]; u < G.inc_ptr[gi + 1]; ++u) {
+      const int64_t he = G.inc_edge[u];
+      int m[2], c = 0;
+      for (uint32_t q = G.hptr[he]; q < G.hptr[he + 1]; ++q)
+        if (G.hmem[q] != i && c < 2) m[c++] = G.hmem[q];
+      put(m[0], c == 2 ? (uint32_t)m[1] : kNone, G.hJ, he);
+      if (c == 2) put(m[1], (uint32_t)m[0], G.hJ, he);
+    }
+    for (; cnt < stride; ++cnt) e[cnt] = make_int4((int)(kPad << 16), 0, 0, 0);
+  }
+}
+
+// LOW: words of low bits (0 exact, 1 and 2 wide).  Wide instances whose energies
+// are not exact in FP64 (InstDesc::fx53 != 1) run them in FP64 as defined, all
+// others as integers in the unit.  FLAT: no leaves (nmax <= kFlatMax).  NR: lane_reads of the launch.  staged: the
+// warp's records sit in shared memory.
+//
+// One move is one dependent chain, and a lone search pays all of it: the lanes
+// scan their words, the warp takes the largest (which brings the spin along),
+// the lanes read the spin's record in one step and change their targets' words,
+// and each lane rescans its target's leaf.  About 155 instructions and 760 cycles
+// a move with a warp alone on its SM (half of the cycles fixed-latency
+// dependencies, a sixth shared memory and shuffles), where fm_kernel takes about
+// 3,900.  61 searches of 2,500 spins: 35.5 -> 10.9 ms; 640 of 256 (int8): 1.70 ->
+// 0.44 ms; 128 uneven cell grids, 32 replicas each: 38.0 -> 12.2 ms, there with
+// the records' trips to L2 on the chain.
+template <int LOW, bool FLAT, int NR>
+__global__ void __launch_bounds__(kFT, 2)
+fm_key_kernel(FmArgs A, int nmax, const int4 *__restrict__ ent, int stride, int rounds, int staged) {
+  constexpr bool WIDE = LOW > 0;
+  using L = std::conditional_t<LOW == 2, unsigned long long, uint32_t>;  // low words
+  using SL = std::conditional_t<LOW == 2, long long, int>;
+  extern __shared__ __align__(16) uint8_t fm_smem[];
+  const DevGraph &G = A.g;
+  const bool fl = G.dtype == ISING_F32, hyper = G.hyper != 0;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const size_t warp_bytes = key_warp_bytes(nmax, LOW) + (staged ? (size_t)nmax * stride * sizeof(int4) : 0);
+  uint8_t *base = fm_smem + (size_t)warp * warp_bytes;
+  constexpr int ls = (NR | 1) * 4;
+  int *hi = reinterpret_cast<int *>(base);
+  L *lo = reinterpret_cast<L *>(hi + key_words(nmax));
+  int4 *rec = reinterpret_cast<int4 *>(base + key_warp_bytes(nmax, LOW));
+  int *top = FLAT ? hi : hi + leaves_of(nmax) * kLeaf;
+  auto lane_pos = [&](int q) -> int { return (q & 31) * ls + (q >> 5); };
+  auto pos = [&](int i) -> int { return FLAT ? lane_pos(i) : i; };
+  // the spin of site i (also while another lane rewrites the word: its bit stays)
+  auto up = [&](int i) -> bool {
+    return WIDE ? *reinterpret_cast<const volatile uint32_t *>(lo + i) & 1u
+                : (uint32_t)*const_cast<const volatile int *>(hi + pos(i)) & 1u;
+  };
+  auto leaf_max = [&](int leaf) -> int {
+    const int4 *p = reinterpret_cast<const int4 *>(hi + leaf * kLeaf);
+    const int4 u = p[0], v = p[1];
+    return max(max4(u), max4(v));
+  };
+  const int4 *mine = reinterpret_cast<const int4 *>(top + lane * ls);
+  int staged_b = -1;
+  unsigned long long c_moves = 0, c_passes = 0, c_starts = 0;
+  for (;;) {
+    int w = 0;
+    if (lane == 0) w = atomicAdd(A.queue, 1);
+    w = __shfl_sync(0xffffffffu, w, 0);
+    if (w >= A.n_work) break;
+    const int it = A.split ? w / A.restarts : w;
+    const int k0 = A.split ? w % A.restarts : 0, k1 = A.split ? k0 + 1 : A.restarts;
+    const int b = A.items[it].x, r = A.items[it].y;
+    const int slot = A.split ? r * A.restarts + k0 : r;
+    const InstDesc I = G.inst[b];
+    const int n = I.n, unit = I.funit;
+    const bool fe = WIDE && I.fx53 != 1;
+    const int64_t so = I.spin_off;
+    const int sh = WIDE ? key_shift(I) : 0;
+    const L low_mask = WIDE ? ((L)1 << sh) - 1 : 0;
+    const int leaves = leaves_of(n);
+    const int4 *row = ent + so * stride;  // (generic loads: global or shared)
+    if (staged) {
+      if (staged_b != b)
+        for (int q = lane; q < n * stride; q += 32) rec[q] = row[q];
+      staged_b = b;
+      row = rec;
+    }
+    const double scale = fl ? __longlong_as_double((long long)(unit - 150 + 1023) << 52) : 1.0;
+    const uint64_t seed = A.seeds[b];
+    // E of the current spins
+    auto energy = [&](long long &Ei) -> double {
+      if (fe) {  // FP64 as fm_energy: lane partial sums, then the warp sum
+        Ei = 0;
+        double acc = 0.0;
+        for (int i = lane; i < n; i += 32) {
+          const int64_t gi = so + i;
+          const double si = up(i) ? 1.0 : -1.0;
+          for (uint32_t k = __ldg(G.row + gi), ke = __ldg(G.row + gi + 1); k < ke; ++k) {
+            const int j = __ldg(G.col + k);
+            if (j > i) acc -= coupling(G, 1, k) * si * (up(j) ? 1.0 : -1.0);
+          }
+          acc -= field_h(G, 1, gi) * si;
+        }
+        for (int e = lane; e < I.n_hyper; e += 32) {
+          const int64_t ge = I.hyper_off + e;
+          double p = 1.0;
+          for (uint32_t q = __ldg(G.hptr + ge), qe = __ldg(G.hptr + ge + 1); q < qe; ++q)
+            p *= up(__ldg(G.hmem + q)) ? 1.0 : -1.0;
+          acc -= coupling_e(G, 1, ge) * p;
+        }
+        return warp_sum(acc);
+      } else {
+        long long acc = 0;
+        for (int i = lane; i < n; i += 32) {
+          const int64_t gi = so + i;
+          const bool ui = up(i);
+          for (uint32_t k = __ldg(G.row + gi), ke = __ldg(G.row + gi + 1); k < ke; ++k) {
+            const int j = __ldg(G.col + k);
+            if (j > i) {
+              const long long t = key_term(G.J, fl, k, I);
+              acc -= ui == up(j) ? t : -t;
+            }
+          }
+          const long long th = key_term(G.h, fl, gi, I);
+          acc -= ui ? th : -th;
+        }
+        for (int e = lane; e < I.n_hyper; e += 32) {
+          const int64_t ge = I.hyper_off + e;
+          const long long t = key_term(G.hJ, fl, ge, I);
+          bool neg = false;
+          for (uint32_t q = __ldg(G.hptr + ge), qe = __ldg(G.hptr + ge + 1); q < qe; ++q)
+            neg ^= !up(__ldg(G.hmem + q));
+          acc -= neg ? -t : t;
+        }
+        Ei = warp_sum(acc);
+        return (double)Ei * scale;
+      }
+    };
+    double E_all = DBL_MAX;
+    int total_passes = 0;
+    int8_t *out = A.spins + (int64_t)A.R_out * so + (int64_t)slot * n;
+    for (int q = lane; q < key_words(nmax); q += 32) hi[q] = kLocked;  // (words of no spin stay so)
+    __syncwarp();
+    for (int k = k0; k < k1; ++k) {
+      for (int i = lane; i < n; i += 32) {
+        const uint4 x = start_bits(seed, (uint32_t)(i >> 7), (uint32_t)r, (uint32_t)k, (uint32_t)b);
+        const uint32_t u = (word_of(x, (i & 127) >> 5) >> (i & 31)) & 1u;
+        if (WIDE) lo[i] = u;
+        else hi[pos(i)] = (int)u;
+      }
+      __syncwarp();
+      long long EstarI;
+      double Estar = energy(EstarI);
+      int passes = 0;
+      for (;;) {
+        ++passes;
+        // words from scratch: g = -s (h + sum J s + hyper-edges) from the spins'
+        // records (a hyper-edge's two entries give its term once)
+        for (int i = lane; i < n; i += 32) {
+          const bool ui = up(i);
+          long long f2 = 2 * key_term(G.h, fl, so + i, I);
+          for (int q = 0; q < stride; ++q) {
+            const int4 en = row[i * stride + q];
+            const uint32_t other = (uint32_t)en.x >> 16;
+            const int c = en.x & 0xfff;
+            if (other == kPad) break;
+            if (other != kNone && (int)other < c) continue;
+            const long long t = ((long long)en.y << sh) + (long long)((unsigned long long)(uint32_t)en.w << 32 | (uint32_t)en.z);
+            f2 += up(c) ^ (other != kNone && !up((int)other)) ? t : -t;
+          }
+          const long long g = (ui ? -f2 : f2) / 2;
+          const uint32_t word = (uint32_t)(int)(g >> sh) << 13 | (uint32_t)(4095 - i) << 1;
+          if (WIDE) {
+            lo[i] = ((L)g & low_mask) << 1 | (L)ui;
+            hi[pos(i)] = (int)word;
+          } else {
+            hi[pos(i)] = (int)(word | (uint32_t)ui);
+          }
+        }
+        __syncwarp();
+        if (!FLAT) {
+          for (int l = lane; l < leaves; l += 32) top[lane_pos(l)] = leaf_max(l);
+          __syncwarp();
+        }
+        long long Ecur = EstarI, Ebest = EstarI;
+        double Ecurd = Estar, Ebestd = Estar;
+        int best_len = 0;
+        for (int step = 0; step < n; ++step) {
+          int m = max4(mine[0]);
+#pragma unroll
+          for (int q = 1; q < NR; ++q) m = max(m, max4(mine[q]));
+          const int best = __reduce_max_sync(0xffffffffu, m);
+          int i = 4095 - ((best >> 1) & 4095);
+          if constexpr (WIDE) {
+            // Does another word have this gq?  The lanes' maxima, then the words
+            // of the one lane that has it (4 NR of them) and of its leaf.
+            const int t = best & ~8191;
+            const unsigned who = __ballot_sync(0xffffffffu, m >= t);
+            const int at = __ffs(who) - 1;
+            int v = kLocked;
+            if (lane < 4 * NR) v = top[at * ls + lane];
+            else if (!FLAT && lane >= 24) v = hi[(i & ~(kLeaf - 1)) + lane - 24];
+            const unsigned eq = __ballot_sync(0xffffffffu, v >= t);
+            if ((who & (who - 1u)) || __popc(eq) != (FLAT ? 1 : 2)) {
+              // the tied spins' low bits decide, then the lowest index
+              L bl = 0;
+              uint32_t bi = 4096u;
+              for (int j = lane; j < n; j += 32)
+                if (hi[pos(j)] >= t) {
+                  const L l = (lo[j] >> 1) + 1;
+                  if (l > bl) {
+                    bl = l;
+                    bi = (uint32_t)j;
+                  }
+                }
+              const uint32_t b1 = LOW == 2 ? (uint32_t)(bl >> 31 >> 1) : 0u, m1 = __reduce_max_sync(0xffffffffu, b1);
+              const uint32_t m0 = __reduce_max_sync(0xffffffffu, b1 == m1 ? (uint32_t)bl : 0u);
+              i = (int)__reduce_min_sync(0xffffffffu, b1 == m1 && (uint32_t)bl == m0 ? bi : 4096u);
+            }
+          }
+          int4 en = make_int4((int)(kPad << 16), 0, 0, 0);
+          if (lane < stride) en = row[i * stride + lane];
+          const L li = WIDE ? lo[i] : (L)(uint32_t)best;
+          const uint32_t other = (uint32_t)en.x >> 16;
+          const bool has = other != kPad;
+          const int c = has ? en.x & 0xfff : i;  // (lanes without an entry repeat the moved spin's leaf)
+          const int pc = pos(c);
+          const int hc = hi[pc];
+          const L lc = WIDE ? lo[c] : (L)(uint32_t)hc;
+          // parity of the (two or three) spins; odd: their product is +1 after
+          // the move, and the target's g falls by 2 J, else it rises
+          uint32_t odd = (uint32_t)li ^ (uint32_t)lc;
+          if (hyper && other < kPad) odd ^= !up((int)other);
+          const bool fall = odd & 1u;
+          const bool open = has && hc >= -(1 << 30);
+          const long long g = ((long long)(best >> 13) << sh) + (WIDE ? (long long)(li >> 1) : 0);
+          if (fe) {
+            Ecurd = __dsub_rn(Ecurd, fx_double(2 * g, unit));
+            if (Ecurd < Ebestd) {
+              Ebestd = Ecurd;
+              best_len = step + 1;
+            }
+          } else {
+            Ecur -= 2 * g;
+            if (Ecur < Ebest) {
+              Ebest = Ecur;
+              best_len = step + 1;
+            }
+          }
+          __syncwarp();
+          if (lane == 31) {
+            hi[pos(i)] = kLocked | step << 1 | (WIDE ? 0 : (int)(~(uint32_t)li & 1u));
+            if (WIDE) lo[i] = li ^ 1;
+          }
+          const SL dl = LOW == 2 ? (SL)((unsigned long long)(uint32_t)en.w << 32 | (uint32_t)en.z) : (SL)en.z;
+          auto change = [&](int h, L l) {
+            if (WIDE) {
+              const SL low = (SL)(l >> 1);
+              const SL sum = fall ? low - dl : low + dl;
+              hi[pc] = h + (int)((uint32_t)((fall ? -en.y : en.y) + (int)(sum >> sh)) << 13);
+              lo[c] = ((L)sum & low_mask) << 1 | (l & 1);
+            } else {
+              hi[pc] = h + (int)((uint32_t)(fall ? -en.y : en.y) << 13);
+            }
+          };
+          if (rounds > 1) {  // some targets occur more than once
+            const int round = (en.x >> 12) & 15;
+            if (open && round == 0) change(hc, lc);
+            for (int q = 1; __any_sync(0xffffffffu, has && round >= q); ++q) {
+              __syncwarp();
+              if (open && round == q) change(hi[pc], WIDE ? lo[c] : (L)0);
+            }
+          } else if (open) {
+            change(hc, lc);
+          }
+          __syncwarp();
+          if (!FLAT) {
+            const int leaf = (lane == 31 ? i : c) / kLeaf;
+            top[lane_pos(leaf)] = leaf_max(leaf);
+            __syncwarp();
+          }
+        }
+        // roll back to the best prefix: spins moved at a later step flip back
+        auto roll = [&](bool inside) {
+          for (int i = lane; i < n; i += 32) {
+            const bool in = ((hi[pos(i)] >> 1) & 4095) < best_len;
+            if (in == inside) {
+              if (WIDE) lo[i] ^= 1;
+              else hi[pos(i)] ^= 1;
+            }
+          }
+          __syncwarp();
+        };
+        roll(false);
+        double Enew;
+        long long EnewI = 0;
+        if (fe) {
+          Enew = energy(EnewI);
+        } else {  // the running energy is exact
+          EnewI = Ebest;
+          Enew = (double)EnewI * scale;
+        }
+        const double margin = fl ? 1e-9 * (1.0 + fabs(Estar)) : 0.0;
+        c_moves += (unsigned long long)n;
+        if (Enew < Estar - margin && (A.max_passes <= 0 || passes < A.max_passes)) {
+          Estar = Enew;
+          EstarI = EnewI;
+          continue;
+        }
+        if (Enew < Estar - margin) Estar = Enew;  // pass cap reached after an improving pass: keep it
+        else if (best_len > 0) roll(true);        // back to the pass's start
+        break;
+      }
+      total_passes += passes;
+      c_passes += (unsigned long long)passes;
+      c_starts += 1;
+      if (Estar < E_all) {  // strictly lower energy; ties keep the earlier
+        E_all = Estar;
+        for (int i = lane; i < n; i += 32) out[i] = up(i) ? 1 : -1;
+      }
+      __syncwarp();
+    }
+    if (lane == 0) {
+      A.energy[(int64_t)b * A.R_out + slot] = E_all;
+      if (A.passes) A.passes[(int64_t)b * A.R_out + slot] = total_passes;
+    }
+    __syncwarp();
+  }
+  if (lane == 0 && c_starts) {
+    atomicAdd(A.stats + 0, c_moves);
+    atomicAdd(A.stats + 1, c_moves);
+    atomicAdd(A.stats + 3, c_starts);
+    atomicAdd(A.stats + 4, c_passes);
+  }
+}
+
 // Small instances in the one-unit integer form (kFx, n <= 32 * S, S = 8 or 16):
 // lane l holds the fields, spin bits, lock bits and best-prefix bits of spins
 // l, l + 32, ... in registers.  A move's arg-max is each lane's maximum over
@@ -805,8 +1211,15 @@ __global__ void fm_best_start_kernel(const InstDesc *inst, int32_t n_inst, int32
   }
 }
 
+// Warps per CTA (one search each) and CTAs per SM of one kernel at one size.
+struct FmShape {
+  int warps = 0, per_sm = 0, one_warp_per_sm = 0;
+  size_t warp_bytes = 0;
+};
+
 // device buffers per handle, kept across calls: the (instance, replica)
-// list, the work-queue counters and, for split starts, every start's result
+// list, the work-queue counters, the change entries and, for split starts,
+// every start's result
 struct FmBufs : FamilyState {
   int2 *items = nullptr;
   size_t items_bytes = 0;
@@ -814,6 +1227,9 @@ struct FmBufs : FamilyState {
   size_t queues_bytes = 0;
   void *scratch = nullptr;
   size_t scratch_bytes = 0;
+  int4 *ent = nullptr;  // [total_spins][ent_stride] (fm_entries_kernel)
+  int ent_stride = -1;  // -1: not built yet, 0: no instance takes the gain keys
+  std::map<std::pair<int, int>, FmShape> shapes;  // by (kernel, size)
   // side streams for overlapping the groups' launches, with fork/join events
   std::vector<cudaStream_t> side;
   std::vector<cudaEvent_t> join;
@@ -835,15 +1251,21 @@ cudaError_t grow(P *&p, size_t &have, size_t need) {
 }
 
 constexpr size_t kSplitScratchMax = size_t(1) << 30;  // bytes of per-start results at most
-constexpr int kSideStreams = 4;
+// Two streams per size class, the larger classes' and within a class the smaller
+// group's of higher priority: with a call queued behind another all groups become
+// ready at once, and a group whose few searches start last ends last.
+constexpr int kClassStreams = 2, kClasses = 5, kSideStreams = kClassStreams * kClasses;
 
 cudaError_t ensure_side(FmBufs &B) {
   if (!B.side.empty()) return cudaSuccess;
-  cudaError_t e = cudaEventCreateWithFlags(&B.fork, cudaEventDisableTiming);
+  int least = 0, greatest = 0;
+  cudaError_t e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&B.fork, cudaEventDisableTiming);
   for (int j = 0; j < kSideStreams && e == cudaSuccess; ++j) {
     cudaStream_t st = nullptr;
     cudaEvent_t ev = nullptr;
-    if ((e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking)) != cudaSuccess) break;
+    const int prio = std::min(least, greatest + j / kClassStreams + j % kClassStreams);
+    if ((e = cudaStreamCreateWithPriority(&st, cudaStreamNonBlocking, prio)) != cudaSuccess) break;
     B.side.push_back(st);
     if ((e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess) break;
     B.join.push_back(ev);
@@ -863,55 +1285,123 @@ cudaError_t ensure_side(FmBufs &B) {
 // One launch group: instances of one arithmetic (FX or FP64) whose size falls
 // in (lo, hi], so that each warp's shared memory is sized for hi.
 struct FmPart {
-  int mode;  // kFp64 / kFx / kFxSpin
+  int mode;  // kFp64 ... kKeyWide64
   int nmax;
   int64_t first, count;  // range of the item list
+  bool one_unit;  // (InstDesc::fx53 == 1: the register kernel could take it)
 };
 
-// Warps per CTA (one search each) and CTAs per SM for instances of up to
-// nmax spins: the most searches per SM that shared memory and registers allow,
-// the larger CTA among equals.
-template <int M, int FL>
-cudaError_t fm_shape(const ising_handle *h, int nmax, int &warps, size_t &smem, int &per_sm) {
-  const size_t per_warp = (fm_warp_bytes(nmax, M) + 15) & ~(size_t)15;
-  int smem_optin = 0;
-  cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
-  cudaError_t e;
-  const int wmax = (int)std::max<size_t>(1, std::min<size_t>(kFW, (size_t)smem_optin / per_warp));
-  if ((e = cudaFuncSetAttribute(fm_kernel<M, FL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(per_warp * wmax))) != cudaSuccess)
-    return e;
-  int best = -1;
-  for (int w = wmax; w >= 1; --w) {
-    int c = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, fm_kernel<M, FL>, w * 32, per_warp * w)) != cudaSuccess)
+// Kernel variants of the launches (FmBufs::shapes is keyed by them).
+enum { kVarReg8 = 8, kVarReg16 = 9, kVarStaged = 16 };  // (the others: the modes)
+
+// Searches per SM: as many as shared memory and registers allow, in the
+// smallest CTAs that come within a tenth of it (a CTA's memory is free for the
+// next size class when its last search ends).  The shared-memory limit is
+// raised to the device's for every size alike: the attribute is the process's,
+// and another thread's handle may launch the same kernel at a larger size.
+template <typename Kern>
+cudaError_t shape_of(const ising_handle *h, Kern kern, size_t warp_bytes, int wmax, FmShape &S) {
+  int optin = 0;
+  cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
+  if (e != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess) return e;
+  S.warp_bytes = warp_bytes;
+  wmax = (int)std::max<size_t>(1, std::min<size_t>(wmax, (size_t)optin / warp_bytes));
+  std::vector<int> ctas(wmax + 1, 0);
+  int best = 0;
+  for (int w = 1; w <= wmax; ++w) {
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas[w], kern, w * 32, warp_bytes * w)) != cudaSuccess)
       return e;
-    if (c * w > best) {
-      best = c * w;
-      warps = w;
-      per_sm = std::max(c, 1);
-    }
+    best = std::max(best, ctas[w] * w);
   }
-  smem = per_warp * warps;
+  S.one_warp_per_sm = ctas[1];
+  int w = 1;
+  while (w < wmax && 10 * ctas[w] * w < 9 * best) ++w;
+  S.warps = w;
+  S.per_sm = std::max(ctas[w], 1);
   return cudaSuccess;
 }
 
+template <int M, int FL>
+cudaError_t fm_shape(const ising_handle *h, int nmax, FmShape &S) {
+  return shape_of(h, fm_kernel<M, FL>, (fm_warp_bytes(nmax, M) + 15) & ~(size_t)15, kFW, S);
+}
+// the gain-key kernel of a mode for instances of up to nmax spins
+using KeyKernel = void (*)(FmArgs, int, const int4 *, int, int, int);
+template <int LOW>
+KeyKernel key_kernel_of(int nmax) {
+  const int r = lane_reads(nmax <= kFlatMax ? nmax : leaves_of(nmax));
+  if (nmax <= kFlatMax)
+    return r == 1 ? fm_key_kernel<LOW, true, 1> : (r == 2 ? fm_key_kernel<LOW, true, 2> : fm_key_kernel<LOW, true, 4>);
+  return r == 1 ? fm_key_kernel<LOW, false, 1> : (r == 2 ? fm_key_kernel<LOW, false, 2> : fm_key_kernel<LOW, false, 4>);
+}
+KeyKernel key_kernel(int mode, int nmax) {
+  return mode == kKeyExact ? key_kernel_of<0>(nmax) : (mode == kKeyWide ? key_kernel_of<1>(nmax) : key_kernel_of<2>(nmax));
+}
 // the register kernel's shape: 8 warps per CTA, as many CTAs per SM as fit
-template <bool FL, int S>
-cudaError_t fm_reg_shape(const ising_handle *h, int &warps, size_t &smem, int &per_sm) {
-  (void)h;
-  warps = kFW;
-  smem = reg_warp_bytes(S) * kFW;
+template <bool FL, int N>
+cudaError_t fm_reg_shape(const ising_handle *h, FmShape &S) {
+  const cudaError_t e = shape_of(h, fm_reg_kernel<FL, N>, reg_warp_bytes(N), kFW, S);
+  if (e != cudaSuccess) return e;
+  S.warps = kFW;
+  int c = 0;
+  const cudaError_t e2 = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, fm_reg_kernel<FL, N>, kFT, S.warp_bytes * kFW);
+  S.per_sm = std::max(c, 1);
+  return e2;
+}
+
+// shape of variant `var` (a mode, or kVarReg*) for instances of up to nmax spins;
+// staged: with the spins' records in shared memory (gain keys)
+cudaError_t variant_shape(const ising_handle *h, FmBufs &B, int var, int nmax, FmShape &S, bool staged = false) {
+  const std::pair<int, int> at{var + (staged ? kVarStaged : 0), nmax};
+  const size_t stage = staged ? (size_t)nmax * B.ent_stride * sizeof(int4) : 0;
+  const auto it = B.shapes.find(at);
+  if (it != B.shapes.end()) {
+    S = it->second;
+    return cudaSuccess;
+  }
+  const bool fl = h->dtype == ISING_F32, f64 = h->dtype == ISING_F64;
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(fm_reg_kernel<FL, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-      cudaSuccess)
-    return e;
-  per_sm = 0;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fm_reg_kernel<FL, S>, kFT, smem)) !=
-      cudaSuccess)
-    return e;
-  per_sm = std::max(per_sm, 1);
-  return cudaSuccess;
+  switch (var) {
+    case kKeyExact:
+    case kKeyWide:
+    case kKeyWide64:
+      e = shape_of(h, key_kernel(var, nmax), key_warp_bytes(nmax, var - kKeyExact) + stage, kFW, S);
+      break;
+    case kVarReg8: e = fl ? fm_reg_shape<true, 8>(h, S) : fm_reg_shape<false, 8>(h, S); break;
+    case kVarReg16: e = fl ? fm_reg_shape<true, 16>(h, S) : fm_reg_shape<false, 16>(h, S); break;
+    // int8 couplings are always exact in one unit (kFx); FP64 couplings take the FP64 form
+    default:
+      e = f64 ? fm_shape<kFp64, 2>(h, nmax, S)
+          : !fl ? fm_shape<kFx, 0>(h, nmax, S)
+          : var == kFx ? fm_shape<kFx, 1>(h, nmax, S)
+          : var == kFxSpin ? fm_shape<kFxSpin, 1>(h, nmax, S)
+                           : fm_shape<kFp64, 1>(h, nmax, S);
+      break;
+  }
+  if (e == cudaSuccess) B.shapes[at] = S;
+  return e;
+}
+
+// The change entries of every instance that can take the gain keys, built by
+// the first call; without room for them the other kernels serve.
+cudaError_t build_entries(ising_handle *h, FmBufs &B, cudaStream_t s) {
+  if (B.ent_stride >= 0) return cudaSuccess;
+  int most = -1;
+  for (const InstDesc &D : h->inst)
+    if (D.fbits >= 0) most = std::max(most, D.fm_ent);
+  B.ent_stride = 0;
+  if (most < 0) return cudaSuccess;
+  const int stride = std::max(4, (most + 3) / 4 * 4);
+  if (cudaMalloc((void **)&B.ent, (size_t)h->total_spins * stride * sizeof(int4)) != cudaSuccess) {
+    cudaGetLastError();
+    B.ent = nullptr;
+    return cudaSuccess;
+  }
+  B.ent_stride = stride;
+  fm_entries_kernel<<<h->n_inst, 256, 0, s>>>(h->graph(), B.ent, stride);
+  h->launches += 1;
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -928,9 +1418,20 @@ cudaError_t launch_fm(ising_handle *h, int32_t R, const ising_fm_params *fp, int
   if (n_items > 0x7fffffff) return cudaErrorInvalidValue;
   FmBufs &B = family_state<FmBufs>(h->fm_st);
   cudaError_t e;
-  // groups: one-unit integer instances, per-spin-unit ones, then FP64;
-  // within each, size classes (0, 256], (256, 512], ... (2048, 4096],
-  // largest first
+  const bool fl = h->dtype == ISING_F32, f64 = h->dtype == ISING_F64;
+  if (!f64 && (e = build_entries(h, B, s)) != cudaSuccess) return e;
+  // The form of an instance: gain keys where its fields are integers of few
+  // enough bits in one unit (the energies then FP64 unless those are too) and
+  // its changes fit the entries; else the arithmetic's general kernel.
+  auto form = [&](const InstDesc &D) -> int {
+    if (B.ent_stride > 0 && D.fm_ent >= 0 && D.fbits >= 0 && D.fx53 > 0) {
+      if (D.fbits <= kGq && D.fx53 == 1) return kKeyExact;
+      if (D.fbits <= kWide64Bits) return D.fbits <= kWideBits ? kKeyWide : kKeyWide64;
+    }
+    return D.fx53;
+  };
+  // groups by form; within each, size classes (0, 256], (256, 512], ...
+  // (2048, 4096], largest first
   auto cls = [](int n) {
     int c = 0;
     while (c < 4 && n > (256 << c)) ++c;
@@ -940,8 +1441,8 @@ cudaError_t launch_fm(ising_handle *h, int32_t R, const ising_fm_params *fp, int
   for (int32_t b = 0; b < h->n_inst; ++b) ord[b] = b;
   std::stable_sort(ord.begin(), ord.end(), [&](int a, int c) {
     const InstDesc &x = h->inst[a], &y = h->inst[c];
-    auto rank = [](int m) { return m == kFx ? 0 : (m == kFxSpin ? 1 : 2); };
-    if (x.fx53 != y.fx53) return rank(x.fx53) < rank(y.fx53);
+    const int fx = form(x), fy = form(y);
+    if (fx != fy) return fx > fy;
     return x.n > y.n;
   });
   std::vector<int2> items;
@@ -949,11 +1450,12 @@ cudaError_t launch_fm(ising_handle *h, int32_t R, const ising_fm_params *fp, int
   items.reserve((size_t)n_items);
   for (int32_t b : ord) {
     const InstDesc &D = h->inst[b];
-    const int mode = D.fx53;
+    const int mode = form(D);
     if (parts.empty() || parts.back().mode != mode || cls(parts.back().nmax) != cls(D.n))
-      parts.push_back({mode, D.n, (int64_t)items.size(), 0});
+      parts.push_back({mode, D.n, (int64_t)items.size(), 0, true});
     for (int32_t r = 0; r < R; ++r) items.push_back(make_int2(b, r));
     parts.back().count += R;
+    parts.back().one_unit = parts.back().one_unit && D.fx53 == 1;
   }
   if ((e = grow(B.items, B.items_bytes, (size_t)n_items * sizeof(int2))) != cudaSuccess) return e;
   if ((e = grow(B.queues, B.queues_bytes, parts.size() * sizeof(int32_t))) != cudaSuccess) return e;
@@ -964,14 +1466,9 @@ cudaError_t launch_fm(ising_handle *h, int32_t R, const ising_fm_params *fp, int
 
   // Starts run in parallel (one per warp, the best chosen afterwards) when
   // the searches alone would leave the GPU underfilled.
-  int warps0 = 0, per_sm0 = 0;
-  size_t smem0 = 0;
-  const bool fl = h->dtype == ISING_F32, f64 = h->dtype == ISING_F64;
-  if ((e = f64  ? fm_shape<kFp64, 2>(h, h->nmax, warps0, smem0, per_sm0)
-           : fl ? fm_shape<kFx, 1>(h, h->nmax, warps0, smem0, per_sm0)
-                : fm_shape<kFx, 0>(h, h->nmax, warps0, smem0, per_sm0)) != cudaSuccess)
-    return e;
-  const int64_t resident = (int64_t)h->sm_count * per_sm0 * warps0;
+  FmShape S0;
+  if ((e = variant_shape(h, B, parts[0].mode, h->nmax, S0)) != cudaSuccess) return e;
+  const int64_t resident = (int64_t)h->sm_count * S0.per_sm * S0.warps;
   const size_t sp_bytes = ((size_t)R * restarts * h->total_spins + 15) & ~(size_t)15;
   const size_t e_bytes = (size_t)n_items * restarts * sizeof(double);
   const size_t p_bytes = (size_t)n_items * restarts * sizeof(int32_t);
@@ -1005,39 +1502,51 @@ cudaError_t launch_fm(ising_handle *h, int32_t R, const ising_fm_params *fp, int
   if (fan) {
     if ((e = ensure_side(B)) != cudaSuccess) return e;
     if ((e = cudaEventRecord(B.fork, s)) != cudaSuccess) return e;
-    for (cudaStream_t st : B.side)
-      if ((e = cudaStreamWaitEvent(st, B.fork, 0)) != cudaSuccess) return e;
   }
+  bool forked[kSideStreams] = {};
   cudaError_t le = cudaSuccess;
+  int used[kClasses] = {0, 0, 0, 0, 0};  // groups launched per size class
   for (size_t o = 0; o < order.size() && le == cudaSuccess; ++o) {
     const size_t q = order[o];
     const FmPart &P = parts[q];
-    cudaStream_t ls = fan ? B.side[o % B.side.size()] : s;
+    const int pc = cls(P.nmax);
+    cudaStream_t ls = s;
+    if (fan) {
+      const int j = (kClasses - 1 - pc) * kClassStreams + used[pc]++ % kClassStreams;
+      ls = B.side[j];
+      if (!forked[j] && (le = cudaStreamWaitEvent(ls, B.fork, 0)) != cudaSuccess) break;
+      forked[j] = true;
+    }
     const int nmax = P.nmax;  // the group's largest instance
-    int warps = 0, per_sm = 0;
-    size_t smem = 0;
-    // Small one-unit instances take the register kernel when the group's
-    // searches fit in one wave of it (latency-bound); larger groups keep the
-    // shared-memory kernel, which holds more searches per SM.
     const int64_t work = split ? P.count * restarts : P.count;
     const bool reg8 = nmax <= 256;
-    bool reg = P.mode == kFx && nmax <= kRegMaxSpins && fp->reg_kernel >= 0;
+    FmShape S;
+    // Small one-unit instances without gain keys take the register kernel when
+    // the group's searches fit in one wave of it.
+    bool reg = P.one_unit && nmax <= kRegMaxSpins && (fp->reg_kernel == 1 || (fp->reg_kernel == 0 && P.mode == kFx));
     if (reg) {
-      le = fl ? (reg8 ? fm_reg_shape<true, 8>(h, warps, smem, per_sm) : fm_reg_shape<true, 16>(h, warps, smem, per_sm))
-              : (reg8 ? fm_reg_shape<false, 8>(h, warps, smem, per_sm)
-                      : fm_reg_shape<false, 16>(h, warps, smem, per_sm));
-      if (le != cudaSuccess) break;
-      reg = work <= (int64_t)h->sm_count * per_sm * warps || fp->reg_kernel == 1;
+      if ((le = variant_shape(h, B, reg8 ? kVarReg8 : kVarReg16, reg8 ? 256 : kRegMaxSpins, S)) != cudaSuccess) break;
+      reg = work <= (int64_t)h->sm_count * S.per_sm * S.warps || fp->reg_kernel == 1;
     }
-    // int8 couplings are always exact in one unit (mode kFx); FP64 couplings
-    // take the FP64 form
-    if (!reg)
-      le = f64 ? fm_shape<kFp64, 2>(h, nmax, warps, smem, per_sm)
-           : !fl ? fm_shape<kFx, 0>(h, nmax, warps, smem, per_sm)
-           : P.mode == kFx ? fm_shape<kFx, 1>(h, nmax, warps, smem, per_sm)
-           : P.mode == kFxSpin ? fm_shape<kFxSpin, 1>(h, nmax, warps, smem, per_sm)
-                               : fm_shape<kFp64, 1>(h, nmax, warps, smem, per_sm);
-    if (le != cudaSuccess) break;
+    if (!reg && (le = variant_shape(h, B, P.mode, nmax, S)) != cudaSuccess) break;
+    // gain keys: the records in shared memory when every search of the call is
+    // then still resident (a record read is on each move's chain)
+    bool staged = false;
+    if (!reg && !fan && P.mode >= kKeyExact) {
+      FmShape T;
+      if ((size_t)nmax * B.ent_stride * sizeof(int4) <= kStageMax) {
+        if ((le = variant_shape(h, B, P.mode, nmax, T, true)) != cudaSuccess) break;
+        staged = work <= (int64_t)h->sm_count * T.one_warp_per_sm;
+        if (staged) S = T;
+      }
+    }
+    // few searches: one per CTA, so that they spread over the SMs
+    if (!reg && work <= (int64_t)h->sm_count * S.one_warp_per_sm) {
+      S.warps = 1;
+      S.per_sm = S.one_warp_per_sm;
+    }
+    const int warps = S.warps, per_sm = S.per_sm;
+    const size_t smem = S.warp_bytes * warps;
     FmArgs A;
     A.g = h->graph();
     A.n_work = (int32_t)(split ? P.count * restarts : P.count);
@@ -1062,6 +1571,8 @@ cudaError_t launch_fm(ising_handle *h, int32_t R, const ising_fm_params *fp, int
       fm_reg_kernel<false, 8><<<grid, warps * 32, smem, ls>>>(A);
     else if (reg)
       fm_reg_kernel<false, 16><<<grid, warps * 32, smem, ls>>>(A);
+    else if (P.mode >= kKeyExact)
+      key_kernel(P.mode, nmax)<<<grid, warps * 32, smem, ls>>>(A, nmax, B.ent, B.ent_stride, h->fm_rounds, staged ? 1 : 0);
     else if (f64)
       fm_kernel<kFp64, 2><<<grid, warps * 32, smem, ls>>>(A, nmax);
     else if (!fl)
@@ -1075,8 +1586,9 @@ cudaError_t launch_fm(ising_handle *h, int32_t R, const ising_fm_params *fp, int
     h->launches += 1;
     le = cudaGetLastError();
   }
-  if (fan)  // join every side stream back into s, also after a failed launch
+  if (fan)  // join every used side stream back into s, also after a failed launch
     for (size_t j = 0; j < B.side.size(); ++j) {
+      if (!forked[j]) continue;
       cudaError_t je = cudaEventRecord(B.join[j], B.side[j]);
       if (je == cudaSuccess) je = cudaStreamWaitEvent(s, B.join[j], 0);
       if (le == cudaSuccess) le = je;
@@ -1096,6 +1608,7 @@ void fm_free(ising_handle *h) {
   cudaFree(B.items);
   cudaFree(B.queues);
   cudaFree(B.scratch);
+  cudaFree(B.ent);
   for (cudaStream_t st : B.side) cudaStreamDestroy(st);
   for (cudaEvent_t ev : B.join) cudaEventDestroy(ev);
   if (B.fork) cudaEventDestroy(B.fork);

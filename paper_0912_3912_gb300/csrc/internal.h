@@ -45,6 +45,16 @@ struct InstDesc {
   // Bits of the largest energy term in fixed-point units: |term| < 2^ebits
   // (int8: 7; FP32 with ebase >= 0: 24 + emax - ebase; else -1).
   int32_t ebits;
+  // Pass-based search with gain keys (fm.cu): change entries of the spin with
+  // the most (its couplings, one per 2-member and two per 3-member hyper-edge),
+  // or -1 when a hyper-edge has more members, a spin more than 31 entries or one
+  // target more than 15 times.
+  int32_t fm_ent;
+  // Bits of the largest possible |field| in units (int8: 1; FP32: 2^(funit - 150),
+  // the largest power of two that divides every term), set with fm_ent >= 0 and,
+  // for FP32, ebase >= 0; else -1.
+  int32_t fbits;
+  int32_t funit;
 };
 
 // Everything a kernel needs to read an instance set.
@@ -82,6 +92,7 @@ struct DevGraph {
   const int16_t *runit;
   int64_t nsp;              // total spins (stride of Jpos)
   int32_t dtype;            // ISING_I8 / ISING_F32
+  int32_t hyper;            // some instance has hyper-edges
 };
 
 // Per-call arguments of the tile kernels (kept in device memory so that a
@@ -128,6 +139,7 @@ struct ising_handle {
   bool dense = false;       // instances given as dense matrices
   bool msc_ok = false;      // every coupling +/-1, every field in {-1,0,+1}, no hyper-edges
   bool has_hyper = false;
+  int32_t fm_rounds = 1;  // most change entries of one spin with one target (InstDesc::fm_ent >= 0)
   int32_t nmax = 0;
   int64_t total_spins = 0, total_nnz = 0, total_edges = 0, total_members = 0;
   int64_t abs_energy_bound = 0;  // sum |J| + |h| + |J_e| (integer instances)

@@ -103,3 +103,53 @@ def test_energy_wide_exponent_range():
     E = h.energy(torch.from_numpy(spins).cuda(), R)[0].cpu().numpy()
     np.testing.assert_allclose(E, oracle.energies(inst, spins), rtol=1e-12)
     h.close()
+
+
+# Pass-based search with gain keys, move for move against the oracle's heap:
+# one word per lane and whole trees (1 to 4096 spins, both sides of the flat
+# layout's 512 and of each number of reads per lane), records of 31 entries (one
+# more goes to the general kernel), hyper-edges of 2 and 3 members over existing
+# pairs (targets that occur twice), values of one, two and three words, and FP32
+# couplings of equal magnitudes (every move tied).
+from test_gpu_fm import _compare as _compare_fm  # noqa: E402
+
+
+def _fm_graph(kind, n):
+    if kind == "pm1":
+        return W.random_graph(n, 4.0, n, dtype="i8", n_hyper=n // 6, hyper_order=(2, 3), int_range=1)
+    if kind == "int":
+        return W.random_graph(n, 6.0, n, dtype="i8", n_hyper=n // 3, hyper_order=(2, 3), int_range=100)
+    g = W.random_graph(n, 4.0, n, dtype="f32", n_hyper=n // 3, hyper_order=(2, 3))
+    if kind == "ties":
+        for k in ("J", "h", "hyper_J"):
+            v = getattr(g, k)
+            if v is not None:
+                setattr(g, k, (np.sign(v) * (1 + np.arange(len(v)) % 2 if k == "h" else 1)).astype(np.float32))
+    if kind == "halves":  # equal magnitudes and one tiny field: ties decided by low bits
+        g.J = (np.sign(g.J) * np.float32(0.75)).astype(np.float32)
+        g.h = np.full(n, 0.0, np.float32)
+        g.h[0] = np.float32(2.0 ** -26)
+    return _exp_spread(g, -14, 3) if kind == "wide" else g
+
+
+@pytest.mark.parametrize("n", [1, 2, 33, 127, 129, 256, 257, 512, 513, 1024, 1025, 2049])
+@pytest.mark.parametrize("kind", ["pm1", "int", "gauss", "ties", "halves", "wide"])
+def test_fm_gain_keys(kind, n):
+    _compare_fm([_fm_graph(kind, n)], 5, 1, kind in ("pm1", "int"))
+
+
+def test_fm_gain_keys_largest_instance_and_mixed_batch():
+    insts = [_fm_graph("gauss", 4096), _fm_graph("wide", 700), _fm_graph("halves", 300), _fm_graph("gauss", 90)]
+    _compare_fm(insts, 3, 2, False)
+
+
+@pytest.mark.parametrize("degree", [31, 32])
+def test_fm_gain_keys_widest_record(degree):
+    n = 64
+    u, v = np.triu_indices(n, 1)
+    keep = ((v - u) % n <= (degree // 2)) | ((u - v) % n <= (degree // 2)) | ((v - u == n // 2) & (degree % 2 == 1))
+    u, v = u[keep], v[keep]
+    w = np.random.default_rng(3).standard_normal(len(u)).astype(np.float32)
+    rp, col, J = W.csr_from_edges(n, u, v, w, "f32")
+    assert np.diff(rp).max() == degree
+    _compare_fm([W.Instance(n=n, row_ptr=rp, col=col, J=J, dtype="f32")], 6, 2, False)
