@@ -16,7 +16,7 @@ namespace isg {
 cudaError_t launch_plain(ising_handle *h, const ising_search_params *p, int32_t R, int8_t *spins, double *E,
                          int32_t *E32, int32_t *minima, const uint64_t *seeds_host, cudaStream_t s);
 cudaError_t launch_sweep(ising_handle *h, const ising_search_params *p, int32_t R, int8_t *spins, double *E,
-                         int32_t *E32, int32_t *minima, const uint64_t *seeds_host, cudaStream_t s);
+                         int32_t *E32, int32_t *minima, cudaStream_t s);
 cudaError_t launch_dense(ising_handle *h, const ising_search_params *p, int32_t R, int8_t *spins, double *E,
                          int32_t *E32, int32_t *minima, const uint64_t *seeds_host, cudaStream_t s);
 bool dense_supported(const ising_handle *h, int32_t R);
@@ -448,10 +448,29 @@ ising_status validate_params(const ising_search_params *p) {
   return ISING_OK;
 }
 
-constexpr int kTileSmemLimit = 200 * 1024;
-
 bool tile_fits(const ising_handle *h, int mode) {
-  return tile_smem_bytes(mode, h->nmax) <= (size_t)kTileSmemLimit;
+  return tile_smem_bytes(mode, h->nmax) <= tile_smem_limit();
+}
+
+// Few large instances on lanes (no multi-spin coding): whether a launch per
+// colour class over the whole GPU beats one CTA per tile and segment, by their
+// times per sweep.  A tile takes about 10 ns per spin (1024 threads) and wave of
+// its units; the sweep family takes its instances and descents one after another,
+// 3.1 us per class launch, 0.35 ns per spin and replica group, and once for a new
+// handle the capture of its graph (about 16 us a sweep over a search's 25).
+// Measured (tile / sweep, us a call): degree-5 graphs of 3,000 spins 975 / 1468, of
+// 6,000 1774 / 1501, of 12,000 3429 / 1597, of 20,000 5690 / 1867 (20 replicas, 2
+// descents); 128 x 128 Gaussian lattices, 4 descents: 32 replicas 2941 / 907, 256
+// replicas 2989 / 3252.
+bool sweep_is_faster(const ising_handle *h, int32_t R, const ising_search_params *p) {
+  const int32_t groups = (R + 31) / 32;
+  if (groups > 32 || p->schedule == ISING_SCHED_SEQUENTIAL) return false;
+  const double descents = p->sweep_budget > 0 ? 1 : p->restarts;
+  const double waves = std::max(1.0, std::ceil((double)h->n_inst * groups * descents / h->sm_count));
+  const double tile = waves * 10e-9 * h->nmax;
+  double sweep = 16e-6;
+  for (const InstDesc &I : h->inst) sweep += descents * ((I.ncls + 1.5) * 3.1e-6 + 0.35e-9 * I.n * groups);
+  return sweep < tile;
 }
 
 // Kernel family for these arguments (ISING_KERNEL_AUTO resolved), or negative status.
@@ -464,8 +483,8 @@ int32_t resolve_kernel(ising_handle *h, int32_t R, const ising_search_params *p)
     if (it != h->tuned.end()) return it->second;
     if (h->dense && dense_supported(h, R)) return ISING_KERNEL_DENSE_TC;
     if (h->msc_ok && tile_fits(h, 2)) return ISING_KERNEL_MSC;
-    if (tile_fits(h, h->dtype == ISING_F32 ? 1 : 0)) return ISING_KERNEL_TILE;
-    return ISING_KERNEL_SWEEP;
+    if (!tile_fits(h, h->dtype == ISING_F32 ? 1 : 0)) return ISING_KERNEL_SWEEP;
+    return sweep_is_faster(h, R, p) ? ISING_KERNEL_SWEEP : ISING_KERNEL_TILE;
   }
   switch (k) {
     case ISING_KERNEL_TILE:
@@ -508,6 +527,63 @@ int msc_cluster_size(const ising_handle *h, int32_t R, const ising_search_params
     if (ok) return P;
   }
   return 0;
+}
+
+// CTA size and segments of the tile kernels for these arguments, null when no
+// CTA fits.  A descent's time in one CTA goes like a constant (barriers, round
+// trips) plus the steps the largest class takes: a warp per spin in the lane
+// modes (constant 6 steps), a thread per spin in the multi-spin-coded ones (30).
+// The tiles' descents (without a budget each descent is a unit of its own) run in
+// waves over the CTA slots; uneven instances fill the waves, a last wave of equal
+// ones does not.  Measured, us a call at 256 / 512 / 1024 threads: one cell grid
+// batch of 64 tiles 1744 / 988 / 680, of 800 2259 / 1563 / 1747, of 4096
+// 7609 / 7676 / 8626; 6,000 spins of degree 5, 20 replicas, 2 descents
+// 5077 / 2712 / 1774 (10046 in one segment); 31^3 +/-J, 1024 replicas, 10 descents
+// 2499 / 1572 / 1279; 16 x 16 +/-J, 64 replicas, 10 descents 52 / 42 / 44 (125 in
+// one segment).
+const TilePlan *tile_plan(ising_handle *h, int mode, int32_t R, const ising_search_params *p) {
+  TilePlan &T = h->tile_plan_cache;
+  const int32_t parallel = p->sweep_budget > 0 ? 1 : p->restarts;
+  if (T.mode == mode && T.R == R && T.parallel == parallel) return T.slots > 0 ? &T : nullptr;
+  T = TilePlan();
+  T.mode = mode;
+  T.R = R;
+  T.parallel = parallel;
+  const int64_t tiles = (int64_t)h->n_inst * ((R + 31) / 32);
+  double weight = 0.0;  // of all units, in units of the largest instance
+  int32_t ncls = 1, nmin = h->nmax;
+  for (const InstDesc &I : h->inst) {
+    weight += (double)I.n / h->nmax;
+    nmin = std::min(nmin, I.n);
+    if (I.n == h->nmax) ncls = std::max(ncls, I.ncls);
+  }
+  weight *= (double)((R + 31) / 32) * parallel;
+  double best = 0.0;
+  for (int threads : {256, 512, 1024}) {
+    // FP32 lanes: fields in shared memory for every instance that fits, within a
+    // budget that lets four CTAs share an SM (one CTA of 1024 threads with four
+    // times as much, and so less L1, was 5 % slower)
+    int fsm_cap = mode == 1 ? tile_fsm_cap(h->nmax, (size_t)48 * 1024) : 0;
+    if (nmin > fsm_cap) fsm_cap = 0;
+    size_t smem = tile_smem_bytes(mode, h->nmax);
+    if (fsm_cap > 0) smem = (smem + 15) / 16 * 16 + (size_t)fsm_cap * 128;
+    const int64_t slots = (int64_t)tile_max_ctas_per_sm(mode, threads, smem) * h->sm_count;
+    if (slots < 1) continue;
+    const double per_step = mode >= 2 ? 2.0 * threads : (double)ncls * threads / 32;
+    const double unit = (mode >= 2 ? 30.0 : 6.0) + std::ceil(h->nmax / per_step);
+    double waves = std::max(1.0, weight / (double)slots);
+    if (nmin == h->nmax && waves < 2.0) waves = std::ceil(waves);
+    if (T.slots == 0 || unit * waves <= best) {  // (ties: the larger CTA)
+      best = unit * waves;
+      T.threads = threads;
+      T.slots = slots;
+      T.fsm_cap = fsm_cap;
+      T.smem = smem;
+    }
+  }
+  if (T.slots == 0) return nullptr;
+  T.segs = (int32_t)std::max<int64_t>(1, std::min<int64_t>(parallel, T.slots / tiles));
+  return &T;
 }
 
 ising_status run_tile(ising_handle *h, int mode, int32_t R, const ising_search_params *p, int8_t *spins,
@@ -560,19 +636,28 @@ ising_status run_tile(ising_handle *h, int mode, int32_t R, const ising_search_p
     h->launches += 1;
     return ISING_OK;
   }
-  // FP32 lanes: fields in shared memory for every instance that fits, within a
-  // budget that still lets two CTAs share an SM (the kernel is built for two)
-  constexpr size_t kFsmBudget = 48 * 1024;
-  const int fsm_cap = mode == 1 ? tile_fsm_cap(h->nmax, kFsmBudget) : 0;
-  const size_t smem = mode == 1 && fsm_cap > 0 ? (tile_smem_bytes(mode, h->nmax) + 15) / 16 * 16 + (size_t)fsm_cap * 128
-                                              : tile_smem_bytes(mode, h->nmax);
-  int per_sm = tile_max_ctas_per_sm(mode, smem);
-  if (per_sm < 1) return ISING_ERR_UNSUPPORTED;
-  const int grid = std::min<int64_t>(h->n_tiles, (int64_t)per_sm * h->sm_count);
-  const size_t f_bytes = mode == 1 ? (size_t)grid * h->nmax * 32 * sizeof(float) : 0;
-  const size_t bw_bytes = (size_t)grid * h->nmax * sizeof(uint32_t);
-  ising_status st = ensure_scratch(h, f_bytes + bw_bytes + 256);
+  const TilePlan *plan = tile_plan(h, mode, R, p);
+  if (!plan) return ISING_ERR_UNSUPPORTED;
+  const int threads = plan->threads, segs = plan->segs, fsm_cap = plan->fsm_cap;
+  const size_t smem = plan->smem;
+  const int64_t work = (int64_t)h->n_tiles * segs;
+  const int grid = (int)std::min<int64_t>(work, plan->slots);
+  auto up256 = [](size_t bytes) { return (bytes + 255) / 256 * 256; };
+  const size_t f_bytes = mode == 1 ? up256((size_t)grid * h->nmax * 32 * sizeof(float)) : 0;
+  const size_t bw_bytes = up256((size_t)grid * h->nmax * sizeof(uint32_t));
+  const size_t seg_bytes = segs > 1 ? up256((size_t)work * h->nmax * sizeof(uint32_t)) : 0;
+  const size_t lane_bytes = segs > 1 ? up256((size_t)work * 32 * sizeof(double)) : 0;
+  ising_status st = ensure_scratch(h, f_bytes + bw_bytes + seg_bytes + 2 * lane_bytes + 256);
   if (st != ISING_OK) return st;
+  const int32_t counters = segs > 1 ? h->n_tiles : 0;  // segments ended, per tile
+  if (counters > h->queue_tiles) {
+    int32_t *q = nullptr;
+    if (cudaMalloc(&q, sizeof(int32_t) * (4 + (size_t)counters)) != cudaSuccess) return ISING_ERR_OOM;
+    cudaFree(h->d_queue);
+    h->d_queue = q;
+    h->queue_tiles = counters;
+    h->tile_exec_key[0] = -1;  // (captured against the old buffer)
+  }
   TileArgs a;
   a.g = h->graph();
   a.tiles = h->d_tiles;
@@ -587,7 +672,12 @@ ising_status run_tile(ising_handle *h, int mode, int32_t R, const ising_search_p
   a.seeds = h->d_seeds;
   a.F = mode == 1 ? (float *)h->d_scratch : nullptr;
   a.fsm_cap = fsm_cap;
-  a.bw = (uint32_t *)((char *)h->d_scratch + ((f_bytes + 255) / 256) * 256);
+  char *scratch = (char *)h->d_scratch + f_bytes;
+  a.bw = (uint32_t *)scratch;
+  a.segs = segs;
+  a.seg_words = (uint32_t *)(scratch + bw_bytes);
+  a.seg_best = (double *)(scratch + bw_bytes + seg_bytes);
+  a.seg_minima = (int32_t *)(scratch + bw_bytes + seg_bytes + lane_bytes);
   a.nmax = h->nmax;
   a.spins = spins;
   a.energy = E;
@@ -596,9 +686,10 @@ ising_status run_tile(ising_handle *h, int mode, int32_t R, const ising_search_p
   a.stats = h->d_stats;
   CUDA_OK(cudaMemcpyAsync(h->d_tile_args, &a, sizeof(a), cudaMemcpyHostToDevice, s));
   // The launch sequence reads its arguments from device memory, so one captured
-  // graph serves every call with the same mode, grid and shared memory.
+  // graph serves every call with the same mode, grid, shared memory, threads and
+  // counters.
   if (!h->tile_exec || h->tile_exec_key[0] != mode || h->tile_exec_key[1] != grid ||
-      h->tile_exec_key[2] != (int32_t)smem) {
+      h->tile_exec_key[2] != (int32_t)smem || h->tile_exec_key[3] != threads || h->tile_exec_key[4] != counters) {
     if (h->tile_exec) cudaGraphExecDestroy(h->tile_exec);
     h->tile_exec = nullptr;
     cudaStream_t cs;
@@ -606,8 +697,8 @@ ising_status run_tile(ising_handle *h, int mode, int32_t R, const ising_search_p
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-      cudaMemsetAsync(h->d_queue, 0, sizeof(int32_t), cs);
-      launch_tile(h, mode, grid, smem, cs);
+      cudaMemsetAsync(h->d_queue, 0, sizeof(int32_t) * (4 + (size_t)counters), cs);
+      launch_tile(h, mode, threads, segs > 1, grid, smem, cs);
       e = cudaStreamEndCapture(cs, &g);
     }
     if (e == cudaSuccess) e = cudaGraphInstantiate(&h->tile_exec, g, 0);
@@ -620,6 +711,8 @@ ising_status run_tile(ising_handle *h, int mode, int32_t R, const ising_search_p
     h->tile_exec_key[0] = mode;
     h->tile_exec_key[1] = grid;
     h->tile_exec_key[2] = (int32_t)smem;
+    h->tile_exec_key[3] = threads;
+    h->tile_exec_key[4] = counters;
   }
   kt_begin(h, "tile_kernel", s);
   CUDA_OK(cudaGraphLaunch(h->tile_exec, s));
@@ -1062,7 +1155,7 @@ ising_status ising_local_search(ising_handle *h, const uint64_t *seeds, int32_t 
                       energy_dev, energy_i32_dev, minima_dev, stream);
         break;
       case ISING_KERNEL_SWEEP:
-        if (launch_sweep(h, p, replicas, spins_dev, energy_dev, energy_i32_dev, minima_dev, seeds, stream) !=
+        if (launch_sweep(h, p, replicas, spins_dev, energy_dev, energy_i32_dev, minima_dev, stream) !=
             cudaSuccess)
           st = ISING_ERR_CUDA;
         break;

@@ -16,7 +16,6 @@
 
 namespace isg {
 
-constexpr int kTileThreads = 256;   // threads per tile CTA (8 warps)
 constexpr int kSweepThreads = 256;  // threads per CTA of the large-instance sweeps
 
 // One instance as the kernels see it.  Spin, edge and class arrays of all
@@ -101,7 +100,12 @@ struct TileArgs {
   DevGraph g;
   const int2 *tiles;        // (instance, 32-replica group), largest instances first
   int32_t n_tiles;
-  int32_t *queue;           // work-queue counter, zeroed before each launch
+  int32_t *queue;           // work-queue counter and, from queue + 4, segments ended per
+                            // tile: zeroed before each launch
+  int32_t segs;             // segments of consecutive descents per tile (1: the whole tile)
+  uint32_t *seg_words;      // [n_tiles * segs][nmax] result words of the segments
+  double *seg_best;         // [n_tiles * segs][32]
+  int32_t *seg_minima;      // [n_tiles * segs][32]
   int32_t R, max_sweeps, restarts, budget, refresh, sequential;
   const uint64_t *seeds;    // [n_inst]
   float *F;                 // [grid][nmax][32] FP32 fields (float lane path)
@@ -120,6 +124,14 @@ struct TileArgs {
 // family's *_free function releases its resources at ising_destroy.
 struct FamilyState {
   virtual ~FamilyState() = default;
+};
+
+// Launch shape of the tile kernels (tile_plan in api.cu).
+struct TilePlan {
+  int32_t mode = -1, R = 0, parallel = 0;  // what it was made for
+  int32_t threads = 0, segs = 1, fsm_cap = 0;
+  int64_t slots = 0;  // resident CTAs, 0: none fits
+  size_t smem = 0;
 };
 
 struct PlanKey {
@@ -177,6 +189,7 @@ struct ising_handle {
   uint64_t *d_seeds = nullptr;
   unsigned long long *d_stats = nullptr;
   int32_t *d_queue = nullptr;
+  int32_t queue_tiles = 0;  // tiles the queue buffer has counters for
   int2 *d_tiles = nullptr;
   int32_t tiles_R = -1;
   int32_t n_tiles = 0;
@@ -196,7 +209,8 @@ struct ising_handle {
   // the tile path's launch sequence (queue reset + persistent kernel) captured
   // once per (mode, grid, shared memory) and replayed
   cudaGraphExec_t tile_exec = nullptr;
-  int32_t tile_exec_key[3] = {-1, -1, -1};
+  isg::TilePlan tile_plan_cache;
+  int32_t tile_exec_key[5] = {-1, -1, -1, -1, -1};
   ising_status latched = ISING_OK;
   uint64_t launches = 0;  // kernel launches enqueued by the current call
   // Optional device timing (ising_set_timing): CUDA events recorded on the
@@ -226,10 +240,11 @@ T &family_state(std::unique_ptr<FamilyState> &slot) {
 void kt_begin(ising_handle *h, const char *name, cudaStream_t s);
 void kt_end(ising_handle *h, cudaStream_t s);
 // launchers (tile.cu / energy.cu / plain.cu / sweep.cu / dense.cu)
-cudaError_t launch_tile(ising_handle *h, int mode, int grid, size_t smem, cudaStream_t s);
+cudaError_t launch_tile(ising_handle *h, int mode, int threads, bool seg, int grid, size_t smem, cudaStream_t s);
 size_t tile_smem_bytes(int mode, int nmax);
+size_t tile_smem_limit();  // dynamic shared memory of a tile CTA at most
 int tile_fsm_cap(int nmax, size_t budget);
-int tile_max_ctas_per_sm(int mode, size_t smem);
+int tile_max_ctas_per_sm(int mode, int threads, size_t smem);
 cudaError_t launch_energy(ising_handle *h, const int8_t *spins, int32_t R, double *E,
                           int32_t *E32, cudaStream_t s);
 void energy_plan_free(ising_handle *h);

@@ -47,7 +47,7 @@ struct SweepArgs {
   InstDesc I;
   int32_t b, R, G, LPS;
   int32_t max_sweeps, restarts, budget, refresh, sequential, lattice;
-  uint64_t seed;
+  const uint64_t *seeds;  // device [instances] (a captured chunk serves every seed)
   uint32_t *sw, *fm, *bw;
   uint32_t *pend;  // [g][n]: lanes in which some neighbour flipped since the spin's last visit
   // Parity-coloured lattices with an even side (class position = site >> 1):
@@ -327,13 +327,22 @@ __global__ void __launch_bounds__(kST, (MODE == 2 && LAT) ? 8 : kVisitCtasPerSm)
     // replicas each), with all loads of one visit independent of each other.
     constexpr int SPW = 32 / LPS;
     const int sub = lane / LPS, ln = lane % LPS;
-    const int nwarps = gridDim.x * (blockDim.x >> 5);
-    const int wid = blockIdx.x * (blockDim.x >> 5) + (tid >> 5);
+    // General graphs: the groups are spread over slices of the warps while every
+    // slice still has a warp for each step of the class.
+    int nwarps = gridDim.x * (blockDim.x >> 5), wid = blockIdx.x * (blockDim.x >> 5) + (tid >> 5);
+    int slices = 1, slice = 0;
+    if constexpr (!LAT) {
+      while (2 * slices <= A.G && cs <= nwarps / (2 * slices) * SPW) slices *= 2;
+      slice = wid % slices;
+      wid /= slices;
+      nwarps /= slices;
+      if (wid >= nwarps) slice = A.G;  // (a remainder of warps stays idle)
+    }
     // class positions per warp step (not the FP32 lattice path): 32, fewer where
     // the class would leave resident warps without work
     int pw = 32;
     while (pw > SPW && cs < nwarps * pw) pw >>= 1;
-    for (int g = 0; g < A.G; ++g) {
+    for (int g = slice; g < A.G; g += slices) {
       const GroupState &S = A.gs[g];
       const uint32_t active = S.active;
       if (!active) continue;
@@ -1334,6 +1343,7 @@ template <int LPS>
 __global__ void __launch_bounds__(kST) sweep_restart(SweepArgs A) {
   pdl_prologue();
   const int n = A.I.n;
+  const uint64_t seed = A.seeds[A.b];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   for (int g = 0; g < A.G; ++g) {
     const GroupState &S = A.gs[g];
@@ -1359,7 +1369,7 @@ __global__ void __launch_bounds__(kST) sweep_restart(SweepArgs A) {
       if (start) {
         const int wl = w0 + lane / LPS, rl = lane % LPS;
         const uint4 x = (wl < nwb && ((start >> rl) & 1u))
-                            ? start_bits(A.seed, (uint32_t)wl, (uint32_t)(32 * g + rl), (uint32_t)S.k, (uint32_t)A.b)
+                            ? start_bits(seed, (uint32_t)wl, (uint32_t)(32 * g + rl), (uint32_t)S.k, (uint32_t)A.b)
                             : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -1585,9 +1595,9 @@ cudaError_t run_instance(ising_handle *h, SweepArgs A, int mode, cudaStream_t s)
   if (use_graph) {
     // everything the captured launches bake in besides the handle's own arrays
     char key[320];
-    std::snprintf(key, sizeof key, "%d/%d/%d/%d/%d/%d/%d/%d/%d/%d/%llu/%p/%d/%d/%d/%d/%p/%d/%d", A.b, A.R, A.G, A.LPS,
+    std::snprintf(key, sizeof key, "%d/%d/%d/%d/%d/%d/%d/%d/%d/%d/%p/%d/%d/%d/%d/%p/%d/%d", A.b, A.R, A.G, A.LPS,
                   A.max_sweeps, A.restarts, A.budget, A.refresh, A.sequential, A.lattice,
-                  (unsigned long long)A.seed, (void *)A.sw, mode, grid_v, chunk, ncls, (void *)A.cflag, A.nchunk,
+                  (void *)A.sw, mode, grid_v, chunk, ncls, (void *)A.cflag, A.nchunk,
                   A.en_fast + 2 * A.en_count);
     auto it = S.graphs.find(key);
     if (it == S.graphs.end()) {
@@ -1664,7 +1674,7 @@ void sweep_free(ising_handle *h) {
 }
 
 cudaError_t launch_sweep(ising_handle *h, const ising_search_params *p, int32_t R, int8_t *spins, double *E,
-                         int32_t *E32, int32_t *minima, const uint64_t *seeds_host, cudaStream_t s) {
+                         int32_t *E32, int32_t *minima, cudaStream_t s) {
   SweepState &S = family_state<SweepState>(h->sweep_st);
   const int LPS = R > 16 ? 32 : (R > 8 ? 16 : 8);
   const int G = (R + 31) / 32;
@@ -1727,6 +1737,7 @@ cudaError_t launch_sweep(ising_handle *h, const ising_search_params *p, int32_t 
   uint16_t *cflag_mem = (uint16_t *)take(cflag_bytes);
   A.nchunk = nchunk;
   A.stats = h->d_stats;
+  A.seeds = h->d_seeds;
   A.spins = spins;
   A.energy = E;
   A.energy_i32 = E32;
@@ -1734,7 +1745,6 @@ cudaError_t launch_sweep(ising_handle *h, const ising_search_params *p, int32_t 
   for (int32_t b = 0; b < h->n_inst; ++b) {
     A.I = h->inst[b];
     A.b = b;
-    A.seed = seeds_host[b];
     A.lattice = (A.I.lat_d > 0 && !A.sequential) ? 1 : 0;
     {
       // site-parallel energies: at most `per_warp` terms, each below 2^ebits,

@@ -1,7 +1,10 @@
-// tile.cu — persistent tile kernels: one CTA (256 threads; four per SM, two for
-// the lattice mode) works on one (instance, 32-replica group) tile at a time,
-// pulled from a work queue largest first, with the instance's spins bit-packed
-// in shared memory (bit r of word i = replica r of spin i is +1).
+// tile.cu — persistent tile kernels: one CTA works on one (instance, 32-replica
+// group) tile at a time, pulled from a work queue largest first, with the
+// instance's spins bit-packed in shared memory (bit r of word i = replica r of
+// spin i is +1).  CTAs of 256 threads (four per SM, two for the lattice mode), or
+// of 512 and 1024 where the tiles are few.  Without a sweep budget a tile's
+// descents are independent, so where the tiles leave CTAs idle each is cut into
+// segments of consecutive descents, and the last segment to end keeps the best.
 //
 // Method (García & Markov, Sec. IV): single-spin moves taken when their gain
 // -2 s_i f_i is positive, whole sweeps repeated until no move is taken (a 1-flip
@@ -238,19 +241,24 @@ __device__ __forceinline__ uint32_t sliced_ge(uint32_t c0, uint32_t c1, uint32_t
 
 }  // namespace
 
-template <int MODE>
-__global__ void __launch_bounds__(kTileThreads, MODE == 3 ? 2 : 4) tile_kernel(const TileArgs *__restrict__ Aptr) {
+// SEG: tiles in segments of descents.  (A separate instantiation: the segments'
+// few values in the whole-tile kernel spill at 64 registers and cost full batches
+// 8 %.)
+template <int MODE, int THREADS, bool SEG>
+__global__ void __launch_bounds__(THREADS, (MODE == 3 ? 512 : 1024) / THREADS < 1 ? 1 : (MODE == 3 ? 512 : 1024) / THREADS)
+tile_kernel(const TileArgs *__restrict__ Aptr) {
   extern __shared__ uint32_t smem[];
-  __shared__ int s_tile;
+  __shared__ int s_tile, s_last, s_segs;
+  __shared__ bool s_merge;
   __shared__ uint32_t s_any, s_active, s_convround, s_upd;
   __shared__ int32_t s_total[32], s_minima[32];
   __shared__ double s_best[32], s_E[32];
-  __shared__ double s_red[(kTileThreads / 32) * 32];
+  __shared__ double s_red[THREADS];
   __shared__ int s_cnt[33];
 
   const TileArgs &A = *Aptr;
   const DevGraph G = A.g;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = THREADS / 32;
   const int nmax = A.nmax;
   uint32_t *sw = smem;
   uint32_t *fm = smem + nmax;
@@ -267,14 +275,16 @@ __global__ void __launch_bounds__(kTileThreads, MODE == 3 ? 2 : 4) tile_kernel(c
   //   s_work: 0 flip_evals, 1 flips, 2 minima, 3 descents, 4 sweeps, 5 evaluated
   __shared__ unsigned long long s_work[6];
   if (tid < 6) s_work[tid] = 0;
+  if (SEG && tid == 0) s_segs = A.segs;  // (read where it is needed: registers are short)
   uint32_t my_flips = 0, my_eval = 0;
 
   for (;;) {
     if (tid == 0) s_tile = atomicAdd(A.queue, 1);
     __syncthreads();
     const int t = s_tile;
-    if (t >= A.n_tiles) break;
-    const int b = A.tiles[t].x, g = A.tiles[t].y;
+    if (t >= (SEG ? A.n_tiles * s_segs : A.n_tiles)) break;
+    const int b = A.tiles[SEG ? t / s_segs : t].x, g = A.tiles[SEG ? t / s_segs : t].y;
+    if (SEG && tid == 0) s_last = (int)((int64_t)A.restarts * (t % s_segs + 1) / s_segs);  // end of its descents
     const InstDesc I = G.inst[b];
     const int n = I.n;
     const int rem = A.R - 32 * g;
@@ -289,10 +299,10 @@ __global__ void __launch_bounds__(kTileThreads, MODE == 3 ? 2 : 4) tile_kernel(c
     }
     __syncthreads();
 
-    for (int k = 0;; ++k) {
+    for (int k = SEG ? (int)((int64_t)A.restarts * (t % s_segs) / s_segs) : 0;; ++k) {
       if (tid == 0) {
         uint32_t start = 0;
-        if (k < A.restarts)
+        if (k < (SEG ? s_last : A.restarts))
           for (int r = 0; r < 32; ++r)
             if (((lane_valid >> r) & 1u) && (A.budget <= 0 || s_total[r] < A.budget)) start |= 1u << r;
         s_active = start;
@@ -344,7 +354,7 @@ __global__ void __launch_bounds__(kTileThreads, MODE == 3 ? 2 : 4) tile_kernel(c
             // field are unsatisfied (3-d: majority of three carries; 2-d: >= 3).
             const int L = I.lat_L, D = I.lat_d;
             const int stride[3] = {1, L, L * L};
-            for (int v = c0 + tid; v < c1; v += blockDim.x) {
+            for (int v = c0 + tid; v < c1; v += THREADS) {
               const int j = __ldg(G.order + I.spin_off + v);
               if (!pending(j)) continue;
               clear_pending(j);
@@ -389,7 +399,7 @@ __global__ void __launch_bounds__(kTileThreads, MODE == 3 ? 2 : 4) tile_kernel(c
           } else if (MODE == 2) {
             const int8_t *Ji = reinterpret_cast<const int8_t *>(G.J);
             const int8_t *hi = reinterpret_cast<const int8_t *>(G.h);
-            for (int v = c0 + tid; v < c1; v += blockDim.x) {
+            for (int v = c0 + tid; v < c1; v += THREADS) {
               const int j = A.sequential ? v : __ldg(G.order + I.spin_off + v);
               if (!pending(j)) continue;
               clear_pending(j);
@@ -693,7 +703,7 @@ __global__ void __launch_bounds__(kTileThreads, MODE == 3 ? 2 : 4) tile_kernel(c
             __syncthreads();
             const uint32_t upd = s_upd;
             if (upd)
-              for (int i = tid; i < n; i += blockDim.x) bw[i] = (bw[i] & ~upd) | (sw[i] & upd);
+              for (int i = tid; i < n; i += THREADS) bw[i] = (bw[i] & ~upd) | (sw[i] & upd);
           }
         }
         __syncthreads();
@@ -701,18 +711,62 @@ __global__ void __launch_bounds__(kTileThreads, MODE == 3 ? 2 : 4) tile_kernel(c
     }
 
     // Result per lane: best converged state, else the final state of its last descent.
+    const int unit = SEG ? s_tile : 0, segs = SEG ? s_segs : 1, tile = unit / segs;
     uint32_t has_best = 0;
     for (int r = 0; r < 32; ++r)
       if (s_minima[r] > 0) has_best |= 1u << r;
-    if (lane_valid & ~has_best) {
+    if ((lane_valid & ~has_best) && (!SEG || unit % segs == segs - 1)) {
       if (MODE == 3) tile_energy_lattice(G, I, sw, s_cnt, s_E);
       else tile_energy_lanes<MODE == 1>(G, I, sw, s_red, s_E);
       if (tid < 32 && !((has_best >> tid) & 1u)) s_best[tid] = s_E[tid];
     }
     __syncthreads();
+    const uint32_t *from = nullptr;  // the words of the tile's segments
+    if constexpr (SEG) {
+      // this segment's words, energies and minima; the last CTA of the tile
+      // chooses per lane among the segments (strictly lower energy, ties keep the
+      // earlier; without a converged descent the last segment)
+      uint32_t *words = A.seg_words + (size_t)unit * nmax;
+      for (int i = tid; i < n; i += THREADS) words[i] = (bw[i] & has_best) | (sw[i] & ~has_best);
+      if (tid < 32) {
+        A.seg_best[(size_t)unit * 32 + tid] = s_best[tid];
+        A.seg_minima[(size_t)unit * 32 + tid] = s_minima[tid];
+      }
+      __threadfence();
+      __syncthreads();
+      if (tid == 0) s_merge = atomicAdd(A.queue + 4 + tile, 1) == segs - 1;
+      __syncthreads();
+      if (!s_merge) continue;
+      __threadfence();
+      from = A.seg_words + (size_t)tile * segs * nmax;
+      if (tid < 32) {
+        double e = DBL_MAX;
+        int m = 0, best = segs - 1;
+        for (int q = 0; q < segs; ++q) {
+          const size_t o = ((size_t)tile * segs + q) * 32 + tid;
+          const int mq = __ldcg(A.seg_minima + o);
+          const double eq = __ldcg(A.seg_best + o);
+          m += mq;
+          if (mq > 0 && eq < e) {
+            e = eq;
+            best = q;
+          }
+        }
+        if (m == 0) e = __ldcg(A.seg_best + ((size_t)tile * segs + best) * 32 + tid);
+        s_best[tid] = e;
+        s_minima[tid] = m;
+        s_total[tid] = best;
+      }
+      __syncthreads();
+    }
     const int64_t out_base = (int64_t)A.R * I.spin_off + (int64_t)(32 * g) * n;
-    for (int i = tid; i < n; i += blockDim.x) {
-      const uint32_t wv = (bw[i] & has_best) | (sw[i] & ~has_best);
+    for (int i = tid; i < n; i += THREADS) {
+      uint32_t wv = 0;
+      if (SEG) {
+        for (int r = 0; r < 32; ++r) wv |= __ldcg(from + (size_t)s_total[r] * nmax + i) & (1u << r);
+      } else {
+        wv = (bw[i] & has_best) | (sw[i] & ~has_best);
+      }
       for (int r = 0; r < 32; ++r)
         if ((lane_valid >> r) & 1u) A.spins[out_base + (int64_t)r * n + i] = ((wv >> r) & 1u) ? 1 : -1;
     }
@@ -734,6 +788,8 @@ size_t tile_smem_bytes(int mode, int nmax) {
   return (size_t)(mode >= 2 ? 1 : 2) * (size_t)nmax * sizeof(uint32_t) + (size_t)((nmax + 31) / 32) * sizeof(uint32_t);
 }
 
+size_t tile_smem_limit() { return 200 * 1024; }
+
 // Spins whose FP32 fields (32 lanes) fit in shared memory next to the tile's
 // words, within `budget` bytes of dynamic shared memory.
 int tile_fsm_cap(int nmax, size_t budget) {
@@ -743,32 +799,41 @@ int tile_fsm_cap(int nmax, size_t budget) {
   return (int)std::min<size_t>(cap, (size_t)nmax);
 }
 
-int tile_max_ctas_per_sm(int mode, size_t smem) {
-  int blocks = 0;
-  cudaError_t e;
-  if (mode == 0) {
-    e = cudaFuncSetAttribute(tile_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, tile_kernel<0>, kTileThreads, smem);
-  } else if (mode == 1) {
-    e = cudaFuncSetAttribute(tile_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, tile_kernel<1>, kTileThreads, smem);
-  } else if (mode == 2) {
-    e = cudaFuncSetAttribute(tile_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, tile_kernel<2>, kTileThreads, smem);
-  } else {
-    e = cudaFuncSetAttribute(tile_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, tile_kernel<3>, kTileThreads, smem);
+namespace {
+using TileKernel = void (*)(const TileArgs *);
+template <int MODE, bool SEG>
+TileKernel tile_kernel_of(int threads) {
+  return threads == 256 ? tile_kernel<MODE, 256, SEG> : (threads == 512 ? tile_kernel<MODE, 512, SEG> : tile_kernel<MODE, 1024, SEG>);
+}
+template <int MODE>
+TileKernel tile_kernel_of(int threads, bool seg) {
+  return seg ? tile_kernel_of<MODE, true>(threads) : tile_kernel_of<MODE, false>(threads);
+}
+TileKernel tile_kernel_for(int mode, int threads, bool seg) {
+  return mode == 0 ? tile_kernel_of<0>(threads, seg)
+                   : (mode == 1 ? tile_kernel_of<1>(threads, seg)
+                                : (mode == 2 ? tile_kernel_of<2>(threads, seg) : tile_kernel_of<3>(threads, seg)));
+}
+}  // namespace
+
+int tile_max_ctas_per_sm(int mode, int threads, size_t smem) {
+  int blocks = 0, least = 0;
+  for (int seg = 0; seg < 2; ++seg) {
+    const TileKernel k = tile_kernel_for(mode, threads, seg != 0);
+    // (the same limit for every size: the attribute is the process's, and another
+    // thread's handle may launch the same kernel at a larger size)
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tile_smem_limit());
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k, threads, smem);
+    if (e != cudaSuccess) return 0;
+    least = seg ? std::min(least, blocks) : blocks;
   }
-  return e == cudaSuccess ? blocks : 0;
+  return least;
 }
 
 // Launch only: the shared-memory attribute was set by tile_max_ctas_per_sm, so
 // this is a plain stream operation and can be captured into a graph.
-cudaError_t launch_tile(ising_handle *h, int mode, int grid, size_t smem, cudaStream_t s) {
-  if (mode == 0) tile_kernel<0><<<grid, kTileThreads, smem, s>>>(h->d_tile_args);
-  else if (mode == 1) tile_kernel<1><<<grid, kTileThreads, smem, s>>>(h->d_tile_args);
-  else if (mode == 2) tile_kernel<2><<<grid, kTileThreads, smem, s>>>(h->d_tile_args);
-  else tile_kernel<3><<<grid, kTileThreads, smem, s>>>(h->d_tile_args);
+cudaError_t launch_tile(ising_handle *h, int mode, int threads, bool seg, int grid, size_t smem, cudaStream_t s) {
+  tile_kernel_for(mode, threads, seg)<<<grid, threads, smem, s>>>(h->d_tile_args);
   return cudaGetLastError();
 }
 

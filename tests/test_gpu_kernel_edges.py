@@ -53,6 +53,42 @@ def test_sweep_general_graph_fp64_refresh(R):
     _compare([inst], [R], R, False, max_sweeps=400, restarts=2, refresh_every=2, kernel=isg.KERNEL_SWEEP)
 
 
+# Tiles cut into segments of descents: more descents than segments and fewer,
+# descents that never converge (the last one's state is the result) or only some,
+# ragged replica groups, both schedules, every mode of the tile kernels.
+def _segment_instance(kind):
+    if kind == "lattice":
+        return W.lattice((9, 9, 9), True, "pm1", "pm1_0", seed=51)
+    if kind == "msc":
+        return W.random_graph(150, 4.0, 52, dtype="i8", int_range=1, fields=False)
+    return W.random_graph(170, 5.0, 53, dtype="f32" if kind == "f32" else "i8", n_hyper=30, hyper_order=(3, 4))
+
+
+@pytest.mark.parametrize("max_sweeps,restarts,R", [(1, 7, 33), (4, 3, 5), (5, 40, 40), (300, 333, 3), (300, 2, 70)])
+@pytest.mark.parametrize("kind", ["lattice", "msc", "i8", "f32"])
+def test_tile_segments(kind, max_sweeps, restarts, R):
+    _compare([_segment_instance(kind)], [R], R, kind != "f32", max_sweeps=max_sweeps, restarts=restarts,
+             refresh_every=3, kernel=isg.KERNEL_MSC if kind in ("lattice", "msc") else isg.KERNEL_TILE)
+
+
+def test_tile_segments_uneven_batch_and_sequential_schedule():
+    insts = [W.random_graph(n, 4.0, 60 + n, dtype="f32", n_hyper=n // 9) for n in (1, 40, 300)]
+    _compare(insts, [1, 2, 3], 34, False, max_sweeps=200, restarts=9, schedule=isg.SCHED_SEQUENTIAL,
+             kernel=isg.KERNEL_TILE)
+
+
+# The planner's line between one CTA per tile and launches over the whole GPU:
+# the same results on both sides of it.
+@pytest.mark.parametrize("n", [2000, 12000])
+def test_auto_family_of_one_general_graph(n):
+    inst = W.random_graph(n, 5.0, 61, dtype="f32", n_hyper=n // 8, hyper_order=(3, 4))
+    kw = dict(max_sweeps=300, restarts=2)
+    h = isg.Handle([inst])
+    assert h.plan_kernel(6, **kw) == (isg.KERNEL_TILE if n == 2000 else isg.KERNEL_SWEEP)
+    h.close()
+    _compare([inst], [n], 6, False, **kw)
+
+
 # ising_energy: one-CTA instances (up to 2048 spins) and larger ones in parts of
 # 1024 sites; 4, 16 and 32 replicas per word group and their remainders; sizes
 # that are no multiple of 4 and spins that start on an odd byte; lattices of
