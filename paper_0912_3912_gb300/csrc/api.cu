@@ -924,6 +924,10 @@ ising_status ising_create(const ising_instance_desc *descs, int32_t n_instances,
         inc_oth.push_back(o);
       }
     }
+    D.has_h = 0;
+    for (float v : I.hf) D.has_h |= v != 0.0f;
+    for (int8_t v : I.hi) D.has_h |= v != 0;
+    for (double v : I.hd) D.has_h |= v != 0.0;
     D.fm_ent = D.fbits = D.funit = -1;
     if (!f64) h->fm_rounds = std::max(h->fm_rounds, fm_entries(I, inc, fl, D));
     for (int32_t e = 0; e < D.n_hyper; ++e) hptr.push_back((uint32_t)(mem_off + I.hptr[e]));

@@ -54,6 +54,7 @@ struct InstDesc {
   // for FP32, ebase >= 0; else -1.
   int32_t fbits;
   int32_t funit;
+  int32_t has_h;  // some field is not zero
 };
 
 // Everything a kernel needs to read an instance set.

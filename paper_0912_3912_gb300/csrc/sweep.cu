@@ -1,6 +1,6 @@
 // sweep.cu — large instances (too big for one CTA's shared memory): every
 // colour class is one launch over the whole GPU; a sweep is the sequence of
-// class launches plus a one-block end-of-sweep launch, with the round-end
+// class launches, the next kernel working out the sweep's end, with the round-end
 // kernels (energy pass, restarts) after every fourth sweep; chunks of sweeps
 // are captured once into a CUDA graph (cached) and replayed until every replica
 // is done, the host polling a done flag one chunk behind.
@@ -9,7 +9,7 @@
 // improving single-spin moves, repeated sweeps to a 1-flip minimum, random
 // restarts, best kept; incremental FP32 field updates for float couplings with
 // an exact refresh).  State lives in global memory: spin words sw[g][n] (bit l =
-// replica 32g + l), flip masks fm[g][n], pending masks pend[g][n] (lanes with a
+// replica g LPS + l), flip masks fm[g][n], pending masks pend[g][n] (lanes with a
 // neighbour that flipped since the spin's last visit), best words bw[g][n], FP32 fields
 // F[g][position][LPS] stored in colour-class order so a class reads them
 // contiguously.  LPS (lanes per spin) = 32, 16 or 8 replicas share one warp
@@ -18,11 +18,12 @@
 // Periodic lattices use the compact per-site metadata (DevGraph::meta/Jpos)
 // instead of the CSR: 4 bytes of neighbour directions and coupling signs plus
 // the couplings in class order, all read contiguously.
+#include <algorithm>
 #include <cfloat>
 #include <cstdio>
-#include <cstdlib>
 #include <map>
 #include <string>
+#include <vector>
 
 #include "device_common.cuh"
 
@@ -36,16 +37,24 @@ constexpr int kST = 256;  // threads per CTA
 constexpr int kVisitCtasPerSm = 4;  // the FP32/int lane visits: 64 registers per thread
 
 struct GroupState {
-  uint32_t lane_valid, active, convround, any, upd, start;
+  uint32_t lane_valid, active, convround, upd, start, pad0;
   int32_t k, d, done, round_end, final_pass, pad;
   int32_t total[32], minima[32];
   double best[32], E[32];
 };
 
+// The groups' state comes in two copies.  A sweep's visits collect the flipped
+// lanes in `any` words of the sweep (four sets, by sweep modulo 4: one is read,
+// one collected and one cleared at a time); the kernel that follows them (the next sweep's
+// first visit, or the round-end pass) works the end of the sweep out from it - in
+// every CTA alike, for its own use - and its first CTA writes the new state to
+// the other copy, which is then the current one.  (A launch of its own for the
+// end of a sweep, one block, took 2.3 us and a launch gap.)
+
 struct SweepArgs {
   DevGraph g;
   InstDesc I;
-  int32_t b, R, G, LPS;
+  int32_t b, R, r0, Rn, G, LPS;  // replicas of the call; first replica, replicas and groups of this run
   int32_t max_sweeps, restarts, budget, refresh, sequential, lattice;
   const uint64_t *seeds;  // device [instances] (a captured chunk serves every seed)
   uint32_t *sw, *fm, *bw;
@@ -64,8 +73,15 @@ struct SweepArgs {
   // below 2^24: q = (x * divL_m) >> divL_k)
   uint64_t divL_m;
   int32_t divL_k;
+  int32_t site_arith;  // 1: the class positions map to sites so (with or without flags)
   float *F;
-  GroupState *gs;
+  GroupState *gs;   // the current copy of the groups' state
+  GroupState *nxt;  // end of the sweep before: where the new state goes (null: none is due)
+  // [G] each: flipped lanes of the sweep whose end is due, of this sweep, and of
+  // the next one (cleared by this sweep's first visit)
+  const uint32_t *any_r;
+  uint32_t *any_w, *any_z;
+  uint32_t *any4;  // the four sets
   double *partial;  // [grid_e][G][32]: FP64 sums of the CTAs (FP64 energies)
   // [G][32][2]: integer and fixed-point energies, high and low halves, summed
   // by atomic adds (order-free); read and zeroed by the last CTA
@@ -79,7 +95,6 @@ struct SweepArgs {
   // counted bit-sliced (E = 2 U - B, U the unsatisfied bonds and fields)
   int32_t en_count;
   // 1: launch the chunk kernels with programmatic stream serialization
-  // (measured faster for the multi-spin-coded visits, slower for the FP32 ones)
   int32_t pdl;
   unsigned int *counter;
   int32_t *all_done;
@@ -100,7 +115,7 @@ __device__ __forceinline__ int lat_nbr(int j, uint32_t meta, int k, int L) {
 }
 
 
-// Programmatic dependent launch (multi-spin-coded lattices; SweepArgs::pdl).
+// Programmatic dependent launch (SweepArgs::pdl).
 // The kernels of a sweep chunk may then be scheduled while their predecessor
 // drains: a visit lets its dependants launch once each of its CTAs has done its
 // main work (launch_dependents), and every chunk kernel waits, before reading
@@ -114,12 +129,12 @@ __global__ void sweep_init(SweepArgs A) {
   const int g = threadIdx.x;
   if (g < A.G) {
     GroupState &S = A.gs[g];
-    const int rem = A.R - 32 * g;
+    const int rem = A.Rn - A.LPS * g;
     const int lanes = rem >= A.LPS ? A.LPS : rem;
     S.lane_valid = lanes >= 32 ? 0xffffffffu : ((1u << lanes) - 1u);
     S.start = S.lane_valid;
     S.active = S.lane_valid;
-    S.convround = S.any = S.upd = 0;
+    S.convround = S.upd = 0;
     S.k = 0;
     S.d = 0;
     S.done = 0;
@@ -131,6 +146,7 @@ __global__ void sweep_init(SweepArgs A) {
       S.best[r] = DBL_MAX;
       S.E[r] = 0.0;
     }
+    for (int q = 0; q < 4; ++q) A.any4[q * A.G + g] = 0u;
     atomicAdd(A.stats + 3, (unsigned long long)__popc(S.start));
   }
   if (threadIdx.x == 0) {
@@ -154,64 +170,98 @@ __device__ __forceinline__ uint32_t sliced_ge4(uint32_t q0, uint32_t q1, uint32_
   return gt | eq;
 }
 
-// End of a sweep: per group, which lanes converged, which descents ended.
-// One warp per group, lane l = replica lane l.  (Folding this into the last
-// class visit - its last CTA closing the sweep - was measured slower than this
-// separate launch.)
-__global__ void sweep_end(SweepArgs A) {
-  pdl_prologue();
-  const int g = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (g >= A.G) return;
-  GroupState &S = A.gs[g];
-  const uint32_t active = S.active;
-  const uint32_t any = S.any;
-  __syncwarp();
-  if (lane == 0) {
-    S.start = 0;
-    S.upd = 0;
+// What a visit needs of the groups' state.
+struct GroupView {
+  uint32_t active[32];
+  int32_t d[32];
+  uint8_t over[32];  // the round is over, or its final pass due
+};
+
+// The groups' state for this kernel: as it stands, or - when A.nxt is set - after
+// the end of the sweep that the visits before closed: which lanes converged,
+// which descents ended.  A warp per group, lane l = replica lane; the first CTA
+// writes the new copy and the counters.  Returns whether some group's round is
+// over (or its final pass due); ends with a block barrier.
+__device__ __forceinline__ bool load_groups(const SweepArgs &A, GroupView &V) {
+  __shared__ int s_over;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) s_over = 0;
+  __syncthreads();
+  for (int g = warp; g < A.G; g += (int)(blockDim.x >> 5)) {
+    const GroupState &S = A.gs[g];
+    uint32_t active = S.active;
+    int32_t d = S.d, round_end = S.round_end;
+    if (A.nxt) {
+      const uint32_t any = A.any_r[g];
+      int32_t t = S.total[lane];
+      uint32_t convround = S.convround, conv = 0u;
+      const uint32_t was = active;
+      if (active) {
+        bool over = false;
+        if ((active >> lane) & 1u) {
+          ++t;
+          over = A.budget > 0 && t >= A.budget;
+        }
+        conv = active & ~any;
+        uint32_t ended = __ballot_sync(0xffffffffu, over) | conv;
+        ++d;
+        if (d >= A.max_sweeps) ended |= active;
+        convround |= conv;
+        active &= ~ended;
+        if (!active) round_end = 1;
+      }
+      if (blockIdx.x == 0 && blockIdx.y == 0) {
+        GroupState &N = A.nxt[g];
+        N.total[lane] = t;
+        N.minima[lane] = S.minima[lane];
+        N.best[lane] = S.best[lane];
+        N.E[lane] = S.E[lane];
+        if (lane == 0) {
+          N.lane_valid = S.lane_valid;
+          N.active = active;
+          N.convround = convround;
+          N.upd = N.start = 0u;
+          N.k = S.k;
+          N.d = d;
+          N.done = S.done;
+          N.round_end = round_end;
+          N.final_pass = 0;
+          if (was) {
+            atomicAdd(A.stats + 4, (unsigned long long)__popc(was));
+            atomicAdd(A.stats + 0, (unsigned long long)__popc(was) * (unsigned long long)A.I.n);
+            atomicAdd(A.stats + 2, (unsigned long long)__popc(conv));
+          }
+        }
+      }
+    }
+    if (lane == 0) {
+      V.active[g] = active;
+      V.d[g] = d;
+      V.over[g] = round_end || S.final_pass;
+      if (round_end || S.final_pass) s_over = 1;
+    }
   }
-  if (!active) return;
-  const bool mine = (active >> lane) & 1u;
-  bool over = false;
-  if (mine) {
-    const int32_t t = S.total[lane] + 1;
-    S.total[lane] = t;
-    over = A.budget > 0 && t >= A.budget;
-  }
-  const uint32_t conv = active & ~any;
-  uint32_t ended = __ballot_sync(0xffffffffu, over) | conv;
-  const int32_t d = S.d + 1;
-  if (d >= A.max_sweeps) ended |= active;
-  if (lane == 0) {
-    S.any = 0;
-    S.d = d;
-    atomicAdd(A.stats + 4, (unsigned long long)__popc(active));
-    atomicAdd(A.stats + 0, (unsigned long long)__popc(active) * (unsigned long long)A.I.n);
-    atomicAdd(A.stats + 2, (unsigned long long)__popc(conv));
-    S.convround |= conv;
-    S.active = active & ~ended;
-    if (!(active & ~ended)) S.round_end = 1;
-  }
+  __syncthreads();
+  return s_over != 0;
 }
 
 // One colour class of one sweep.  MODE 0 int lanes, 1 FP32 lanes, 2 multi-spin
 // coded.  Groups are walked in an outer loop so the per-group state is read once
 // per warp and no index needs a division.
 template <int MODE, int LPS, bool LAT>
-__global__ void __launch_bounds__(kST, (MODE == 2 && LAT) ? 8 : kVisitCtasPerSm) sweep_visit(SweepArgs A, int32_t c) {
+__global__ void __launch_bounds__(kST, (MODE == 2 && LAT) ? 8 : kVisitCtasPerSm)
+sweep_visit(SweepArgs A, int32_t c, int32_t c0, int32_t c1) {
+  __shared__ GroupView s_grp;
   __shared__ uint32_t s_any[32];
-  __shared__ unsigned long long s_red[kST / 32];
   __shared__ int s_off[6], s_wrap[6];
-  __shared__ unsigned int s_eval;
+  __shared__ unsigned long long s_eval, s_flips;
   const DevGraph &G = A.g;
   const InstDesc &I = A.I;
   const int n = I.n, L = I.lat_L;
   const int64_t so = I.spin_off;
   const int tid = threadIdx.x, lane = threadIdx.x & 31;
-  pdl_prologue();
   if (tid < 32) s_any[tid] = 0;
-  if (tid == 0) s_eval = 0;
+  if (tid == 0) s_eval = s_flips = 0;
   if (LAT && tid < 6) {
     // direction d: +x, -x, +y, -y, +z, -z; stride and wrap-around correction
     const int a = tid >> 1;
@@ -219,16 +269,10 @@ __global__ void __launch_bounds__(kST, (MODE == 2 && LAT) ? 8 : kVisitCtasPerSm)
     s_off[tid] = (tid & 1) ? -st : st;
     s_wrap[tid] = (tid & 1) ? L * st : -L * st;
   }
-  __syncthreads();
-  int c0, c1;
-  if (A.sequential) {
-    c0 = c;
-    c1 = c + 1;
-  } else {
-    c0 = __ldg(G.cls + I.cls_off + c);
-    c1 = __ldg(G.cls + I.cls_off + c + 1);
-  }
-  const int cs = c1 - c0;
+  pdl_prologue();
+  load_groups(A, s_grp);
+  if (A.any_z && blockIdx.x == 0 && blockIdx.y == 0 && tid < A.G) A.any_z[tid] = 0u;
+  const int cs = c1 - c0;  // the class's positions c0 .. c1
   // per-thread counts of one launch (each below 2^32: a thread visits at most
   // n / threads positions of LPS replicas)
   uint32_t my_flips = 0;
@@ -240,19 +284,27 @@ __global__ void __launch_bounds__(kST, (MODE == 2 && LAT) ? 8 : kVisitCtasPerSm)
     const int8_t *Ji = reinterpret_cast<const int8_t *>(G.J);
     const int D = I.lat_d;
     for (int g = 0; g < A.G; ++g) {
-      const uint32_t active = A.gs[g].active & lmask;
+      const uint32_t active = s_grp.active[g] & lmask;
       if (!active) continue;
-      const bool fresh = A.gs[g].d == 0;
+      const bool fresh = s_grp.d[g] == 0;
       uint32_t *swg = A.sw + (size_t)g * n;
       uint32_t *pendg = A.pend + (size_t)g * n;
       uint32_t anyg = 0;
       for (int t = blockIdx.x * blockDim.x + tid; t < cs; t += gridDim.x * blockDim.x) {
         const int v = c0 + t;
-        const int j = A.sequential ? v : __ldg(G.order + so + v);
+        int j;
+        if (LAT && A.site_arith) {
+          const uint32_t p2 = 2u * (uint32_t)t;
+          const uint32_t rho = (uint32_t)(((uint64_t)p2 * A.divL_m) >> A.divL_k);
+          const uint32_t z = (uint32_t)(((uint64_t)rho * A.divL_m) >> A.divL_k);
+          j = (int)(p2 + (((uint32_t)c + rho - z * (uint32_t)L + z) & 1u));
+        } else {
+          j = A.sequential ? v : __ldg(G.order + so + v);
+        }
         // everything indexed by the site itself is read in one round trip
         const uint32_t pj = pendg[j];
         const uint32_t wj = swg[j];
-        const int hv = __ldg(hi + so + j);
+        const int hv = I.has_h ? __ldg(hi + so + j) : 0;
         const uint32_t info = LAT ? __ldg(G.latinfo + so + v) : 0u;
         if (!fresh && !(pj & active)) continue;  // no neighbour flipped: still stable
         if (pj) pendg[j] = 0u;
@@ -327,26 +379,18 @@ __global__ void __launch_bounds__(kST, (MODE == 2 && LAT) ? 8 : kVisitCtasPerSm)
     // replicas each), with all loads of one visit independent of each other.
     constexpr int SPW = 32 / LPS;
     const int sub = lane / LPS, ln = lane % LPS;
-    // General graphs: the groups are spread over slices of the warps while every
-    // slice still has a warp for each step of the class.
-    int nwarps = gridDim.x * (blockDim.x >> 5), wid = blockIdx.x * (blockDim.x >> 5) + (tid >> 5);
-    int slices = 1, slice = 0;
-    if constexpr (!LAT) {
-      while (2 * slices <= A.G && cs <= nwarps / (2 * slices) * SPW) slices *= 2;
-      slice = wid % slices;
-      wid /= slices;
-      nwarps /= slices;
-      if (wid >= nwarps) slice = A.G;  // (a remainder of warps stays idle)
-    }
+    // The groups are spread over blockIdx.y; on FP32 lattices, whose registers are
+    // short, every group has CTAs of its own, so that there is no loop.
+    constexpr bool kOneGroup = MODE == 1 && LAT;
+    const int nwarps = gridDim.x * (blockDim.x >> 5), wid = blockIdx.x * (blockDim.x >> 5) + (tid >> 5);
     // class positions per warp step (not the FP32 lattice path): 32, fewer where
     // the class would leave resident warps without work
     int pw = 32;
     while (pw > SPW && cs < nwarps * pw) pw >>= 1;
-    for (int g = slice; g < A.G; g += slices) {
-      const GroupState &S = A.gs[g];
-      const uint32_t active = S.active;
+    for (int g = blockIdx.y; g < (kOneGroup ? (int)blockIdx.y + 1 : A.G); g += kOneGroup ? 1 : gridDim.y) {
+      const uint32_t active = s_grp.active[g];
       if (!active) continue;
-      const int dd = S.d;
+      const int dd = s_grp.d[g];
       const bool refresh = (dd == 0) || (A.refresh > 0 && dd % A.refresh == 0);
       uint32_t *swg = A.sw + (size_t)g * n;
       uint32_t *fmg = A.fm + (size_t)g * n;
@@ -400,7 +444,7 @@ __global__ void __launch_bounds__(kST, (MODE == 2 && LAT) ? 8 : kVisitCtasPerSm)
             continue;
           }
           // replica visits of the positions not skipped (one shared add per warp step)
-          if (lane == 0) atomicAdd(&s_eval, (uint32_t)__popc(todo) * (uint32_t)__popc(active));
+          if (lane == 0) atomicAdd(&s_eval, (unsigned long long)(__popc(todo) * __popc(active)));
           if (!refresh) {
             // Site-parallel: the position lane pulls, for each of its pending
             // replicas, the flips of the neighbours since the site's previous
@@ -841,12 +885,14 @@ __global__ void __launch_bounds__(kST, (MODE == 2 && LAT) ? 8 : kVisitCtasPerSm)
     }
   }
   pdl_trigger();
+  my_flips = __reduce_add_sync(0xffffffffu, my_flips);
+  my_eval = __reduce_add_sync(0xffffffffu, my_eval);
+  if (lane == 0 && my_flips) atomicAdd(&s_flips, (unsigned long long)my_flips);
+  if (lane == 0 && my_eval) atomicAdd(&s_eval, (unsigned long long)my_eval);
   __syncthreads();
-  if (tid < A.G && s_any[tid]) atomicOr(&A.gs[tid].any, s_any[tid]);
-  const unsigned long long flips_b = block_sum((unsigned long long)my_flips, s_red);
-  if (tid == 0 && flips_b) atomicAdd(A.stats + 1, flips_b);
-  const unsigned long long eval_b = block_sum((unsigned long long)my_eval, s_red) + s_eval;
-  if (tid == 0 && eval_b) atomicAdd(A.stats + 5, eval_b);
+  if (tid < A.G && s_any[tid]) atomicOr(A.any_w + tid, s_any[tid]);
+  if (tid == 32 && s_flips) atomicAdd(A.stats + 1, s_flips);
+  if (tid == 64 && s_eval) atomicAdd(A.stats + 5, s_eval);
 }
 
 // Warp sums of NV per-lane values at once: NV halving exchange steps leave
@@ -895,18 +941,17 @@ __global__ void __launch_bounds__(kST, 4) sweep_energy(SweepArgs A) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int ub = I.ebase;
   const bool fx = FLOAT && ub >= 0;
+  __shared__ GroupView s_grp;
   pdl_prologue();
-  bool any = false;
-  for (int g = 0; g < A.G; ++g) any = any || A.gs[g].round_end || A.gs[g].final_pass;
-  if (!any) return;
+  if (!load_groups(A, s_grp)) return;
+  GroupState *const cur = A.nxt ? A.nxt : A.gs;  // (read by the last CTA only: the first one may be writing it)
   constexpr int SPW = 32 / LPS;
   const int sub = lane / LPS, ln = lane % LPS;
   for (int g = 0; g < A.G; ++g) {
-    const GroupState &S = A.gs[g];
     double accd = 0.0;
     long long acci = 0;
     unsigned long long accl = 0;
-    if (S.round_end || S.final_pass) {
+    if (s_grp.over[g]) {
       const uint32_t *swg = A.sw + (size_t)g * n;
       if (LAT && !FLOAT && A.en_count) {
         // Multi-spin-coded lattice, site-parallel in site order: with J = +/-1
@@ -1228,7 +1273,7 @@ __global__ void __launch_bounds__(kST, 4) sweep_energy(SweepArgs A) {
       acci += __shfl_xor_sync(0xffffffffu, acci, o);
       accl += __shfl_xor_sync(0xffffffffu, accl, o);
     }
-    if (!(S.round_end || S.final_pass)) continue;  // (uniform across the grid)
+    if (!s_grp.over[g]) continue;  // (uniform across the grid)
     const bool dbl = FLOAT && !fx;
     long long *ri = reinterpret_cast<long long *>(&s_red[0][0]);
     __syncthreads();
@@ -1265,8 +1310,8 @@ __global__ void __launch_bounds__(kST, 4) sweep_energy(SweepArgs A) {
   __threadfence();
   // last CTA: totals in CTA order, then per-group bookkeeping
   for (int g = 0; g < A.G; ++g) {
-    GroupState &S = A.gs[g];
-    if (!(S.round_end || S.final_pass)) continue;
+    GroupState &S = cur[g];
+    if (!s_grp.over[g]) continue;
     if (FLOAT && !fx) {
       // FP64: warp w adds the partials of CTAs w, w + nw, ... (fixed order),
       // then warp 0 adds the warps' sums in ascending order: deterministic
@@ -1329,7 +1374,7 @@ __global__ void __launch_bounds__(kST, 4) sweep_energy(SweepArgs A) {
   }
   if (tid == 0) {
     int all = 1;
-    for (int g = 0; g < A.G; ++g) all = all && A.gs[g].done;
+    for (int g = 0; g < A.G; ++g) all = all && cur[g].done;
     *A.all_done = all;
     *A.counter = 0;
   }
@@ -1359,29 +1404,49 @@ __global__ void __launch_bounds__(kST) sweep_restart(SweepArgs A) {
     // the same 32-site quarter of block w0 + j.
     constexpr int P = 32 / LPS;
     constexpr uint32_t lmask = LPS == 32 ? 0xffffffffu : ((1u << LPS) - 1u);
+    // Every lane of the group restarting (the usual round's end): the words are
+    // replaced, not merged, and no read of the old ones is waited for.
+    const bool whole = start == S.lane_valid;
     for (int w0 = (blockIdx.x * nw + warp) * P; w0 < nwb; w0 += gridDim.x * nw * P) {
-      if (upd)
-        for (int t = lane; t < 128 * P; t += 32) {
-          const int i = w0 * 128 + t;
-          if (i < n) bwg[i] = (bwg[i] & ~upd) | (swg[i] & upd);
+      if (upd) {
+        uint32_t sv[4 * P], bv[4 * P];
+#pragma unroll
+        for (int t = 0; t < 4 * P; ++t) {
+          const int i = w0 * 128 + t * 32 + lane;
+          sv[t] = i < n ? swg[i] : 0u;
+          bv[t] = i < n ? bwg[i] : 0u;
         }
+#pragma unroll
+        for (int t = 0; t < 4 * P; ++t) {
+          const int i = w0 * 128 + t * 32 + lane;
+          if (i < n) bwg[i] = (bv[t] & ~upd) | (sv[t] & upd);
+        }
+      }
       __syncwarp();
       if (start) {
         const int wl = w0 + lane / LPS, rl = lane % LPS;
         const uint4 x = (wl < nwb && ((start >> rl) & 1u))
-                            ? start_bits(seed, (uint32_t)wl, (uint32_t)(32 * g + rl), (uint32_t)S.k, (uint32_t)A.b)
+                            ? start_bits(seed, (uint32_t)wl, (uint32_t)(A.r0 + LPS * g + rl), (uint32_t)S.k, (uint32_t)A.b)
                             : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const uint32_t mine = warp_transpose32(word_of(x, q), lane);  // field j: site u of block w0 + j
+          uint32_t sv[P], fv[P];
+#pragma unroll
+          for (int j = 0; j < P; ++j) {
+            const int i = (w0 + j) * 128 + q * 32 + lane;
+            sv[j] = fv[j] = 0u;
+            if (!whole && i < n) {
+              sv[j] = swg[i] & ~start;
+              fv[j] = fmg[i] & ~start;
+            }
+          }
 #pragma unroll
           for (int j = 0; j < P; ++j) {
             const int i = (w0 + j) * 128 + q * 32 + lane;
             if (i < n) {
-              const uint32_t word = (mine >> (j * LPS)) & lmask;
-              swg[i] = (swg[i] & ~start) | (word & start);
-              const uint32_t f = fmg[i];
-              if (f & start) fmg[i] = f & ~start;
+              swg[i] = sv[j] | ((mine >> (j * LPS)) & lmask & start);
+              fmg[i] = fv[j];
             }
           }
         }
@@ -1404,20 +1469,20 @@ __global__ void sweep_mark_final(SweepArgs A) {
 
 __global__ void sweep_output(SweepArgs A) {
   const int n = A.I.n;
-  const int64_t tot = (int64_t)A.R * n;
+  const int64_t tot = (int64_t)A.Rn * n;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < tot; t += (int64_t)gridDim.x * blockDim.x) {
     const int r = (int)(t / n), i = (int)(t % n);
-    const int g = r / 32, l = r % 32;
+    const int g = r / A.LPS, l = r % A.LPS;
     const GroupState &S = A.gs[g];
     const uint32_t w = S.minima[l] > 0 ? A.bw[(size_t)g * n + i] : A.sw[(size_t)g * n + i];
-    A.spins[(int64_t)A.R * A.I.spin_off + t] = ((w >> l) & 1u) ? 1 : -1;
+    A.spins[(int64_t)A.R * A.I.spin_off + (int64_t)A.r0 * n + t] = ((w >> l) & 1u) ? 1 : -1;
   }
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < A.R) {
-    const int g = (int)t / 32, l = (int)t % 32;
+  if (t < A.Rn) {
+    const int g = (int)t / A.LPS, l = (int)t % A.LPS;
     const GroupState &S = A.gs[g];
     const double e = S.minima[l] > 0 ? S.best[l] : S.E[l];
-    const int64_t o = (int64_t)A.b * A.R + t;
+    const int64_t o = (int64_t)A.b * A.R + A.r0 + t;
     A.energy[o] = e;
     if (A.energy_i32) A.energy_i32[o] = (int32_t)e;
     if (A.minima) A.minima[o] = S.minima[l];
@@ -1438,36 +1503,13 @@ struct SweepState : FamilyState {
 };
 
 
-// ISING_SWEEP_DEBUG=1: launch without graphs, synchronise and report after
-// every launch (diagnostics only).
-bool sweep_debug() {
-  static const int on = [] {
-    const char *v = std::getenv("ISING_SWEEP_DEBUG");
-    return v && v[0] == '1' ? 1 : 0;
-  }();
-  return on != 0;
-}
-
-void debug_step(const char *what, int c, cudaStream_t s) {
-  if (!sweep_debug()) return;
-  const cudaError_t e1 = cudaGetLastError();
-  const cudaError_t e2 = cudaStreamSynchronize(s);
-  std::fprintf(stderr, "[sweep] %s %d: launch=%s sync=%s\n", what, c, cudaGetErrorString(e1), cudaGetErrorString(e2));
-  std::fflush(stderr);
-}
-
-constexpr size_t visit_smem(int, int, bool) {
-  return 0;  // the visits keep their per-position data in registers
-}
-
 // Launch, with programmatic stream serialization when pdl is set (see
 // pdl_prologue); a launch error is left for the caller's cudaGetLastError.
 template <typename... KArgs, typename... Args>
-void launch_pdl(bool pdl, void (*kern)(KArgs...), int grid, int block, size_t smem, cudaStream_t s, Args... args) {
+void launch_pdl(bool pdl, void (*kern)(KArgs...), dim3 grid, int block, cudaStream_t s, Args... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1477,65 +1519,64 @@ void launch_pdl(bool pdl, void (*kern)(KArgs...), int grid, int block, size_t sm
   cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-template <int MODE, int LPS, bool LAT>
-void enqueue_visit(const SweepArgs &A, int c, int grid, cudaStream_t s) {
-  launch_pdl(A.pdl != 0, sweep_visit<MODE, LPS, LAT>, grid, kST, visit_smem(MODE, LPS, LAT), s, A, (int32_t)c);
-  debug_step("visit", c, s);
-}
-
-template <int LPS, bool LAT>
-void enqueue_round_end(const SweepArgs &A, int mode, cudaStream_t s) {
-  if (mode == 1) launch_pdl(A.pdl != 0, sweep_energy<true, LPS, LAT>, A.grid_e, kST, 0, s, A);
-  else launch_pdl(A.pdl != 0, sweep_energy<false, LPS, LAT>, A.grid_e, kST, 0, s, A);
-  debug_step("energy", 0, s);
-  launch_pdl(A.pdl != 0, sweep_restart<LPS>, A.grid_e, kST, 0, s, A);
-  debug_step("restart", 0, s);
-}
-
-template <int LPS, bool LAT>
-void enqueue_sweep(const SweepArgs &A, int mode, int ncls, int grid_v, cudaStream_t s, bool round_end = true) {
-  for (int c = 0; c < ncls; ++c) {
-    if (mode == 0) enqueue_visit<0, LPS, LAT>(A, c, grid_v, s);
-    else if (mode == 1) enqueue_visit<1, LPS, LAT>(A, c, grid_v, s);
-    else enqueue_visit<2, LPS, LAT>(A, c, grid_v, s);
+// Where a run stands: the current copy of the groups' state, the sweeps enqueued
+// (modulo 4: the `any` sets) and whether the last one's end is due.
+struct Phase {
+  GroupState *copy[2];
+  int cur = 0, sweep = 0;
+  bool due = false;
+};
+// the arguments of the next kernel, which works out the end of a sweep that is due
+SweepArgs at_phase(const SweepArgs &A, Phase &ph) {
+  SweepArgs B = A;
+  B.gs = ph.copy[ph.cur];
+  B.nxt = nullptr;
+  if (ph.due) {
+    B.nxt = ph.copy[ph.cur ^ 1];
+    B.any_r = A.any4 + ((ph.sweep + 3) & 3) * A.G;
+    ph.cur ^= 1;
+    ph.due = false;
   }
-  launch_pdl(A.pdl != 0, sweep_end, (A.G + 7) / 8, 256, 0, s, A);
-  debug_step("end", 0, s);
-  if (round_end) enqueue_round_end<LPS, LAT>(A, mode, s);
+  B.any_w = A.any4 + (ph.sweep & 3) * A.G;
+  B.any_z = nullptr;
+  return B;
+}
+
+template <int LPS, bool LAT>
+void enqueue_sweep(const SweepArgs &A, Phase &ph, int mode, const std::vector<int2> &cls, dim3 grid, cudaStream_t s,
+                   bool round_end) {
+  const int ncls = A.sequential ? A.I.n : (int)cls.size();
+  for (int c = 0; c < ncls; ++c) {
+    SweepArgs B = at_phase(A, ph);
+    if (c == 0) B.any_z = A.any4 + ((ph.sweep + 1) & 3) * A.G;
+    const int32_t c0 = A.sequential ? c : cls[c].x, c1 = A.sequential ? c + 1 : cls[c].y;
+    if (mode == 0) launch_pdl(A.pdl != 0, sweep_visit<0, LPS, LAT>, grid, kST, s, B, (int32_t)c, c0, c1);
+    else if (mode == 1) launch_pdl(A.pdl != 0, sweep_visit<1, LPS, LAT>, grid, kST, s, B, (int32_t)c, c0, c1);
+    else launch_pdl(A.pdl != 0, sweep_visit<2, LPS, LAT>, grid, kST, s, B, (int32_t)c, c0, c1);
+  }
+  ph.due = true;
+  ph.sweep = (ph.sweep + 1) & 3;
+  if (!round_end) return;
+  const SweepArgs B = at_phase(A, ph);
+  if (mode == 1) launch_pdl(A.pdl != 0, sweep_energy<true, LPS, LAT>, dim3(A.grid_e), kST, s, B);
+  else launch_pdl(A.pdl != 0, sweep_energy<false, LPS, LAT>, dim3(A.grid_e), kST, s, B);
+  launch_pdl(A.pdl != 0, sweep_restart<LPS>, dim3(A.grid_e), kST, s, at_phase(A, ph));
 }
 
 // Load every kernel of this configuration before any graph capture, so the
-// capture never triggers module loading.
+// capture never triggers module loading; resident CTAs per SM of the visits.
 template <int LPS, bool LAT>
-cudaError_t preload(int mode) {
+cudaError_t preload(int mode, int *ctas_per_sm) {
   cudaFuncAttributes fa;
-  cudaError_t e = cudaSuccess;
-  if (mode == 0) e = cudaFuncGetAttributes(&fa, sweep_visit<0, LPS, LAT>);
-  else if (mode == 1) {
-    e = cudaFuncSetAttribute(sweep_visit<1, LPS, LAT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)visit_smem(1, LPS, LAT));
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, sweep_visit<1, LPS, LAT>);
-  }
-  else e = cudaFuncGetAttributes(&fa, sweep_visit<2, LPS, LAT>);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, sweep_end);
+  const void *visit = mode == 0   ? (const void *)sweep_visit<0, LPS, LAT>
+                      : mode == 1 ? (const void *)sweep_visit<1, LPS, LAT>
+                                  : (const void *)sweep_visit<2, LPS, LAT>;
+  cudaError_t e = cudaFuncGetAttributes(&fa, visit);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, sweep_energy<true, LPS, LAT>);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, sweep_energy<false, LPS, LAT>);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, sweep_restart<LPS>);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, visit, kST, 0);
   return e;
-}
-
-// Resident CTAs per SM of the visit kernel of this configuration.
-template <int LPS, bool LAT>
-int visit_ctas_per_sm(int mode) {
-  int k = 0;
-  cudaError_t e;
-  if (mode == 0)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, sweep_visit<0, LPS, LAT>, kST, visit_smem(0, LPS, LAT));
-  else if (mode == 1)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, sweep_visit<1, LPS, LAT>, kST, visit_smem(1, LPS, LAT));
-  else
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, sweep_visit<2, LPS, LAT>, kST, visit_smem(2, LPS, LAT));
-  return (e == cudaSuccess && k > 0) ? k : 8;
 }
 
 template <int LPS, bool LAT>
@@ -1543,28 +1584,38 @@ cudaError_t run_instance(ising_handle *h, SweepArgs A, int mode, cudaStream_t s)
   SweepState &S = family_state<SweepState>(h->sweep_st);
   const InstDesc &I = A.I;
   const int ncls = A.sequential ? I.n : I.ncls;
+  std::vector<int2> cls;  // the classes' position ranges
   int maxcls = 1;
-  if (A.sequential) maxcls = 1;
-  else
-    for (int c = 0; c < I.ncls; ++c)
-      maxcls = std::max(maxcls, h->h_cls[I.cls_off + c + 1] - h->h_cls[I.cls_off + c]);
-  const int64_t items = mode == 2 ? (int64_t)A.G * maxcls : (int64_t)A.G * ((maxcls + 32 / LPS - 1) / (32 / LPS)) * 32;
-  cudaError_t e0 = preload<LPS, LAT>(mode);
-  if (e0 != cudaSuccess) return e0;
-  // one wave of resident CTAs at most: the visits loop over their positions,
-  // so a larger grid only adds CTA start-up and barrier cost per visit
-  const int grid_v = (int)std::max<int64_t>(
-      1, std::min<int64_t>((items + kST - 1) / kST, (int64_t)h->sm_count * visit_ctas_per_sm<LPS, LAT>(mode)));
-  if (sweep_debug())
-    std::fprintf(stderr, "[sweep] n=%d ncls=%d G=%d LPS=%d mode=%d grid_v=%d grid_e=%d lattice=%d seq=%d\n", I.n,
-                 ncls, A.G, LPS, mode, grid_v, A.grid_e, A.lattice, A.sequential);
+  if (!A.sequential)
+    for (int c = 0; c < I.ncls; ++c) {
+      cls.push_back(make_int2(h->h_cls[I.cls_off + c], h->h_cls[I.cls_off + c + 1]));
+      maxcls = std::max(maxcls, cls[c].y - cls[c].x);
+    }
+  int ctas_per_sm = 0;
+  cudaError_t e = preload<LPS, LAT>(mode, &ctas_per_sm);
+  if (e != cudaSuccess) return e;
+  // One wave of resident CTAs at most: the visits loop over their positions, so a
+  // larger grid only adds CTA start-up and barrier cost per visit.  The lane
+  // visits' groups are spread over the grid's y as far as every group keeps a warp
+  // for each step of the largest class.
+  constexpr int kW = kST / 32;
+  const int64_t slots = (int64_t)h->sm_count * std::max(1, ctas_per_sm);
+  const int64_t step = mode == 2 ? 32 : ((mode == 1 && LAT) ? 32 : 32 / LPS);
+  const int64_t need = ((maxcls + step - 1) / step + kW - 1) / kW;  // CTAs of one group
+  const int64_t gy = mode == 2 ? 1 : ((mode == 1 && LAT) ? A.G : std::max<int64_t>(1, std::min<int64_t>(A.G, slots / need)));
+  const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(need, slots / gy)), (unsigned)gy);
+  // Programmatic launches: measured faster for the multi-spin-coded visits and for
+  // FP32 lattices whose classes leave warps idle (45^3, 21 replicas: 1533 against
+  // 1653 us), slower for larger ones (100^3, 16 replicas: 49.4 against 48.3 ms) and
+  // on general graphs (3801 against 3753 us)
+  A.pdl = mode == 2 || (mode == 1 && LAT && need * A.G * 2 <= slots);
+  Phase ph;
+  ph.copy[0] = A.gs;
+  ph.copy[1] = A.gs + A.G;
   sweep_init<<<1, 32, 0, s>>>(A);
-  debug_step("init", 0, s);
   sweep_restart<LPS><<<A.grid_e, kST, 0, s>>>(A);
   h->launches += 2;
-  debug_step("restart0", 0, s);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // The round-end kernels (energy pass, restarts) follow every kRoundEnd-th
   // sweep of a captured chunk: most of their launches find no round ended, and
   // a group whose round ended only waits (no active lane: it visits and counts
@@ -1575,30 +1626,33 @@ cudaError_t run_instance(ising_handle *h, SweepArgs A, int mode, cudaStream_t s)
   int64_t max_sweeps_total = (int64_t)A.restarts * (A.max_sweeps + kRoundEnd) + A.restarts;
   if (A.budget > 0)
     max_sweeps_total =
-        std::min<int64_t>(max_sweeps_total, (int64_t)A.R * A.budget * kRoundEnd + A.max_sweeps + kRoundEnd);
+        std::min<int64_t>(max_sweeps_total, (int64_t)A.Rn * A.budget * kRoundEnd + A.max_sweeps + kRoundEnd);
   // Capture a chunk of sweeps once per configuration (cached) and replay it
   // until every group is done, polling a done flag one chunk behind so the GPU
-  // always has queued work.  A graph holds at most kMaxNodes launches; when one
-  // sweep alone needs more (many colour classes, e.g. the sequential schedule)
+  // always has queued work.  A graph holds at most kMaxNodes launches and a
+  // multiple of 4 sweeps (after which the phase is what it was); when that many
+  // sweeps need more launches (many colour classes, e.g. the sequential schedule)
   // sweeps are launched directly instead.  (A device-side loop - a conditional
   // WHILE node, optionally with an IF node around the round-end kernels - was
-  // measured slightly slower on GB300, and its kernels are not visible to ncu.)
+  // measured slightly slower on GB300, and its kernels are not visible to ncu; one
+  // persistent kernel with grid barriers for the whole search no faster on a
+  // 45^3 lattice and 10 % slower on 100^3, with the visits' registers short.)
   constexpr int kMaxNodes = 512;
-  const int per_sweep = ncls + 3;
-  const bool use_graph = per_sweep <= kMaxNodes && !sweep_debug();
-  const int chunk = use_graph ? std::max(1, std::min(16, kMaxNodes / per_sweep)) : 1;
+  const int per_sweep = ncls + 2;
+  const bool use_graph = 4 * per_sweep <= kMaxNodes;
+  const int chunk = use_graph ? std::min(16, kMaxNodes / per_sweep & ~3) : 1;
   // the first sweep runs with direct launches, the rest from the graph
-  enqueue_sweep<LPS, LAT>(A, mode, ncls, grid_v, s);
+  enqueue_sweep<LPS, LAT>(A, ph, mode, cls, grid, s, true);
   h->launches += per_sweep;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   cudaGraphExec_t exec = nullptr;
   if (use_graph) {
     // everything the captured launches bake in besides the handle's own arrays
     char key[320];
-    std::snprintf(key, sizeof key, "%d/%d/%d/%d/%d/%d/%d/%d/%d/%d/%p/%d/%d/%d/%d/%p/%d/%d", A.b, A.R, A.G, A.LPS,
-                  A.max_sweeps, A.restarts, A.budget, A.refresh, A.sequential, A.lattice,
-                  (void *)A.sw, mode, grid_v, chunk, ncls, (void *)A.cflag, A.nchunk,
-                  A.en_fast + 2 * A.en_count);
+    std::snprintf(key, sizeof key, "%d/%d/%d/%d/%d/%d/%d/%d/%d/%d/%d/%d/%p/%d/%u/%u/%d/%d/%p/%d/%d/%d", A.b, A.R, A.r0,
+                  A.Rn, A.G, A.LPS, A.max_sweeps, A.restarts, A.budget, A.refresh, A.sequential, A.lattice,
+                  (void *)A.sw, mode, grid.x, grid.y, chunk, ncls, (void *)A.cflag, A.nchunk,
+                  A.en_fast + 2 * A.en_count, A.pdl);
     auto it = S.graphs.find(key);
     if (it == S.graphs.end()) {
       SweepGraph sg;
@@ -1606,8 +1660,9 @@ cudaError_t run_instance(ising_handle *h, SweepArgs A, int mode, cudaStream_t s)
       if ((e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking)) != cudaSuccess) return e;
       e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
       if (e == cudaSuccess) {
+        Phase pc = ph;
         for (int k = 0; k < chunk; ++k)
-          enqueue_sweep<LPS, LAT>(A, mode, ncls, grid_v, cs, (k % kRoundEnd) == kRoundEnd - 1 || k == chunk - 1);
+          enqueue_sweep<LPS, LAT>(A, pc, mode, cls, grid, cs, (k % kRoundEnd) == kRoundEnd - 1);
         e = cudaStreamEndCapture(cs, &sg.graph);
       }
       if (e == cudaSuccess) e = cudaGraphInstantiate(&sg.exec, sg.graph, 0);
@@ -1623,22 +1678,18 @@ cudaError_t run_instance(ising_handle *h, SweepArgs A, int mode, cudaStream_t s)
   const int64_t max_chunks = max_sweeps_total / chunk + 2;
   int64_t launched = 0;
   for (;;) {
-    // sweeps of a captured chunk without round-end kernels launch two fewer
-    int with_re = 0;
-    for (int k = 0; k < chunk; ++k) with_re += ((k % kRoundEnd) == kRoundEnd - 1 || k == chunk - 1) ? 1 : 0;
-    h->launches += (uint64_t)chunk * per_sweep - (use_graph ? (uint64_t)(chunk - with_re) * 2 : 0);
+    h->launches += (uint64_t)chunk * ncls + (use_graph ? chunk / kRoundEnd : 1) * 2;
     kt_begin(h, "sweep_chunk", s);
     if (use_graph) {
       if ((e = cudaGraphLaunch(exec, s)) != cudaSuccess) break;
     } else {
-      enqueue_sweep<LPS, LAT>(A, mode, ncls, grid_v, s);
+      enqueue_sweep<LPS, LAT>(A, ph, mode, cls, grid, s, true);
       if ((e = cudaGetLastError()) != cudaSuccess) break;
     }
     kt_end(h, s);
     cudaMemcpyAsync(S.h_done + (launched & 1), A.all_done, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
     cudaEventRecord(S.ev[launched & 1], s);
     ++launched;
-    if (sweep_debug()) std::fprintf(stderr, "[sweep] chunk %lld queued\n", (long long)launched);
     if (launched >= 2) {
       // look one chunk behind so the GPU always has queued work
       cudaEventSynchronize(S.ev[launched & 1]);
@@ -1648,13 +1699,25 @@ cudaError_t run_instance(ising_handle *h, SweepArgs A, int mode, cudaStream_t s)
   }
   if (e != cudaSuccess) return e;
   // energies of the final states of replicas that never converged
-  sweep_mark_final<<<1, 32, 0, s>>>(A);
+  const SweepArgs F = at_phase(A, ph);
+  sweep_mark_final<<<1, 32, 0, s>>>(F);
   h->launches += 3;
-  if (mode == 1) sweep_energy<true, LPS, LAT><<<A.grid_e, kST, 0, s>>>(A);
-  else sweep_energy<false, LPS, LAT><<<A.grid_e, kST, 0, s>>>(A);
-  const int64_t tot = (int64_t)A.R * I.n;
-  sweep_output<<<(int)std::min<int64_t>((tot + kST - 1) / kST, (int64_t)h->sm_count * 16), kST, 0, s>>>(A);
+  if (mode == 1) sweep_energy<true, LPS, LAT><<<A.grid_e, kST, 0, s>>>(F);
+  else sweep_energy<false, LPS, LAT><<<A.grid_e, kST, 0, s>>>(F);
+  const int64_t tot = (int64_t)A.Rn * I.n;
+  sweep_output<<<(int)std::min<int64_t>((tot + kST - 1) / kST, (int64_t)h->sm_count * 16), kST, 0, s>>>(F);
   return cudaGetLastError();
+}
+
+// Replicas of a group.  Words of 8 or 16 lanes waste none of a lattice position's
+// work on absent replicas and take the site-parallel energies; general graphs
+// share a row's reads among up to 32.  FP32 lattices, us a call in groups of 32 /
+// 16: 45^3 with 21 replicas 1760 / 1620.
+int lanes_per_spin(const ising_handle *h, int mode, bool sequential, int32_t R) {
+  if (R <= 8) return 8;
+  if (R <= 16) return 16;
+  if (mode == 1 && h->all_lattice && !sequential && R <= 512) return 16;
+  return 32;
 }
 
 }  // namespace
@@ -1676,20 +1739,20 @@ void sweep_free(ising_handle *h) {
 cudaError_t launch_sweep(ising_handle *h, const ising_search_params *p, int32_t R, int8_t *spins, double *E,
                          int32_t *E32, int32_t *minima, cudaStream_t s) {
   SweepState &S = family_state<SweepState>(h->sweep_st);
-  const int LPS = R > 16 ? 32 : (R > 8 ? 16 : 8);
-  const int G = (R + 31) / 32;
-  if (LPS < 32 && R > LPS) return cudaErrorInvalidValue;
   const bool fl = h->dtype == ISING_F32;
   const int mode = fl ? 1 : (h->msc_ok ? 2 : 0);
+  const int LPS = lanes_per_spin(h, mode, p->schedule == ISING_SCHED_SEQUENTIAL, R);
+  const int32_t Rb = std::min(R, 32 * LPS);  // replicas of one run: at most 32 groups
+  const int G = (Rb + LPS - 1) / LPS;
   const int grid_e = h->sm_count * 4;
-  // scratch: sw, fm, bw, pend [G][nmax]; F [G][nmax][LPS]; gs [G]; partial [grid_e][G][32]; eacc [G][32][2];
+  // scratch: sw, fm, bw, pend [G][nmax]; F [G][nmax][LPS]; gs [2][G]; any [4][G]; partial [grid_e][G][32]; eacc [G][32][2];
   // counter; done
   const size_t words = (size_t)G * h->nmax;
   auto up256 = [](size_t b) { return (b + 255) / 256 * 256; };
   const int32_t nchunk = (h->nmax / 2 + 31) / 32 + 1;
   const size_t cflag_bytes = (size_t)G * 2 * nchunk * sizeof(uint16_t);
-  const size_t need = 4 * up256(words * 4) + (fl ? up256(words * LPS * 4) : 0) + up256(G * sizeof(GroupState)) +
-                      up256((size_t)grid_e * G * 32 * 8) + up256((size_t)G * 32 * 16) + 2 * 256 +
+  const size_t need = 4 * up256(words * 4) + (fl ? up256(words * LPS * 4) : 0) + up256(2 * G * sizeof(GroupState)) +
+                      up256((size_t)grid_e * G * 32 * 8) + up256((size_t)G * 32 * 16) + 2 * 256 + up256((size_t)4 * G * 4) +
                       up256(cflag_bytes);
   cudaError_t e;
   if (need > S.bytes) {
@@ -1716,7 +1779,6 @@ cudaError_t launch_sweep(ising_handle *h, const ising_search_params *p, int32_t 
   SweepArgs A;
   A.g = h->graph();
   A.R = R;
-  A.G = G;
   A.LPS = LPS;
   A.max_sweeps = p->max_sweeps;
   A.restarts = p->restarts;
@@ -1728,7 +1790,11 @@ cudaError_t launch_sweep(ising_handle *h, const ising_search_params *p, int32_t 
   A.bw = (uint32_t *)take(words * 4);
   A.pend = (uint32_t *)take(words * 4);
   A.F = fl ? (float *)take(words * LPS * 4) : nullptr;
-  A.gs = (GroupState *)take(G * sizeof(GroupState));
+  A.gs = (GroupState *)take(2 * G * sizeof(GroupState));
+  A.nxt = nullptr;
+  A.any_r = nullptr;
+  A.any_w = A.any_z = nullptr;
+  A.any4 = (uint32_t *)take((size_t)4 * G * 4);
   A.grid_e = grid_e;
   A.partial = (double *)take((size_t)grid_e * G * 32 * 8);
   A.eacc = (unsigned long long *)take((size_t)G * 32 * 16);
@@ -1757,11 +1823,7 @@ cudaError_t launch_sweep(ising_handle *h, const ising_search_params *p, int32_t 
       A.en_fast = (A.lattice && LPS <= 16 && A.I.ebits >= 0 && A.I.ebits + lg + 1 <= 62) ? 1 : 0;
       // bit-sliced counts: at most 4 terms per site, sites_lane sites per lane, below 2^8
       A.en_count = (A.lattice && mode == 2 && 4 * sites_lane <= 255) ? 1 : 0;
-      A.pdl = mode == 2 ? 1 : 0;
     }
-    if ((e = cudaMemsetAsync(A.fm, 0, words * 4, s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(A.eacc, 0, (size_t)G * 32 * 16, s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(A.pend, 0, words * 4, s)) != cudaSuccess) return e;
     // chunk flags: the two-class parity colouring of an even-sided lattice puts
     // site j at class position j >> 1 (class order is index order)
     // (FP32 lattices only: in the multi-spin-coded visits, a thread per site,
@@ -1779,17 +1841,25 @@ cudaError_t launch_sweep(ising_handle *h, const ising_search_params *p, int32_t 
     }
     // (the flagged visits find their sites by that division)
     A.cflag = (chunked && A.divL_m) ? cflag_mem : nullptr;
-    if (A.cflag && (e = cudaMemsetAsync(cflag_mem, 0, cflag_bytes, s)) != cudaSuccess) return e;
-    if (A.lattice) {
-      if (LPS == 32) e = run_instance<32, true>(h, A, mode, s);
-      else if (LPS == 16) e = run_instance<16, true>(h, A, mode, s);
-      else e = run_instance<8, true>(h, A, mode, s);
-    } else {
-      if (LPS == 32) e = run_instance<32, false>(h, A, mode, s);
-      else if (LPS == 16) e = run_instance<16, false>(h, A, mode, s);
-      else e = run_instance<8, false>(h, A, mode, s);
+    A.site_arith = A.divL_m && h->lat_parity && A.I.ncls == 2 && A.I.lat_L % 2 == 0;
+    for (A.r0 = 0; A.r0 < R; A.r0 += Rb) {
+      A.Rn = std::min(Rb, R - A.r0);
+      A.G = (A.Rn + LPS - 1) / LPS;
+      if ((e = cudaMemsetAsync(A.fm, 0, words * 4, s)) != cudaSuccess) return e;
+      if ((e = cudaMemsetAsync(A.eacc, 0, (size_t)G * 32 * 16, s)) != cudaSuccess) return e;
+      if ((e = cudaMemsetAsync(A.pend, 0, words * 4, s)) != cudaSuccess) return e;
+      if (A.cflag && (e = cudaMemsetAsync(cflag_mem, 0, cflag_bytes, s)) != cudaSuccess) return e;
+      if (A.lattice) {
+        if (LPS == 32) e = run_instance<32, true>(h, A, mode, s);
+        else if (LPS == 16) e = run_instance<16, true>(h, A, mode, s);
+        else e = run_instance<8, true>(h, A, mode, s);
+      } else {
+        if (LPS == 32) e = run_instance<32, false>(h, A, mode, s);
+        else if (LPS == 16) e = run_instance<16, false>(h, A, mode, s);
+        else e = run_instance<8, false>(h, A, mode, s);
+      }
+      if (e != cudaSuccess) return e;
     }
-    if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }

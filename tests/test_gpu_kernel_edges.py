@@ -53,6 +53,34 @@ def test_sweep_general_graph_fp64_refresh(R):
     _compare([inst], [R], R, False, max_sweeps=400, restarts=2, refresh_every=2, kernel=isg.KERNEL_SWEEP)
 
 
+# Groups of 16 replicas on FP32 lattices (odd and even sides, a last group with
+# one replica and with 15), chunks of 4, 8 and 16 sweeps and none (by the number
+# of classes), and more replicas than one run's 32 groups hold.
+@pytest.mark.parametrize("dims,R", [((9, 9, 9), 17), ((12, 12), 31), ((10, 10, 10), 40), ((7, 7), 513)])
+def test_sweep_fp32_lattice_groups(dims, R):
+    inst = W.lattice(dims, True, "gauss", "gauss", seed=sum(dims))
+    _compare([inst], [R], R, False, max_sweeps=300, restarts=3, refresh_every=5, kernel=isg.KERNEL_SWEEP)
+
+
+@pytest.mark.parametrize("dtype,R", [("i8", 1030), ("f32", 1025)])
+def test_sweep_more_replicas_than_one_run(dtype, R):
+    inst = W.random_graph(60, 4.0, 71, dtype=dtype, n_hyper=8)
+    _compare([inst], [R], R, dtype == "i8", max_sweeps=60, restarts=2, kernel=isg.KERNEL_SWEEP)
+
+
+@pytest.mark.parametrize("ncls", [30, 60, 120, 130])
+def test_sweep_chunk_lengths(ncls):
+    n = 2 * ncls
+    inst = W.random_graph(n, 3.0, ncls, dtype="f32")
+    order = np.random.default_rng(ncls).permutation(n)
+    inst.colour = np.empty(n, np.int32)
+    inst.colour[order] = np.arange(n) % ncls  # classes of two spins; conflicting pairs get a class of their own
+    rows = np.repeat(np.arange(n), np.diff(inst.row_ptr))
+    clash = np.unique(rows[inst.colour[rows] == inst.colour[inst.col]])
+    inst.colour[clash] = ncls + np.arange(len(clash))
+    _compare([inst], [ncls], 9, False, max_sweeps=200, restarts=3, refresh_every=4, kernel=isg.KERNEL_SWEEP)
+
+
 # Tiles cut into segments of descents: more descents than segments and fewer,
 # descents that never converge (the last one's state is the result) or only some,
 # ragged replica groups, both schedules, every mode of the tile kernels.
