@@ -148,6 +148,18 @@ __device__ __forceinline__ uint32_t warp_transpose32(uint32_t v, int lane) {
   return v;
 }
 
+// 32 spins of one replica (bit u = spin u is +1) as bytes +1 / -1 at out: eight
+// words of four bytes, a nibble's bits spread by one multiplication (bit b to bit
+// 8 b; the partial products do not meet), 0xff ^ 0xfe where the bit is set.
+__device__ __forceinline__ void store_spins32(int8_t *out, uint32_t bits) {
+  uint32_t w[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q)
+    w[q] = ~((((bits >> (4 * q)) & 0xfu) * 0x00204081u & 0x01010101u) * 0xfeu);
+  reinterpret_cast<uint4 *>(out)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+  reinterpret_cast<uint4 *>(out)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+}
+
 // Warp total of bit-sliced per-lane counters: plane q of every lane holds bit
 // q of 32 counters (one per bit position r).  A butterfly of bit-sliced adds
 // leaves every lane with the warp-wide sums (Q + 5 planes); lane r then reads

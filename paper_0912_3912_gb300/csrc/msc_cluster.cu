@@ -10,18 +10,22 @@
 // memory.  The two checkerboard classes are separated by cluster barriers, so
 // one lattice uses P SMs instead of one.
 //
-// Work layout: a warp visits a chunk of 64 consecutive sites per step, lane t
-// taking the t-th site of the current class in the chunk (each row segment of
-// even length holds equally many sites of both parities), so all 32 lanes do
-// useful work and site indices, neighbours and wrap-around follow from the
-// coordinates.  Coupling signs and the field of every site are one byte in
-// shared memory.  Pending flags per (class, chunk) say whether some site of the
-// class in the chunk has a neighbour that flipped since its last visit; a chunk
-// without one is stable and skipped (only the first sweep of a descent visits
-// everything).  All per-lane bookkeeping (sweep counts, convergence, best
-// energies) is replicated identically in every CTA of the cluster, so the
-// cluster's control flow stays uniform and every barrier is matched.
+// Work layout: words lie by colour class, the site o of a CTA at place o >> 1 of
+// its class's half (each row holds equally many sites of both parities).  A
+// warp visits a chunk of 64 consecutive sites per step, lane t taking place t of
+// the current class in the chunk; its neighbours are then the places t and t + 1
+// or t - 1 of the row in the other class and the same places of the rows above and
+// below, so the warp reads consecutive words (by site index they would lie two
+// apart, two words to a bank) and the slab axis's remote reads are uniform.
+// Coupling signs and the field of every site are one byte in shared memory.
+// Pending flags per (class, chunk) say whether some site of the class in the chunk
+// has a neighbour that flipped since its last visit; a chunk without one is
+// stable and skipped (only the first sweep of a descent visits everything).  All
+// per-lane bookkeeping (sweep counts, convergence, best energies) is replicated
+// identically in every CTA of the cluster, so the cluster's control flow stays
+// uniform and every barrier is matched.  C2NOTE
 #include <cfloat>
+#include <type_traits>
 
 #include "device_common.cuh"
 #include "tc.cuh"
@@ -34,7 +38,10 @@ namespace {
 // 8, measured slower on the 32^3 lattice)
 constexpr int kCT = 512;
 
-template <int D>
+// MASKS: the signs and fields as bytes of 0 or -1, one plane per direction and two
+// for the field, which the loads extend to whole words; else packed in one byte
+// per site (large slabs, for shared memory's sake).
+template <int D, bool MASKS>
 __global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const TileArgs *__restrict__ Aptr, int P) {
   extern __shared__ uint32_t smem[];
   __shared__ uint32_t s_any[2], s_active, s_convround, s_upd;
@@ -55,46 +62,81 @@ __global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const TileArgs *__r
   const int lgc = 31 - __clz(csz);
   const int nch = csz >> 6;  // 64-site chunks per CTA
   const int lo = (int)rank * csz;
-  uint32_t *sw = smem;                                          // words of sites lo .. lo + csz - 1
+  const int half = csz >> 1, hl = L >> 1, lghl = lgL - 1;       // places per class, per row
+  uint32_t *sw = smem;                                          // [2][half] words of sites lo .. lo + csz - 1
   uint32_t *pend = smem + csz;                                  // [2][nch] pending flags
-  uint8_t *tab = reinterpret_cast<uint8_t *>(smem + csz + 2 * nch);  // [csz]: neg bits 0..5, h != 0, h > 0
-  uint32_t *bw = smem + csz + 2 * nch + csz / 4;                      // [csz]: best words of my sites
+  uint32_t *bw = smem + csz + 2 * nch;                          // [2][half]: best words of my sites
+  // [2][half]: coupling signs (0 the x neighbour at the same place, 1 the other one,
+  // 2, 3 +y, -y, 4, 5 +z, -z), h != 0, h > 0: bits of a byte, or eight planes
+  uint8_t *tab = reinterpret_cast<uint8_t *>(smem + 2 * csz + 2 * nch);
   const int rem = A.R - 32 * g;
   const uint32_t lane_valid = rem >= 32 ? 0xffffffffu : ((1u << rem) - 1u);
   const uint64_t seed = A.seeds[b];
   const int64_t so = I.spin_off;
-  const int lgp = min(lgL, 6) - 1;  // log2 of the class sites per row segment of a chunk
-  unsigned long long my_flips = 0, my_evals = 0, my_sweeps = 0, my_minima = 0, my_desc = 0;
+  unsigned long long my_evals = 0, my_sweeps = 0, my_minima = 0, my_desc = 0;
+  uint32_t my_flips = 0;  // of the current sweep
+  unsigned long long all_flips = 0;
   unsigned long long my_eval = 0;  // (site, replica) pairs of the chunks visited (skipped chunks excluded)
 
-  // word of site j (any CTA of the cluster).  Only neighbours along the slab
-  // axis (z in 3D, y in 2D) can lie in another CTA, and a warp's sites share
-  // that axis coordinate, so the branch is uniform.
-  auto word = [&](int j) -> uint32_t {
-    const uint32_t owner = (uint32_t)j >> lgc;
-    if (owner == rank) return sw[j - lo];
-    return tc::ld_cluster_u32(tc::map_shared(sw + (j & (csz - 1)), owner));
+  // class of global site j; place of a site of mine: cls * half + ((j - lo) >> 1)
+  auto cls_of = [&](int j) -> int { return (j + (j >> lgL) + (D == 3 ? j >> (2 * lgL) : 0)) & 1; };
+  auto place = [&](int j) -> int { return cls_of(j) * half + ((j - lo) >> 1); };
+  // The neighbour words of place q of class c: x[0], x[1] in the row (the same place
+  // of the other class, and the one beside it), then +y, -y (and +z, -z).  Only
+  // neighbours along the slab axis (z in 3D, y in 2D) can lie in another CTA: those of
+  // the slab's first and last step along it (`edge`; a chunk has one such coordinate).
+  const int sstep = D == 3 ? hl << lgL : hl;  // places per step along the slab axis
+  auto nwords = [&](auto edge, int c, int q, uint32_t (&x)[6]) {
+    const uint32_t *oth = sw + (c ^ 1) * half;
+    const int row = q >> lghl;  // local row
+    const int s = ((lo >> lgL) + row + (D == 3 ? (lo >> (2 * lgL)) + (row >> lgL) : 0) + c) & 1;
+    x[0] = oth[q];
+    x[1] = oth[(q & ~(hl - 1)) | ((q + (s ? 1 : -1)) & (hl - 1))];  // (s: the site's x is odd)
+    if (D == 3) {
+      const int ym = (L - 1) << lghl;
+      x[2] = oth[(q & ~ym) | ((q + hl) & ym)];
+      x[3] = oth[(q & ~ym) | ((q - hl) & ym)];
+    }
+#pragma unroll
+    for (int dn = 0; dn < 2; ++dn) {
+      const int t = dn ? q - sstep : q + sstep;
+      uint32_t w;
+      if (!decltype(edge)::value || (t >= 0 && t < half))
+        w = oth[t];
+      else
+        w = tc::ld_cluster_u32(tc::map_shared(oth + (t & (half - 1)), (rank + (dn ? P - 1 : 1)) & (P - 1)));
+      x[2 * D - 2 + dn] = w;
+    }
   };
-  auto mark = [&](int j, int cls) {
-    const uint32_t owner = (uint32_t)j >> lgc;
-    uint32_t *f = pend + cls * nch + ((j & (csz - 1)) >> 6);
-    if (owner == rank) *f = 1u;
-    else tc::st_cluster_u32(tc::map_shared(f, owner), 1u);
+  // Chunks holding the neighbours of a chunk's flipped sites (lanes: one target
+  // each): the chunk itself, those of the rows above and below, of the planes above
+  // and below and, in rows longer than a chunk, the next ones in the row; a lane's
+  // target is due when one of the flipping lanes in its mask m_from flipped.
+  //   target = (ch & ~m_wrap) | ((ch + m_step) & m_wrap), in the CTA m_rank once it
+  //   leaves the slab
+  const int cpr = L > 64 ? L >> 6 : 1, cpp = (L * L) >> 6;  // chunks per row, per plane
+  const int m_edge = D == 3 ? cpp : cpr;  // chunks of the slab's first (last) step
+  const uint32_t m_inner = __ballot_sync(0xffffffffu, warp + lane * nwarps >= m_edge && warp + lane * nwarps < nch - m_edge);
+  uint32_t m_from = 0u;
+  int m_step = 0, m_wrap = 0, m_rank = (int)rank;
+  {
+    const int dir = lane & 1 ? 1 : -1, kind = lane == 0 ? 0 : (lane + 1) >> 1;  // lanes 1, 2: y; 3, 4: z; 5, 6: x
+    const uint32_t lastrow = hl >= 32 ? 0xffffffffu : ~0u << (32 - hl), firstrow = hl >= 32 ? 0xffffffffu : (1u << hl) - 1u;
+    const bool slab = kind == D - 1;
+    if (lane == 0) {
+      m_from = 0xffffffffu;
+    } else if (lane < 2 * D - 1 || (kind == 3 && L > 64)) {
+      m_step = dir * (kind == 3 ? 1 : (kind == 2 ? cpp : cpr));
+      m_wrap = slab ? nch - 1 : (kind == 3 ? cpr - 1 : cpp - 1);
+      m_from = kind == 3 ? (dir > 0 ? 0x80000000u : 1u) : (slab ? 0xffffffffu : (dir > 0 ? lastrow : firstrow));
+      if (slab) m_rank = (int)((rank + (dir > 0 ? 1 : P - 1)) & (P - 1));
+    }
+  }
+  // sign (or field) mask d of place o: all ones or zeros in every replica
+  auto mask = [&](int o, uint32_t t, int d) -> uint32_t {
+    if (MASKS) return (uint32_t)(int32_t)reinterpret_cast<const int8_t *>(tab)[d * csz + o];
+    return (t >> d) & 1u ? 0xffffffffu : 0u;
   };
-  // neighbour of site j in direction d (+x, -x, +y, -y, +z, -z), periodic:
-  // step the axis coordinate inside its bit field (L is a power of two)
-  auto nbr = [&](int j, int d) -> int {
-    const int sh = (d >> 1) * lgL, m = (L - 1) << sh;
-    const int t = (d & 1) ? j - (1 << sh) : j + (1 << sh);
-    return (j & ~m) | (t & m);
-  };
-  // neighbour word in direction d of a site of mine (local off the slab axis)
-  auto nword = [&](int j, int d) -> uint32_t {
-    const int nb = nbr(j, d);
-    if ((d >> 1) == D - 1) return word(nb);
-    return sw[nb - lo];
-  };
-
   // my part of each colour class (positions whose site lies in [lo, lo + csz))
   if (tid < 2) {
     const int c = tid;
@@ -128,7 +170,14 @@ __global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const TileArgs *__r
       const int j = __ldg(G.order + so + v);
       const uint32_t info = __ldg(G.latinfo + so + v);
       const int hv = __ldg(reinterpret_cast<const int8_t *>(G.h) + so + j);
-      tab[j - lo] = (uint8_t)(((info >> 8) & 63u) | (hv != 0 ? 64u : 0u) | (hv > 0 ? 128u : 0u));
+      uint32_t neg = (info >> 8) & 63u;  // by direction: +x, -x, +y, -y, +z, -z
+      if (j & 1) neg = (neg & ~3u) | ((neg >> 1) & 1u) | ((neg & 1u) << 1);  // (odd x: -x lies at the same place)
+      neg |= (hv != 0 ? 64u : 0u) | (hv > 0 ? 128u : 0u);
+      if (MASKS) {
+        for (int d = 0; d < 8; ++d) tab[d * csz + place(j)] = (neg >> d) & 1u ? 0xffu : 0u;
+      } else {
+        tab[place(j)] = (uint8_t)neg;
+      }
     }
   __syncthreads();
 
@@ -136,7 +185,7 @@ __global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const TileArgs *__r
   // sites (one site per thread, the forward bonds +x, +y, +z and the field),
   // the counts are summed over the cluster in rank order
   auto energies = [&]() {
-    constexpr int Q = 10;  // per-thread counts stay below 2^10 (csz / blockDim sites, D + 1 terms each)
+    constexpr int Q = 8;  // per-thread counts stay below 2^8: at most 32 sites of D + 1 terms (csz <= 16384)
     uint32_t acc[Q];
 #pragma unroll
     for (int q = 0; q < Q; ++q) acc[q] = 0u;
@@ -144,14 +193,23 @@ __global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const TileArgs *__r
     if (tid < 33) s_cnt[tid] = 0;
     __syncthreads();
     for (int o = tid; o < csz; o += blockDim.x) {
-      const int j = lo + o;
-      const uint32_t wj = sw[o], t = tab[o];
+      const int c = o >= half, q = o - c * half;
+      const uint32_t wj = sw[o], t = MASKS ? 0u : tab[o];
+      const uint32_t *oth = sw + (c ^ 1) * half;
+      // +x is the neighbour at the same place for even x, else the one beside it
+      const int row = q >> lghl;
+      const int odd = ((lo >> lgL) + row + (D == 3 ? (lo >> (2 * lgL)) + (row >> lgL) : 0) + c) & 1;
       uint32_t f[3] = {0u, 0u, 0u};
-#pragma unroll
-      for (int a = 0; a < 3; ++a)
-        if (a < D) f[a] = wj ^ nword(j, 2 * a) ^ (((t >> (2 * a)) & 1u) ? 0xffffffffu : 0u);
-      const uint32_t uf = (t & 64u) ? ((t & 128u) ? ~wj : wj) : 0u;
-      nz += (t & 64u) ? 1 : 0;
+      f[0] = wj ^ oth[(q & ~(hl - 1)) | ((q + odd) & (hl - 1))] ^ mask(o, t, odd);
+      if (D == 3) {
+        const int ym = (L - 1) << lghl;
+        f[1] = wj ^ oth[(q & ~ym) | ((q + hl) & ym)] ^ mask(o, t, 2);
+      }
+      const int up = q + sstep;
+      f[D - 1] = wj ^ mask(o, t, 2 * D - 2) ^
+                 (up < half ? oth[up] : tc::ld_cluster_u32(tc::map_shared(oth + (up - half), (rank + 1) & (P - 1))));
+      const uint32_t field = mask(o, t, 6), uf = (wj ^ mask(o, t, 7)) & field;
+      nz += field & 1u;
       const uint32_t s1 = f[0] ^ f[1] ^ f[2], c1 = (f[0] & f[1]) | (f[0] & f[2]) | (f[1] & f[2]);
       const uint32_t s2 = s1 ^ uf, c2 = s1 & uf;
       const uint32_t t1 = c1 ^ c2, t2 = c1 & c2;
@@ -170,14 +228,19 @@ __global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const TileArgs *__r
         cy = c;
       }
     }
-    const long long mine = warp_sliced_total<Q>(acc, lane);  // lane r: replica r's warp total
+    // lane r: replica r's warp total (a plane's transpose counts its bits: a third
+    // of the exchanges of adding the planes across the lanes)
+    int mine = 0;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) mine += __popc(warp_transpose32(acc[q], lane)) << q;
     nz = warp_sum(nz);
-    atomicAdd(&s_cnt[lane], (int)mine);
+    atomicAdd(&s_cnt[lane], mine);
     if (lane == 0) atomicAdd(&s_cnt[32], nz);
     __syncthreads();
     tc::cluster_sync();
     if (tid < 32) {
       long long u = 0, z = 0;
+#pragma unroll 4
       for (int c = 0; c < P; ++c) {
         u += (int)tc::ld_cluster_u32(tc::map_shared(&s_cnt[tid], (uint32_t)c));
         z += (int)tc::ld_cluster_u32(tc::map_shared(&s_cnt[32], (uint32_t)c));
@@ -207,8 +270,8 @@ __global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const TileArgs *__r
       for (int q = 0; q < 4; ++q) {
         const uint32_t xw = word_of(x, q);
         const uint32_t mine = warp_transpose32(xw, lane);  // lane u: site u's word
-        const int o = w * 128 + q * 32 + lane - lo;
-        sw[o] = (sw[o] & ~active) | (mine & active);
+        const int o = place(w * 128 + q * 32 + lane);
+        sw[o] = active == lane_valid ? mine : (sw[o] & ~active) | (mine & active);
       }
     }
     tc::cluster_sync();
@@ -218,27 +281,26 @@ __global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const TileArgs *__r
       const int pb = sc & 1;
       uint32_t anyf = 0;
       for (int c = 0; c < 2; ++c) {
-        for (int ch = warp; ch < nch; ch += nwarps) {
-          uint32_t *pf = pend + c * nch + ch;
-          if (!fresh && !*pf) continue;  // no site of the class here has a neighbour that flipped
-          __syncwarp();
-          if (lane == 0) {
-            *pf = 0u;  // marks made in this phase go to the other class
-            my_eval += 32ull * (unsigned long long)__popc(active);
-          }
-          // lane's site: the lane-th site of class c in the chunk
-          const int r = lane >> lgp, q = lane & ((1 << lgp) - 1);
-          const int rowbase = lo + (ch << 6) + (r << (lgp + 1));
-          const int yz = (rowbase >> lgL) + (D == 3 ? (rowbase >> (2 * lgL)) : 0);
-          const int j = rowbase + 2 * q + ((yz + c) & 1);
-          const uint32_t wj = sw[j - lo], t = tab[j - lo];
-          uint32_t x[6];
+        // the warp's chunks ch = warp + k nwarps: lane k reads chunk k's flag
+        const int mych = warp + lane * nwarps;
+        const bool pending = mych < nch && (fresh || pend[c * nch + mych]);
+        if (pending) pend[c * nch + mych] = 0u;  // marks made in this phase go to the other class
+        uint32_t todo = __ballot_sync(0xffffffffu, pending);
+        if (lane == 0) my_eval += 32ull * (unsigned long long)(__popc(active) * __popc(todo));
+        // one chunk: its words, then its decisions and the pending flags of the chunks
+        // holding the flipped sites' neighbours (few branches: they cost more than what
+        // they skip)
+        auto load = [&](auto edge, int ch, uint32_t &wj, uint32_t &uf, uint32_t (&x)[6]) {
+          const int q = ch * 32 + lane, o = c * half + q;
+          wj = sw[o];
+          const uint32_t t = MASKS ? 0u : tab[o];
+          nwords(edge, c, q, x);
+          uf = (wj ^ mask(o, t, 7)) & mask(o, t, 6);
 #pragma unroll
-          for (int dd = 0; dd < 6; ++dd) {
-            x[dd] = 0u;
-            if (dd < 2 * D) x[dd] = wj ^ nword(j, dd) ^ (((t >> dd) & 1u) ? 0xffffffffu : 0u);
-          }
-          const uint32_t uf = (t & 64u) ? ((t & 128u) ? ~wj : wj) : 0u;
+          for (int dd = 0; dd < 2 * D; ++dd) x[dd] ^= wj ^ mask(o, t, dd);
+        };
+        auto decide = [&](auto edge, int ch, uint32_t wj, uint32_t uf, uint32_t (&x)[6]) {
+          const int q = ch * 32 + lane;
           const uint32_t s1 = x[0] ^ x[1] ^ x[2], c1 = (x[0] & x[1]) | (x[0] & x[2]) | (x[1] & x[2]);
           uint32_t flip;
           if (D == 3) {
@@ -250,37 +312,52 @@ __global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const TileArgs *__r
             flip = (c1 & c2) | ((c1 | c2) & s2);
           }
           flip &= active;
-          if (flip) {
-            sw[j - lo] = wj ^ flip;
-            anyf |= flip;
-            my_flips += __popc(flip);
-          }
-          // Pending flags of the chunks holding the flipped sites' neighbours.
-          // Per direction those chunks are at most two, and lanes are ordered
-          // so that they are the targets of the lowest and the highest
-          // flipping lane (checked exhaustively for every accepted shape).
+          sw[c * half + q] = wj ^ flip;
+          anyf |= flip;
+          my_flips += __popc(flip);
           const uint32_t fb = __ballot_sync(0xffffffffu, flip != 0u);
-          if (fb) {
-            const int jl = __shfl_sync(0xffffffffu, j, __ffs(fb) - 1);
-            const int jh = __shfl_sync(0xffffffffu, j, 31 - __clz(fb));
-            if (lane < 4 * D) {
-              const int dd = lane < 2 * D ? lane : lane - 2 * D;
-              mark(nbr(lane < 2 * D ? jl : jh, dd), c ^ 1);
-            }
-          }
+          const int t0 = ch + m_step;
+          uint32_t *f = pend + (c ^ 1) * nch + ((ch & ~m_wrap) | (t0 & m_wrap));
+          const bool due = fb & m_from, far = decltype(edge)::value && m_rank != (int)rank && (t0 < 0 || t0 >= nch);
+          if (due && !far) *f = 1u;
+          if (due && far) tc::st_cluster_u32(tc::map_shared(f, (uint32_t)m_rank), 1u);
+        };
+        // the slab's inner chunks two at a time (a class's sites do not read each other)
+        uint32_t inner = todo & m_inner, outer = todo & ~m_inner;
+        while (inner) {
+          const int a = warp + (__ffs(inner) - 1) * nwarps;
+          inner &= inner - 1u;
+          const bool two = inner != 0u;
+          const int b2 = two ? warp + (__ffs(inner) - 1) * nwarps : a;
+          inner &= inner - 1u;
+          uint32_t wa, ta, xa[6], wb, tb, xb[6];
+          load(std::false_type(), a, wa, ta, xa);
+          load(std::false_type(), b2, wb, tb, xb);
+          decide(std::false_type(), a, wa, ta, xa);
+          if (two) decide(std::false_type(), b2, wb, tb, xb);
+        }
+        while (outer) {
+          const int ch = warp + (__ffs(outer) - 1) * nwarps;
+          outer &= outer - 1u;
+          uint32_t wj, t, x[6];
+          load(std::true_type(), ch, wj, t, x);
+          decide(std::true_type(), ch, wj, t, x);
         }
         if (c == 1) {
+          // this warp's flipped replicas to every CTA of the cluster
           anyf = __reduce_or_sync(0xffffffffu, anyf);
-          if (lane == 0 && anyf) atomicOr(&s_any[pb], anyf);
+          if (lane < P && anyf)
+            asm volatile("red.relaxed.cluster.shared::cluster.or.b32 [%0], %1;" ::"r"(
+                             tc::map_shared(&s_any[pb], (uint32_t)lane)),
+                         "r"(anyf)
+                         : "memory");
         }
         tc::cluster_sync();  // class done in every CTA: its flips, marks and flags visible
-        // every CTA read the other buffer's flags before this barrier: reset it
+        // (the other buffer was read after the last sweep; peers add to it after the next barrier)
         if (c == 0 && tid == 0) s_any[pb ^ 1] = 0u;
       }
       if (warp == 0) {
-        // lane = replica; lanes < P read the peers' convergence words
-        const uint32_t any = __reduce_or_sync(
-            0xffffffffu, lane < P ? tc::ld_cluster_u32(tc::map_shared(&s_any[pb], (uint32_t)lane)) : 0u);
+        const uint32_t any = s_any[pb];  // lane = replica
         const bool act = (active >> lane) & 1u;
         int tot = s_total[lane];
         if (act) s_total[lane] = ++tot;
@@ -297,6 +374,8 @@ __global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const TileArgs *__r
           s_active = active & ~ended;
         }
       }
+      all_flips += my_flips;
+      my_flips = 0;
       __syncthreads();
       active = s_active;
       if (!active) {
@@ -335,10 +414,21 @@ __global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const TileArgs *__r
   }
   __syncthreads();
   const int64_t out_base = (int64_t)A.R * I.spin_off + (int64_t)(32 * g) * n;
-  for (int o = tid; o < csz; o += blockDim.x) {
-    const uint32_t wv = (bw[o] & has_best) | (sw[o] & ~has_best);
-    for (int r = 0; r < 32; ++r)
-      if ((lane_valid >> r) & 1u) A.spins[out_base + (int64_t)r * n + lo + o] = ((wv >> r) & 1u) ? 1 : -1;
+  if (((uintptr_t)(A.spins + out_base) & 15) == 0) {
+    // (n is a multiple of 32 here) 32 sites a warp step: the transpose hands lane r
+    // replica r's spins, 32 bytes of its row
+    for (int o = 32 * warp; o < csz; o += blockDim.x) {
+      const int pl = place(lo + o + lane);
+      const uint32_t mine = warp_transpose32((bw[pl] & has_best) | (sw[pl] & ~has_best), lane);
+      if ((lane_valid >> lane) & 1u) store_spins32(A.spins + out_base + (int64_t)lane * n + lo + o, mine);
+    }
+  } else {
+    for (int o = tid; o < csz; o += blockDim.x) {
+      const int pl = place(lo + o);
+      const uint32_t wv = (bw[pl] & has_best) | (sw[pl] & ~has_best);
+      for (int r = 0; r < 32; ++r)
+        if ((lane_valid >> r) & 1u) A.spins[out_base + (int64_t)r * n + lo + o] = ((wv >> r) & 1u) ? 1 : -1;
+    }
   }
   if (rank == 0 && tid < 32 && ((lane_valid >> tid) & 1u)) {
     const int64_t o = (int64_t)b * A.R + 32 * g + tid;
@@ -354,8 +444,8 @@ __global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const TileArgs *__r
     atomicAdd(A.stats + 4, my_sweeps);
   }
   __shared__ unsigned long long s_fl[kCT / 32];
-  my_flips = block_sum(my_flips, s_fl);
-  if (tid == 0) atomicAdd(A.stats + 1, my_flips);
+  all_flips = block_sum(all_flips, s_fl);
+  if (tid == 0) atomicAdd(A.stats + 1, all_flips);
   my_eval = block_sum(my_eval, s_fl);
   if (tid == 0) atomicAdd(A.stats + 5, my_eval);
   tc::cluster_sync();  // no CTA leaves while peers may still read its shared memory
@@ -363,12 +453,15 @@ __global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const TileArgs *__r
 
 }  // namespace
 
-// words, pending flags, per-site bytes, best words
-size_t msc_cluster_smem(int csz) { return (size_t)csz * 4 + (size_t)(csz / 64) * 2 * 4 + (size_t)csz + (size_t)csz * 4; }
+// words, pending flags, best words, per-site signs (in planes while those fit)
+static bool cluster_masks(int csz) { return csz <= 8192; }
+size_t msc_cluster_smem(int csz) {
+  return (size_t)csz * 4 + (size_t)(csz / 64) * 2 * 4 + (size_t)csz * 4 + (size_t)csz * (cluster_masks(csz) ? 8 : 1);
+}
 
-template <int D>
+template <int D, bool MASKS>
 cudaError_t launch_cfg(cudaLaunchConfig_t &cfg, const TileArgs *args, int P, size_t smem, int *max_active) {
-  auto kern = msc_cluster_kernel<D>;
+  auto kern = msc_cluster_kernel<D, MASKS>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   if (max_active) return cudaOccupancyMaxActiveClusters(max_active, kern, &cfg);
@@ -393,7 +486,9 @@ cudaError_t msc_cluster_launch_or_query(ising_handle *h, int n_tiles, int P, int
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   const TileArgs *args = (const TileArgs *)h->d_tile_args;
-  return D == 3 ? launch_cfg<3>(cfg, args, P, smem, max_active) : launch_cfg<2>(cfg, args, P, smem, max_active);
+  if (cluster_masks(csz_max))
+    return D == 3 ? launch_cfg<3, true>(cfg, args, P, smem, max_active) : launch_cfg<2, true>(cfg, args, P, smem, max_active);
+  return D == 3 ? launch_cfg<3, false>(cfg, args, P, smem, max_active) : launch_cfg<2, false>(cfg, args, P, smem, max_active);
 }
 
 cudaError_t launch_msc_cluster(ising_handle *h, int n_tiles, int P, int csz_max, int D, cudaStream_t s) {
