@@ -498,13 +498,24 @@ int32_t resolve_kernel(ising_handle *h, int32_t R, const ising_search_params *p)
   }
 }
 
-// Cluster split of the multi-spin-coded lattice path: worth it when the tiles
-// alone would leave most SMs idle.  Every instance must split into P
-// power-of-two chunks of at least 1024 sites (whole Philox blocks).
-int msc_cluster_size(const ising_handle *h, int32_t R, const ising_search_params *p) {
-  if (!h->msc_ok || !h->all_lattice || !h->lat_parity || p->schedule != ISING_SCHED_COLOUR) return 0;
-  if (p->cluster_ctas == 1) return 0;
+// Cluster split of the multi-spin-coded lattice path.  Every instance must split
+// into P power-of-two slabs of at least 1024 sites (whole Philox blocks).  A
+// cluster of P CTAs runs a descent about P^0.8 times as fast as one CTA (a barrier
+// per class and the exchange of flags stay); tiles whose descents are independent
+// run as many segments at once as clusters are resident.  Taken is the P whose
+// clusters get through the call's descents soonest, in whole waves (ties: the
+// smaller), so long as the tiles alone would leave most SMs idle.
+const ClusterPlan &cluster_plan(ising_handle *h, int32_t R, const ising_search_params *p) {
+  ClusterPlan &T = h->cluster_plan_cache;
+  const int32_t parallel = p->sweep_budget > 0 ? 1 : p->restarts;
+  if (T.R == R && T.parallel == parallel && T.only == p->cluster_ctas) return T;
+  T = ClusterPlan();
+  T.R = R;
+  T.parallel = parallel;
+  T.only = p->cluster_ctas;
+  if (!h->msc_ok || !h->all_lattice || !h->lat_parity || p->cluster_ctas == 1) return T;
   const int64_t tiles = (int64_t)h->n_inst * ((R + 31) / 32);
+  double best = 0.0;
   for (int P : {8, 4, 2}) {
     if (p->cluster_ctas > 1 && p->cluster_ctas != P) continue;  // restricted to one size
     if (tiles * P > 2 * (int64_t)h->sm_count) continue;
@@ -517,16 +528,21 @@ int msc_cluster_size(const ising_handle *h, int32_t R, const ising_search_params
       if (d >= 0 && I.lat_d != d) ok = false;
       d = I.lat_d;
     }
-    // Clusters of 8 only when every CTA gets an SM of its own and all clusters
-    // are resident at once: few replica groups, each spread wider.  With more
-    // groups, 4-CTA clusters measured faster than two 8-CTA clusters per SM set.
-    if (ok && P == 8 &&
-        (tiles * P > (int64_t)h->sm_count ||
-         msc_cluster_max_active(const_cast<ising_handle *>(h), (int)tiles, P, h->nmax / P, d) < tiles))
-      ok = false;
-    if (ok) return P;
+    if (!ok) continue;
+    const int64_t active = std::max(1, msc_cluster_max_active(h, (int)std::min<int64_t>(tiles * parallel, 4096), P, h->nmax / P, d));
+    // Clusters of 8 only when every CTA gets an SM of its own and all clusters of
+    // one segment are resident at once.
+    if (P == 8 && (tiles * P > (int64_t)h->sm_count || active < tiles)) continue;
+    const int64_t segs = std::max<int64_t>(1, std::min<int64_t>(parallel, active / tiles));
+    const double waves = std::max(1.0, std::ceil((double)(tiles * segs) / (double)active));
+    const double time = waves * std::ceil((double)parallel / (double)segs) / std::pow((double)P, 0.8);
+    if (T.P == 0 || time <= best) {
+      best = time;
+      T.P = P;
+      T.segs = (int32_t)segs;
+    }
   }
-  return 0;
+  return T;
 }
 
 // CTA size and segments of the tile kernels for these arguments, null when no
@@ -604,65 +620,22 @@ ising_status run_tile(ising_handle *h, int mode, int32_t R, const ising_search_p
     h->n_tiles = (int32_t)tiles.size();
     h->tiles_R = R;
   }
-  const int P = mode == 3 ? msc_cluster_size(h, R, p) : 0;
-  if (P > 0) {
-    const size_t bw_bytes = (size_t)h->n_tiles * h->nmax * sizeof(uint32_t);
-    ising_status st = ensure_scratch(h, bw_bytes + 256);
-    if (st != ISING_OK) return st;
-    TileArgs a;
-    a.g = h->graph();
-    a.tiles = h->d_tiles;
-    a.n_tiles = h->n_tiles;
-    a.queue = h->d_queue;
-    a.R = R;
-    a.max_sweeps = p->max_sweeps;
-    a.restarts = p->restarts;
-    a.budget = p->sweep_budget;
-    a.refresh = p->refresh_every;
-    a.sequential = 0;
-    a.seeds = h->d_seeds;
-    a.F = nullptr;
-    a.bw = (uint32_t *)h->d_scratch;
-    a.nmax = h->nmax;
-    a.spins = spins;
-    a.energy = E;
-    a.energy_i32 = E32;
-    a.minima = minima;
-    a.stats = h->d_stats;
-    CUDA_OK(cudaMemcpyAsync(h->d_tile_args, &a, sizeof(a), cudaMemcpyHostToDevice, s));
-    kt_begin(h, "msc_cluster_kernel", s);
-    CUDA_OK(launch_msc_cluster(h, h->n_tiles, P, h->nmax / P, h->inst[0].lat_d, s));
-    kt_end(h, s);
-    h->launches += 1;
-    return ISING_OK;
-  }
-  const TilePlan *plan = tile_plan(h, mode, R, p);
-  if (!plan) return ISING_ERR_UNSUPPORTED;
-  const int threads = plan->threads, segs = plan->segs, fsm_cap = plan->fsm_cap;
-  const size_t smem = plan->smem;
-  const int64_t work = (int64_t)h->n_tiles * segs;
-  const int grid = (int)std::min<int64_t>(work, plan->slots);
   auto up256 = [](size_t bytes) { return (bytes + 255) / 256 * 256; };
-  const size_t f_bytes = mode == 1 ? up256((size_t)grid * h->nmax * 32 * sizeof(float)) : 0;
-  const size_t bw_bytes = up256((size_t)grid * h->nmax * sizeof(uint32_t));
-  const size_t seg_bytes = segs > 1 ? up256((size_t)work * h->nmax * sizeof(uint32_t)) : 0;
-  const size_t lane_bytes = segs > 1 ? up256((size_t)work * 32 * sizeof(double)) : 0;
-  ising_status st = ensure_scratch(h, f_bytes + bw_bytes + seg_bytes + 2 * lane_bytes + 256);
-  if (st != ISING_OK) return st;
-  const int32_t counters = segs > 1 ? h->n_tiles : 0;  // segments ended, per tile
-  if (counters > h->queue_tiles) {
+  // counters of the segments ended, per tile, behind the work queue's
+  auto ensure_counters = [&](int32_t counters) -> ising_status {
+    if (counters <= h->queue_tiles) return ISING_OK;
     int32_t *q = nullptr;
     if (cudaMalloc(&q, sizeof(int32_t) * (4 + (size_t)counters)) != cudaSuccess) return ISING_ERR_OOM;
     cudaFree(h->d_queue);
     h->d_queue = q;
     h->queue_tiles = counters;
     h->tile_exec_key[0] = -1;  // (captured against the old buffer)
-  }
-  TileArgs a;
+    return ISING_OK;
+  };
+  TileArgs a = {};
   a.g = h->graph();
   a.tiles = h->d_tiles;
   a.n_tiles = h->n_tiles;
-  a.queue = h->d_queue;
   a.R = R;
   a.max_sweeps = p->max_sweeps;
   a.restarts = p->restarts;
@@ -670,6 +643,50 @@ ising_status run_tile(ising_handle *h, int mode, int32_t R, const ising_search_p
   a.refresh = p->refresh_every;
   a.sequential = p->schedule == ISING_SCHED_SEQUENTIAL ? 1 : 0;
   a.seeds = h->d_seeds;
+  a.nmax = h->nmax;
+  a.spins = spins;
+  a.energy = E;
+  a.energy_i32 = E32;
+  a.minima = minima;
+  a.stats = h->d_stats;
+  if (mode == 3) {
+    const ClusterPlan &C = cluster_plan(h, R, p);
+    if (C.P > 0) {
+      const int units = h->n_tiles * C.segs;
+      const size_t seg_bytes = C.segs > 1 ? up256((size_t)units * h->nmax * sizeof(uint32_t)) : 0;
+      const size_t lane_bytes = C.segs > 1 ? up256((size_t)units * 32 * sizeof(double)) : 0;
+      ising_status st = ensure_scratch(h, seg_bytes + 2 * lane_bytes + 256);
+      if (st == ISING_OK && C.segs > 1) st = ensure_counters(h->n_tiles);
+      if (st != ISING_OK) return st;
+      a.queue = h->d_queue;
+      a.segs = C.segs;
+      a.seg_words = (uint32_t *)h->d_scratch;
+      a.seg_best = (double *)((char *)h->d_scratch + seg_bytes);
+      a.seg_minima = (int32_t *)((char *)h->d_scratch + seg_bytes + lane_bytes);
+      CUDA_OK(cudaMemcpyAsync(h->d_tile_args, &a, sizeof(a), cudaMemcpyHostToDevice, s));
+      if (C.segs > 1) CUDA_OK(cudaMemsetAsync(h->d_queue, 0, sizeof(int32_t) * (4 + (size_t)h->n_tiles), s));
+      kt_begin(h, "msc_cluster_kernel", s);
+      CUDA_OK(launch_msc_cluster(h, units, C.P, h->nmax / C.P, h->inst[0].lat_d, s));
+      kt_end(h, s);
+      h->launches += 1;
+      return ISING_OK;
+    }
+  }
+  const TilePlan *plan = tile_plan(h, mode, R, p);
+  if (!plan) return ISING_ERR_UNSUPPORTED;
+  const int threads = plan->threads, segs = plan->segs, fsm_cap = plan->fsm_cap;
+  const size_t smem = plan->smem;
+  const int64_t work = (int64_t)h->n_tiles * segs;
+  const int grid = (int)std::min<int64_t>(work, plan->slots);
+  const size_t f_bytes = mode == 1 ? up256((size_t)grid * h->nmax * 32 * sizeof(float)) : 0;
+  const size_t bw_bytes = up256((size_t)grid * h->nmax * sizeof(uint32_t));
+  const size_t seg_bytes = segs > 1 ? up256((size_t)work * h->nmax * sizeof(uint32_t)) : 0;
+  const size_t lane_bytes = segs > 1 ? up256((size_t)work * 32 * sizeof(double)) : 0;
+  ising_status st = ensure_scratch(h, f_bytes + bw_bytes + seg_bytes + 2 * lane_bytes + 256);
+  if (st != ISING_OK) return st;
+  const int32_t counters = segs > 1 ? h->n_tiles : 0;
+  if ((st = ensure_counters(counters)) != ISING_OK) return st;
+  a.queue = h->d_queue;
   a.F = mode == 1 ? (float *)h->d_scratch : nullptr;
   a.fsm_cap = fsm_cap;
   char *scratch = (char *)h->d_scratch + f_bytes;
@@ -678,12 +695,6 @@ ising_status run_tile(ising_handle *h, int mode, int32_t R, const ising_search_p
   a.seg_words = (uint32_t *)(scratch + bw_bytes);
   a.seg_best = (double *)(scratch + bw_bytes + seg_bytes);
   a.seg_minima = (int32_t *)(scratch + bw_bytes + seg_bytes + lane_bytes);
-  a.nmax = h->nmax;
-  a.spins = spins;
-  a.energy = E;
-  a.energy_i32 = E32;
-  a.minima = minima;
-  a.stats = h->d_stats;
   CUDA_OK(cudaMemcpyAsync(h->d_tile_args, &a, sizeof(a), cudaMemcpyHostToDevice, s));
   // The launch sequence reads its arguments from device memory, so one captured
   // graph serves every call with the same mode, grid, shared memory, threads and

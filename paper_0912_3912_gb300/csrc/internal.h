@@ -135,6 +135,12 @@ struct TilePlan {
   size_t smem = 0;
 };
 
+// The same of the lattice clusters (cluster_plan in api.cu).
+struct ClusterPlan {
+  int32_t R = 0, parallel = 0, only = -1;  // what it was made for (only: cluster_ctas)
+  int32_t P = 0, segs = 1;                 // CTAs per cluster (0: no clusters), segments per tile
+};
+
 struct PlanKey {
   int32_t R, kernel, schedule;
   bool operator<(const PlanKey &o) const {
@@ -211,6 +217,7 @@ struct ising_handle {
   // once per (mode, grid, shared memory) and replayed
   cudaGraphExec_t tile_exec = nullptr;
   isg::TilePlan tile_plan_cache;
+  isg::ClusterPlan cluster_plan_cache;
   int32_t tile_exec_key[5] = {-1, -1, -1, -1, -1};
   ising_status latched = ISING_OK;
   uint64_t launches = 0;  // kernel launches enqueued by the current call
@@ -250,7 +257,7 @@ cudaError_t launch_energy(ising_handle *h, const int8_t *spins, int32_t R, doubl
                           int32_t *E32, cudaStream_t s);
 void energy_plan_free(ising_handle *h);
 size_t msc_cluster_smem(int csz);
-cudaError_t launch_msc_cluster(ising_handle *h, int n_tiles, int P, int csz_max, int D, cudaStream_t s);
+cudaError_t launch_msc_cluster(ising_handle *h, int units, int P, int csz_max, int D, cudaStream_t s);
 // the pass-based search (fm.cu)
 int fm_max_spins();
 cudaError_t launch_fm(ising_handle *h, int32_t R, const ising_fm_params *p, int8_t *spins, double *E,

@@ -23,7 +23,13 @@
 // stable and skipped (only the first sweep of a descent visits everything).  All
 // per-lane bookkeeping (sweep counts, convergence, best energies) is replicated
 // identically in every CTA of the cluster, so the cluster's control flow stays
-// uniform and every barrier is matched.  C2NOTE
+// uniform and every barrier is matched.
+//
+// A visit is bound by its logic instructions (64 lanes a cycle and SM): the class
+// layout, sign planes, one pending target per lane and two chunks at a time took
+// 32^3 with fields, 1,024 replicas, 10 descents from 719 to 535 us a call with four
+// CTAs a cluster; two CTAs and two segments of descents each: 504.  With 32
+// replicas, ten segments of eight CTAs: 467 -> 84 us.
 #include <cfloat>
 #include <type_traits>
 
@@ -35,7 +41,7 @@ namespace isg {
 namespace {
 
 // CTAs of 512 threads, one per SM (two per SM at 64 registers, in clusters of
-// 8, measured slower on the 32^3 lattice)
+// 8, measured slower on the 32^3 lattice; 768 threads 640, 1,024 740 against 602 us)
 constexpr int kCT = 512;
 
 // MASKS: the signs and fields as bytes of 0 or -1, one plane per direction and two
@@ -53,7 +59,9 @@ __global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const TileArgs *__r
   const TileArgs &A = *Aptr;
   const DevGraph G = A.g;
   const uint32_t rank = tc::cluster_rank();
-  const int tile = blockIdx.x / P;
+  // one cluster per tile and segment of its descents (see the tile kernels)
+  const int unit = blockIdx.x / P, segs = A.segs, tile = unit / segs;
+  const int k0 = (int)((int64_t)A.restarts * (unit % segs) / segs), k1 = (int)((int64_t)A.restarts * (unit % segs + 1) / segs);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
   const int b = A.tiles[tile].x, g = A.tiles[tile].y;
   const InstDesc I = G.inst[b];
@@ -251,10 +259,10 @@ __global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const TileArgs *__r
   };
 
   uint32_t sc = 0;  // sweeps so far (all descents): picks the convergence buffer
-  for (int k = 0;; ++k) {
+  for (int k = k0;; ++k) {
     if (warp == 0) {
       const uint32_t start = __ballot_sync(
-          0xffffffffu, k < A.restarts && ((lane_valid >> lane) & 1u) && (A.budget <= 0 || s_total[lane] < A.budget));
+          0xffffffffu, k < k1 && ((lane_valid >> lane) & 1u) && (A.budget <= 0 || s_total[lane] < A.budget));
       if (lane == 0) {
         s_active = start;
         s_convround = 0;
@@ -408,13 +416,64 @@ __global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const TileArgs *__r
   uint32_t has_best = 0;
   for (int r = 0; r < 32; ++r)
     if (s_minima[r] > 0) has_best |= 1u << r;
-  if (lane_valid & ~has_best) {
+  if ((lane_valid & ~has_best) && unit % segs == segs - 1) {
     energies();
     if (tid < 32 && !((has_best >> tid) & 1u)) s_best[tid] = s_E[tid];
   }
   __syncthreads();
+  bool write = true;  // this cluster writes the tile's results (the same in every CTA of it)
+  if (segs > 1) {
+    // this segment's words (by place), energies and minima; the last cluster of the
+    // tile chooses per lane among the segments (strictly lower energy, ties keep the
+    // earlier; without a converged descent the last segment)
+    uint32_t *words = A.seg_words + (size_t)unit * A.nmax + lo;
+    for (int o = tid; o < csz; o += blockDim.x) words[o] = (bw[o] & has_best) | (sw[o] & ~has_best);
+    if (rank == 0 && tid < 32) {
+      A.seg_best[(size_t)unit * 32 + tid] = s_best[tid];
+      A.seg_minima[(size_t)unit * 32 + tid] = s_minima[tid];
+    }
+    __threadfence();
+    __syncthreads();
+    tc::cluster_sync();
+    if (rank == 0 && tid == 0) s_upd = atomicAdd(A.queue + 4 + tile, 1) == segs - 1;
+    __syncthreads();
+    tc::cluster_sync();
+    write = rank == 0 ? s_upd : tc::ld_cluster_u32(tc::map_shared(&s_upd, 0u));
+    tc::cluster_sync();  // read before that CTA goes on
+    if (write) {
+      __threadfence();
+      if (tid < 32) {
+        double e = DBL_MAX;
+        int m = 0, best = segs - 1;
+        for (int q = 0; q < segs; ++q) {
+          const size_t o = ((size_t)tile * segs + q) * 32 + tid;
+          const int mq = __ldcg(A.seg_minima + o);
+          const double eq = __ldcg(A.seg_best + o);
+          m += mq;
+          if (mq > 0 && eq < e) {
+            e = eq;
+            best = q;
+          }
+        }
+        if (m == 0) e = __ldcg(A.seg_best + ((size_t)tile * segs + best) * 32 + tid);
+        s_best[tid] = e;
+        s_minima[tid] = m;
+        s_total[tid] = best;
+      }
+      __syncthreads();
+      // the chosen words in place of the best ones
+      const uint32_t *from = A.seg_words + (size_t)tile * segs * A.nmax + lo;
+      for (int o = tid; o < csz; o += blockDim.x) {
+        uint32_t wv = 0u;
+        for (int r = 0; r < 32; ++r) wv |= __ldcg(from + (size_t)s_total[r] * A.nmax + o) & (1u << r);
+        bw[o] = wv;
+      }
+      has_best = 0xffffffffu;
+      __syncthreads();
+    }
+  }
   const int64_t out_base = (int64_t)A.R * I.spin_off + (int64_t)(32 * g) * n;
-  if (((uintptr_t)(A.spins + out_base) & 15) == 0) {
+  if (write && ((uintptr_t)(A.spins + out_base) & 15) == 0) {
     // (n is a multiple of 32 here) 32 sites a warp step: the transpose hands lane r
     // replica r's spins, 32 bytes of its row
     for (int o = 32 * warp; o < csz; o += blockDim.x) {
@@ -422,7 +481,7 @@ __global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const TileArgs *__r
       const uint32_t mine = warp_transpose32((bw[pl] & has_best) | (sw[pl] & ~has_best), lane);
       if ((lane_valid >> lane) & 1u) store_spins32(A.spins + out_base + (int64_t)lane * n + lo + o, mine);
     }
-  } else {
+  } else if (write) {
     for (int o = tid; o < csz; o += blockDim.x) {
       const int pl = place(lo + o);
       const uint32_t wv = (bw[pl] & has_best) | (sw[pl] & ~has_best);
@@ -430,7 +489,7 @@ __global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const TileArgs *__r
         if ((lane_valid >> r) & 1u) A.spins[out_base + (int64_t)r * n + lo + o] = ((wv >> r) & 1u) ? 1 : -1;
     }
   }
-  if (rank == 0 && tid < 32 && ((lane_valid >> tid) & 1u)) {
+  if (write && rank == 0 && tid < 32 && ((lane_valid >> tid) & 1u)) {
     const int64_t o = (int64_t)b * A.R + 32 * g + tid;
     A.energy[o] = s_best[tid];
     if (A.energy_i32) A.energy_i32[o] = (int32_t)s_best[tid];
@@ -491,8 +550,8 @@ cudaError_t msc_cluster_launch_or_query(ising_handle *h, int n_tiles, int P, int
   return D == 3 ? launch_cfg<3, false>(cfg, args, P, smem, max_active) : launch_cfg<2, false>(cfg, args, P, smem, max_active);
 }
 
-cudaError_t launch_msc_cluster(ising_handle *h, int n_tiles, int P, int csz_max, int D, cudaStream_t s) {
-  return msc_cluster_launch_or_query(h, n_tiles, P, csz_max, D, s, nullptr);
+cudaError_t launch_msc_cluster(ising_handle *h, int units, int P, int csz_max, int D, cudaStream_t s) {
+  return msc_cluster_launch_or_query(h, units, P, csz_max, D, s, nullptr);
 }
 
 int msc_cluster_max_active(ising_handle *h, int n_tiles, int P, int csz_max, int D) {

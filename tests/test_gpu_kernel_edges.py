@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 isg = pytest.importorskip("paper_0912_3912_gb300")
 
-from test_gpu_parity import _compare, _exp_spread  # noqa: E402
+from test_gpu_parity import _compare, _exp_spread, _oracle, _run  # noqa: E402
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -103,6 +103,30 @@ def test_tile_segments_uneven_batch_and_sequential_schedule():
     insts = [W.random_graph(n, 4.0, 60 + n, dtype="f32", n_hyper=n // 9) for n in (1, 40, 300)]
     _compare(insts, [1, 2, 3], 34, False, max_sweeps=200, restarts=9, schedule=isg.SCHED_SEQUENTIAL,
              kernel=isg.KERNEL_TILE)
+
+
+# Lattice clusters: every cluster size, both dimensions, rows shorter than, as long
+# as and longer than a chunk, slabs of one plane, signs in planes and (slabs of
+# 16,384 sites) packed; segments of descents with none, some and all converged;
+# results written to an odd address.
+@pytest.mark.parametrize("dims,ctas", [((16, 16, 16), 2), ((16, 16, 16), 4), ((32, 32, 32), 2), ((32, 32, 32), 8),
+                                       ((64, 64), 4), ((64, 64), 2), ((128, 128), 8), ((128, 128), 2)])
+@pytest.mark.parametrize("max_sweeps,restarts,R", [(1, 5, 33), (5, 3, 7), (200, 4, 40)])
+def test_lattice_cluster_segments(dims, ctas, max_sweeps, restarts, R):
+    inst = W.lattice(dims, True, "pm1", "pm1_0" if dims[0] != 64 else None, seed=dims[0])
+    if max_sweeps == 1 and R == 33:
+        h = isg.Handle([inst])
+        kw = dict(max_sweeps=max_sweeps, restarts=restarts, kernel=isg.KERNEL_MSC, cluster_ctas=ctas)
+        ref = h.local_search([R], R, **kw)
+        buf = torch.zeros(R * inst.n + 1, dtype=torch.int8, device="cuda")[1:]
+        h.local_search([R], R, out=(buf, ref.energy.clone(), None, ref.minima.clone()), **kw)
+        assert torch.equal(buf, ref.spins)
+        h.close()
+    g, gst, _ = _run([inst], [R], R, max_sweeps=max_sweeps, restarts=restarts, kernel=isg.KERNEL_MSC, cluster_ctas=ctas)
+    o, ost = _oracle([inst], [R], R, max_sweeps=max_sweeps, restarts=restarts)
+    for k in range(3):
+        assert np.array_equal(g[0][k], o[0][k])
+    assert {k: gst[k] for k in ost} == ost
 
 
 # The planner's line between one CTA per tile and launches over the whole GPU:
