@@ -34,6 +34,7 @@
 #include <cfloat>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "device_common.cuh"
 
@@ -158,6 +159,95 @@ __device__ void tile_energy_lanes(const DevGraph &G, const InstDesc &I, const ui
     }
   }
   __syncthreads();
+}
+
+// The same in integers with a lane per spin (and per hyper-edge): with p the parity
+// word of a term's spins (bit r: their product in replica r is -1), the term is
+// -t + 2 t p_r, so a predicated add per replica for 32 spins at once, where the form
+// above spends that and the term's decoding on every spin for itself (bound by
+// issue).  FP32: 64-bit fixed point, NV = 8 replicas at a time, the rows read again
+// from L1 for each (1,024 cell grids of 512 spins, two descents: 1,754 us with the
+// form above, 1,623 / 1,577 / 1,699 with 4 / 8 / 16); integers: all 32 (1,000 random
+// graphs of 1,024 spins: 1,112 -> 1,036 us).  False, and nothing done, when FP32
+// terms are not integers of one unit, or so wide or so many that a lane's sum could
+// leave its 62 bits (integers: a warp's its 31); the same for the whole CTA.
+template <bool FLOAT, int THREADS>
+__device__ bool tile_energy_sites(const DevGraph &G, const InstDesc &I, const uint32_t *sw, double *red, double *E) {
+  using T = std::conditional_t<FLOAT, long long, int>;
+  constexpr int NV = FLOAT ? 8 : 32;
+  const int n = I.n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int ub = I.ebase;
+  // (a lane's terms; 64-bit: the degree is not bounded by the tile's size)
+  const int64_t terms = (int64_t)((n + THREADS - 1) / THREADS) * (I.max_deg + 1) + (I.n_hyper + THREADS - 1) / THREADS;
+  if (FLOAT ? ub < 0 || I.ebits + (64 - __clzll(terms)) + 1 > 62 : terms > 1 << 19) return false;
+  long long hi = 0;  // lane r: replica r's warp total
+  unsigned long long lo = 0;
+#pragma unroll 1
+  for (int r0 = 0; r0 < 32; r0 += NV) {
+    T acc[NV], csum = 0;
+#pragma unroll
+    for (int r = 0; r < NV; ++r) acc[r] = 0;
+    auto value = [&](const void *arr, int64_t at) -> T {
+      if constexpr (FLOAT) return (T)xr_term(__ldg(reinterpret_cast<const float *>(arr) + at), ub);
+      else return (T)__ldg(reinterpret_cast<const int8_t *>(arr) + at);
+    };
+    auto add = [&](T t, uint32_t p) {
+      csum += t;
+      p >>= r0;
+#pragma unroll
+      for (int r = 0; r < NV; ++r)
+        if ((p >> r) & 1u) acc[r] += t;
+    };
+    for (int i = tid; i < n; i += THREADS) {
+      const int64_t gi = I.spin_off + i;
+      const uint32_t w = sw[i];
+      add(value(G.h, gi), ~w);
+      for (uint32_t k = __ldg(G.row + gi), k1 = __ldg(G.row + gi + 1); k < k1; ++k) {
+        const int j = __ldg(G.col + k);
+        if (j > i) add(value(G.J, k), w ^ sw[j]);
+      }
+    }
+    for (int e = tid; e < I.n_hyper; e += THREADS) {
+      const int64_t ge = I.hyper_off + e;
+      uint32_t p = 0u;
+      for (uint32_t q = __ldg(G.hptr + ge), qe = __ldg(G.hptr + ge + 1); q < qe; ++q) p ^= ~sw[__ldg(G.hmem + q)];
+      add(value(G.hJ, ge), p);
+    }
+#pragma unroll
+    for (int r = 0; r < NV; ++r) {
+      const T v = 2 * acc[r] - csum;
+      if constexpr (FLOAT) {  // (20-bit pieces: 32 of them add up in 32 bits)
+        const int p0 = __reduce_add_sync(0xffffffffu, (int)(v & 0xfffff));
+        const int p1 = __reduce_add_sync(0xffffffffu, (int)((v >> 20) & 0xfffff));
+        const int p2 = __reduce_add_sync(0xffffffffu, (int)(v >> 40));
+        if (lane == r0 + r) {
+          hi = (long long)p2 << 8;
+          lo = ((unsigned long long)(unsigned)p1 << 20) + (unsigned)p0;
+        }
+      } else {
+        const int t = __reduce_add_sync(0xffffffffu, v);
+        if (lane == r) hi = t;
+      }
+    }
+  }
+  long long *ri = reinterpret_cast<long long *>(red);
+  __syncthreads();
+  ri[warp * 32 + lane] = hi;
+  __syncthreads();
+  hi = 0;
+  if (warp == 0)
+    for (int w = 0; w < THREADS / 32; ++w) hi += ri[w * 32 + lane];
+  if (FLOAT) {
+    __syncthreads();
+    reinterpret_cast<unsigned long long *>(red)[warp * 32 + lane] = lo;
+    __syncthreads();
+    lo = 0;
+    if (warp == 0)
+      for (int w = 0; w < THREADS / 32; ++w) lo += reinterpret_cast<unsigned long long *>(red)[w * 32 + lane];
+  }
+  if (warp == 0) E[lane] = FLOAT ? xe_value(hi, lo, ub) : (double)hi;
+  __syncthreads();
+  return true;
 }
 
 // Energies of all 32 lanes for a +/-1 periodic lattice with |h| <= 1 (the
@@ -683,7 +773,8 @@ tile_kernel(const TileArgs *__restrict__ Aptr) {
           const uint32_t cr = s_convround;
           if (cr) {
             if (MODE == 3) tile_energy_lattice(G, I, sw, s_cnt, s_E);
-            else tile_energy_lanes<MODE == 1>(G, I, sw, s_red, s_E);
+            else if (!tile_energy_sites<MODE == 1, THREADS>(G, I, sw, s_red, s_E))
+              tile_energy_lanes<MODE == 1>(G, I, sw, s_red, s_E);
             if (tid == 0) {
               uint32_t upd = 0;
               for (int r = 0; r < 32; ++r)
@@ -713,7 +804,8 @@ tile_kernel(const TileArgs *__restrict__ Aptr) {
       if (s_minima[r] > 0) has_best |= 1u << r;
     if ((lane_valid & ~has_best) && (!SEG || unit % segs == segs - 1)) {
       if (MODE == 3) tile_energy_lattice(G, I, sw, s_cnt, s_E);
-      else tile_energy_lanes<MODE == 1>(G, I, sw, s_red, s_E);
+      else if (!tile_energy_sites<MODE == 1, THREADS>(G, I, sw, s_red, s_E))
+        tile_energy_lanes<MODE == 1>(G, I, sw, s_red, s_E);
       if (tid < 32 && !((has_best >> tid) & 1u)) s_best[tid] = s_E[tid];
     }
     __syncthreads();

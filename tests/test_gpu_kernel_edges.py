@@ -105,6 +105,20 @@ def test_tile_segments_uneven_batch_and_sequential_schedule():
              kernel=isg.KERNEL_TILE)
 
 
+# Tile energies, a lane per spin: fewer spins than lanes and one more than a CTA's
+# threads, hyper-edges of 2 to 9 members, the highest replica alone in its group of
+# 8, and exponents too far apart for one unit or for a lane's sum.
+@pytest.mark.parametrize("n,R", [(1, 1), (33, 9), (257, 17), (1025, 32)])
+@pytest.mark.parametrize("kind", ["i8", "f32", "wide", "wider"])
+def test_tile_energy_sums(kind, n, R):
+    inst = W.random_graph(n, 5.0 if n > 1 else 0.0, n, dtype="i8" if kind == "i8" else "f32",
+                          n_hyper=n // 4, hyper_order=(2, 3, 4, 9))
+    if kind.startswith("wide"):
+        inst = _exp_spread(inst, *((-12, 12) if kind == "wide" else (-45, 25)))
+    for restarts, max_sweeps in ((1, 100), (3, 2)):
+        _compare([inst], [n], R, kind == "i8", max_sweeps=max_sweeps, restarts=restarts, kernel=isg.KERNEL_TILE)
+
+
 # Lattice clusters: every cluster size, both dimensions, rows shorter than, as long
 # as and longer than a chunk, slabs of one plane, signs in planes and (slabs of
 # 16,384 sites) packed; segments of descents with none, some and all converged;
