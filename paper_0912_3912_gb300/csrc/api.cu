@@ -421,7 +421,6 @@ void free_handle(ising_handle *h) {
   for (void *p : ptrs)
     if (p) cudaFree(p);
   if (h->h_stats_pinned) cudaFreeHost(h->h_stats_pinned);
-  if (h->tile_exec) cudaGraphExecDestroy(h->tile_exec);
   cudaSetDevice(cur);
   delete h;
 }
@@ -629,7 +628,6 @@ ising_status run_tile(ising_handle *h, int mode, int32_t R, const ising_search_p
     cudaFree(h->d_queue);
     h->d_queue = q;
     h->queue_tiles = counters;
-    h->tile_exec_key[0] = -1;  // (captured against the old buffer)
     return ISING_OK;
   };
   TileArgs a = {};
@@ -695,38 +693,12 @@ ising_status run_tile(ising_handle *h, int mode, int32_t R, const ising_search_p
   a.seg_words = (uint32_t *)(scratch + bw_bytes);
   a.seg_best = (double *)(scratch + bw_bytes + seg_bytes);
   a.seg_minima = (int32_t *)(scratch + bw_bytes + seg_bytes + lane_bytes);
-  CUDA_OK(cudaMemcpyAsync(h->d_tile_args, &a, sizeof(a), cudaMemcpyHostToDevice, s));
-  // The launch sequence reads its arguments from device memory, so one captured
-  // graph serves every call with the same mode, grid, shared memory, threads and
-  // counters.
-  if (!h->tile_exec || h->tile_exec_key[0] != mode || h->tile_exec_key[1] != grid ||
-      h->tile_exec_key[2] != (int32_t)smem || h->tile_exec_key[3] != threads || h->tile_exec_key[4] != counters) {
-    if (h->tile_exec) cudaGraphExecDestroy(h->tile_exec);
-    h->tile_exec = nullptr;
-    cudaStream_t cs;
-    CUDA_OK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-    cudaGraph_t g = nullptr;
-    cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-    if (e == cudaSuccess) {
-      cudaMemsetAsync(h->d_queue, 0, sizeof(int32_t) * (4 + (size_t)counters), cs);
-      launch_tile(h, mode, threads, segs > 1, grid, smem, cs);
-      e = cudaStreamEndCapture(cs, &g);
-    }
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&h->tile_exec, g, 0);
-    if (g) cudaGraphDestroy(g);
-    cudaStreamDestroy(cs);
-    if (e != cudaSuccess) {
-      h->tile_exec = nullptr;
-      return ISING_ERR_CUDA;
-    }
-    h->tile_exec_key[0] = mode;
-    h->tile_exec_key[1] = grid;
-    h->tile_exec_key[2] = (int32_t)smem;
-    h->tile_exec_key[3] = threads;
-    h->tile_exec_key[4] = counters;
-  }
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  CUDA_OK(cudaStreamIsCapturing(s, &cap));
+  if (cap != cudaStreamCaptureStatusNone) return ISING_ERR_CUDA;  // (scratch and work queue are the handle's)
+  CUDA_OK(cudaMemsetAsync(h->d_queue, 0, sizeof(int32_t) * (4 + (size_t)counters), s));
   kt_begin(h, "tile_kernel", s);
-  CUDA_OK(cudaGraphLaunch(h->tile_exec, s));
+  CUDA_OK(launch_tile(a, mode, threads, segs > 1, grid, smem, s));
   kt_end(h, s);
   h->launches += 1;
   return ISING_OK;

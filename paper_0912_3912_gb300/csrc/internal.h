@@ -213,12 +213,8 @@ struct ising_handle {
 
   // tuned kernel family per replica count (autotuner cache)
   std::map<int32_t, int32_t> tuned;
-  // the tile path's launch sequence (queue reset + persistent kernel) captured
-  // once per (mode, grid, shared memory) and replayed
-  cudaGraphExec_t tile_exec = nullptr;
   isg::TilePlan tile_plan_cache;
   isg::ClusterPlan cluster_plan_cache;
-  int32_t tile_exec_key[5] = {-1, -1, -1, -1, -1};
   ising_status latched = ISING_OK;
   uint64_t launches = 0;  // kernel launches enqueued by the current call
   // Optional device timing (ising_set_timing): CUDA events recorded on the
@@ -248,7 +244,7 @@ T &family_state(std::unique_ptr<FamilyState> &slot) {
 void kt_begin(ising_handle *h, const char *name, cudaStream_t s);
 void kt_end(ising_handle *h, cudaStream_t s);
 // launchers (tile.cu / energy.cu / plain.cu / sweep.cu / dense.cu)
-cudaError_t launch_tile(ising_handle *h, int mode, int threads, bool seg, int grid, size_t smem, cudaStream_t s);
+cudaError_t launch_tile(const TileArgs &a, int mode, int threads, bool seg, int grid, size_t smem, cudaStream_t s);
 size_t tile_smem_bytes(int mode, int nmax);
 size_t tile_smem_limit();  // dynamic shared memory of a tile CTA at most
 int tile_fsm_cap(int nmax, size_t budget);

@@ -329,6 +329,118 @@ __device__ __forceinline__ uint32_t sliced_ge(uint32_t c0, uint32_t c1, uint32_t
   return gt | eq;
 }
 
+// FP32 visits: four lanes share a pending spin, 8 replicas each from r0, and a warp
+// takes 8 spins at a time.  A visit by the whole warp, a lane per replica, spent the
+// row, the neighbours' words and each term's decoding on one spin (some 380
+// instructions) and was bound by issue; here a term is a predicated add per replica
+// for 8 spins at once, and 8 pending spins of a class fill a warp.  1,024 cell grids
+// of 512 spins, one descent: 1,577 -> 965 us (one lane for all 32 replicas of a spin:
+// 1,127, and slower than a whole warp on small classes); 4,096 of them: 5,983 ->
+// 3,265; one graph of 6,000 spins: 1,718 -> 964.  Both forms return the replicas in
+// which the spin is against its field and leave the fields in F.
+
+// The parities of the other members' spins (flips) of incident hyper-edge q of j.
+__device__ __forceinline__ uint32_t own_parity(const DevGraph &G, const uint32_t *words, uint32_t inv, int j, uint32_t q) {
+  const int2 oth = __ldg(G.inc_oth + q);
+  if (oth.x >= 0) return words[oth.x] ^ words[oth.y];
+  const int e = __ldg(G.inc_edge + q);
+  uint32_t p = 0u;
+  for (uint32_t m = __ldg(G.hptr + e), me = __ldg(G.hptr + e + 1); m < me; ++m) {
+    const int mm = __ldg(G.hmem + m);
+    if (mm != j) p ^= words[mm] ^ inv;
+  }
+  return p;
+}
+
+// Replica r's place in spin j's row of fields: quads of replicas are turned by the
+// spin, so that lanes reading the same quad of several spins spread over the banks
+// of shared memory (cell grids' classes visit every 16th spin).
+__device__ __forceinline__ int field_at(int j, int r) { return r ^ (((j ^ (j >> 4)) & 7) << 2); }
+
+// The fields are stored; those against the spins (word w) are returned, in place.
+__device__ __forceinline__ uint32_t own_store(float *F, int j, int r0, const float *f, uint32_t w) {
+  F += (size_t)j * 32;
+  *reinterpret_cast<float4 *>(F + field_at(j, r0)) = make_float4(f[0], f[1], f[2], f[3]);
+  *reinterpret_cast<float4 *>(F + field_at(j, r0 + 4)) = make_float4(f[4], f[5], f[6], f[7]);
+  uint32_t m = 0u;
+  w >>= r0;
+#pragma unroll
+  for (int r = 0; r < 8; ++r)
+    if ((w >> r) & 1u ? f[r] < 0.0f : f[r] > 0.0f) m |= 1u << r;
+  return m << r0;
+}
+
+// From scratch: the exact sum in fixed point (the spin's unit), rounded to FP32.
+__device__ __forceinline__ uint32_t own_refresh(const DevGraph &G, const InstDesc &I, const uint32_t *sw, float *F, int j,
+                                                int r0, uint32_t k0, uint32_t k1, uint32_t e0, uint32_t e1, int unit) {
+  const float *Jf = reinterpret_cast<const float *>(G.J), *hJ = reinterpret_cast<const float *>(G.hJ);
+  int64_t sum = xr_term(__ldg(reinterpret_cast<const float *>(G.h) + I.spin_off + j), unit), acc[8] = {};
+  auto add = [&](int64_t t, uint32_t minus) {
+    sum += t;
+    minus >>= r0;
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+      if ((minus >> r) & 1u) acc[r] += t;
+  };
+  for (uint32_t k = k0; k < k1; ++k) add(xr_term(__ldg(Jf + k), unit), ~sw[__ldg(G.col + k)]);
+  for (uint32_t q = e0; q < e1; ++q)
+    add(xr_term(__ldg(hJ + __ldg(G.inc_edge + q)), unit), own_parity(G, sw, 0xffffffffu, j, q));
+  float f[8];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) f[r] = xr_round(sum - 2 * acc[r], unit);
+  return own_store(F, j, r0, f, sw[j]);
+}
+
+// By the neighbours' flips since the previous visit (their words in fm), in CSR order
+// and then by hyper-edge; a replica with none keeps its field and its spin.
+__device__ __forceinline__ uint32_t own_visit(const DevGraph &G, const uint32_t *sw, const uint32_t *fm, float *F, int j,
+                                              int r0, uint32_t k0, uint32_t k1, uint32_t e0, uint32_t e1) {
+  const float *Jf = reinterpret_cast<const float *>(G.J), *hJ = reinterpret_cast<const float *>(G.hJ);
+  constexpr int kPre = 6;  // row entries fetched together
+  const int dg = (int)(k1 - k0);
+  uint32_t pf[kPre], ps[kPre], dirty = 0u;
+  float pw[kPre];
+#pragma unroll
+  for (int q = 0; q < kPre; ++q) {
+    pf[q] = 0u;
+    if (q < dg) {
+      const int i = __ldg(G.col + k0 + q);
+      pw[q] = 2.0f * __ldg(Jf + k0 + q);
+      pf[q] = fm[i];
+      ps[q] = ~sw[i];
+      dirty |= pf[q];
+    }
+  }
+  const bool more = dg > kPre || e1 > e0;
+  if (!more && !((dirty >> r0) & 0xffu)) return 0u;
+  const float4 a = *reinterpret_cast<const float4 *>(F + (size_t)j * 32 + field_at(j, r0));
+  const float4 b = *reinterpret_cast<const float4 *>(F + (size_t)j * 32 + field_at(j, r0 + 4));
+  float f[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+  auto pull = [&](float w2, uint32_t flipped, uint32_t minus) {
+    flipped >>= r0;
+    minus >>= r0;
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+      if ((flipped >> r) & 1u)
+        f[r] = __fadd_rn(f[r], __uint_as_float(__float_as_uint(w2) ^ ((minus << (31 - r)) & 0x80000000u)));
+  };
+#pragma unroll
+  for (int q = 0; q < kPre; ++q) pull(pw[q], pf[q], ps[q]);
+  if (more) {
+    for (uint32_t k = k0 + kPre; k < k1; ++k) {
+      const int i = __ldg(G.col + k);
+      dirty |= fm[i];
+      pull(2.0f * __ldg(Jf + k), fm[i], ~sw[i]);
+    }
+    for (uint32_t q = e0; q < e1; ++q) {
+      const uint32_t p = own_parity(G, fm, 0u, j, q);
+      dirty |= p;
+      pull(2.0f * __ldg(hJ + __ldg(G.inc_edge + q)), p, own_parity(G, sw, 0xffffffffu, j, q));
+    }
+  }
+  return own_store(F, j, r0, f, sw[j]) & dirty;
+}
+
 }  // namespace
 
 // SEG: tiles in segments of descents.  (A separate instantiation: the segments'
@@ -336,7 +448,9 @@ __device__ __forceinline__ uint32_t sliced_ge(uint32_t c0, uint32_t c1, uint32_t
 // 8 %.)
 template <int MODE, int THREADS, bool SEG>
 __global__ void __launch_bounds__(THREADS, (MODE == 3 ? 512 : 1024) / THREADS < 1 ? 1 : (MODE == 3 ? 512 : 1024) / THREADS)
-tile_kernel(const TileArgs *__restrict__ Aptr) {
+tile_kernel(const __grid_constant__ TileArgs A) {
+  // (a parameter, so that its pointers stay in constant memory: read through a pointer
+  // they took registers, and the 64 spilled)
   extern __shared__ uint32_t smem[];
   __shared__ int s_tile, s_last, s_segs;
   __shared__ bool s_merge;
@@ -344,10 +458,10 @@ tile_kernel(const TileArgs *__restrict__ Aptr) {
   __shared__ int32_t s_total[32], s_minima[32];
   __shared__ double s_best[32], s_E[32];
   __shared__ double s_red[THREADS];
+  __shared__ uint8_t s_slot[MODE == 1 ? THREADS : 32];
   __shared__ int s_cnt[33];
 
-  const TileArgs &A = *Aptr;
-  const DevGraph G = A.g;
+  const DevGraph &G = A.g;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = THREADS / 32;
   const int nmax = A.nmax;
   uint32_t *sw = smem;
@@ -553,6 +667,53 @@ tile_kernel(const TileArgs *__restrict__ Aptr) {
                 e1l = __ldg(G.inc_ptr + g + 1);
               }
               uint32_t todo = __ballot_sync(0xffffffffu, pl);
+              if constexpr (MODE == 1) {
+                const int ul = refresh && pl ? __ldg(G.runit + I.spin_off + jl) : 0;
+                const uint32_t own = __ballot_sync(0xffffffffu, pl && ul >= 0);
+                if ((own >> lane) & 1u) s_slot[(tid & ~31) + __popc(own & ((1u << lane) - 1u))] = (uint8_t)lane;
+                __syncwarp();
+                const int cnt = __popc(own), r0 = 8 * (lane & 3);
+                for (int p = lane >> 2; p - (lane >> 2) < cnt; p += 8) {
+                  const bool on = p < cnt;
+                  const int src = on ? s_slot[(tid & ~31) + p] : 0;
+                  const int j = __shfl_sync(0xffffffffu, jl, src);
+                  const uint32_t k0 = __shfl_sync(0xffffffffu, k0l, src), k1 = __shfl_sync(0xffffffffu, k1l, src);
+                  const uint32_t e0 = __shfl_sync(0xffffffffu, e0l, src), e1 = __shfl_sync(0xffffffffu, e1l, src);
+                  const int u = __shfl_sync(0xffffffffu, ul, src);
+                  uint32_t m = 0u;
+                  if (on)
+                    m = active & (refresh ? own_refresh(G, I, sw, Fc, j, r0, k0, k1, e0, e1, u)
+                                          : own_visit(G, sw, fm, Fc, j, r0, k0, k1, e0, e1));
+                  m |= __shfl_xor_sync(0xffffffffu, m, 1);
+                  m |= __shfl_xor_sync(0xffffffffu, m, 2);
+                  if (!on) continue;
+                  if (r0 == 0) {
+                    my_eval += __popc(active);
+                    my_flips += __popc(m);
+                    clear_pending(j);
+                    sw[j] ^= m;
+                    fm[j] = m;
+                    anyf |= m;
+                  }
+                  if (m) {
+                    for (uint32_t kk = k0 + (lane & 3); kk < k1; kk += 4) mark(__ldg(G.col + kk));
+                    for (uint32_t q = e0; q < e1; ++q) {
+                      const int2 oth = __ldg(G.inc_oth + q);
+                      if (oth.x >= 0) {
+                        if ((lane & 3) < 2) mark((lane & 3) == 0 ? oth.x : oth.y);
+                        continue;
+                      }
+                      const int e = __ldg(G.inc_edge + q);
+                      for (uint32_t mm = __ldg(G.hptr + e) + (lane & 3), me = __ldg(G.hptr + e + 1); mm < me; mm += 4) {
+                        const int o = __ldg(G.hmem + mm);
+                        if (o != j) mark(o);
+                      }
+                    }
+                  }
+                }
+                todo &= ~own;
+                __syncwarp();
+              }
               while (todo) {
               const int src = __ffs(todo) - 1;
               todo &= todo - 1u;
@@ -591,120 +752,32 @@ tile_kernel(const TileArgs *__restrict__ Aptr) {
               } else {
                 const float *Jf = reinterpret_cast<const float *>(G.J);
                 const float *hJ = reinterpret_cast<const float *>(G.hJ);
-                float f;
-                if (refresh) {
-                  // from scratch: the FP64 sum rounded to FP32, formed exactly in
-                  // fixed point with the spin's precomputed unit when that is exact
-                  const float hj = __ldg(reinterpret_cast<const float *>(G.h) + gj);
-                  const int u = __ldg(G.runit + gj);
-                  if (u >= 0) {
-                    int64_t acc = xr_term(hj, u);
-                    for (uint32_t kk = k0; kk < k1; ++kk) {
-                      const int64_t t = xr_term(__ldg(Jf + kk), u);
-                      acc += ((sw[__ldg(G.col + kk)] >> lane) & 1u) ? t : -t;
-                    }
-                    for (uint32_t q = e0; q < e1; ++q) {
-                      const int e = __ldg(G.inc_edge + q);
-                      const int2 oth = __ldg(G.inc_oth + q);
-                      uint32_t neg = 0;
-                      if (oth.x >= 0) {
-                        neg = (~(sw[oth.x] >> lane) & 1u) ^ (~(sw[oth.y] >> lane) & 1u);
-                      } else {
-                        for (uint32_t m = __ldg(G.hptr + e), me = __ldg(G.hptr + e + 1); m < me; ++m) {
-                          const int mm = __ldg(G.hmem + m);
-                          if (mm != j) neg ^= ~(sw[mm] >> lane) & 1u;
-                        }
-                      }
-                      const int64_t t = xr_term(__ldg(hJ + e), u);
-                      acc += neg ? -t : t;
-                    }
-                    f = xr_round(acc, u);
-                  } else {
-                    double acc = (double)hj;
-                    for (uint32_t kk = k0; kk < k1; ++kk) {
-                      const int i = __ldg(G.col + kk);
-                      const double w = (double)__ldg(Jf + kk);
-                      acc = __dadd_rn(acc, ((sw[i] >> lane) & 1u) ? w : -w);
-                    }
-                    for (uint32_t q = e0; q < e1; ++q) {
-                      const int e = __ldg(G.inc_edge + q);
-                      const int2 oth = __ldg(G.inc_oth + q);
-                      uint32_t neg = 0;
-                      if (oth.x >= 0) {
-                        neg = (~(sw[oth.x] >> lane) & 1u) ^ (~(sw[oth.y] >> lane) & 1u);
-                      } else {
-                        for (uint32_t m = __ldg(G.hptr + e), me = __ldg(G.hptr + e + 1); m < me; ++m) {
-                          const int mm = __ldg(G.hmem + m);
-                          if (mm != j) neg ^= ~(sw[mm] >> lane) & 1u;
-                        }
-                      }
-                      const double w = (double)__ldg(hJ + e);
-                      acc = __dadd_rn(acc, neg ? -w : w);
-                    }
-                    f = __double2float_rn(acc);
-                  }
-                } else {
-                  // Pull the flips of the neighbours since this spin's previous
-                  // visit (CSR order, then hyper-edges ascending), one pass; with
-                  // none for this lane, field and decision are unchanged.  The
-                  // neighbours' words are the warp's, so they are all read and the
-                  // lanes take each term or leave it without a branch (with a
-                  // branch per entry 1,024 cell grids of 512 spins took
-                  // 1,844 us, without it 1,754).
-                  f = Fc[(size_t)j * 32 + lane];
-                  const uint32_t bit = 1u << lane;
-                  uint32_t dirtyw = 0u;  // replicas whose field changes
-                  auto pull = [&](float w2, uint32_t flipped, uint32_t plus) {
-                    const float g = __fadd_rn(f, plus & bit ? w2 : -w2);
-                    f = flipped & bit ? g : f;
-                    dirtyw |= flipped;
-                  };
-                  // the first kPre entries of the row fetched together (one round
-                  // trip instead of one per entry), then applied in CSR order
-                  constexpr int kPre = 6;
-                  const int dg = (int)(k1 - k0);
-                  int ci[kPre];
-                  float cw[kPre];
-#pragma unroll
-                  for (int q = 0; q < kPre; ++q)
-                    if (q < dg) {
-                      ci[q] = __ldg(G.col + k0 + q);
-                      cw[q] = __ldg(Jf + k0 + q);
-                    }
-#pragma unroll
-                  for (int q = 0; q < kPre; ++q)
-                    if (q < dg) pull(2.0f * cw[q], fm[ci[q]], sw[ci[q]]);
-                  for (uint32_t kk = k0 + kPre; kk < k1; ++kk) {
-                    const int i = __ldg(G.col + kk);
-                    pull(2.0f * __ldg(Jf + kk), fm[i], sw[i]);
-                  }
-                  for (uint32_t q = e0; q < e1; ++q) {
-                    const int e = __ldg(G.inc_edge + q);
-                    const int2 oth = __ldg(G.inc_oth + q);  // a 3-member edge's other two, with the id
-                    uint32_t plus = 0xffffffffu, par = 0u;
-                    if (oth.x >= 0) {
-                      plus = ~(sw[oth.x] ^ sw[oth.y]);
-                      par = fm[oth.x] ^ fm[oth.y];
-                    } else {
-                      for (uint32_t m = __ldg(G.hptr + e), me = __ldg(G.hptr + e + 1); m < me; ++m) {
-                        const int mm = __ldg(G.hmem + m);
-                        if (mm != j) {
-                          plus ^= ~sw[mm];
-                          par ^= fm[mm];
-                        }
-                      }
-                    }
-                    pull(2.0f * __ldg(hJ + e), par, plus);
-                  }
-                  const bool dirty = dirtyw & bit;
-                  if (!dirty) {
-                    flip = false;
-                    goto decided;
-                  }
+                // a refresh without an exact unit: the FP64 sum in order, rounded
+                const float hj = __ldg(reinterpret_cast<const float *>(G.h) + gj);
+                double acc = (double)hj;
+                for (uint32_t kk = k0; kk < k1; ++kk) {
+                  const int i = __ldg(G.col + kk);
+                  const double w = (double)__ldg(Jf + kk);
+                  acc = __dadd_rn(acc, ((sw[i] >> lane) & 1u) ? w : -w);
                 }
-                Fc[(size_t)j * 32 + lane] = f;
+                for (uint32_t q = e0; q < e1; ++q) {
+                  const int e = __ldg(G.inc_edge + q);
+                  const int2 oth = __ldg(G.inc_oth + q);
+                  uint32_t neg = 0;
+                  if (oth.x >= 0) {
+                    neg = (~(sw[oth.x] >> lane) & 1u) ^ (~(sw[oth.y] >> lane) & 1u);
+                  } else {
+                    for (uint32_t m = __ldg(G.hptr + e), me = __ldg(G.hptr + e + 1); m < me; ++m) {
+                      const int mm = __ldg(G.hmem + m);
+                      if (mm != j) neg ^= ~(sw[mm] >> lane) & 1u;
+                    }
+                  }
+                  const double w = (double)__ldg(hJ + e);
+                  acc = __dadd_rn(acc, neg ? -w : w);
+                }
+                const float f = __double2float_rn(acc);
+                Fc[(size_t)j * 32 + field_at(j, lane)] = f;
                 flip = up ? (f < 0.0f) : (f > 0.0f);
-              decided:;
               }
               flip = flip && ((active >> lane) & 1u);
               const uint32_t m = __ballot_sync(0xffffffffu, flip);
@@ -888,7 +961,7 @@ int tile_fsm_cap(int nmax, size_t budget) {
 }
 
 namespace {
-using TileKernel = void (*)(const TileArgs *);
+using TileKernel = void (*)(const TileArgs);
 template <int MODE, bool SEG>
 TileKernel tile_kernel_of(int threads) {
   return threads == 256 ? tile_kernel<MODE, 256, SEG> : (threads == 512 ? tile_kernel<MODE, 512, SEG> : tile_kernel<MODE, 1024, SEG>);
@@ -918,10 +991,9 @@ int tile_max_ctas_per_sm(int mode, int threads, size_t smem) {
   return least;
 }
 
-// Launch only: the shared-memory attribute was set by tile_max_ctas_per_sm, so
-// this is a plain stream operation and can be captured into a graph.
-cudaError_t launch_tile(ising_handle *h, int mode, int threads, bool seg, int grid, size_t smem, cudaStream_t s) {
-  tile_kernel_for(mode, threads, seg)<<<grid, threads, smem, s>>>(h->d_tile_args);
+// Launch only: the shared-memory attribute was set by tile_max_ctas_per_sm.
+cudaError_t launch_tile(const TileArgs &a, int mode, int threads, bool seg, int grid, size_t smem, cudaStream_t s) {
+  tile_kernel_for(mode, threads, seg)<<<grid, threads, smem, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -119,6 +119,21 @@ def test_tile_energy_sums(kind, n, R):
         _compare([inst], [n], R, kind == "i8", max_sweeps=max_sweeps, restarts=restarts, kernel=isg.KERNEL_TILE)
 
 
+# FP32 tile visits, eight spins at a time: classes of fewer and more spins than that,
+# rows of more than the entries fetched together, hyper-edges of 2 to 9 members,
+# refreshes in fixed point, in FP64 and (wider) both in one class.
+@pytest.mark.parametrize("n,R,schedule", [(7, 5, isg.SCHED_COLOUR), (100, 32, isg.SCHED_COLOUR),
+                                          (300, 41, isg.SCHED_COLOUR), (3000, 9, isg.SCHED_COLOUR),
+                                          (7, 32, isg.SCHED_SEQUENTIAL), (100, 8, isg.SCHED_SEQUENTIAL)])
+@pytest.mark.parametrize("kind", ["f32", "wide", "wider"])
+def test_tile_fp32_visits(kind, n, R, schedule):
+    inst = _star_graph(n, "f32", n) if n >= 100 else W.random_graph(n, 3.0, n, n_hyper=3, hyper_order=(2, 3, 4))
+    if kind.startswith("wide"):
+        inst = _exp_spread(inst, *((-12, 12) if kind == "wide" else (-45, 25)))
+    _compare([inst], [n], R, False, max_sweeps=200, restarts=2, refresh_every=3, schedule=schedule,
+             kernel=isg.KERNEL_TILE)
+
+
 # Lattice clusters: every cluster size, both dimensions, rows shorter than, as long
 # as and longer than a chunk, slabs of one plane, signs in planes and (slabs of
 # 16,384 sites) packed; segments of descents with none, some and all converged;
