@@ -416,8 +416,7 @@ void free_handle(ising_handle *h) {
   plain_free(h);
   void *ptrs[] = {h->d_inst, h->d_row, h->d_col, h->d_J, h->d_h, h->d_inc_ptr, h->d_inc_edge, h->d_inc_oth, h->d_hptr,
                   h->d_hmem, h->d_hJ, h->d_order, h->d_cls, h->d_Jdense, h->d_meta, h->d_Jpos, h->d_Jfwd, h->d_latinfo, h->d_runit,
-                  h->d_scratch, h->d_tile_args,
-                  h->d_seeds, h->d_stats, h->d_queue, h->d_tiles};
+                  h->d_scratch, h->d_seeds, h->d_stats, h->d_queue, h->d_tiles};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   if (h->h_stats_pinned) cudaFreeHost(h->h_stats_pinned);
@@ -528,7 +527,7 @@ const ClusterPlan &cluster_plan(ising_handle *h, int32_t R, const ising_search_p
       d = I.lat_d;
     }
     if (!ok) continue;
-    const int64_t active = std::max(1, msc_cluster_max_active(h, (int)std::min<int64_t>(tiles * parallel, 4096), P, h->nmax / P, d));
+    const int64_t active = std::max(1, msc_cluster_max_active((int)std::min<int64_t>(tiles * parallel, 4096), P, h->nmax / P, d));
     // Clusters of 8 only when every CTA gets an SM of its own and all clusters of
     // one segment are resident at once.
     if (P == 8 && (tiles * P > (int64_t)h->sm_count || active < tiles)) continue;
@@ -661,10 +660,9 @@ ising_status run_tile(ising_handle *h, int mode, int32_t R, const ising_search_p
       a.seg_words = (uint32_t *)h->d_scratch;
       a.seg_best = (double *)((char *)h->d_scratch + seg_bytes);
       a.seg_minima = (int32_t *)((char *)h->d_scratch + seg_bytes + lane_bytes);
-      CUDA_OK(cudaMemcpyAsync(h->d_tile_args, &a, sizeof(a), cudaMemcpyHostToDevice, s));
       if (C.segs > 1) CUDA_OK(cudaMemsetAsync(h->d_queue, 0, sizeof(int32_t) * (4 + (size_t)h->n_tiles), s));
       kt_begin(h, "msc_cluster_kernel", s);
-      CUDA_OK(launch_msc_cluster(h, units, C.P, h->nmax / C.P, h->inst[0].lat_d, s));
+      CUDA_OK(launch_msc_cluster(a, units, C.P, h->nmax / C.P, h->inst[0].lat_d, s));
       kt_end(h, s);
       h->launches += 1;
       return ISING_OK;
@@ -1058,8 +1056,7 @@ ising_status ising_create(const ising_instance_desc *descs, int32_t n_instances,
       Jd.insert(Jd.end(), descs[b].J_dense, descs[b].J_dense + (int64_t)descs[b].n * descs[b].n);
     ok = upload(&h->d_Jdense, Jd) == cudaSuccess;
   }
-  ok = ok && cudaMalloc(&h->d_tile_args, sizeof(TileArgs)) == cudaSuccess &&
-       cudaMalloc(&h->d_seeds, sizeof(uint64_t) * n_instances) == cudaSuccess &&
+  ok = ok && cudaMalloc(&h->d_seeds, sizeof(uint64_t) * n_instances) == cudaSuccess &&
        cudaMalloc(&h->d_stats, sizeof(unsigned long long) * 8) == cudaSuccess &&
        cudaMalloc(&h->d_queue, sizeof(int32_t) * 4) == cudaSuccess &&
        cudaMallocHost(&h->h_stats_pinned, sizeof(unsigned long long) * 8) == cudaSuccess;

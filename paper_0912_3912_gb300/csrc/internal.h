@@ -192,7 +192,6 @@ struct ising_handle {
   // scratch and per-call state, grown on demand
   void *d_scratch = nullptr;
   size_t scratch_bytes = 0;
-  isg::TileArgs *d_tile_args = nullptr;
   uint64_t *d_seeds = nullptr;
   unsigned long long *d_stats = nullptr;
   int32_t *d_queue = nullptr;
@@ -253,11 +252,11 @@ cudaError_t launch_energy(ising_handle *h, const int8_t *spins, int32_t R, doubl
                           int32_t *E32, cudaStream_t s);
 void energy_plan_free(ising_handle *h);
 size_t msc_cluster_smem(int csz);
-cudaError_t launch_msc_cluster(ising_handle *h, int units, int P, int csz_max, int D, cudaStream_t s);
+cudaError_t launch_msc_cluster(const TileArgs &args, int units, int P, int csz_max, int D, cudaStream_t s);
 // the pass-based search (fm.cu)
 int fm_max_spins();
 cudaError_t launch_fm(ising_handle *h, int32_t R, const ising_fm_params *p, int8_t *spins, double *E,
                       int32_t *passes, cudaStream_t s);
 void fm_free(ising_handle *h);
-int msc_cluster_max_active(ising_handle *h, int n_tiles, int P, int csz_max, int D);
+int msc_cluster_max_active(int n_tiles, int P, int csz_max, int D);
 }  // namespace isg

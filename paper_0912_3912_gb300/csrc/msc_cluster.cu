@@ -48,7 +48,7 @@ constexpr int kCT = 512;
 // for the field, which the loads extend to whole words; else packed in one byte
 // per site (large slabs, for shared memory's sake).
 template <int D, bool MASKS>
-__global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const TileArgs *__restrict__ Aptr, int P) {
+__global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const __grid_constant__ TileArgs A, int P) {
   extern __shared__ uint32_t smem[];
   __shared__ uint32_t s_any[2], s_active, s_convround, s_upd;
   __shared__ int32_t s_total[32], s_minima[32];
@@ -56,8 +56,7 @@ __global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const TileArgs *__r
   __shared__ int32_t s_cnt[33];
   __shared__ int32_t s_rng[2][2];
 
-  const TileArgs &A = *Aptr;
-  const DevGraph G = A.g;
+  const DevGraph &G = A.g;
   const uint32_t rank = tc::cluster_rank();
   // one cluster per tile and segment of its descents (see the tile kernels)
   const int unit = blockIdx.x / P, segs = A.segs, tile = unit / segs;
@@ -519,7 +518,7 @@ size_t msc_cluster_smem(int csz) {
 }
 
 template <int D, bool MASKS>
-cudaError_t launch_cfg(cudaLaunchConfig_t &cfg, const TileArgs *args, int P, size_t smem, int *max_active) {
+cudaError_t launch_cfg(cudaLaunchConfig_t &cfg, const TileArgs &args, int P, size_t smem, int *max_active) {
   auto kern = msc_cluster_kernel<D, MASKS>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -528,7 +527,7 @@ cudaError_t launch_cfg(cudaLaunchConfig_t &cfg, const TileArgs *args, int P, siz
 }
 
 // Launch (max_active == nullptr) or report how many clusters can be resident at once.
-cudaError_t msc_cluster_launch_or_query(ising_handle *h, int n_tiles, int P, int csz_max, int D, cudaStream_t s,
+static cudaError_t msc_cluster_launch_or_query(const TileArgs &args, int n_tiles, int P, int csz_max, int D, cudaStream_t s,
                                         int *max_active) {
   const size_t smem = msc_cluster_smem(csz_max);
 
@@ -544,19 +543,18 @@ cudaError_t msc_cluster_launch_or_query(ising_handle *h, int n_tiles, int P, int
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const TileArgs *args = (const TileArgs *)h->d_tile_args;
   if (cluster_masks(csz_max))
     return D == 3 ? launch_cfg<3, true>(cfg, args, P, smem, max_active) : launch_cfg<2, true>(cfg, args, P, smem, max_active);
   return D == 3 ? launch_cfg<3, false>(cfg, args, P, smem, max_active) : launch_cfg<2, false>(cfg, args, P, smem, max_active);
 }
 
-cudaError_t launch_msc_cluster(ising_handle *h, int units, int P, int csz_max, int D, cudaStream_t s) {
-  return msc_cluster_launch_or_query(h, units, P, csz_max, D, s, nullptr);
+cudaError_t launch_msc_cluster(const TileArgs &args, int units, int P, int csz_max, int D, cudaStream_t s) {
+  return msc_cluster_launch_or_query(args, units, P, csz_max, D, s, nullptr);
 }
 
-int msc_cluster_max_active(ising_handle *h, int n_tiles, int P, int csz_max, int D) {
+int msc_cluster_max_active(int n_tiles, int P, int csz_max, int D) {
   int m = 0;
-  if (msc_cluster_launch_or_query(h, n_tiles, P, csz_max, D, nullptr, &m) != cudaSuccess) {
+  if (msc_cluster_launch_or_query(TileArgs(), n_tiles, P, csz_max, D, nullptr, &m) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
