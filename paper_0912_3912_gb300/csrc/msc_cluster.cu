@@ -28,8 +28,9 @@
 // A visit is bound by its logic instructions (64 lanes a cycle and SM): the class
 // layout, sign planes, one pending target per lane and two chunks at a time took
 // 32^3 with fields, 1,024 replicas, 10 descents from 719 to 535 us a call with four
-// CTAs a cluster; two CTAs and two segments of descents each: 504.  With 32
-// replicas, ten segments of eight CTAs: 467 -> 84 us.
+// CTAs a cluster; two CTAs and two segments of descents each: 504, and 482 with the
+// arguments as a parameter (their pointers in constant memory).  With 32 replicas,
+// ten segments of eight CTAs: 467 -> 84 us.
 #include <cfloat>
 #include <type_traits>
 

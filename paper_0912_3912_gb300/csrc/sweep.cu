@@ -21,6 +21,7 @@
 #include <algorithm>
 #include <cfloat>
 #include <cstdio>
+#include <cstdlib>
 #include <map>
 #include <string>
 #include <vector>
@@ -1519,6 +1520,24 @@ void launch_pdl(bool pdl, void (*kern)(KArgs...), dim3 grid, int block, cudaStre
   cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
+// ISING_SWEEP_DEBUG=1: launch without graphs, synchronise and report after
+// every launch (diagnostics only).
+bool sweep_debug() {
+  static const int on = [] {
+    const char *v = std::getenv("ISING_SWEEP_DEBUG");
+    return v && v[0] == '1' ? 1 : 0;
+  }();
+  return on != 0;
+}
+
+void debug_step(const char *what, int c, cudaStream_t s) {
+  if (!sweep_debug()) return;
+  const cudaError_t e1 = cudaGetLastError();
+  const cudaError_t e2 = cudaStreamSynchronize(s);
+  std::fprintf(stderr, "[sweep] %s %d: launch=%s sync=%s\n", what, c, cudaGetErrorString(e1), cudaGetErrorString(e2));
+  std::fflush(stderr);
+}
+
 // Where a run stands: the current copy of the groups' state, the sweeps enqueued
 // (modulo 4: the `any` sets) and whether the last one's end is due.
 struct Phase {
@@ -1553,6 +1572,7 @@ void enqueue_sweep(const SweepArgs &A, Phase &ph, int mode, const std::vector<in
     if (mode == 0) launch_pdl(A.pdl != 0, sweep_visit<0, LPS, LAT>, grid, kST, s, B, (int32_t)c, c0, c1);
     else if (mode == 1) launch_pdl(A.pdl != 0, sweep_visit<1, LPS, LAT>, grid, kST, s, B, (int32_t)c, c0, c1);
     else launch_pdl(A.pdl != 0, sweep_visit<2, LPS, LAT>, grid, kST, s, B, (int32_t)c, c0, c1);
+    debug_step("visit", c, s);
   }
   ph.due = true;
   ph.sweep = (ph.sweep + 1) & 3;
@@ -1560,7 +1580,9 @@ void enqueue_sweep(const SweepArgs &A, Phase &ph, int mode, const std::vector<in
   const SweepArgs B = at_phase(A, ph);
   if (mode == 1) launch_pdl(A.pdl != 0, sweep_energy<true, LPS, LAT>, dim3(A.grid_e), kST, s, B);
   else launch_pdl(A.pdl != 0, sweep_energy<false, LPS, LAT>, dim3(A.grid_e), kST, s, B);
+  debug_step("energy", 0, s);
   launch_pdl(A.pdl != 0, sweep_restart<LPS>, dim3(A.grid_e), kST, s, at_phase(A, ph));
+  debug_step("restart", 0, s);
 }
 
 // Load every kernel of this configuration before any graph capture, so the
@@ -1612,8 +1634,13 @@ cudaError_t run_instance(ising_handle *h, SweepArgs A, int mode, cudaStream_t s)
   Phase ph;
   ph.copy[0] = A.gs;
   ph.copy[1] = A.gs + A.G;
+  if (sweep_debug())
+    std::fprintf(stderr, "[sweep] n=%d ncls=%d G=%d LPS=%d mode=%d grid_v=%ux%u grid_e=%d lattice=%d seq=%d\n", I.n, ncls,
+                 A.G, LPS, mode, grid.x, grid.y, A.grid_e, A.lattice, A.sequential);
   sweep_init<<<1, 32, 0, s>>>(A);
+  debug_step("init", 0, s);
   sweep_restart<LPS><<<A.grid_e, kST, 0, s>>>(A);
+  debug_step("restart0", 0, s);
   h->launches += 2;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // The round-end kernels (energy pass, restarts) follow every kRoundEnd-th
@@ -1639,7 +1666,7 @@ cudaError_t run_instance(ising_handle *h, SweepArgs A, int mode, cudaStream_t s)
   // 45^3 lattice and 10 % slower on 100^3, with the visits' registers short.)
   constexpr int kMaxNodes = 512;
   const int per_sweep = ncls + 2;
-  const bool use_graph = 4 * per_sweep <= kMaxNodes;
+  const bool use_graph = 4 * per_sweep <= kMaxNodes && !sweep_debug();
   const int chunk = use_graph ? std::min(16, kMaxNodes / per_sweep & ~3) : 1;
   // the first sweep runs with direct launches, the rest from the graph
   enqueue_sweep<LPS, LAT>(A, ph, mode, cls, grid, s, true);
@@ -1690,6 +1717,7 @@ cudaError_t run_instance(ising_handle *h, SweepArgs A, int mode, cudaStream_t s)
     cudaMemcpyAsync(S.h_done + (launched & 1), A.all_done, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
     cudaEventRecord(S.ev[launched & 1], s);
     ++launched;
+    if (sweep_debug()) std::fprintf(stderr, "[sweep] chunk %lld queued\n", (long long)launched);
     if (launched >= 2) {
       // look one chunk behind so the GPU always has queued work
       cudaEventSynchronize(S.ev[launched & 1]);

@@ -14,12 +14,13 @@
 // Four evaluators share the sweep/restart machinery:
 //   MODE 0  integer couplings, one warp per spin, lane = replica, exact int32
 //           fields recomputed from the neighbours' bits at each visit;
-//   MODE 1  FP32 couplings, one warp per spin, lane = replica, FP32 fields kept
-//           per (spin, replica) and updated at each visit from the neighbours
+//   MODE 1  FP32 couplings, four lanes per spin with 8 replicas each, FP32 fields
+//           kept per (spin, replica) and updated at each visit from the neighbours
 //           that flipped since the previous visit (the paper's incremental gain
 //           update), with a from-scratch refresh at descent sweeps
 //           d % refresh == 0 (always d == 0): the FP64 sum rounded to FP32,
-//           formed exactly in fixed point when that is exact (runit >= 0);
+//           formed exactly in fixed point when that is exact (runit >= 0; else a
+//           warp per spin, lane = replica);
 //           fields of instances that fit stay in shared memory;
 //   MODE 2  multi-spin coding for J in {-1,+1}, h in {-1,0,+1}: one thread per
 //           spin evaluates all 32 replicas with bitwise logic (unsatisfied-bond
