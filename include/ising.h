@@ -124,8 +124,8 @@ typedef enum { ISING_SCHED_COLOUR = 0, ISING_SCHED_SEQUENTIAL = 1 } ising_schedu
 /* Kernel families.  AUTO lets the planner (and its tuning cache) choose. */
 typedef enum {
   ISING_KERNEL_AUTO = 0,
-  ISING_KERNEL_TILE = 1,     /* one CTA per (instance, 32-replica group), lane = replica,
-                                persistent work queue over all tiles                    */
+  ISING_KERNEL_TILE = 1,     /* one CTA per (instance, 32-replica group) and segment of
+                                its descents, persistent work queue over all of them    */
   ISING_KERNEL_MSC = 2,      /* multi-spin coded tile: 32 replicas as bits of a word;
                                 needs J in {-1,+1}, h in {-1,0,+1}, no hyper-edges      */
   ISING_KERNEL_SWEEP = 3,    /* large instances: one launch per colour class over the
@@ -295,9 +295,10 @@ typedef struct {
                           in one warp; 2 = one start per warp, the best chosen
                           afterwards (same results either way)                    */
   int32_t reg_kernel;  /* instances of at most 512 spins in the one-unit integer
-                          form: 0 = automatic (registers when the searches fit one
-                          wave), 1 = always the register-resident kernel, -1 =
-                          always the shared-memory kernel (same results)          */
+                          form: 0 = automatic (gain keys in shared memory where
+                          they serve the instance, else registers when the
+                          searches fit one wave), 1 = always the register-resident
+                          kernel, -1 = never (same results)                       */
 } ising_fm_params;
 
 /* The paper's pass-based search with hill climbing (Sec. IV, Fig. 3), for
