@@ -545,16 +545,18 @@ const ClusterPlan &cluster_plan(ising_handle *h, int32_t R, const ising_search_p
 
 // CTA size and segments of the tile kernels for these arguments, null when no
 // CTA fits.  A descent's time in one CTA goes like a constant (barriers, round
-// trips) plus the steps the largest class takes: a warp per spin in the lane
-// modes (constant 6 steps), a thread per spin in the multi-spin-coded ones (30).
-// The tiles' descents (without a budget each descent is a unit of its own) run in
-// waves over the CTA slots; uneven instances fill the waves, a last wave of equal
-// ones does not.  Measured, us a call at 256 / 512 / 1024 threads: one cell grid
-// batch of 64 tiles 1744 / 988 / 680, of 800 2259 / 1563 / 1747, of 4096
-// 7609 / 7676 / 8626; 6,000 spins of degree 5, 20 replicas, 2 descents
-// 5077 / 2712 / 1774 (10046 in one segment); 31^3 +/-J, 1024 replicas, 10 descents
-// 2499 / 1572 / 1279; 16 x 16 +/-J, 64 replicas, 10 descents 52 / 42 / 44 (125 in
-// one segment).
+// trips) plus the steps the largest class takes: a warp's spins in the lane modes
+// (constant 6 steps; 10, or 15 with 1024 threads, in the FP32 visits, eight spins a
+// warp), a thread per spin in the multi-spin-coded ones (30).  The tiles' descents
+// (without a budget each descent is a unit of its own) run in waves over the CTA
+// slots; uneven instances fill the waves, a last wave of equal ones does not.
+// Measured, us a call at 256 / 512 / 1024 threads (FP32): cell grids of up to 2,048
+// spins, 64 tiles 603 / 370 / 338, 512 tiles 816 / 501 / 742, 1,024 tiles 971 / 950 /
+// 1395, 4,096 tiles 3197 / 3555 / 5318, of 128 spins each, 700 tiles 210 / 319 / 577;
+// 6,000 spins of degree 5, 20 replicas, 2 descents 2579 / 1340 / 979; 45 x 45, 10
+// descents of 64 replicas 323 / 230 / 218, of 1,024 447 / 561 / 553.  +/-J: 31^3, 1,024
+// replicas, 10 descents 2499 / 1572 / 1279; 16 x 16, 64 replicas, 10 descents 52 / 42 /
+// 44 (125 in one segment).
 const TilePlan *tile_plan(ising_handle *h, int mode, int32_t R, const ising_search_params *p) {
   TilePlan &T = h->tile_plan_cache;
   const int32_t parallel = p->sweep_budget > 0 ? 1 : p->restarts;
@@ -584,9 +586,17 @@ const TilePlan *tile_plan(ising_handle *h, int mode, int32_t R, const ising_sear
     const int64_t slots = (int64_t)tile_max_ctas_per_sm(mode, threads, smem) * h->sm_count;
     if (slots < 1) continue;
     const double per_step = mode >= 2 ? 2.0 * threads : (double)ncls * threads / 32;
-    const double unit = (mode >= 2 ? 30.0 : 6.0) + std::ceil(h->nmax / per_step);
-    double waves = std::max(1.0, weight / (double)slots);
-    if (nmin == h->nmax && waves < 2.0) waves = std::ceil(waves);
+    const double fixed = mode >= 2 ? 30.0 : (mode == 0 ? 6.0 : (threads == 1024 ? 15.0 : 10.0));
+    const double unit = fixed + std::ceil(h->nmax / per_step);
+    double waves = weight / (double)slots;
+    if (mode != 1) {
+      waves = std::max(1.0, waves);
+      if (nmin == h->nmax && waves < 2.0) waves = std::ceil(waves);
+    } else if (waves < 1.0) {
+      waves = 0.6 + 0.4 * waves;  // (SMs with fewer CTAs than they hold run them faster)
+    } else if (nmin == h->nmax && waves < 2.0) {
+      waves = 0.5 * (waves + std::ceil(waves));
+    }
     if (T.slots == 0 || unit * waves <= best) {  // (ties: the larger CTA)
       best = unit * waves;
       T.threads = threads;
