@@ -12,8 +12,9 @@
 // classes are independent sets, so all spins of a class decide at once.
 //
 // Four evaluators share the sweep/restart machinery:
-//   MODE 0  integer couplings, one warp per spin, lane = replica, exact int32
-//           fields recomputed from the neighbours' bits at each visit;
+//   MODE 0  integer couplings, exact int32 fields recomputed from the neighbours'
+//           bits at each visit, four lanes per spin with 8 replicas each where a
+//           warp has several pending spins, else a warp per spin, lane = replica;
 //   MODE 1  FP32 couplings, four lanes per spin with 8 replicas each, FP32 fields
 //           kept per (spin, replica) and updated at each visit from the neighbours
 //           that flipped since the previous visit (the paper's incremental gain
@@ -392,6 +393,36 @@ __device__ __forceinline__ uint32_t own_refresh(const DevGraph &G, const InstDes
   return own_store(F, j, r0, f, sw[j]);
 }
 
+// Integer couplings: the exact field from scratch, not kept.  Fewer than kOwnInt
+// pending spins of a warp's 32 positions are visited by the whole warp, a lane per
+// replica, whose marks take fewer steps: 6,000 spins of degree 5, 20 replicas, 2
+// descents 889 -> 623 us (all by four lanes 639), 300 spins 110 -> 114 (144); 1,000
+// spins, 1,024 replicas, 20 descents 982 -> 792 (3 / 6 spins: 802 / 806).
+constexpr int kOwnInt = 4;
+__device__ __forceinline__ uint32_t own_int(const DevGraph &G, const InstDesc &I, const uint32_t *sw, int j, int r0,
+                                            uint32_t k0, uint32_t k1, uint32_t e0, uint32_t e1) {
+  const int8_t *Ji = reinterpret_cast<const int8_t *>(G.J), *hJ = reinterpret_cast<const int8_t *>(G.hJ);
+  int sum = __ldg(reinterpret_cast<const int8_t *>(G.h) + I.spin_off + j), acc[8] = {};
+  auto add = [&](int t, uint32_t minus) {
+    sum += t;
+    minus >>= r0;
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+      if ((minus >> r) & 1u) acc[r] += t;
+  };
+  for (uint32_t k = k0; k < k1; ++k) add(__ldg(Ji + k), ~sw[__ldg(G.col + k)]);
+  for (uint32_t q = e0; q < e1; ++q)
+    add(__ldg(hJ + __ldg(G.inc_edge + q)), own_parity(G, sw, 0xffffffffu, j, q));
+  const uint32_t w = sw[j] >> r0;
+  uint32_t m = 0u;
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const int f = sum - 2 * acc[r];
+    if ((w >> r) & 1u ? f < 0 : f > 0) m |= 1u << r;
+  }
+  return m << r0;
+}
+
 // By the neighbours' flips since the previous visit (their words in fm), in CSR order
 // and then by hyper-edge; a replica with none keeps its field and its spin.
 __device__ __forceinline__ uint32_t own_visit(const DevGraph &G, const uint32_t *sw, const uint32_t *fm, float *F, int j,
@@ -459,7 +490,7 @@ tile_kernel(const __grid_constant__ TileArgs A) {
   __shared__ int32_t s_total[32], s_minima[32];
   __shared__ double s_best[32], s_E[32];
   __shared__ double s_red[THREADS];
-  __shared__ uint8_t s_slot[MODE == 1 ? THREADS : 32];
+  __shared__ uint8_t s_slot[MODE <= 1 ? THREADS : 32];
   __shared__ int s_cnt[33];
 
   const DevGraph &G = A.g;
@@ -668,52 +699,57 @@ tile_kernel(const __grid_constant__ TileArgs A) {
                 e1l = __ldg(G.inc_ptr + g + 1);
               }
               uint32_t todo = __ballot_sync(0xffffffffu, pl);
-              if constexpr (MODE == 1) {
-                const int ul = refresh && pl ? __ldg(G.runit + I.spin_off + jl) : 0;
-                const uint32_t own = __ballot_sync(0xffffffffu, pl && ul >= 0);
-                if ((own >> lane) & 1u) s_slot[(tid & ~31) + __popc(own & ((1u << lane) - 1u))] = (uint8_t)lane;
-                __syncwarp();
-                const int cnt = __popc(own), r0 = 8 * (lane & 3);
-                for (int p = lane >> 2; p - (lane >> 2) < cnt; p += 8) {
-                  const bool on = p < cnt;
-                  const int src = on ? s_slot[(tid & ~31) + p] : 0;
-                  const int j = __shfl_sync(0xffffffffu, jl, src);
-                  const uint32_t k0 = __shfl_sync(0xffffffffu, k0l, src), k1 = __shfl_sync(0xffffffffu, k1l, src);
-                  const uint32_t e0 = __shfl_sync(0xffffffffu, e0l, src), e1 = __shfl_sync(0xffffffffu, e1l, src);
-                  const int u = __shfl_sync(0xffffffffu, ul, src);
-                  uint32_t m = 0u;
-                  if (on)
-                    m = active & (refresh ? own_refresh(G, I, sw, Fc, j, r0, k0, k1, e0, e1, u)
-                                          : own_visit(G, sw, fm, Fc, j, r0, k0, k1, e0, e1));
-                  m |= __shfl_xor_sync(0xffffffffu, m, 1);
-                  m |= __shfl_xor_sync(0xffffffffu, m, 2);
-                  if (!on) continue;
-                  if (r0 == 0) {
-                    my_eval += __popc(active);
-                    my_flips += __popc(m);
-                    clear_pending(j);
-                    sw[j] ^= m;
-                    fm[j] = m;
-                    anyf |= m;
-                  }
-                  if (m) {
-                    for (uint32_t kk = k0 + (lane & 3); kk < k1; kk += 4) mark(__ldg(G.col + kk));
-                    for (uint32_t q = e0; q < e1; ++q) {
-                      const int2 oth = __ldg(G.inc_oth + q);
-                      if (oth.x >= 0) {
-                        if ((lane & 3) < 2) mark((lane & 3) == 0 ? oth.x : oth.y);
-                        continue;
-                      }
-                      const int e = __ldg(G.inc_edge + q);
-                      for (uint32_t mm = __ldg(G.hptr + e) + (lane & 3), me = __ldg(G.hptr + e + 1); mm < me; mm += 4) {
-                        const int o = __ldg(G.hmem + mm);
-                        if (o != j) mark(o);
+              {
+                const int ul = MODE == 1 && refresh && pl ? __ldg(G.runit + I.spin_off + jl) : 0;
+                uint32_t own = __ballot_sync(0xffffffffu, pl && ul >= 0);
+                if (MODE == 0 && __popc(own) < kOwnInt) own = 0u;
+                if (own) {
+                  if ((own >> lane) & 1u) s_slot[(tid & ~31) + __popc(own & ((1u << lane) - 1u))] = (uint8_t)lane;
+                  __syncwarp();
+                  const int cnt = __popc(own), r0 = 8 * (lane & 3);
+                  for (int p = lane >> 2; p - (lane >> 2) < cnt; p += 8) {
+                    const bool on = p < cnt;
+                    const int src = on ? s_slot[(tid & ~31) + p] : 0;
+                    const int j = __shfl_sync(0xffffffffu, jl, src);
+                    const uint32_t k0 = __shfl_sync(0xffffffffu, k0l, src), k1 = __shfl_sync(0xffffffffu, k1l, src);
+                    const uint32_t e0 = __shfl_sync(0xffffffffu, e0l, src), e1 = __shfl_sync(0xffffffffu, e1l, src);
+                    const int u = __shfl_sync(0xffffffffu, ul, src);
+                    uint32_t m = 0u;
+                    if (MODE == 0) {
+                      if (on) m = active & own_int(G, I, sw, j, r0, k0, k1, e0, e1);
+                    } else if (on)
+                      m = active & (refresh ? own_refresh(G, I, sw, Fc, j, r0, k0, k1, e0, e1, u)
+                                            : own_visit(G, sw, fm, Fc, j, r0, k0, k1, e0, e1));
+                    m |= __shfl_xor_sync(0xffffffffu, m, 1);
+                    m |= __shfl_xor_sync(0xffffffffu, m, 2);
+                    if (!on) continue;
+                    if (r0 == 0) {
+                      my_eval += __popc(active);
+                      my_flips += __popc(m);
+                      clear_pending(j);
+                      sw[j] ^= m;
+                      if (MODE == 1) fm[j] = m;
+                      anyf |= m;
+                    }
+                    if (m) {
+                      for (uint32_t kk = k0 + (lane & 3); kk < k1; kk += 4) mark(__ldg(G.col + kk));
+                      for (uint32_t q = e0; q < e1; ++q) {
+                        const int2 oth = __ldg(G.inc_oth + q);
+                        if (oth.x >= 0) {
+                          if ((lane & 3) < 2) mark((lane & 3) == 0 ? oth.x : oth.y);
+                          continue;
+                        }
+                        const int e = __ldg(G.inc_edge + q);
+                        for (uint32_t mm = __ldg(G.hptr + e) + (lane & 3), me = __ldg(G.hptr + e + 1); mm < me; mm += 4) {
+                          const int o = __ldg(G.hmem + mm);
+                          if (o != j) mark(o);
+                        }
                       }
                     }
                   }
+                  todo &= ~own;
+                  __syncwarp();
                 }
-                todo &= ~own;
-                __syncwarp();
               }
               while (todo) {
               const int src = __ffs(todo) - 1;

@@ -119,18 +119,20 @@ def test_tile_energy_sums(kind, n, R):
         _compare([inst], [n], R, kind == "i8", max_sweeps=max_sweeps, restarts=restarts, kernel=isg.KERNEL_TILE)
 
 
-# FP32 tile visits, eight spins at a time: classes of fewer and more spins than that,
+# Tile visits, eight spins at a time: classes of fewer and more spins than that,
 # rows of more than the entries fetched together, hyper-edges of 2 to 9 members,
 # refreshes in fixed point, in FP64 and (wider) both in one class.
 @pytest.mark.parametrize("n,R,schedule", [(7, 5, isg.SCHED_COLOUR), (100, 32, isg.SCHED_COLOUR),
                                           (300, 41, isg.SCHED_COLOUR), (3000, 9, isg.SCHED_COLOUR),
                                           (7, 32, isg.SCHED_SEQUENTIAL), (100, 8, isg.SCHED_SEQUENTIAL)])
-@pytest.mark.parametrize("kind", ["f32", "wide", "wider"])
-def test_tile_fp32_visits(kind, n, R, schedule):
-    inst = _star_graph(n, "f32", n) if n >= 100 else W.random_graph(n, 3.0, n, n_hyper=3, hyper_order=(2, 3, 4))
+@pytest.mark.parametrize("kind", ["i8", "f32", "wide", "wider"])
+def test_tile_visits(kind, n, R, schedule):
+    dtype = "i8" if kind == "i8" else "f32"
+    inst = (_star_graph(n, dtype, n) if n >= 100 else
+            W.random_graph(n, 3.0, n, dtype=dtype, n_hyper=3, hyper_order=(2, 3, 4)))
     if kind.startswith("wide"):
         inst = _exp_spread(inst, *((-12, 12) if kind == "wide" else (-45, 25)))
-    _compare([inst], [n], R, False, max_sweeps=200, restarts=2, refresh_every=3, schedule=schedule,
+    _compare([inst], [n], R, kind == "i8", max_sweeps=200, restarts=2, refresh_every=3, schedule=schedule,
              kernel=isg.KERNEL_TILE)
 
 
