@@ -168,9 +168,9 @@ __device__ void tile_energy_lanes(const DevGraph &G, const InstDesc &I, const ui
 // -t + 2 t p_r, so a predicated add per replica for 32 spins at once, where the form
 // above spends that and the term's decoding on every spin for itself (bound by
 // issue).  FP32: 64-bit fixed point, NV = 8 replicas at a time, the rows read again
-// from L1 for each (1,024 cell grids of 512 spins, two descents: 1,754 us with the
-// form above, 1,623 / 1,577 / 1,699 with 4 / 8 / 16); integers: all 32 (1,000 random
-// graphs of 1,024 spins: 1,112 -> 1,036 us).  False, and nothing done, when FP32
+// from L1 for each (1,024 cell grids of 128 to 2,048 spins: 1,754 us a call with
+// the form above, 1,623 / 1,577 / 1,699 with 4 / 8 / 16); integers: all 32 (a graph of
+// 1,000 spins, 1,024 replicas, 20 descents: 1,112 -> 1,036 us).  False, and nothing done, when FP32
 // terms are not integers of one unit, or so wide or so many that a lane's sum could
 // leave its 62 bits (integers: a warp's its 31); the same for the whole CTA.
 template <bool FLOAT, int THREADS>
@@ -336,7 +336,7 @@ __device__ __forceinline__ uint32_t sliced_ge(uint32_t c0, uint32_t c1, uint32_t
 // row, the neighbours' words and each term's decoding on one spin (some 380
 // instructions) and was bound by issue; here a term is a predicated add per replica
 // for 8 spins at once, and 8 pending spins of a class fill a warp.  1,024 cell grids
-// of 512 spins, one descent: 1,577 -> 965 us (one lane for all 32 replicas of a spin:
+// of 128 to 2,048 spins: 1,577 -> 965 us (one lane for all 32 replicas of a spin:
 // 1,127, and slower than a whole warp on small classes); 4,096 of them: 5,983 ->
 // 3,265; one graph of 6,000 spins: 1,718 -> 964.  Both forms return the replicas in
 // which the spin is against its field and leave the fields in F.
