@@ -420,6 +420,7 @@ void free_handle(ising_handle *h) {
   for (void *p : ptrs)
     if (p) cudaFree(p);
   if (h->h_stats_pinned) cudaFreeHost(h->h_stats_pinned);
+  if (h->setup) cudaStreamDestroy(h->setup);
   cudaSetDevice(cur);
   delete h;
 }
@@ -779,6 +780,13 @@ struct NvtxRange {
   NvtxRange(const NvtxRange &) = delete;
   NvtxRange &operator=(const NvtxRange &) = delete;
 };
+
+cudaError_t setup_stream(ising_handle *h, cudaStream_t *s) {
+  cudaError_t e = cudaSuccess;
+  if (!h->setup) e = cudaStreamCreateWithFlags(&h->setup, cudaStreamNonBlocking);
+  *s = h->setup;
+  return e;
+}
 
 void kt_begin(ising_handle *h, const char *name, cudaStream_t s) {
   if (!h->timing) return;

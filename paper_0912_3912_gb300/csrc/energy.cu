@@ -438,9 +438,9 @@ bool integer_sums(const ising_handle *h) {
 }
 
 template <typename T>
-cudaError_t put(T **dst, const std::vector<T> &src) {
+cudaError_t put(T **dst, const std::vector<T> &src, cudaStream_t setup) {
   const cudaError_t e = cudaMalloc((void **)dst, src.size() * sizeof(T));
-  return e != cudaSuccess ? e : cudaMemcpy(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice);
+  return e != cudaSuccess ? e : cudaMemcpyAsync(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice, setup);
 }
 
 // Work list, words and accumulators of the packed form.  On failure nothing
@@ -459,10 +459,13 @@ cudaError_t plan_parts(ising_handle *h, int32_t R, int32_t groups) {
   if (work.size() > 0x7fffffffu) return cudaErrorInvalidValue;
   const size_t slots = (size_t)h->n_inst * groups;
   const size_t acc_bytes = slots * 32 * 2 * sizeof(unsigned long long);
-  cudaError_t e = put(&h->d_en_work, work);
+  cudaStream_t setup = nullptr;
+  cudaError_t e = setup_stream(h, &setup);
+  if (e == cudaSuccess) e = put(&h->d_en_work, work, setup);
   if (e == cudaSuccess) e = cudaMalloc((void **)&h->d_en_words, (size_t)groups * h->total_spins * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc((void **)&h->d_en_acc, acc_bytes + slots * sizeof(unsigned int));
-  if (e == cudaSuccess) e = cudaMemset(h->d_en_acc, 0, acc_bytes + slots * sizeof(unsigned int));
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->d_en_acc, 0, acc_bytes + slots * sizeof(unsigned int), setup);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(setup);  // (before the caller's stream reads them)
   if (e != cudaSuccess) {
     energy_plan_free(h);
     return e;
@@ -482,8 +485,11 @@ cudaError_t plan_partials(ising_handle *h, int32_t R) {
       for (int c = 0; c < nch; ++c) work.push_back(make_int4(b, r, c, nch));
     }
   }
-  cudaError_t e = put(&h->d_en_work, work);
-  if (e == cudaSuccess) e = put(&h->d_en_first, first);
+  cudaStream_t setup = nullptr;
+  cudaError_t e = setup_stream(h, &setup);
+  if (e == cudaSuccess) e = put(&h->d_en_work, work, setup);
+  if (e == cudaSuccess) e = put(&h->d_en_first, first, setup);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(setup);
   if (e == cudaSuccess) e = cudaMalloc(&h->d_en_partd, work.size() * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&h->d_en_parti, work.size() * sizeof(long long));
   if (e != cudaSuccess) {

@@ -158,6 +158,11 @@ struct ising_handle {
   bool dense = false;       // instances given as dense matrices
   bool msc_ok = false;      // every coupling +/-1, every field in {-1,0,+1}, no hyper-edges
   bool has_hyper = false;
+  // (setup_stream) what the handle builds once and keeps - work lists, zeroed sums,
+  // change entries - is written on this stream and waited for: a caller's
+  // non-blocking stream is not ordered after the default stream, and a stream that
+  // is being captured would only record the writes
+  cudaStream_t setup = nullptr;
   int32_t fm_rounds = 1;  // most change entries of one spin with one target (InstDesc::fm_ent >= 0)
   int32_t nmax = 0;
   int64_t total_spins = 0, total_nnz = 0, total_edges = 0, total_members = 0;
@@ -239,6 +244,8 @@ T &family_state(std::unique_ptr<FamilyState> &slot) {
   if (!slot) slot.reset(new T());
   return static_cast<T &>(*slot);
 }
+// the handle's own non-blocking stream, created on first use (api.cu)
+cudaError_t setup_stream(ising_handle *h, cudaStream_t *s);
 // device timing around a launch (no-ops unless timing is on); name: a static string
 void kt_begin(ising_handle *h, const char *name, cudaStream_t s);
 void kt_end(ising_handle *h, cudaStream_t s);

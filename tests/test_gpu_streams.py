@@ -1,0 +1,94 @@
+"""Calls on the caller's own streams: what a handle builds on a first call is in
+place before that call's kernels read it, whatever else the GPU is doing.
+
+The caller's stream is non-blocking (every torch.cuda.Stream is), so nothing
+orders it after the default stream, which is kept busy with ordinary work here.
+Results are compared with the CPU oracle."""
+import numpy as np
+import pytest
+
+import oracle
+import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+isg = pytest.importorskip("paper_0912_3912_gb300")
+
+from test_gpu_parity import _exp_spread  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_0912_3912_gb300 import build as B
+    B.build()
+    oracle.build()
+
+
+@pytest.fixture(scope="module")
+def busy():
+    """Queue some 50 ms of copies on the default stream."""
+    a = torch.zeros(1 << 28, dtype=torch.float32, device="cuda")
+    b = torch.empty_like(a)
+
+    def go():
+        torch.cuda.synchronize()
+        with torch.cuda.stream(torch.cuda.default_stream()):
+            for _ in range(150):
+                b.copy_(a)
+    return go
+
+
+def _energy_instance(kind):
+    if kind == "lattice":
+        return W.lattice((14, 14, 14), True, "pm1", "pm1_0", seed=14)
+    g = W.random_graph(5000, 5.0, 5, dtype="f32", n_hyper=300, hyper_order=(2, 3))
+    return _exp_spread(g, -45, 25) if kind == "wide" else g  # (wide: the FP64 passes)
+
+
+def _check_energy(inst, spins, E):
+    ref = oracle.energies(inst, spins)
+    if inst.dtype == "i8":
+        assert np.array_equal(E.cpu().numpy()[0], ref)
+    else:  # exact sums rounded once (wide: FP64 sums); the oracle's are FP64
+        np.testing.assert_allclose(E.cpu().numpy()[0], ref, rtol=1e-12, atol=1e-9)
+
+
+@pytest.mark.parametrize("kind", ["lattice", "graph", "wide"])
+def test_first_energy_call_on_a_side_stream(kind, busy):
+    inst = _energy_instance(kind)
+    h = isg.Handle([inst])
+    side = torch.cuda.Stream()
+    for R in (33, 5):  # (a new replica count builds anew)
+        spins = (np.random.default_rng(R).integers(0, 2, size=(R, inst.n)) * 2 - 1).astype(np.int8)
+        dev = torch.from_numpy(spins).cuda()
+        busy()
+        with torch.cuda.stream(side):
+            E = [h.energy(dev, R) for _ in range(2)]
+        side.synchronize()
+        for e in E:
+            _check_energy(inst, spins, e)
+    torch.cuda.synchronize()
+    h.close()
+
+
+# A first call that is only captured builds what the handle keeps all the same.
+@pytest.mark.parametrize("kind", ["lattice", "graph", "wide"])
+def test_first_energy_call_under_capture(kind):
+    inst = _energy_instance(kind)
+    R = 9
+    spins = (np.random.default_rng(R).integers(0, 2, size=(R, inst.n)) * 2 - 1).astype(np.int8)
+    dev = torch.from_numpy(spins).cuda()
+    h = isg.Handle([inst])
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, capture_error_mode="relaxed"):
+        captured = h.energy(dev, R)
+    _check_energy(inst, spins, h.energy(dev, R))
+    for _ in range(2):
+        g.replay()
+    _check_energy(inst, spins, captured)
+    torch.cuda.synchronize()
+    del g
+    h.close()
