@@ -392,12 +392,14 @@ bool fault_is(const char *what) {
 int g_alloc_countdown = 0;  // allocations left before the injected failure (0: none)
 
 template <class T>
-cudaError_t upload(T **dst, const std::vector<T> &src) {
+cudaError_t upload(ising_handle *h, T **dst, const std::vector<T> &src) {
   if (g_alloc_countdown > 0 && --g_alloc_countdown == 0) return cudaErrorMemoryAllocation;
-  cudaError_t e = cudaMalloc((void **)dst, std::max<size_t>(1, src.size()) * sizeof(T));
-  if (e != cudaSuccess) return e;
-  if (!src.empty()) e = cudaMemcpy(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice);
-  return e;
+  cudaStream_t setup = nullptr;
+  cudaError_t e = setup_stream(h, &setup);
+  if (e == cudaSuccess) e = cudaMalloc((void **)dst, std::max<size_t>(1, src.size()) * sizeof(T));
+  if (e != cudaSuccess || src.empty()) return e;
+  e = cudaMemcpyAsync(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice, setup);
+  return e != cudaSuccess ? e : cudaStreamSynchronize(setup);  // (before any stream reads it)
 }
 
 void free_handle(ising_handle *h) {
@@ -625,7 +627,8 @@ ising_status run_tile(ising_handle *h, int mode, int32_t R, const ising_search_p
       for (int32_t g = 0; g < groups; ++g) tiles.push_back(make_int2(b, g));
     if (h->d_tiles) cudaFree(h->d_tiles);
     h->d_tiles = nullptr;
-    if (upload(&h->d_tiles, tiles) != cudaSuccess) return ISING_ERR_CUDA;
+    h->tiles_R = -1;
+    if (upload(h, &h->d_tiles, tiles) != cudaSuccess) return ISING_ERR_CUDA;
     h->n_tiles = (int32_t)tiles.size();
     h->tiles_R = R;
   }
@@ -995,23 +998,23 @@ ising_status ising_create(const ising_instance_desc *descs, int32_t n_instances,
   h->total_edges = edge_off;
   h->total_members = mem_off;
 
-  bool ok = upload(&h->d_inst, inst) == cudaSuccess && upload(&h->d_row, row) == cudaSuccess &&
-            upload(&h->d_col, col) == cudaSuccess && upload(&h->d_inc_ptr, inc_ptr) == cudaSuccess &&
-            upload(&h->d_inc_edge, inc_edge) == cudaSuccess && upload(&h->d_inc_oth, inc_oth) == cudaSuccess &&
-            upload(&h->d_hptr, hptr) == cudaSuccess &&
-            upload(&h->d_hmem, hmem) == cudaSuccess && upload(&h->d_order, order) == cudaSuccess &&
-            upload(&h->d_cls, cls) == cudaSuccess;
+  bool ok = upload(h, &h->d_inst, inst) == cudaSuccess && upload(h, &h->d_row, row) == cudaSuccess &&
+            upload(h, &h->d_col, col) == cudaSuccess && upload(h, &h->d_inc_ptr, inc_ptr) == cudaSuccess &&
+            upload(h, &h->d_inc_edge, inc_edge) == cudaSuccess && upload(h, &h->d_inc_oth, inc_oth) == cudaSuccess &&
+            upload(h, &h->d_hptr, hptr) == cudaSuccess &&
+            upload(h, &h->d_hmem, hmem) == cudaSuccess && upload(h, &h->d_order, order) == cudaSuccess &&
+            upload(h, &h->d_cls, cls) == cudaSuccess;
   if (ok) {
     if (fl) {
-      ok = upload((float **)&h->d_J, Jf) == cudaSuccess && upload((float **)&h->d_h, hf) == cudaSuccess &&
-           upload((float **)&h->d_hJ, hJf) == cudaSuccess;
-      ok = ok && upload(&h->d_runit, runit) == cudaSuccess;
+      ok = upload(h, (float **)&h->d_J, Jf) == cudaSuccess && upload(h, (float **)&h->d_h, hf) == cudaSuccess &&
+           upload(h, (float **)&h->d_hJ, hJf) == cudaSuccess;
+      ok = ok && upload(h, &h->d_runit, runit) == cudaSuccess;
     } else if (f64) {
-      ok = upload((double **)&h->d_J, Jd) == cudaSuccess && upload((double **)&h->d_h, hd) == cudaSuccess &&
-           upload((double **)&h->d_hJ, hJd) == cudaSuccess;
+      ok = upload(h, (double **)&h->d_J, Jd) == cudaSuccess && upload(h, (double **)&h->d_h, hd) == cudaSuccess &&
+           upload(h, (double **)&h->d_hJ, hJd) == cudaSuccess;
     } else {
-      ok = upload((int8_t **)&h->d_J, Ji) == cudaSuccess && upload((int8_t **)&h->d_h, hi) == cudaSuccess &&
-           upload((int8_t **)&h->d_hJ, hJi) == cudaSuccess;
+      ok = upload(h, (int8_t **)&h->d_J, Ji) == cudaSuccess && upload(h, (int8_t **)&h->d_h, hi) == cudaSuccess &&
+           upload(h, (int8_t **)&h->d_hJ, hJi) == cudaSuccess;
     }
   }
   if (ok && h->any_lattice) {
@@ -1064,15 +1067,15 @@ ising_status ising_create(const ising_instance_desc *descs, int32_t n_instances,
         meta[D.spin_off + v] = m;
       }
     }
-    ok = upload(&h->d_meta, meta) == cudaSuccess && upload(&h->d_latinfo, latinfo) == cudaSuccess &&
-         (fl ? upload((float **)&h->d_Jpos, Jpf) : upload((int8_t **)&h->d_Jpos, Jpi)) == cudaSuccess &&
-         (fl ? upload((float **)&h->d_Jfwd, Jff) : upload((int8_t **)&h->d_Jfwd, Jfi)) == cudaSuccess;
+    ok = upload(h, &h->d_meta, meta) == cudaSuccess && upload(h, &h->d_latinfo, latinfo) == cudaSuccess &&
+         (fl ? upload(h, (float **)&h->d_Jpos, Jpf) : upload(h, (int8_t **)&h->d_Jpos, Jpi)) == cudaSuccess &&
+         (fl ? upload(h, (float **)&h->d_Jfwd, Jff) : upload(h, (int8_t **)&h->d_Jfwd, Jfi)) == cudaSuccess;
   }
   if (ok && dense) {
     std::vector<float> Jd;
     for (int32_t b = 0; b < n_instances; ++b)
       Jd.insert(Jd.end(), descs[b].J_dense, descs[b].J_dense + (int64_t)descs[b].n * descs[b].n);
-    ok = upload(&h->d_Jdense, Jd) == cudaSuccess;
+    ok = upload(h, &h->d_Jdense, Jd) == cudaSuccess;
   }
   ok = ok && cudaMalloc(&h->d_seeds, sizeof(uint64_t) * n_instances) == cudaSuccess &&
        cudaMalloc(&h->d_stats, sizeof(unsigned long long) * 8) == cudaSuccess &&

@@ -444,7 +444,7 @@ cudaError_t launch_dense(ising_handle *h, const ising_search_params *p, int32_t 
       if ((e = cudaMalloc(&D.best, (size_t)R * n)) != cudaSuccess) return e;
       if ((e = cudaMalloc(&D.active, 64)) != cudaSuccess) return e;
       if ((e = cudaMallocHost(&D.h_active, 64)) != cudaSuccess) return e;
-      if ((e = cudaMemset(D.S, 0, (size_t)n * Rp * 2)) != cudaSuccess) return e;
+      if ((e = cudaMemsetAsync(D.S, 0, (size_t)n * Rp * 2, s)) != cudaSuccess) return e;
       dense_split<<<h->sm_count * 8, 256, 0, s>>>(h->d_Jdense + joff, D.hi, D.lo, (int64_t)n * n);
     }
     const float *J = h->d_Jdense + joff;
@@ -474,7 +474,7 @@ cudaError_t launch_dense(ising_handle *h, const ising_search_params *p, int32_t 
           h->launches += 1;
         }
         if ((e = cudaMalloc(&D.S_tc, (size_t)Rp128 * np * 2)) != cudaSuccess) return e;
-        if ((e = cudaMemset(D.S_tc, 0, (size_t)Rp128 * np * 2)) != cudaSuccess) return e;
+        if ((e = cudaMemsetAsync(D.S_tc, 0, (size_t)Rp128 * np * 2, s)) != cudaSuccess) return e;
         if ((e = cudaMalloc(&D.planes, (size_t)4 * np * np * 2)) != cudaSuccess) return e;
         if ((e = cudaMalloc(&D.bands, (size_t)4 * np * 128 * 2)) != cudaSuccess) return e;
         if ((e = cudaMalloc(&D.Se, (size_t)Rp128 * np * 2)) != cudaSuccess) return e;

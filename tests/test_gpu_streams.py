@@ -92,3 +92,49 @@ def test_first_energy_call_under_capture(kind):
     torch.cuda.synchronize()
     del g
     h.close()
+
+
+# First searches of a fresh handle, family by family: the instance's own copies,
+# work lists and zeroed buffers; the dense family against a second call.
+@pytest.mark.parametrize("kind", ["tile", "msc", "cluster", "sweep", "passes", "dense", "dense_library"])
+def test_first_search_on_a_side_stream(kind, busy):
+    if kind == "tile":
+        inst, R, kw = W.random_graph(500, 5.0, 3, dtype="f32", n_hyper=40), 40, dict(kernel=isg.KERNEL_TILE)
+    elif kind == "sweep":
+        inst, R, kw = W.random_graph(500, 5.0, 4, dtype="i8", n_hyper=40), 20, dict(kernel=isg.KERNEL_SWEEP)
+    elif kind == "passes":
+        inst, R, kw = W.random_graph(400, 5.0, 6, dtype="f32", n_hyper=40), 6, {}
+    elif kind.startswith("dense"):
+        inst, R = W.sk(300, seed=8), 70
+        kw = dict(kernel=isg.KERNEL_DENSE_TC, schedule=isg.SCHED_SEQUENTIAL,
+                  dense_variant=isg.DENSE_LIBRARY if kind == "dense_library" else isg.DENSE_OWN)
+    else:
+        inst = W.lattice((16, 16, 16), True, "pm1", "pm1_0", seed=9)
+        R, kw = 33, dict(kernel=isg.KERNEL_MSC, cluster_ctas=1 if kind == "msc" else 4)
+    side = torch.cuda.Stream()
+    busy()
+    h = isg.Handle([inst])
+    with torch.cuda.stream(side):
+        if kind == "passes":
+            spins, E, extra, _ = h.fm_search([5], R, stats=False)
+        else:
+            r = h.local_search([5], R, max_sweeps=200, stats=False, **kw)
+            spins, E, extra = r.spins, r.energy, r.minima
+    side.synchronize()
+    spins, E = spins.cpu().numpy().reshape(R, inst.n), E[0].cpu().numpy()
+    extra = extra[0].cpu().numpy()
+    torch.cuda.synchronize()
+    if kind == "passes":
+        for k in range(R):
+            s, e, p = oracle.fm_search(inst, oracle.random_start(inst.n, 5, 0, k, 0))
+            assert np.array_equal(spins[k], s) and extra[k] == p
+            assert abs(E[k] - e) <= 1e-9 * (1 + abs(e))
+    elif kind.startswith("dense"):
+        again = h.local_search([5], R, max_sweeps=200, **kw)
+        assert np.array_equal(spins, again.spins.cpu().numpy().reshape(R, inst.n))
+        assert np.array_equal(E, again.energy[0].cpu().numpy())
+    else:
+        s, e, m, _ = oracle.descent(inst, 5, 0, R, max_sweeps=200)
+        assert np.array_equal(spins, s) and np.array_equal(extra, m)
+        np.testing.assert_allclose(E, e, rtol=1e-9, atol=1e-9)
+    h.close()
