@@ -1384,24 +1384,39 @@ cudaError_t variant_shape(const ising_handle *h, FmBufs &B, int var, int nmax, F
 }
 
 // The change entries of every instance that can take the gain keys, built by
-// the first call; without room for them the other kernels serve.
-cudaError_t build_entries(ising_handle *h, FmBufs &B, cudaStream_t s) {
+// the first call (on the handle's own stream and waited for, so that they are
+// there whatever becomes of the caller's stream, also one that is being
+// captured); without room for them the other kernels serve.
+cudaError_t build_entries(ising_handle *h, FmBufs &B) {
   if (B.ent_stride >= 0) return cudaSuccess;
   int most = -1;
   for (const InstDesc &D : h->inst)
     if (D.fbits >= 0) most = std::max(most, D.fm_ent);
-  B.ent_stride = 0;
-  if (most < 0) return cudaSuccess;
-  const int stride = std::max(4, (most + 3) / 4 * 4);
-  if (cudaMalloc((void **)&B.ent, (size_t)h->total_spins * stride * sizeof(int4)) != cudaSuccess) {
-    cudaGetLastError();
-    B.ent = nullptr;
+  if (most < 0) {
+    B.ent_stride = 0;
     return cudaSuccess;
   }
-  B.ent_stride = stride;
-  fm_entries_kernel<<<h->n_inst, 256, 0, s>>>(h->graph(), B.ent, stride);
+  const int stride = std::max(4, (most + 3) / 4 * 4);
+  cudaStream_t setup = nullptr;
+  cudaError_t e = setup_stream(h, &setup);
+  if (e != cudaSuccess) return e;
+  if ((e = cudaMalloc((void **)&B.ent, (size_t)h->total_spins * stride * sizeof(int4))) != cudaSuccess) {
+    B.ent = nullptr;
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    B.ent_stride = 0;
+    return cudaSuccess;
+  }
+  fm_entries_kernel<<<h->n_inst, 256, 0, setup>>>(h->graph(), B.ent, stride);
   h->launches += 1;
-  return cudaGetLastError();
+  if ((e = cudaGetLastError()) == cudaSuccess) e = cudaStreamSynchronize(setup);
+  if (e != cudaSuccess) {
+    cudaFree(B.ent);
+    B.ent = nullptr;
+    return e;
+  }
+  B.ent_stride = stride;
+  return cudaSuccess;
 }
 
 }  // namespace
@@ -1419,7 +1434,7 @@ cudaError_t launch_fm(ising_handle *h, int32_t R, const ising_fm_params *fp, int
   FmBufs &B = family_state<FmBufs>(h->fm_st);
   cudaError_t e;
   const bool fl = h->dtype == ISING_F32, f64 = h->dtype == ISING_F64;
-  if (!f64 && (e = build_entries(h, B, s)) != cudaSuccess) return e;
+  if (!f64 && (e = build_entries(h, B)) != cudaSuccess) return e;
   // The form of an instance: gain keys where its fields are integers of few
   // enough bits in one unit (the energies then FP64 unless those are too) and
   // its changes fit the entries; else the arithmetic's general kernel.

@@ -138,3 +138,24 @@ def test_first_search_on_a_side_stream(kind, busy):
         assert np.array_equal(spins, s) and np.array_equal(extra, m)
         np.testing.assert_allclose(E, e, rtol=1e-9, atol=1e-9)
     h.close()
+
+
+# The same for the pass-based search, whose first call builds the move records:
+# that call is captured and never run.
+@pytest.mark.parametrize("dtype", ["i8", "f32"])
+def test_first_passes_call_under_capture(dtype):
+    inst = W.random_graph(300, 5.0, 12, dtype=dtype, n_hyper=40, hyper_order=(2, 3))
+    R = 4
+    h = isg.Handle([inst])
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, capture_error_mode="relaxed"):
+        h.fm_search([5], R, stats=False)
+    torch.cuda.synchronize()
+    del g
+    spins, E, passes, _ = h.fm_search([5], R)
+    spins = spins.cpu().numpy().reshape(R, inst.n)
+    for k in range(R):
+        s, e, p = oracle.fm_search(inst, oracle.random_start(inst.n, 5, 0, k, 0))
+        assert np.array_equal(spins[k], s) and int(passes[0, k]) == p
+        assert abs(float(E[0, k]) - e) <= 1e-9 * (1 + abs(e))
+    h.close()
