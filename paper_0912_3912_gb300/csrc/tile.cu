@@ -20,8 +20,8 @@
 //           that flipped since the previous visit (the paper's incremental gain
 //           update), with a from-scratch refresh at descent sweeps
 //           d % refresh == 0 (always d == 0): the FP64 sum rounded to FP32,
-//           formed exactly in fixed point when that is exact (runit >= 0; else a
-//           warp per spin, lane = replica);
+//           formed exactly in fixed point when that is exact (runit >= 0; else, and
+//           for a warp's lone pending spin, a warp per spin, lane = replica);
 //           fields of instances that fit stay in shared memory;
 //   MODE 2  multi-spin coding for J in {-1,+1}, h in {-1,0,+1}: one thread per
 //           spin evaluates all 32 replicas with bitwise logic (unsatisfied-bond
@@ -393,12 +393,20 @@ __device__ __forceinline__ uint32_t own_refresh(const DevGraph &G, const InstDes
   return own_store(F, j, r0, f, sw[j]);
 }
 
-// Integer couplings: the exact field from scratch, not kept.  Fewer than kOwnInt
-// pending spins of a warp's 32 positions are visited by the whole warp, a lane per
-// replica, whose marks take fewer steps: 6,000 spins of degree 5, 20 replicas, 2
-// descents 889 -> 623 us (all by four lanes 639), 300 spins 110 -> 114 (144); 1,000
-// spins, 1,024 replicas, 20 descents 982 -> 792 (3 / 6 spins: 802 / 806).
-constexpr int kOwnInt = 4;
+// Fewer than this many pending spins of a warp's 32 positions are visited by the
+// whole warp, a lane per replica: its terms cost one add where four lanes take
+// eight predicated ones each, and its marks take fewer steps.  Integers: 6,000 spins
+// of degree 5, 20 replicas, 2 descents 889 -> 623 us (all by four lanes 639), 300
+// spins 110 -> 114 (144); 1,000 spins, 1,024 replicas, 20 descents 982 -> 792 (3 / 6
+// spins: 802 / 806).  FP32, where the fields are read and written besides: one spin,
+// as in the index order, dense rows and the last sweeps (1,000 spins in index order
+// 11.0 -> 7.6 ms, 256 fully coupled spins given as rows, 32 replicas, 100 -> 44, 200
+// spins of degree 40 1,127 -> 614 us, 4,096 cell grids 3.27 -> 3.28 ms; from 3 spins
+// the grids take 3.32 ms).
+template <int MODE>
+constexpr int kOwnLeast = MODE == 0 ? 4 : 2;
+
+// Integer couplings: the exact field from scratch, not kept.
 __device__ __forceinline__ uint32_t own_int(const DevGraph &G, const InstDesc &I, const uint32_t *sw, int j, int r0,
                                             uint32_t k0, uint32_t k1, uint32_t e0, uint32_t e1) {
   const int8_t *Ji = reinterpret_cast<const int8_t *>(G.J), *hJ = reinterpret_cast<const int8_t *>(G.hJ);
@@ -702,7 +710,7 @@ tile_kernel(const __grid_constant__ TileArgs A) {
               {
                 const int ul = MODE == 1 && refresh && pl ? __ldg(G.runit + I.spin_off + jl) : 0;
                 uint32_t own = __ballot_sync(0xffffffffu, pl && ul >= 0);
-                if (MODE == 0 && __popc(own) < kOwnInt) own = 0u;
+                if (__popc(own) < kOwnLeast<MODE>) own = 0u;
                 if (own) {
                   if ((own >> lane) & 1u) s_slot[(tid & ~31) + __popc(own & ((1u << lane) - 1u))] = (uint8_t)lane;
                   __syncwarp();
@@ -789,32 +797,71 @@ tile_kernel(const __grid_constant__ TileArgs A) {
               } else {
                 const float *Jf = reinterpret_cast<const float *>(G.J);
                 const float *hJ = reinterpret_cast<const float *>(G.hJ);
-                // a refresh without an exact unit: the FP64 sum in order, rounded
-                const float hj = __ldg(reinterpret_cast<const float *>(G.h) + gj);
-                double acc = (double)hj;
-                for (uint32_t kk = k0; kk < k1; ++kk) {
-                  const int i = __ldg(G.col + kk);
-                  const double w = (double)__ldg(Jf + kk);
-                  acc = __dadd_rn(acc, ((sw[i] >> lane) & 1u) ? w : -w);
-                }
-                for (uint32_t q = e0; q < e1; ++q) {
-                  const int e = __ldg(G.inc_edge + q);
-                  const int2 oth = __ldg(G.inc_oth + q);
-                  uint32_t neg = 0;
-                  if (oth.x >= 0) {
-                    neg = (~(sw[oth.x] >> lane) & 1u) ^ (~(sw[oth.y] >> lane) & 1u);
-                  } else {
-                    for (uint32_t m = __ldg(G.hptr + e), me = __ldg(G.hptr + e + 1); m < me; ++m) {
-                      const int mm = __ldg(G.hmem + m);
-                      if (mm != j) neg ^= ~(sw[mm] >> lane) & 1u;
+                const uint32_t bit = 1u << lane;
+                // +1 products of an incidence's other spins
+                auto product = [&](uint32_t q) -> uint32_t { return ~own_parity(G, sw, 0xffffffffu, j, q); };
+                float f;
+                bool dirty = true;
+                if (refresh) {
+                  const float hj = __ldg(reinterpret_cast<const float *>(G.h) + gj);
+                  const int u = __ldg(G.runit + gj);
+                  if (u >= 0) {
+                    int64_t acc = xr_term(hj, u);
+                    for (uint32_t kk = k0; kk < k1; ++kk) {
+                      const int64_t t = xr_term(__ldg(Jf + kk), u);
+                      acc += sw[__ldg(G.col + kk)] & bit ? t : -t;
                     }
+                    for (uint32_t q = e0; q < e1; ++q) {
+                      const int64_t t = xr_term(__ldg(hJ + __ldg(G.inc_edge + q)), u);
+                      acc += product(q) & bit ? t : -t;
+                    }
+                    f = xr_round(acc, u);
+                  } else {  // no exact unit: the FP64 sum in order, rounded
+                    double acc = (double)hj;
+                    for (uint32_t kk = k0; kk < k1; ++kk) {
+                      const double w = (double)__ldg(Jf + kk);
+                      acc = __dadd_rn(acc, sw[__ldg(G.col + kk)] & bit ? w : -w);
+                    }
+                    for (uint32_t q = e0; q < e1; ++q) {
+                      const double w = (double)__ldg(hJ + __ldg(G.inc_edge + q));
+                      acc = __dadd_rn(acc, product(q) & bit ? w : -w);
+                    }
+                    f = __double2float_rn(acc);
                   }
-                  const double w = (double)__ldg(hJ + e);
-                  acc = __dadd_rn(acc, neg ? -w : w);
+                } else {
+                  // the flips of the neighbours since the previous visit, in order; the
+                  // words are the warp's, so every lane takes each term or leaves it
+                  // without a branch
+                  f = Fc[(size_t)j * 32 + field_at(j, lane)];
+                  uint32_t dirtyw = 0u;  // replicas whose field changes
+                  auto pull = [&](float w2, uint32_t flipped, uint32_t plus) {
+                    const float g = __fadd_rn(f, plus & bit ? w2 : -w2);
+                    f = flipped & bit ? g : f;
+                    dirtyw |= flipped;
+                  };
+                  constexpr int kPre = 6;  // row entries fetched together
+                  const int dg = (int)(k1 - k0);
+                  int ci[kPre];
+                  float cw[kPre];
+#pragma unroll
+                  for (int q = 0; q < kPre; ++q)
+                    if (q < dg) {
+                      ci[q] = __ldg(G.col + k0 + q);
+                      cw[q] = __ldg(Jf + k0 + q);
+                    }
+#pragma unroll
+                  for (int q = 0; q < kPre; ++q)
+                    if (q < dg) pull(2.0f * cw[q], fm[ci[q]], sw[ci[q]]);
+                  for (uint32_t kk = k0 + kPre; kk < k1; ++kk) {
+                    const int i = __ldg(G.col + kk);
+                    pull(2.0f * __ldg(Jf + kk), fm[i], sw[i]);
+                  }
+                  for (uint32_t q = e0; q < e1; ++q)
+                    pull(2.0f * __ldg(hJ + __ldg(G.inc_edge + q)), own_parity(G, fm, 0u, j, q), product(q));
+                  dirty = dirtyw & bit;
                 }
-                const float f = __double2float_rn(acc);
-                Fc[(size_t)j * 32 + field_at(j, lane)] = f;
-                flip = up ? (f < 0.0f) : (f > 0.0f);
+                if (dirty) Fc[(size_t)j * 32 + field_at(j, lane)] = f;
+                flip = dirty && (up ? f < 0.0f : f > 0.0f);
               }
               flip = flip && ((active >> lane) & 1u);
               const uint32_t m = __ballot_sync(0xffffffffu, flip);

@@ -287,3 +287,26 @@ def test_fm_gain_keys_widest_record(degree):
     rp, col, J = W.csr_from_edges(n, u, v, w, "f32")
     assert np.diff(rp).max() == degree
     _compare_fm([W.Instance(n=n, row_ptr=rp, col=col, J=J, dtype="f32")], 6, 2, False)
+
+
+# A warp's lone pending FP32 spin (classes of one spin: fully coupled rows) and two
+# and three of them, with refreshes in fixed point, in FP64 and none but the first.
+@pytest.mark.parametrize("refresh_every", [0, 1, 3])
+@pytest.mark.parametrize("per_class", [1, 2, 3])
+@pytest.mark.parametrize("kind", ["f32", "wide", "wider"])
+def test_tile_lone_spins(kind, per_class, refresh_every):
+    n = 40 * per_class
+    u, v = np.triu_indices(n, 1)
+    keep = u // per_class != v // per_class  # (spins of one class are not coupled)
+    u, v = u[keep], v[keep]
+    rng = np.random.default_rng(per_class)
+    rp, col, J = W.csr_from_edges(n, u, v, rng.standard_normal(len(u)).astype(np.float32), "f32")
+    cls = rng.permutation(n // per_class)
+    hyper = np.array([[0, per_class, 2 * per_class], [per_class, 3 * per_class, 4 * per_class]], np.int32).ravel()
+    inst = W.Instance(n=n, row_ptr=rp, col=col, J=J, h=rng.standard_normal(n).astype(np.float32),
+                      hyper_ptr=np.array([0, 3, 6], np.int64), hyper_members=hyper,
+                      hyper_J=np.array([0.5, -0.25], np.float32),
+                      colour=cls[np.arange(n) // per_class].astype(np.int32), dtype="f32")
+    if kind != "f32":
+        inst = _exp_spread(inst, *((-12, 12) if kind == "wide" else (-45, 25)))
+    _compare([inst], [n], 37, False, max_sweeps=200, restarts=2, refresh_every=refresh_every, kernel=isg.KERNEL_TILE)
