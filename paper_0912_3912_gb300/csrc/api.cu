@@ -560,12 +560,17 @@ const ClusterPlan &cluster_plan(ising_handle *h, int32_t R, const ising_search_p
 // descents of 64 replicas 323 / 230 / 218, of 1,024 447 / 561 / 553.  +/-J: 31^3, 1,024
 // replicas, 10 descents 2499 / 1572 / 1279; 16 x 16, 64 replicas, 10 descents 52 / 42 /
 // 44 (125 in one segment).
+// In the index order a CTA of any size decides a spin at a time; multi-spin coded, its
+// barrier per spin takes longer the more warps wait at it (64 x 64, 64 replicas 9.1 /
+// 9.3 / 10.1 ms).
 const TilePlan *tile_plan(ising_handle *h, int mode, int32_t R, const ising_search_params *p) {
   TilePlan &T = h->tile_plan_cache;
   const int32_t parallel = p->sweep_budget > 0 ? 1 : p->restarts;
-  if (T.mode == mode && T.R == R && T.parallel == parallel) return T.slots > 0 ? &T : nullptr;
+  const bool sequential = p->schedule == ISING_SCHED_SEQUENTIAL;
+  if (T.mode == mode && T.R == R && T.parallel == parallel && T.sequential == sequential) return T.slots > 0 ? &T : nullptr;
   T = TilePlan();
   T.mode = mode;
+  T.sequential = sequential;
   T.R = R;
   T.parallel = parallel;
   const int64_t tiles = (int64_t)h->n_inst * ((R + 31) / 32);
@@ -590,9 +595,9 @@ const TilePlan *tile_plan(ising_handle *h, int mode, int32_t R, const ising_sear
     if (slots < 1) continue;
     const double per_step = mode >= 2 ? 2.0 * threads : (double)ncls * threads / 32;
     const double fixed = mode >= 2 ? 30.0 : (mode == 0 ? 6.0 : (threads == 1024 ? 15.0 : 10.0));
-    const double unit = fixed + std::ceil(h->nmax / per_step);
+    const double unit = sequential ? 1.0 + (mode >= 2 ? 1e-4 * threads : 0.0) : fixed + std::ceil(h->nmax / per_step);
     double waves = weight / (double)slots;
-    if (mode != 1) {
+    if (mode != 1 || sequential) {
       waves = std::max(1.0, waves);
       if (nmin == h->nmax && waves < 2.0) waves = std::ceil(waves);
     } else if (waves < 1.0) {
@@ -710,7 +715,7 @@ ising_status run_tile(ising_handle *h, int mode, int32_t R, const ising_search_p
   if (cap != cudaStreamCaptureStatusNone) return ISING_ERR_CUDA;  // (scratch and work queue are the handle's)
   CUDA_OK(cudaMemsetAsync(h->d_queue, 0, sizeof(int32_t) * (4 + (size_t)counters), s));
   kt_begin(h, "tile_kernel", s);
-  CUDA_OK(launch_tile(a, mode, threads, segs > 1, grid, smem, s));
+  CUDA_OK(launch_tile(a, mode, threads, segs > 1 || a.sequential, grid, smem, s));
   kt_end(h, s);
   h->launches += 1;
   return ISING_OK;

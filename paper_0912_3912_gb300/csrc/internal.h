@@ -130,6 +130,7 @@ struct FamilyState {
 // Launch shape of the tile kernels (tile_plan in api.cu).
 struct TilePlan {
   int32_t mode = -1, R = 0, parallel = 0;  // what it was made for
+  bool sequential = false;
   int32_t threads = 0, segs = 1, fsm_cap = 0;
   int64_t slots = 0;  // resident CTAs, 0: none fits
   size_t smem = 0;

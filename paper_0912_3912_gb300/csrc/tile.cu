@@ -399,10 +399,10 @@ __device__ __forceinline__ uint32_t own_refresh(const DevGraph &G, const InstDes
 // of degree 5, 20 replicas, 2 descents 889 -> 623 us (all by four lanes 639), 300
 // spins 110 -> 114 (144); 1,000 spins, 1,024 replicas, 20 descents 982 -> 792 (3 / 6
 // spins: 802 / 806).  FP32, where the fields are read and written besides: one spin,
-// as in the index order, dense rows and the last sweeps (1,000 spins in index order
-// 11.0 -> 7.6 ms, 256 fully coupled spins given as rows, 32 replicas, 100 -> 44, 200
-// spins of degree 40 1,127 -> 614 us, 4,096 cell grids 3.27 -> 3.28 ms; from 3 spins
-// the grids take 3.32 ms).
+// as in the index order, dense rows and the last sweeps (32 replicas: 1,000 spins in
+// index order 10.7 -> 5.3 ms, 64 fully coupled spins given as rows 3.5 -> 1.5 ms, 200
+// spins of degree 40 1,096 -> 556 us; 4,096 cell grids 3.26 -> 3.20 ms, and 1 % more
+// from 3 spins).
 template <int MODE>
 constexpr int kOwnLeast = MODE == 0 ? 4 : 2;
 
@@ -485,7 +485,8 @@ __device__ __forceinline__ uint32_t own_visit(const DevGraph &G, const uint32_t 
 
 // SEG: tiles in segments of descents.  (A separate instantiation: the segments'
 // few values in the whole-tile kernel spill at 64 registers and cost full batches
-// 8 %.)
+// 8 %.  For the same reason only the segments' instantiations know the index order:
+// one segment of them where there is one.)
 template <int MODE, int THREADS, bool SEG>
 __global__ void __launch_bounds__(THREADS, (MODE == 3 ? 512 : 1024) / THREADS < 1 ? 1 : (MODE == 3 ? 512 : 1024) / THREADS)
 tile_kernel(const __grid_constant__ TileArgs A) {
@@ -534,7 +535,12 @@ tile_kernel(const __grid_constant__ TileArgs A) {
     const int rem = A.R - 32 * g;
     const uint32_t lane_valid = rem >= 32 ? 0xffffffffu : ((1u << rem) - 1u);
     const uint64_t seed = A.seeds[b];
-    const int ncls = A.sequential ? n : I.ncls;
+    const bool index_order = SEG && A.sequential;  // (launched with SEG alone)
+    // On lanes, warp 0 takes the spins of the index order one after another and the
+    // others wait for the sweep's end; multi-spin coded, a thread takes one and the
+    // CTA waits for it.
+    const bool seq = MODE <= 1 && index_order;
+    const int ncls = seq ? 1 : (index_order ? n : I.ncls);
     float *Fc = (MODE == 1 && n <= A.fsm_cap) ? Fs : F;
     if (tid < 32) {
       s_total[tid] = 0;
@@ -585,9 +591,9 @@ tile_kernel(const __grid_constant__ TileArgs A) {
         uint32_t anyf = 0;
         for (int c = 0; c < ncls; ++c) {
           int c0, c1;
-          if (A.sequential) {
+          if (index_order) {
             c0 = c;
-            c1 = c + 1;
+            c1 = seq ? n : c + 1;
           } else {
             c0 = __ldg(G.cls + I.cls_off + c);
             c1 = __ldg(G.cls + I.cls_off + c + 1);
@@ -644,7 +650,7 @@ tile_kernel(const __grid_constant__ TileArgs A) {
             const int8_t *Ji = reinterpret_cast<const int8_t *>(G.J);
             const int8_t *hi = reinterpret_cast<const int8_t *>(G.h);
             for (int v = c0 + tid; v < c1; v += THREADS) {
-              const int j = A.sequential ? v : __ldg(G.order + I.spin_off + v);
+              const int j = index_order ? v : __ldg(G.order + I.spin_off + v);
               if (!pending(j)) continue;
               clear_pending(j);
               my_eval += __popc(active);
@@ -691,11 +697,14 @@ tile_kernel(const __grid_constant__ TileArgs A) {
             // reads position k's spin and pending bit (one round trip for the 32),
             // a position with nothing pending is settled at once (its visit flips
             // nothing), and the others are visited in order.
-            for (int vb = c0 + warp; vb < c1; vb += 32 * nwarps) {
-              const int vl = vb + lane * nwarps;
+            // (In index order warp 0's next 32 spins; each one's pending bit is read
+            // when its turn comes.)
+            const int vstep = seq ? 1 : nwarps;
+            for (int vb = seq && warp ? c1 : c0 + warp; vb < c1; vb += 32 * vstep) {
+              const int vl = vb + lane * vstep;
               const bool inr = vl < c1;
-              const int jl = inr ? (A.sequential ? vl : __ldg(G.order + I.spin_off + vl)) : 0;
-              const bool pl = inr && pending(jl);
+              const int jl = inr ? (seq ? vl : __ldg(G.order + I.spin_off + vl)) : 0;
+              const bool pl = inr && (seq || pending(jl));
               if (MODE == 1 && inr && !pl && fm[jl]) fm[jl] = 0u;
               // a pending position's row and hyper-edge bounds, read with the batch
               uint32_t k0l = 0, k1l = 0, e0l = 0, e1l = 0;
@@ -707,7 +716,7 @@ tile_kernel(const __grid_constant__ TileArgs A) {
                 e1l = __ldg(G.inc_ptr + g + 1);
               }
               uint32_t todo = __ballot_sync(0xffffffffu, pl);
-              {
+              if (!seq) {
                 const int ul = MODE == 1 && refresh && pl ? __ldg(G.runit + I.spin_off + jl) : 0;
                 uint32_t own = __ballot_sync(0xffffffffu, pl && ul >= 0);
                 if (__popc(own) < kOwnLeast<MODE>) own = 0u;
@@ -763,6 +772,13 @@ tile_kernel(const __grid_constant__ TileArgs A) {
               const int src = __ffs(todo) - 1;
               todo &= todo - 1u;
               const int j = __shfl_sync(0xffffffffu, jl, src);
+              if (seq) {
+                __syncwarp();  // the flips and marks of the spins before
+                if (!pending(j)) {
+                  if (MODE == 1 && lane == 0) fm[j] = 0u;
+                  continue;
+                }
+              }
               const int64_t gj = I.spin_off + j;
               const uint32_t wj = sw[j];
               const bool up = (wj >> lane) & 1u;
@@ -839,20 +855,8 @@ tile_kernel(const __grid_constant__ TileArgs A) {
                     f = flipped & bit ? g : f;
                     dirtyw |= flipped;
                   };
-                  constexpr int kPre = 6;  // row entries fetched together
-                  const int dg = (int)(k1 - k0);
-                  int ci[kPre];
-                  float cw[kPre];
-#pragma unroll
-                  for (int q = 0; q < kPre; ++q)
-                    if (q < dg) {
-                      ci[q] = __ldg(G.col + k0 + q);
-                      cw[q] = __ldg(Jf + k0 + q);
-                    }
-#pragma unroll
-                  for (int q = 0; q < kPre; ++q)
-                    if (q < dg) pull(2.0f * cw[q], fm[ci[q]], sw[ci[q]]);
-                  for (uint32_t kk = k0 + kPre; kk < k1; ++kk) {
+#pragma unroll 4
+                  for (uint32_t kk = k0; kk < k1; ++kk) {
                     const int i = __ldg(G.col + kk);
                     pull(2.0f * __ldg(Jf + kk), fm[i], sw[i]);
                   }
@@ -967,7 +971,7 @@ tile_kernel(const __grid_constant__ TileArgs A) {
     }
     __syncthreads();
     const uint32_t *from = nullptr;  // the words of the tile's segments
-    if constexpr (SEG) {
+    if (SEG && segs > 1) {
       // this segment's words, energies and minima; the last CTA of the tile
       // chooses per lane among the segments (strictly lower energy, ties keep the
       // earlier; without a converged descent the last segment)
@@ -1010,7 +1014,7 @@ tile_kernel(const __grid_constant__ TileArgs A) {
     const bool wide = (n & 31) == 0 && ((uintptr_t)(A.spins + out_base) & 15) == 0;
     for (int i = tid; i < n; i += THREADS) {
       uint32_t wv = 0;
-      if (SEG) {
+      if (SEG && from) {
         for (int r = 0; r < 32; ++r) wv |= __ldcg(from + (size_t)s_total[r] * nmax + i) & (1u << r);
       } else {
         wv = (bw[i] & has_best) | (sw[i] & ~has_best);

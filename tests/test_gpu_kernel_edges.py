@@ -310,3 +310,37 @@ def test_tile_lone_spins(kind, per_class, refresh_every):
     if kind != "f32":
         inst = _exp_spread(inst, *((-12, 12) if kind == "wide" else (-45, 25)))
     _compare([inst], [n], 37, False, max_sweeps=200, restarts=2, refresh_every=refresh_every, kernel=isg.KERNEL_TILE)
+
+
+# The index order: sizes around a warp's batch of 32, one segment and several, more
+# tiles than CTAs fit, and both orders in turn on one handle.
+@pytest.mark.parametrize("restarts,R", [(1, 33), (5, 4)])
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 65, 300])
+@pytest.mark.parametrize("kind", ["i8", "f32", "wider", "msc"])
+def test_tile_index_order(kind, n, restarts, R):
+    if kind == "msc":
+        inst = W.random_graph(n, min(4.0, n - 1.0), n, dtype="i8", int_range=1, fields=False)
+    else:
+        inst = W.random_graph(n, min(5.0, n - 1.0), n, dtype="i8" if kind == "i8" else "f32",
+                              n_hyper=n // 6, hyper_order=(2, 3, 4))
+        inst = _exp_spread(inst, -45, 25) if kind == "wider" else inst
+    _compare([inst], [n], R, kind in ("i8", "msc"), max_sweeps=200, restarts=restarts, refresh_every=3,
+             schedule=isg.SCHED_SEQUENTIAL, kernel=isg.KERNEL_MSC if kind == "msc" else isg.KERNEL_TILE)
+
+
+@pytest.mark.parametrize("dtype", ["i8", "f32"])
+def test_tile_index_order_of_more_tiles_than_ctas(dtype):
+    insts = [W.random_graph(3 + b % 9, 2.0, b, dtype=dtype) for b in range(1300)]
+    _compare(insts, list(range(1, 1301)), 3, dtype == "i8", max_sweeps=50, restarts=2,
+             schedule=isg.SCHED_SEQUENTIAL, kernel=isg.KERNEL_TILE)
+
+
+def test_tile_both_orders_on_one_handle():
+    inst = W.random_graph(200, 5.0, 8, dtype="f32", n_hyper=20)
+    h = isg.Handle([inst])
+    for schedule in (isg.SCHED_COLOUR, isg.SCHED_SEQUENTIAL) * 2:
+        r = h.local_search([3], 40, max_sweeps=200, restarts=2, schedule=schedule, kernel=isg.KERNEL_TILE)
+        s, _, m, _ = oracle.descent(inst, 3, 0, 40, max_sweeps=200, restarts=2, schedule=schedule)
+        assert np.array_equal(r.spins.cpu().numpy().reshape(40, -1), s)
+        assert np.array_equal(r.minima[0].cpu().numpy(), m)
+    h.close()
