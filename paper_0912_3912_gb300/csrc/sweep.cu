@@ -1739,13 +1739,19 @@ cudaError_t run_instance(ising_handle *h, SweepArgs A, int mode, cudaStream_t s)
 
 // Replicas of a group.  Words of 8 or 16 lanes waste none of a lattice position's
 // work on absent replicas and take the site-parallel energies; general graphs
-// share a row's reads among up to 32.  FP32 lattices, us a call in groups of 32 /
-// 16: 45^3 with 21 replicas 1760 / 1620.
+// share a row's reads among up to 32.  FP32 lattices beyond 16 replicas: a group of
+// 16 takes little more than half the time of one of 32 in the dense visits, so 33 to
+// 48 replicas take three of them instead of two (100^3, 40 replicas, 2 descents, 32 /
+// 16 lanes: 2,771 / 2,457 us); where launches are most of the time more groups spread
+// further over the chip (24^3, 32 replicas 579 / 506, 32^3, 48 655 / 571, 200^2, 32
+// 450 / 398; no longer at 32^3, 96 760 / 761); else two groups read each position
+// twice (45^3, 21 replicas 921 / 1,031, 64^3, 32 840 / 892, 24^3, 512 1,325 / 1,576).
 int lanes_per_spin(const ising_handle *h, int mode, bool sequential, int32_t R) {
   if (R <= 8) return 8;
   if (R <= 16) return 16;
-  if (mode == 1 && h->all_lattice && !sequential && R <= 512) return 16;
-  return 32;
+  if (mode != 1 || !h->all_lattice || sequential) return 32;
+  const int64_t groups = (R + 15) / 16;
+  return groups == 3 || (groups <= 32 && groups * h->nmax <= 150000) ? 16 : 32;
 }
 
 }  // namespace

@@ -344,3 +344,12 @@ def test_tile_both_orders_on_one_handle():
         assert np.array_equal(r.spins.cpu().numpy().reshape(40, -1), s)
         assert np.array_equal(r.minima[0].cpu().numpy(), m)
     h.close()
+
+
+# FP32 lattices on both sides of the rule between groups of 16 and of 32 replicas
+# (three groups of 16; few sites; many), odd and even sides, last groups of one.
+@pytest.mark.parametrize("dims,R", [((41, 41, 41), 17), ((41, 41, 41), 33), ((260, 260), 18), ((34, 34, 34), 49),
+                                    ((20, 20, 20), 100), ((12, 12, 12), 400), ((16, 16, 16), 513)])
+def test_sweep_fp32_lattice_group_sizes(dims, R):
+    inst = W.lattice(dims, True, "gauss", "gauss", seed=R)
+    _compare([inst], [R], R, False, max_sweeps=12, restarts=2, refresh_every=5, kernel=isg.KERNEL_SWEEP)
