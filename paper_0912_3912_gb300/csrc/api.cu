@@ -463,6 +463,9 @@ bool tile_fits(const ising_handle *h, int mode) {
 // spins 670 / 1380, 6,000 1045 / 1422, 9,000 1465 / 1326, 12,000 1902 / 1531, 20,000
 // 3037 / 1786; Gaussian squares, 32 replicas, 4 descents: 64 x 64 348 / 551, 96 x 96
 // 668 / 592, 128 x 128 1113 / 739 and with 256 replicas 1112 / 1439.
+// Asked only for calls that wait for their search anyway: the sweep family holds the
+// host until the search is nearly done, a tile launch returns at once, and a program
+// that drives several handles or streams from one thread counts on that.
 bool sweep_is_faster(const ising_handle *h, int32_t R, const ising_search_params *p) {
   const int32_t groups = (R + 31) / 32;
   if (groups > 32 || p->schedule == ISING_SCHED_SEQUENTIAL) return false;
@@ -475,7 +478,8 @@ bool sweep_is_faster(const ising_handle *h, int32_t R, const ising_search_params
 }
 
 // Kernel family for these arguments (ISING_KERNEL_AUTO resolved), or negative status.
-int32_t resolve_kernel(ising_handle *h, int32_t R, const ising_search_params *p) {
+// waits: the call waits for its search (it was asked for the work counters).
+int32_t resolve_kernel(ising_handle *h, int32_t R, const ising_search_params *p, bool waits) {
   int32_t k = p->kernel;
   if (h->dtype == ISING_F64)  // FP64 couplings: the plain family only
     return (k == ISING_KERNEL_AUTO || k == ISING_KERNEL_PLAIN) ? ISING_KERNEL_PLAIN : -(int32_t)ISING_ERR_UNSUPPORTED;
@@ -485,7 +489,7 @@ int32_t resolve_kernel(ising_handle *h, int32_t R, const ising_search_params *p)
     if (h->dense && dense_supported(h, R)) return ISING_KERNEL_DENSE_TC;
     if (h->msc_ok && tile_fits(h, 2)) return ISING_KERNEL_MSC;
     if (!tile_fits(h, h->dtype == ISING_F32 ? 1 : 0)) return ISING_KERNEL_SWEEP;
-    return sweep_is_faster(h, R, p) ? ISING_KERNEL_SWEEP : ISING_KERNEL_TILE;
+    return waits && sweep_is_faster(h, R, p) ? ISING_KERNEL_SWEEP : ISING_KERNEL_TILE;
   }
   switch (k) {
     case ISING_KERNEL_TILE:
@@ -1118,7 +1122,7 @@ int32_t ising_plan_kernel(ising_handle *h, int32_t replicas, const ising_search_
   if (!h || replicas < 1) return -(int32_t)ISING_ERR_INVALID_ARG;
   ising_status st = validate_params(p);
   if (st != ISING_OK) return -(int32_t)st;
-  return resolve_kernel(h, replicas, p);
+  return resolve_kernel(h, replicas, p, true);
 }
 
 ising_status ising_local_search(ising_handle *h, const uint64_t *seeds, int32_t replicas,
@@ -1137,7 +1141,7 @@ ising_status ising_local_search(ising_handle *h, const uint64_t *seeds, int32_t 
   if (energy_i32_dev && (h->dtype != ISING_I8 || h->abs_energy_bound > 0x7fffffffLL))
     return ISING_ERR_UNSUPPORTED;
   if ((int64_t)replicas * h->total_spins > (int64_t)1 << 40) return ISING_ERR_UNSUPPORTED;
-  const int32_t kernel = resolve_kernel(h, replicas, p);
+  const int32_t kernel = resolve_kernel(h, replicas, p, stats != nullptr);
   if (kernel < 0) return (ising_status)(-kernel);
   int cur = 0;
   cudaGetDevice(&cur);
@@ -1222,7 +1226,7 @@ ising_status ising_autotune(ising_handle *h, int32_t replicas, const ising_searc
   if (cached > 0) {
     ising_search_params q = *p;
     q.kernel = (ising_kernel)cached;
-    if (resolve_kernel(h, replicas, &q) == cached) {
+    if (resolve_kernel(h, replicas, &q, true) == cached) {
       h->tuned[replicas] = cached;
       if (chosen) *chosen = cached;
       return ISING_OK;
@@ -1252,7 +1256,7 @@ ising_status ising_autotune(ising_handle *h, int32_t replicas, const ising_searc
   for (int32_t fam : families) {
     ising_search_params q = *p;
     q.kernel = (ising_kernel)fam;
-    if (resolve_kernel(h, replicas, &q) != fam) continue;
+    if (resolve_kernel(h, replicas, &q, true) != fam) continue;
     ising_stats s1;
     if (ising_local_search(h, seeds.data(), replicas, &q, spins, E, nullptr, mins, &s1, stream) != ISING_OK) continue;
     cudaEventRecord(e0, stream);

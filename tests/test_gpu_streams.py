@@ -159,3 +159,24 @@ def test_first_passes_call_under_capture(dtype):
         assert np.array_equal(spins[k], s) and int(passes[0, k]) == p
         assert abs(float(E[0, k]) - e) <= 1e-9 * (1 + abs(e))
     h.close()
+
+
+# A search without work counters returns to the host once it is queued where one
+# kernel serves the instance: also for the few large instances that AUTO gives to
+# the sweep family when the call waits anyway.
+def test_auto_search_without_stats_does_not_hold_the_host(busy):
+    inst = W.random_graph(12000, 5.0, 61, dtype="f32", n_hyper=1500, hyper_order=(3, 4))
+    kw = dict(max_sweeps=300, restarts=2)
+    h = isg.Handle([inst])
+    assert h.plan_kernel(6, **kw) == isg.KERNEL_SWEEP
+    waited = h.local_search([5], 6, **kw)
+    h.local_search([5], 6, stats=False, **kw)  # (grows the scratch)
+    before = torch.cuda.Event()
+    busy()
+    before.record()
+    r = h.local_search([5], 6, stats=False, **kw)
+    assert not before.query(), "the call held the host until the stream had caught up"
+    torch.cuda.synchronize()
+    assert torch.equal(r.spins, waited.spins) and torch.equal(r.minima, waited.minima)
+    torch.testing.assert_close(r.energy, waited.energy, rtol=1e-12, atol=0)
+    h.close()
