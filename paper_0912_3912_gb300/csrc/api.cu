@@ -383,8 +383,9 @@ ising_status load_desc(const ising_instance_desc &d, ising_dtype dtype, HostInst
 
 // Host-side fault injection for tests (ISING_FAULT): "alloc:k" makes the k-th
 // device upload of ising_create fail ("alloc" = the first); "launch" makes
-// ising_local_search fail as a failed launch would; "device_timeout" (read by
-// the dense tensor-core path) makes one CTA's bounded wait run out.
+// ising_local_search fail as a failed launch would; "scratch:k" makes scratch
+// requests of more than k bytes fail; "device_timeout" (read by the dense
+// tensor-core path) makes one CTA's bounded wait run out.
 bool fault_is(const char *what) {
   const char *f = std::getenv("ISING_FAULT");
   return f && std::strncmp(f, what, std::strlen(what)) == 0;
@@ -428,11 +429,15 @@ void free_handle(ising_handle *h) {
 }
 
 ising_status ensure_scratch(ising_handle *h, size_t bytes) {
+  if (fault_is("scratch:") && bytes > (size_t)std::atoll(std::getenv("ISING_FAULT") + 8)) return ISING_ERR_OOM;
   if (bytes <= h->scratch_bytes) return ISING_OK;
   if (h->d_scratch) cudaFree(h->d_scratch);
   h->d_scratch = nullptr;
   h->scratch_bytes = 0;
-  if (cudaMalloc(&h->d_scratch, bytes) != cudaSuccess) return ISING_ERR_OOM;
+  if (cudaMalloc(&h->d_scratch, bytes) != cudaSuccess) {
+    cudaGetLastError();  // (the caller may do with less)
+    return ISING_ERR_OOM;
+  }
   h->scratch_bytes = bytes;
   return ISING_OK;
 }
@@ -646,7 +651,10 @@ ising_status run_tile(ising_handle *h, int mode, int32_t R, const ising_search_p
   auto ensure_counters = [&](int32_t counters) -> ising_status {
     if (counters <= h->queue_tiles) return ISING_OK;
     int32_t *q = nullptr;
-    if (cudaMalloc(&q, sizeof(int32_t) * (4 + (size_t)counters)) != cudaSuccess) return ISING_ERR_OOM;
+    if (cudaMalloc(&q, sizeof(int32_t) * (4 + (size_t)counters)) != cudaSuccess) {
+      cudaGetLastError();
+      return ISING_ERR_OOM;
+    }
     cudaFree(h->d_queue);
     h->d_queue = q;
     h->queue_tiles = counters;
@@ -672,18 +680,20 @@ ising_status run_tile(ising_handle *h, int mode, int32_t R, const ising_search_p
   if (mode == 3) {
     const ClusterPlan &C = cluster_plan(h, R, p);
     if (C.P > 0) {
-      const int units = h->n_tiles * C.segs;
-      const size_t seg_bytes = C.segs > 1 ? up256((size_t)units * h->nmax * sizeof(uint32_t)) : 0;
-      const size_t lane_bytes = C.segs > 1 ? up256((size_t)units * 32 * sizeof(double)) : 0;
-      ising_status st = ensure_scratch(h, seg_bytes + 2 * lane_bytes + 256);
-      if (st == ISING_OK && C.segs > 1) st = ensure_counters(h->n_tiles);
-      if (st != ISING_OK) return st;
+      const size_t seg_bytes = up256((size_t)h->n_tiles * C.segs * h->nmax * sizeof(uint32_t));
+      const size_t lane_bytes = up256((size_t)h->n_tiles * C.segs * 32 * sizeof(double));
+      // without room for the segments' results the tiles run whole, which needs none
+      const int segs = C.segs > 1 && ensure_scratch(h, seg_bytes + 2 * lane_bytes + 256) == ISING_OK &&
+                               ensure_counters(h->n_tiles) == ISING_OK
+                           ? C.segs
+                           : 1;
+      const int units = h->n_tiles * segs;
       a.queue = h->d_queue;
-      a.segs = C.segs;
+      a.segs = segs;
       a.seg_words = (uint32_t *)h->d_scratch;
       a.seg_best = (double *)((char *)h->d_scratch + seg_bytes);
       a.seg_minima = (int32_t *)((char *)h->d_scratch + seg_bytes + lane_bytes);
-      if (C.segs > 1) CUDA_OK(cudaMemsetAsync(h->d_queue, 0, sizeof(int32_t) * (4 + (size_t)h->n_tiles), s));
+      if (segs > 1) CUDA_OK(cudaMemsetAsync(h->d_queue, 0, sizeof(int32_t) * (4 + (size_t)h->n_tiles), s));
       kt_begin(h, "msc_cluster_kernel", s);
       CUDA_OK(launch_msc_cluster(a, units, C.P, h->nmax / C.P, h->inst[0].lat_d, s));
       kt_end(h, s);
@@ -693,18 +703,23 @@ ising_status run_tile(ising_handle *h, int mode, int32_t R, const ising_search_p
   }
   const TilePlan *plan = tile_plan(h, mode, R, p);
   if (!plan) return ISING_ERR_UNSUPPORTED;
-  const int threads = plan->threads, segs = plan->segs, fsm_cap = plan->fsm_cap;
+  const int threads = plan->threads, fsm_cap = plan->fsm_cap;
   const size_t smem = plan->smem;
-  const int64_t work = (int64_t)h->n_tiles * segs;
-  const int grid = (int)std::min<int64_t>(work, plan->slots);
-  const size_t f_bytes = mode == 1 ? up256((size_t)grid * h->nmax * 32 * sizeof(float)) : 0;
-  const size_t bw_bytes = up256((size_t)grid * h->nmax * sizeof(uint32_t));
-  const size_t seg_bytes = segs > 1 ? up256((size_t)work * h->nmax * sizeof(uint32_t)) : 0;
-  const size_t lane_bytes = segs > 1 ? up256((size_t)work * 32 * sizeof(double)) : 0;
-  ising_status st = ensure_scratch(h, f_bytes + bw_bytes + seg_bytes + 2 * lane_bytes + 256);
-  if (st != ISING_OK) return st;
+  int segs = plan->segs, grid;
+  size_t f_bytes, bw_bytes, seg_bytes, lane_bytes;
+  for (;; segs = 1) {  // without room for the segments' results and CTAs the tiles run whole
+    const int64_t work = (int64_t)h->n_tiles * segs;
+    grid = (int)std::min<int64_t>(work, plan->slots);
+    f_bytes = mode == 1 ? up256((size_t)grid * h->nmax * 32 * sizeof(float)) : 0;
+    bw_bytes = up256((size_t)grid * h->nmax * sizeof(uint32_t));
+    seg_bytes = segs > 1 ? up256((size_t)work * h->nmax * sizeof(uint32_t)) : 0;
+    lane_bytes = segs > 1 ? up256((size_t)work * 32 * sizeof(double)) : 0;
+    ising_status st = ensure_scratch(h, f_bytes + bw_bytes + seg_bytes + 2 * lane_bytes + 256);
+    if (st == ISING_OK && segs > 1) st = ensure_counters(h->n_tiles);
+    if (st == ISING_OK) break;
+    if (segs == 1) return st;
+  }
   const int32_t counters = segs > 1 ? h->n_tiles : 0;
-  if ((st = ensure_counters(counters)) != ISING_OK) return st;
   a.queue = h->d_queue;
   a.F = mode == 1 ? (float *)h->d_scratch : nullptr;
   a.fsm_cap = fsm_cap;

@@ -87,3 +87,38 @@ def test_device_wait_that_runs_out_returns_timeout(monkeypatch):
     assert np.array_equal(again.spins.cpu().numpy(), sp_ref)
     assert np.array_equal(again.energy.cpu().numpy(), E_ref)
     h.close()
+
+
+# Descents in segments need scratch for every segment's result (and FP32 fields for
+# every CTA): where that cannot be had the tiles run whole, with the same results.
+@pytest.mark.parametrize("kind", ["i8", "f32", "msc", "lattice", "cluster"])
+def test_no_room_for_segments(kind, monkeypatch):
+    if kind in ("lattice", "cluster"):
+        inst = W.lattice((16, 16, 16), True, "pm1", "pm1_0", seed=4)
+    else:
+        inst = W.random_graph(700, 4.0, 5, dtype="f32" if kind == "f32" else "i8", n_hyper=0 if kind == "msc" else 60,
+                              int_range=1 if kind == "msc" else 3, fields=kind != "msc")
+    kw = dict(max_sweeps=100, restarts=6, cluster_ctas=4 if kind == "cluster" else 1,
+              kernel=isg.KERNEL_TILE if kind in ("i8", "f32") else isg.KERNEL_MSC)
+    R = 33  # two tiles
+    h = isg.Handle([inst])
+    ref = h.local_search([9], R, **kw)
+    h.close()
+    whole = 0 if kind == "cluster" else 2 * inst.n * (132 if kind == "f32" else 4) + 1024
+    monkeypatch.setenv("ISING_FAULT", f"scratch:{whole}")
+    h = isg.Handle([inst])
+    for _ in range(2):
+        r = h.local_search([9], R, **kw)
+        assert torch.equal(r.spins, ref.spins) and torch.equal(r.energy, ref.energy)
+        assert torch.equal(r.minima, ref.minima)
+        assert {k: r.stats[k] for k in ("flips", "minima", "descents", "sweeps")} == \
+            {k: ref.stats[k] for k in ("flips", "minima", "descents", "sweeps")}
+    if kind != "cluster":
+        monkeypatch.setenv("ISING_FAULT", "scratch:0")
+        with pytest.raises(isg.IsingError) as ei:
+            h.local_search([9], R, **kw)
+        assert ei.value.code == ERR_OOM
+    monkeypatch.delenv("ISING_FAULT")
+    r = h.local_search([9], R, **kw)
+    assert torch.equal(r.spins, ref.spins)
+    h.close()
