@@ -260,6 +260,7 @@ cudaError_t launch_energy(ising_handle *h, const int8_t *spins, int32_t R, doubl
                           int32_t *E32, cudaStream_t s);
 void energy_plan_free(ising_handle *h);
 size_t msc_cluster_smem(int csz);
+size_t msc_cluster_smem_limit();
 cudaError_t launch_msc_cluster(const TileArgs &args, int units, int P, int csz_max, int D, cudaStream_t s);
 // the pass-based search (fm.cu)
 int fm_max_spins();

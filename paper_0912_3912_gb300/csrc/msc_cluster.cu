@@ -514,14 +514,18 @@ __global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const __grid_consta
 
 // words, pending flags, best words, per-site signs (in planes while those fit)
 static bool cluster_masks(int csz) { return csz <= 8192; }
+// dynamic shared memory of a CTA at most (232,448 bytes less the static part)
+size_t msc_cluster_smem_limit() { return 232448 - 4096; }
 size_t msc_cluster_smem(int csz) {
   return (size_t)csz * 4 + (size_t)(csz / 64) * 2 * 4 + (size_t)csz * 4 + (size_t)csz * (cluster_masks(csz) ? 8 : 1);
 }
 
 template <int D, bool MASKS>
-cudaError_t launch_cfg(cudaLaunchConfig_t &cfg, const TileArgs &args, int P, size_t smem, int *max_active) {
+cudaError_t launch_cfg(cudaLaunchConfig_t &cfg, const TileArgs &args, int P, int *max_active) {
   auto kern = msc_cluster_kernel<D, MASKS>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // (the same limit for every size: the attribute is the process's, and another
+  // thread's handle may launch the same kernel at a larger size)
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)msc_cluster_smem_limit());
   if (e != cudaSuccess) return e;
   if (max_active) return cudaOccupancyMaxActiveClusters(max_active, kern, &cfg);
   return cudaLaunchKernelEx(&cfg, kern, args, P);
@@ -530,12 +534,10 @@ cudaError_t launch_cfg(cudaLaunchConfig_t &cfg, const TileArgs &args, int P, siz
 // Launch (max_active == nullptr) or report how many clusters can be resident at once.
 static cudaError_t msc_cluster_launch_or_query(const TileArgs &args, int n_tiles, int P, int csz_max, int D, cudaStream_t s,
                                         int *max_active) {
-  const size_t smem = msc_cluster_smem(csz_max);
-
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(n_tiles * P);
   cfg.blockDim = dim3(kCT);
-  cfg.dynamicSmemBytes = smem;
+  cfg.dynamicSmemBytes = msc_cluster_smem(csz_max);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -545,8 +547,8 @@ static cudaError_t msc_cluster_launch_or_query(const TileArgs &args, int n_tiles
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   if (cluster_masks(csz_max))
-    return D == 3 ? launch_cfg<3, true>(cfg, args, P, smem, max_active) : launch_cfg<2, true>(cfg, args, P, smem, max_active);
-  return D == 3 ? launch_cfg<3, false>(cfg, args, P, smem, max_active) : launch_cfg<2, false>(cfg, args, P, smem, max_active);
+    return D == 3 ? launch_cfg<3, true>(cfg, args, P, max_active) : launch_cfg<2, true>(cfg, args, P, max_active);
+  return D == 3 ? launch_cfg<3, false>(cfg, args, P, max_active) : launch_cfg<2, false>(cfg, args, P, max_active);
 }
 
 cudaError_t launch_msc_cluster(const TileArgs &args, int units, int P, int csz_max, int D, cudaStream_t s) {

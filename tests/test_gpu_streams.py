@@ -180,3 +180,43 @@ def test_auto_search_without_stats_does_not_hold_the_host(busy):
     assert torch.equal(r.spins, waited.spins) and torch.equal(r.minima, waited.minima)
     torch.testing.assert_close(r.energy, waited.energy, rtol=1e-12, atol=0)
     h.close()
+
+
+# Two handles of one kernel and different sizes, from two host threads: neither
+# changes what the other may launch.
+def test_cluster_launches_of_two_sizes_from_two_threads():
+    import threading
+    cases = [(W.lattice((32, 32, 32), True, "pm1", seed=1), 8), (W.lattice((16, 16, 16), True, "pm1", seed=2), 4)]
+    failures, results = [], {}
+
+    def work(k):
+        inst, ctas = cases[k]
+        kw = dict(max_sweeps=2, kernel=isg.KERNEL_MSC, cluster_ctas=ctas, stats=False)
+        try:
+            h = isg.Handle([inst])
+            out = None
+            wide = (torch.empty(64 * inst.n, dtype=torch.int8, device="cuda"),
+                    torch.empty((1, 64), dtype=torch.float64, device="cuda"), None,
+                    torch.empty((1, 64), dtype=torch.int32, device="cuda"))
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for i in range(4000):
+                    if k and i % 2:  # (the small one is planned anew for every call)
+                        h.local_search([7], 64, out=wide, **kw)
+                        continue
+                    r = h.local_search([7], 32, out=out, **kw)
+                    out = (r.spins, r.energy, None, r.minima)
+            torch.cuda.synchronize()
+            results[k] = r.spins.cpu().numpy()
+            h.close()
+        except Exception as e:  # noqa: BLE001 (reported by the main thread)
+            failures.append(e)
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failures, failures
+    for k, (inst, _) in enumerate(cases):
+        s, _, _, _ = oracle.descent(inst, 7, 0, 32, max_sweeps=2)
+        assert np.array_equal(results[k].reshape(32, inst.n), s)
