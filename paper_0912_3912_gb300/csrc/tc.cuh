@@ -202,7 +202,10 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   return r;
 }
 
+// Every thread of every CTA.  The aligned forms ask for converged warps, so lanes
+// that come out of a branch meet first.
 __device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
