@@ -89,7 +89,7 @@ __global__ void dense_start(int32_t n, int32_t R, int32_t Rp, uint64_t seed, int
 __global__ void __launch_bounds__(256) dense_decide(int32_t n, int32_t R, int32_t Rp, int32_t b0, int32_t bsz,
                                                     const float *__restrict__ J, const float *__restrict__ hf,
                                                     const float *__restrict__ F, __nv_bfloat16 *S, DenseRep *rep) {
-  extern __shared__ float sJ[];  // [kDB][kDB] block of J
+  extern __shared__ __align__(16) float sJ[];  // [kDB][kDB] block of J
   for (int t = threadIdx.x; t < bsz * bsz; t += blockDim.x) {
     const int a = t / bsz, c = t % bsz;
     sJ[a * kDB + c] = J[(int64_t)(b0 + a) * n + b0 + c];

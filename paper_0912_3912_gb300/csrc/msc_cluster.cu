@@ -50,7 +50,7 @@ constexpr int kCT = 512;
 // per site (large slabs, for shared memory's sake).
 template <int D, bool MASKS>
 __global__ void __launch_bounds__(kCT, 1) msc_cluster_kernel(const __grid_constant__ TileArgs A, int P) {
-  extern __shared__ uint32_t smem[];
+  extern __shared__ __align__(16) uint32_t smem[];
   __shared__ uint32_t s_any[2], s_active, s_convround, s_upd;
   __shared__ int32_t s_total[32], s_minima[32];
   __shared__ double s_best[32], s_E[32];

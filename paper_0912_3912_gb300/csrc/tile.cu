@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(THREADS, (MODE == 3 ? 512 : 1024) / THREADS < 
 tile_kernel(const __grid_constant__ TileArgs A) {
   // (a parameter, so that its pointers stay in constant memory: read through a pointer
   // they took registers, and the 64 spilled)
-  extern __shared__ uint32_t smem[];
+  extern __shared__ __align__(16) uint32_t smem[];
   __shared__ int s_tile, s_last, s_segs;
   __shared__ bool s_merge;
   __shared__ uint32_t s_any, s_active, s_convround, s_upd;

@@ -15,3 +15,15 @@ def test_aligned_cluster_barrier_after_the_warp_has_met():
     assert body.index("__syncwarp();") < body.index("barrier.cluster.arrive.release.aligned")
     for name in sorted(os.listdir(CSRC)):  # ... and no such barrier elsewhere
         assert name == "tc.cuh" or "barrier.cluster" not in _source(name), name
+
+
+def test_dynamic_shared_memory_is_declared_aligned():
+    """Kernels read it in 16-byte vectors; its base follows the static variables.  (Two
+    kernels round the address up to 1,024 bytes themselves.)"""
+    found = 0
+    for name in sorted(os.listdir(CSRC)):
+        src = _source(name)
+        for m in re.finditer(r"extern __shared__ ([^;]*);", src):
+            found += 1
+            assert "__align__(16)" in m.group(1) or "1023" in src[m.end(): m.end() + 400], (name, m.group(0))
+    assert found >= 8
