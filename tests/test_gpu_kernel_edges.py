@@ -187,8 +187,8 @@ def test_auto_family_of_one_general_graph(n):
     _compare([inst], [n], 6, False, **kw)
 
 
-# ising_energy: one-CTA instances (up to 2048 spins) and larger ones in parts of
-# 1024 sites; 4, 16 and 32 replicas per word group and their remainders; sizes
+# ising_energy: one-CTA instances (handles of up to 1024 spins) and larger ones in
+# parts of 256 sites (below: others of both); 4, 16 and 32 replicas per word group and their remainders; sizes
 # that are no multiple of 4 and spins that start on an odd byte; lattices of
 # both dimensions; rows of 48 entries and more; hyper-edges.  Integer energies
 # are equal; float ones are exact sums rounded once, the oracle's FP64 sums of
@@ -353,3 +353,70 @@ def test_tile_both_orders_on_one_handle():
 def test_sweep_fp32_lattice_group_sizes(dims, R):
     inst = W.lattice(dims, True, "gauss", "gauss", seed=R)
     _compare([inst], [R], R, False, max_sweeps=12, restarts=2, refresh_every=5, kernel=isg.KERNEL_SWEEP)
+
+
+# ... and the shapes those do not reach: lattices in one CTA, many instances of up
+# to 2048 spins (one CTA each), parts of more than one site a thread with a ragged
+# last one (lattices of both dimensions, rows walked by a thread and by a warp).
+def _check_energies(insts, R, rtol):
+    h = isg.Handle(insts)
+    spins = (np.random.default_rng(R).integers(0, 2, size=R * h.total_spins) * 2 - 1).astype(np.int8)
+    dev = torch.from_numpy(spins).cuda()
+    for _ in range(2):
+        E = h.energy(dev, R).cpu().numpy()
+    off = 0
+    for b, inst in enumerate(insts):
+        ref = oracle.energies(inst, spins[off: off + R * inst.n].reshape(R, inst.n))
+        off += R * inst.n
+        if inst.dtype == "i8":
+            assert np.array_equal(E[b], ref)
+        else:
+            np.testing.assert_allclose(E[b], ref, rtol=rtol, atol=1e-9)
+    h.close()
+
+
+@pytest.mark.parametrize("R", [1, 6, 33])
+@pytest.mark.parametrize("J", ["pm1", "gauss"])
+@pytest.mark.parametrize("dims", [(3, 3), (31, 31), (32, 32), (10, 10, 10)])
+def test_energy_lattice_in_one_cta(dims, J, R):
+    _check_energies([W.lattice(dims, True, J, "pm1_0" if J == "pm1" else "gauss", seed=sum(dims))], R, 1e-12)
+
+
+@pytest.mark.parametrize("kind", ["lattice", "i8", "f32"])
+def test_energy_many_instances_of_one_cta(kind):
+    rng = np.random.default_rng(7)
+    if kind == "lattice":
+        insts = [W.lattice((L, L), True, "gauss", "gauss", seed=L) for L in list(range(33, 46)) * 12]
+    else:
+        insts = [W.random_graph(int(n), 3.0, int(n), dtype=kind, n_hyper=50, hyper_order=(2, 3, 5))
+                 for n in np.concatenate([[1025, 2047, 2048], rng.integers(1025, 2049, size=21)])] * 7
+    _check_energies(insts, 2, 1e-12)
+
+
+@pytest.mark.parametrize("dims,J,R", [((45, 45, 45), "gauss", 40), ((64, 64, 64), "pm1", 33), ((90, 90, 90), "gauss", 5),
+                                      ((701, 701), "pm1", 17)])
+def test_energy_lattice_large_parts(dims, J, R):
+    # (a relative bound on sums of up to 3e6 terms of order one that partly cancel)
+    _check_energies([W.lattice(dims, True, J, "pm1_0" if J == "pm1" else None, seed=R)], R, 1e-10)
+
+
+@pytest.mark.parametrize("dtype,R", [("i8", 40), ("f32", 70)])
+def test_energy_graph_large_parts(dtype, R):
+    n = 90001
+    rng = np.random.default_rng(n)
+    key = np.unique(rng.integers(0, n, size=3 * n) * np.int64(n) + rng.integers(0, n, size=3 * n))
+    u, v = key // n, key % n
+    lo, hi = np.minimum(u, v), np.maximum(u, v)
+    key = np.unique((lo * np.int64(n) + hi)[lo != hi])
+    u, v = key // n, key % n
+    w = rng.standard_normal(len(u)).astype(np.float32) if dtype == "f32" else \
+        (rng.integers(1, 128, size=len(u)) * (rng.integers(0, 2, size=len(u)) * 2 - 1)).astype(np.int8)
+    for hub in (False, True):  # (a hub: rows by warps)
+        if hub:
+            keep = (u != 17) & (v != 17)
+            ends = np.arange(18, n, 3)
+            u, v = np.concatenate([u[keep], np.full(len(ends), 17)]), np.concatenate([v[keep], ends])
+            w = np.concatenate([w[keep], np.resize(w, len(ends))])
+        rp, col, J = W.csr_from_edges(n, u, v, w, dtype)
+        h = np.resize(w, n).astype(w.dtype)
+        _check_energies([W.Instance(n=n, row_ptr=rp, col=col, J=J, h=h, dtype=dtype)], R, 1e-10)
