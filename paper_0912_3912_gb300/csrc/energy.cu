@@ -417,22 +417,26 @@ void energy_plan_free(ising_handle *h) {
 
 namespace {
 
-// Whether every instance's terms can be summed in integers: integer couplings,
-// or FP32 ones with a unit whose terms, as many as one lane adds, fit 62 bits
-// (doubled and offset by the constant: two more bits, within the 64).
+// Whether every instance's terms can be summed in integers: FP32 couplings with a
+// unit whose terms, as many as one lane adds, fit 62 bits (doubled and offset by the
+// constant: two more bits, within the 64); int8 ones whose sums fit 30 bits of 32 (not
+// with some 2^27 couplings in the rows of a few spins).
 bool integer_sums(const ising_handle *h) {
-  if (h->dtype == ISING_I8) return true;
+  const bool fl = h->dtype == ISING_F32;
   for (const InstDesc &I : h->inst) {
-    if (I.ebase < 0) return false;
+    if (fl && I.ebase < 0) return false;
+    const bool by_row = I.max_deg >= 48;
     const int64_t sites = std::min<int64_t>(I.n, kPartMax);  // (a tile holds fewer)
     const int64_t parts = (I.n + sites - 1) / sites;
-    const int64_t lane_sites = I.max_deg >= 48 ? (sites + kWarps - 1) / kWarps : (sites + kThreads - 1) / kThreads;
-    const int64_t lane_row = I.max_deg >= 48 ? (I.max_deg + 31) / 32 : I.max_deg;
+    const int64_t lane_sites = by_row ? (sites + kWarps - 1) / kWarps : (sites + kThreads - 1) / kThreads;
+    // entries: the longest row at every site, or every row of the handle
+    int64_t entries = lane_sites * (by_row ? (I.max_deg + 31) / 32 : I.max_deg);
+    if (by_row) entries = std::min(entries, lane_sites + h->total_nnz / 32);
     const int64_t edges = ((I.n_hyper + parts - 1) / parts + kThreads - 1) / kThreads;
-    const int64_t terms = lane_sites * (lane_row + 1) + edges;
+    const int64_t terms = lane_sites + entries + edges;
     int lg = 0;
     while (((int64_t)1 << lg) < terms) ++lg;
-    if (I.ebits + lg > 62 - 1) return false;
+    if (I.ebits + lg > (fl ? 62 : 30) - 1) return false;
   }
   return true;
 }
