@@ -392,6 +392,8 @@ bool fault_is(const char *what) {
 }
 int g_alloc_countdown = 0;  // allocations left before the injected failure (0: none)
 
+// Enqueued on the handle's own stream: uploads_done() before src goes and before
+// any stream reads *dst.
 template <class T>
 cudaError_t upload(ising_handle *h, T **dst, const std::vector<T> &src) {
   if (g_alloc_countdown > 0 && --g_alloc_countdown == 0) return cudaErrorMemoryAllocation;
@@ -399,9 +401,9 @@ cudaError_t upload(ising_handle *h, T **dst, const std::vector<T> &src) {
   cudaError_t e = setup_stream(h, &setup);
   if (e == cudaSuccess) e = cudaMalloc((void **)dst, std::max<size_t>(1, src.size()) * sizeof(T));
   if (e != cudaSuccess || src.empty()) return e;
-  e = cudaMemcpyAsync(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice, setup);
-  return e != cudaSuccess ? e : cudaStreamSynchronize(setup);  // (before any stream reads it)
+  return cudaMemcpyAsync(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice, setup);
 }
+bool uploads_done(ising_handle *h) { return !h->setup || cudaStreamSynchronize(h->setup) == cudaSuccess; }
 
 void free_handle(ising_handle *h) {
   if (!h) return;
@@ -642,7 +644,8 @@ ising_status run_tile(ising_handle *h, int mode, int32_t R, const ising_search_p
     if (h->d_tiles) cudaFree(h->d_tiles);
     h->d_tiles = nullptr;
     h->tiles_R = -1;
-    if (upload(h, &h->d_tiles, tiles) != cudaSuccess) return ISING_ERR_CUDA;
+    const cudaError_t e = upload(h, &h->d_tiles, tiles);
+    if (!uploads_done(h) || e != cudaSuccess) return ISING_ERR_CUDA;
     h->n_tiles = (int32_t)tiles.size();
     h->tiles_R = R;
   }
@@ -1094,17 +1097,20 @@ ising_status ising_create(const ising_instance_desc *descs, int32_t n_instances,
     ok = upload(h, &h->d_meta, meta) == cudaSuccess && upload(h, &h->d_latinfo, latinfo) == cudaSuccess &&
          (fl ? upload(h, (float **)&h->d_Jpos, Jpf) : upload(h, (int8_t **)&h->d_Jpos, Jpi)) == cudaSuccess &&
          (fl ? upload(h, (float **)&h->d_Jfwd, Jff) : upload(h, (int8_t **)&h->d_Jfwd, Jfi)) == cudaSuccess;
+    ok = uploads_done(h) && ok;
   }
   if (ok && dense) {
     std::vector<float> Jd;
     for (int32_t b = 0; b < n_instances; ++b)
       Jd.insert(Jd.end(), descs[b].J_dense, descs[b].J_dense + (int64_t)descs[b].n * descs[b].n);
     ok = upload(h, &h->d_Jdense, Jd) == cudaSuccess;
+    ok = uploads_done(h) && ok;
   }
   ok = ok && cudaMalloc(&h->d_seeds, sizeof(uint64_t) * n_instances) == cudaSuccess &&
        cudaMalloc(&h->d_stats, sizeof(unsigned long long) * 8) == cudaSuccess &&
        cudaMalloc(&h->d_queue, sizeof(int32_t) * 4) == cudaSuccess &&
        cudaMallocHost(&h->h_stats_pinned, sizeof(unsigned long long) * 8) == cudaSuccess;
+  ok = uploads_done(h) && ok;
   if (!ok) {
     cudaGetLastError();
     free_handle(h);
