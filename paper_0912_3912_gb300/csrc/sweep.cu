@@ -400,14 +400,11 @@ sweep_visit(SweepArgs A, int32_t c, int32_t c0, int32_t c1) {
       const bool fresh = MODE == 1 ? refresh : dd == 0;  // every spin is evaluated
       uint32_t anyg = 0;
       if constexpr (MODE == 1 && LAT) {
-        // Periodic lattice, FP32 fields.  Lane = position for every read a
-        // visit needs (its word, the neighbour words, their flip masks, the
-        // couplings, the field), so a warp step costs one round trip to memory.
-        // Refresh sweeps evaluate every (site, replica) pair: SPW sites at a
-        // time, LPS lanes each, values taken by shuffle.  Other sweeps evaluate
-        // only the pairs with a pending bit: the positions stage their reads and
-        // stored fields in shared memory, the pairs are listed, and all 32 lanes
-        // work through the list; the flips are then applied per position.
+        // Periodic lattice, FP32 fields.  Lane = position: it reads its word, the
+        // neighbours' words and flip masks, the couplings and the field in one round
+        // trip and takes all LPS replicas of its site from registers.  Refresh sweeps
+        // evaluate every (site, replica) pair; other sweeps only the positions with a
+        // pending replica.
         const int D2 = 2 * I.lat_d;
         const float *Jp0 = reinterpret_cast<const float *>(G.Jpos) + so;
         const float *hf = reinterpret_cast<const float *>(G.h) + so;
@@ -613,7 +610,6 @@ sweep_visit(SweepArgs A, int32_t c, int32_t c0, int32_t c1) {
             const bool fl = __any_sync(0xffffffffu, segr != 0u);
             if (lane == 0) cf_own[base >> 5] = fl ? (uint16_t)0x0100 : (uint16_t)0;
           }
-          __syncwarp();  // staging read before the next batch overwrites it
         }
       } else if constexpr (LAT) {
       // Integer lattice: a warp takes `pw` consecutive class positions at a time
@@ -1180,69 +1176,48 @@ __global__ void __launch_bounds__(kST, 4) sweep_energy(SweepArgs A) {
           __syncwarp();
         }
       } else {
-      // 32 positions per warp step: one coalesced read of their site indices
-        // and lattice metadata, then SPW sites at a time, several steps unrolled
-        // so that their neighbour reads are in flight together
+        // General graphs: 32 spins per warp step, SPW at a time, several steps
+        // unrolled so that their neighbour reads are in flight together
         for (int base = (blockIdx.x * nw + warp) * 32; base < n; base += gridDim.x * nw * 32) {
-          const int v1 = base + lane;
-          const int j1 = v1 < n ? ((LAT && !A.sequential) ? __ldg(G.order + I.spin_off + v1) : v1) : 0;
-          const uint32_t meta1 = (LAT && v1 < n) ? __ldg(G.meta + I.spin_off + v1) : 0u;
-  #pragma unroll 4
-        for (int st = 0; st < 32 / SPW; ++st) {
-          const int src = st * SPW + sub;
-          const int v = base + src;
-          const int j = __shfl_sync(0xffffffffu, j1, src);
-          const uint32_t meta = __shfl_sync(0xffffffffu, meta1, src);
-          if (v >= n) continue;
-          const int64_t gj = I.spin_off + j;
-          const uint32_t bj = (swg[j] >> ln) & 1u;
-          const uint32_t k0 = LAT ? 0u : __ldg(G.row + gj);
-          const uint32_t k1 = LAT ? (uint32_t)(2 * I.lat_d) : __ldg(G.row + gj + 1);
-          if (FLOAT) {
-            const float hv = __ldg(reinterpret_cast<const float *>(G.h) + gj);
-            double e = bj ? (double)hv : -(double)hv;
-            if (fx) {
-              const int64_t th = xr_term(hv, ub);
-              xe_add(acci, accl, bj ? -th : th);
-            }
-            for (uint32_t kk = k0; kk < k1; ++kk) {
-              int i;
-              float w;
-              if (LAT) {
-                i = lat_nbr(j, meta, (int)kk, L);
-                w = __ldg(reinterpret_cast<const float *>(G.Jpos) + (int64_t)kk * G.nsp + I.spin_off + v);
-              } else {
-                i = __ldg(G.col + kk);
-                w = __ldg(reinterpret_cast<const float *>(G.J) + kk);
+#pragma unroll 4
+          for (int st = 0; st < 32 / SPW; ++st) {
+            const int j = base + st * SPW + sub;
+            if (j >= n) continue;
+            const int64_t gj = I.spin_off + j;
+            const uint32_t bj = (swg[j] >> ln) & 1u;
+            const uint32_t k0 = __ldg(G.row + gj), k1 = __ldg(G.row + gj + 1);
+            if (FLOAT) {
+              const float hv = __ldg(reinterpret_cast<const float *>(G.h) + gj);
+              double e = bj ? (double)hv : -(double)hv;
+              if (fx) {
+                const int64_t th = xr_term(hv, ub);
+                xe_add(acci, accl, bj ? -th : th);
               }
-              if (i > j) {
-                const bool differ = ((swg[i] >> ln) & 1u) ^ bj;
-                if (fx) {
-                  const int64_t t = xr_term(w, ub);
-                  xe_add(acci, accl, differ ? t : -t);
-                } else {
-                  e += differ ? -(double)w : (double)w;
+              for (uint32_t kk = k0; kk < k1; ++kk) {
+                const int i = __ldg(G.col + kk);
+                const float w = __ldg(reinterpret_cast<const float *>(G.J) + kk);
+                if (i > j) {
+                  const bool differ = ((swg[i] >> ln) & 1u) ^ bj;
+                  if (fx) {
+                    const int64_t t = xr_term(w, ub);
+                    xe_add(acci, accl, differ ? t : -t);
+                  } else {
+                    e += differ ? -(double)w : (double)w;
+                  }
                 }
               }
-            }
-            if (!fx) accd -= e;
-          } else {
-            const int hv = __ldg(reinterpret_cast<const int8_t *>(G.h) + gj);
-            int e = bj ? hv : -hv;
-            for (uint32_t kk = k0; kk < k1; ++kk) {
-              int i, w;
-              if (LAT) {
-                i = lat_nbr(j, meta, (int)kk, L);
-                w = __ldg(reinterpret_cast<const int8_t *>(G.Jpos) + (int64_t)kk * G.nsp + I.spin_off + v);
-              } else {
-                i = __ldg(G.col + kk);
-                w = __ldg(reinterpret_cast<const int8_t *>(G.J) + kk);
+              if (!fx) accd -= e;
+            } else {
+              const int hv = __ldg(reinterpret_cast<const int8_t *>(G.h) + gj);
+              int e = bj ? hv : -hv;
+              for (uint32_t kk = k0; kk < k1; ++kk) {
+                const int i = __ldg(G.col + kk);
+                const int w = __ldg(reinterpret_cast<const int8_t *>(G.J) + kk);
+                if (i > j) e += (((swg[i] >> ln) & 1u) ^ bj) ? -w : w;
               }
-              if (i > j) e += (((swg[i] >> ln) & 1u) ^ bj) ? -w : w;
+              acci -= e;
             }
-            acci -= e;
           }
-        }
         }
       }
       // hyper-edges (CSR instances only)
