@@ -95,8 +95,7 @@ struct DevGraph {
   int32_t hyper;            // some instance has hyper-edges
 };
 
-// Per-call arguments of the tile kernels (kept in device memory so that a
-// captured graph can be replayed with new outputs and seeds).
+// Per-call arguments of the tile and cluster kernels (a kernel parameter).
 struct TileArgs {
   DevGraph g;
   const int2 *tiles;        // (instance, 32-replica group), largest instances first

@@ -25,8 +25,9 @@
 // identically in every CTA of the cluster, so the cluster's control flow stays
 // uniform and every barrier is matched.
 //
-// A visit is bound by its logic instructions (64 lanes a cycle and SM): the class
-// layout, sign planes, one pending target per lane and two chunks at a time took
+// A visit is bound by its logic instructions (64 lanes a cycle and SM): on the 128 SMs
+// that hold a CTA the ALU pipe is 74 % busy and 69 % of the issue slots are, the top
+// stalls are not_selected 1.4, math pipe 1.2 and wait 1.1 per issue.  The class layout, sign planes, one pending target per lane and two chunks at a time took
 // 32^3 with fields, 1,024 replicas, 10 descents from 719 to 535 us a call with four
 // CTAs a cluster; two CTAs and two segments of descents each: 504, and 482 with the
 // arguments as a parameter (their pointers in constant memory).  With 32 replicas,

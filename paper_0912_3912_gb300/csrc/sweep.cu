@@ -1602,8 +1602,8 @@ cudaError_t run_instance(ising_handle *h, SweepArgs A, int mode, cudaStream_t s)
   const int64_t gy = mode == 2 ? 1 : ((mode == 1 && LAT) ? A.G : std::max<int64_t>(1, std::min<int64_t>(A.G, slots / need)));
   const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(need, slots / gy)), (unsigned)gy);
   // Programmatic launches: measured faster for the multi-spin-coded visits and for
-  // FP32 lattices whose classes leave warps idle (45^3, 21 replicas: 1533 against
-  // 1653 us), slower for larger ones (100^3, 16 replicas: 49.4 against 48.3 ms) and
+  // FP32 lattices whose classes leave warps idle (45^3, 21 replicas: 1521 against
+  // 1624 us), slower for larger ones (100^3, 16 replicas: 49.4 against 48.3 ms) and
   // on general graphs (3801 against 3753 us)
   A.pdl = mode == 2 || (mode == 1 && LAT && need * A.G * 2 <= slots);
   Phase ph;

@@ -29,6 +29,8 @@
 //           thresholds);
 //   MODE 3  the same on periodic 2-d/3-d lattices, with neighbours computed
 //           from the lattice geometry and the field folded into the count.
+// In the index order the lane modes give a tile's spins to one warp, one after
+// another, multi-spin coding to one thread a step.
 // Replicas of a tile run their descents in lockstep rounds: descent k of every
 // lane starts together; a lane whose descent ended waits (masked) until the
 // round ends.  Each replica's own sequence of states is exactly the one its
