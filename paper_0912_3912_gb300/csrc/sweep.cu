@@ -1443,25 +1443,36 @@ __global__ void sweep_mark_final(SweepArgs A) {
   if (threadIdx.x == 0) *A.counter = 0;
 }
 
-__global__ void sweep_output(SweepArgs A) {
-  const int n = A.I.n;
-  const int64_t tot = (int64_t)A.Rn * n;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < tot; t += (int64_t)gridDim.x * blockDim.x) {
-    const int r = (int)(t / n), i = (int)(t % n);
-    const int g = r / A.LPS, l = r % A.LPS;
-    const GroupState &S = A.gs[g];
-    const uint32_t w = S.minima[l] > 0 ? A.bw[(size_t)g * n + i] : A.sw[(size_t)g * n + i];
-    A.spins[(int64_t)A.R * A.I.spin_off + (int64_t)A.r0 * n + t] = ((w >> l) & 1u) ? 1 : -1;
+// Results: a warp per 32 sites of a group (blockIdx.y).  With whole words of spins at
+// 16-byte addresses a transpose hands lane r replica r's 32 spins, 32 bytes of its
+// row; else byte by byte.  Bound by the writes (a thread per spin, with its index's
+// divisions, took 435 us for 128^3 sites and 64 replicas, 316 with one division less).
+__global__ void __launch_bounds__(kST) sweep_output(SweepArgs A) {
+  const int n = A.I.n, g = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const GroupState &S = A.gs[g];
+  const uint32_t valid = S.lane_valid, best = __ballot_sync(0xffffffffu, S.minima[lane] > 0);
+  const uint32_t *swg = A.sw + (size_t)g * n, *bwg = A.bw + (size_t)g * n;
+  int8_t *out = A.spins + (int64_t)A.R * A.I.spin_off + ((int64_t)A.r0 + A.LPS * g) * n;
+  const bool wide = (n & 31) == 0 && ((uintptr_t)out & 15) == 0;
+  for (int64_t i0 = ((int64_t)blockIdx.x * nw + warp) * 32; i0 < n; i0 += (int64_t)gridDim.x * nw * 32) {
+    const int64_t i = i0 + lane;
+    const uint32_t w = i < n ? (bwg[i] & best) | (swg[i] & ~best) : 0u;
+    if (wide) {
+      const uint32_t mine = warp_transpose32(w, lane);
+      if ((valid >> lane) & 1u) store_spins32(out + (int64_t)lane * n + i0, mine);
+    } else if (i < n) {
+      for (uint32_t m = valid; m; m &= m - 1u) {
+        const int r = __ffs(m) - 1;
+        out[(int64_t)r * n + i] = ((w >> r) & 1u) ? 1 : -1;
+      }
+    }
   }
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < A.Rn) {
-    const int g = (int)t / A.LPS, l = (int)t % A.LPS;
-    const GroupState &S = A.gs[g];
-    const double e = S.minima[l] > 0 ? S.best[l] : S.E[l];
-    const int64_t o = (int64_t)A.b * A.R + A.r0 + t;
+  if (blockIdx.x == 0 && warp == 0 && ((valid >> lane) & 1u)) {
+    const double e = (best >> lane) & 1u ? S.best[lane] : S.E[lane];
+    const int64_t o = (int64_t)A.b * A.R + A.r0 + A.LPS * g + lane;
     A.energy[o] = e;
     if (A.energy_i32) A.energy_i32[o] = (int32_t)e;
-    if (A.minima) A.minima[o] = S.minima[l];
+    if (A.minima) A.minima[o] = S.minima[lane];
   }
 }
 
@@ -1707,8 +1718,8 @@ cudaError_t run_instance(ising_handle *h, SweepArgs A, int mode, cudaStream_t s)
   h->launches += 3;
   if (mode == 1) sweep_energy<true, LPS, LAT><<<A.grid_e, kST, 0, s>>>(F);
   else sweep_energy<false, LPS, LAT><<<A.grid_e, kST, 0, s>>>(F);
-  const int64_t tot = (int64_t)A.Rn * I.n;
-  sweep_output<<<(int)std::min<int64_t>((tot + kST - 1) / kST, (int64_t)h->sm_count * 16), kST, 0, s>>>(F);
+  const int64_t blocks = ((int64_t)I.n + 32 * kW - 1) / (32 * kW), most = std::max(1, h->sm_count * 16 / A.G);
+  sweep_output<<<dim3((unsigned)std::min(blocks, most), (unsigned)A.G), kST, 0, s>>>(F);
   return cudaGetLastError();
 }
 

@@ -420,3 +420,25 @@ def test_energy_graph_large_parts(dtype, R):
         rp, col, J = W.csr_from_edges(n, u, v, w, dtype)
         h = np.resize(w, n).astype(w.dtype)
         _check_energies([W.Instance(n=n, row_ptr=rp, col=col, J=J, h=h, dtype=dtype)], R, 1e-10)
+
+
+# Results of the sweep family in whole words of spins and (an odd address, an odd
+# size) byte by byte: groups of 8, 16 and 32, a last one partly filled, results of
+# converged descents and of some that never converge.
+@pytest.mark.parametrize("max_sweeps", [3, 200])
+@pytest.mark.parametrize("R", [5, 16, 33, 70])
+@pytest.mark.parametrize("kind,n", [("i8", 96), ("f32", 96), ("f32", 97), ("pm1", 512), ("gauss", 343)])
+def test_sweep_result_addresses(kind, n, R, max_sweeps):
+    if kind in ("pm1", "gauss"):
+        inst = W.lattice((round(n ** (1 / 3)),) * 3, True, kind, None, seed=n)
+    else:
+        inst = W.random_graph(n, 4.0, n, dtype=kind)
+    kw = dict(max_sweeps=max_sweeps, restarts=2, kernel=isg.KERNEL_SWEEP)
+    _, o = _compare([inst], [n], R, inst.dtype == "i8", **kw)
+    h = isg.Handle([inst])
+    ref = h.local_search([n], R, **kw)
+    for at in (0, 1, 8, 16):
+        buf = torch.zeros(R * n + 16, dtype=torch.int8, device="cuda")[at:at + R * n]
+        h.local_search([n], R, out=(buf, ref.energy.clone(), None, ref.minima.clone()), **kw)
+        assert np.array_equal(buf.cpu().numpy().reshape(R, n), o[0][0])
+    h.close()
