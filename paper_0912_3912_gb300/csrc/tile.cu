@@ -21,7 +21,7 @@
 //           update), with a from-scratch refresh at descent sweeps
 //           d % refresh == 0 (always d == 0): the FP64 sum rounded to FP32,
 //           formed exactly in fixed point when that is exact (runit >= 0; else, and
-//           for a warp's lone pending spin, a warp per spin, lane = replica);
+//           for one or two pending spins of a warp, a warp per spin, lane = replica);
 //           fields of instances that fit stay in shared memory;
 //   MODE 2  multi-spin coding for J in {-1,+1}, h in {-1,0,+1}: one thread per
 //           spin evaluates all 32 replicas with bitwise logic (unsatisfied-bond
@@ -172,7 +172,9 @@ __device__ void tile_energy_lanes(const DevGraph &G, const InstDesc &I, const ui
 // issue).  FP32: 64-bit fixed point, NV = 8 replicas at a time, the rows read again
 // from L1 for each (1,024 cell grids of 128 to 2,048 spins: 1,754 us a call with
 // the form above, 1,623 / 1,577 / 1,699 with 4 / 8 / 16); integers: all 32 (a graph of
-// 1,000 spins, 1,024 replicas, 20 descents: 1,112 -> 1,036 us).  False, and nothing done, when FP32
+// 1,000 spins, 1,024 replicas, 20 descents: 1,112 -> 1,036 us).  Instances of up to
+// kFewSpins leave most lanes without a spin and take the form above (5,000 of 40 spins,
+// 10 descents: 6.04 against 5.31 ms).  False, and nothing done, when FP32
 // terms are not integers of one unit, or so wide or so many that a lane's sum could
 // leave its 62 bits (integers: a warp's its 31); the same for the whole CTA.
 template <bool FLOAT, int THREADS>
@@ -400,13 +402,17 @@ __device__ __forceinline__ uint32_t own_refresh(const DevGraph &G, const InstDes
 // eight predicated ones each, and its marks take fewer steps.  Integers: 6,000 spins
 // of degree 5, 20 replicas, 2 descents 889 -> 623 us (all by four lanes 639), 300
 // spins 110 -> 114 (144); 1,000 spins, 1,024 replicas, 20 descents 982 -> 792 (3 / 6
-// spins: 802 / 806).  FP32, where the fields are read and written besides: one spin,
-// as in the index order, dense rows and the last sweeps (32 replicas: 1,000 spins in
-// index order 10.7 -> 5.3 ms, 64 fully coupled spins given as rows 3.5 -> 1.5 ms, 200
-// spins of degree 40 1,096 -> 556 us; 4,096 cell grids 3.26 -> 3.20 ms, and 1 % more
-// from 3 spins).
+// spins: 802 / 806).  FP32, where the fields are read and written besides: one or two,
+// as in dense rows, small classes and the last sweeps (32 replicas, all by four lanes /
+// from 2 / 3 / 4 / 5 spins: 200 spins of degree 40 1,096 / 561 / 543 / 535 / 545 us,
+// 1,000 of degree 100 10.0 / 9.2 / 8.3 / 8.6 / 8.6 ms, 4,096 cell grids 3.26 / 3.22 /
+// 3.24 / 3.28 / 3.33), up to three in instances of few spins (5,000 of 40 spins 748 /
+// 654 / 527 / 516 / 520 us, 3,000 of 64 spins 515 / 498 / 465 / 432 / 433).
+constexpr int kFewSpins = 80;  // ten a warp of the smallest CTA
 template <int MODE>
-constexpr int kOwnLeast = MODE == 0 ? 4 : 2;
+__device__ __forceinline__ int own_least(int n) {
+  return MODE == 0 || n <= kFewSpins ? 4 : 3;
+}
 
 // Integer couplings: the exact field from scratch, not kept.
 __device__ __forceinline__ uint32_t own_int(const DevGraph &G, const InstDesc &I, const uint32_t *sw, int j, int r0,
@@ -721,7 +727,7 @@ tile_kernel(const __grid_constant__ TileArgs A) {
               if (!seq) {
                 const int ul = MODE == 1 && refresh && pl ? __ldg(G.runit + I.spin_off + jl) : 0;
                 uint32_t own = __ballot_sync(0xffffffffu, pl && ul >= 0);
-                if (__popc(own) < kOwnLeast<MODE>) own = 0u;
+                if (__popc(own) < own_least<MODE>(n)) own = 0u;
                 if (own) {
                   if ((own >> lane) & 1u) s_slot[(tid & ~31) + __popc(own & ((1u << lane) - 1u))] = (uint8_t)lane;
                   __syncwarp();
@@ -936,7 +942,7 @@ tile_kernel(const __grid_constant__ TileArgs A) {
           const uint32_t cr = s_convround;
           if (cr) {
             if (MODE == 3) tile_energy_lattice(G, I, sw, s_cnt, s_E);
-            else if (!tile_energy_sites<MODE == 1, THREADS>(G, I, sw, s_red, s_E))
+            else if (n <= kFewSpins || !tile_energy_sites<MODE == 1, THREADS>(G, I, sw, s_red, s_E))
               tile_energy_lanes<MODE == 1>(G, I, sw, s_red, s_E);
             if (tid == 0) {
               uint32_t upd = 0;
@@ -967,7 +973,7 @@ tile_kernel(const __grid_constant__ TileArgs A) {
       if (s_minima[r] > 0) has_best |= 1u << r;
     if ((lane_valid & ~has_best) && (!SEG || unit % segs == segs - 1)) {
       if (MODE == 3) tile_energy_lattice(G, I, sw, s_cnt, s_E);
-      else if (!tile_energy_sites<MODE == 1, THREADS>(G, I, sw, s_red, s_E))
+      else if (n <= kFewSpins || !tile_energy_sites<MODE == 1, THREADS>(G, I, sw, s_red, s_E))
         tile_energy_lanes<MODE == 1>(G, I, sw, s_red, s_E);
       if (tid < 32 && !((has_best >> tid) & 1u)) s_best[tid] = s_E[tid];
     }

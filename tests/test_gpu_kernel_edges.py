@@ -442,3 +442,17 @@ def test_sweep_result_addresses(kind, n, R, max_sweeps):
         h.local_search([n], R, out=(buf, ref.energy.clone(), None, ref.minima.clone()), **kw)
         assert np.array_equal(buf.cpu().numpy().reshape(R, n), o[0][0])
     h.close()
+
+
+# Both sides of the size up to which a tile's energies and few pending spins are the
+# whole warp's.
+@pytest.mark.parametrize("R", [9, 33])
+@pytest.mark.parametrize("n", [80, 81])
+@pytest.mark.parametrize("kind", ["i8", "f32", "wide", "wider"])
+def test_tile_few_spins(kind, n, R):
+    inst = W.random_graph(n, 5.0, n, dtype="i8" if kind == "i8" else "f32", n_hyper=n // 4, hyper_order=(2, 3, 4, 9))
+    if kind.startswith("wide"):
+        inst = _exp_spread(inst, *((-12, 12) if kind == "wide" else (-45, 25)))
+    for restarts, max_sweeps in ((1, 100), (3, 2)):
+        _compare([inst] * 2, [n, 7], R, kind == "i8", max_sweeps=max_sweeps, restarts=restarts, refresh_every=3,
+                 kernel=isg.KERNEL_TILE)
