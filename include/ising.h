@@ -239,21 +239,19 @@ ising_status ising_energy(ising_handle *h, const int8_t *spins_dev, int32_t repl
  * [instance][replica][spin].  energy_dev: device double out [instance][replica].
  * energy_i32_dev, minima_dev (device int32 [instance][replica], converged
  * descents per replica) may be NULL.  stats (host) may be NULL; when given, the
- * call waits for the stream to finish and fills it.  Without stats, families TILE
- * and MSC return once their kernel is enqueued; SWEEP and DENSE_TC read the search's
- * progress on the host and hold it until the search is nearly done.
- * ISING_KERNEL_AUTO takes SWEEP for an instance that TILE could run only where it is
- * faster and the call has stats (spins, minima and counters are the same either way,
- * energies too but for the rounding of FP64 sums).                              */
+ * call waits for the stream to finish and fills it.  Without stats the call returns
+ * once the search is enqueued, but for families SWEEP and DENSE_TC, which follow it
+ * on the host and return when it is nearly done; where ISING_KERNEL_AUTO takes SWEEP
+ * for an instance that TILE could run, because it is faster, the call without stats
+ * still returns at once (its sweeps loop on the device).                          */
 ising_status ising_local_search(ising_handle *h, const uint64_t *seeds, int32_t replicas,
                                 const ising_search_params *p, int8_t *spins_dev,
                                 double *energy_dev, int32_t *energy_i32_dev,
                                 int32_t *minima_dev, ising_stats *stats,
                                 cudaStream_t stream);
 
-/* The kernel family the planner would use for these arguments in a call with
- * stats (after resolving ISING_KERNEL_AUTO), or a negative ising_status on invalid
- * input.                                                                       */
+/* The kernel family the planner would use for these arguments (after
+ * resolving ISING_KERNEL_AUTO), or a negative ising_status on invalid input.   */
 int32_t ising_plan_kernel(ising_handle *h, int32_t replicas, const ising_search_params *p);
 
 /* Time every eligible kernel family on this handle (on `stream`, synchronising

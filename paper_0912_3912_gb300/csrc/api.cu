@@ -16,7 +16,7 @@ namespace isg {
 cudaError_t launch_plain(ising_handle *h, const ising_search_params *p, int32_t R, int8_t *spins, double *E,
                          int32_t *E32, int32_t *minima, const uint64_t *seeds_host, cudaStream_t s);
 cudaError_t launch_sweep(ising_handle *h, const ising_search_params *p, int32_t R, int8_t *spins, double *E,
-                         int32_t *E32, int32_t *minima, cudaStream_t s);
+                         int32_t *E32, int32_t *minima, bool detached, cudaStream_t s);
 cudaError_t launch_dense(ising_handle *h, const ising_search_params *p, int32_t R, int8_t *spins, double *E,
                          int32_t *E32, int32_t *minima, const uint64_t *seeds_host, cudaStream_t s);
 bool dense_supported(const ising_handle *h, int32_t R);
@@ -470,12 +470,14 @@ bool tile_fits(const ising_handle *h, int mode) {
 // spins 670 / 1380, 6,000 1045 / 1422, 9,000 1465 / 1326, 12,000 1902 / 1531, 20,000
 // 3037 / 1786; Gaussian squares, 32 replicas, 4 descents: 64 x 64 348 / 551, 96 x 96
 // 668 / 592, 128 x 128 1113 / 739 and with 256 replicas 1112 / 1439.
-// Asked only for calls that wait for their search anyway: the sweep family holds the
-// host until the search is nearly done, a tile launch returns at once, and a program
-// that drives several handles or streams from one thread counts on that.
+// A tile launch returns at once, and a program that drives several handles or streams
+// from one thread counts on that: without counters to wait for, the sweep family runs
+// such a search detached (launch_sweep) instead of following it on the host.
 bool sweep_is_faster(const ising_handle *h, int32_t R, const ising_search_params *p) {
   const int32_t groups = (R + 31) / 32;
   if (groups > 32 || p->schedule == ISING_SCHED_SEQUENTIAL) return false;
+  for (const InstDesc &I : h->inst)
+    if (I.ncls > 120) return false;  // (a detached search's loop holds 4 sweeps of 512 launches at most)
   const double descents = p->sweep_budget > 0 ? 1 : p->restarts;
   const double waves = std::max(1.0, std::ceil((double)h->n_inst * groups * descents / h->sm_count));
   const double tile = waves * 10e-9 * h->nmax;
@@ -485,8 +487,8 @@ bool sweep_is_faster(const ising_handle *h, int32_t R, const ising_search_params
 }
 
 // Kernel family for these arguments (ISING_KERNEL_AUTO resolved), or negative status.
-// waits: the call waits for its search (it was asked for the work counters).
-int32_t resolve_kernel(ising_handle *h, int32_t R, const ising_search_params *p, bool waits) {
+// *by_time is set where the sweep family was taken though a tile could run the call.
+int32_t resolve_kernel(ising_handle *h, int32_t R, const ising_search_params *p, bool *by_time = nullptr) {
   int32_t k = p->kernel;
   if (h->dtype == ISING_F64)  // FP64 couplings: the plain family only
     return (k == ISING_KERNEL_AUTO || k == ISING_KERNEL_PLAIN) ? ISING_KERNEL_PLAIN : -(int32_t)ISING_ERR_UNSUPPORTED;
@@ -496,7 +498,9 @@ int32_t resolve_kernel(ising_handle *h, int32_t R, const ising_search_params *p,
     if (h->dense && dense_supported(h, R)) return ISING_KERNEL_DENSE_TC;
     if (h->msc_ok && tile_fits(h, 2)) return ISING_KERNEL_MSC;
     if (!tile_fits(h, h->dtype == ISING_F32 ? 1 : 0)) return ISING_KERNEL_SWEEP;
-    return waits && sweep_is_faster(h, R, p) ? ISING_KERNEL_SWEEP : ISING_KERNEL_TILE;
+    if (!sweep_is_faster(h, R, p)) return ISING_KERNEL_TILE;
+    if (by_time) *by_time = true;
+    return ISING_KERNEL_SWEEP;
   }
   switch (k) {
     case ISING_KERNEL_TILE:
@@ -1143,7 +1147,7 @@ int32_t ising_plan_kernel(ising_handle *h, int32_t replicas, const ising_search_
   if (!h || replicas < 1) return -(int32_t)ISING_ERR_INVALID_ARG;
   ising_status st = validate_params(p);
   if (st != ISING_OK) return -(int32_t)st;
-  return resolve_kernel(h, replicas, p, true);
+  return resolve_kernel(h, replicas, p);
 }
 
 ising_status ising_local_search(ising_handle *h, const uint64_t *seeds, int32_t replicas,
@@ -1162,7 +1166,8 @@ ising_status ising_local_search(ising_handle *h, const uint64_t *seeds, int32_t 
   if (energy_i32_dev && (h->dtype != ISING_I8 || h->abs_energy_bound > 0x7fffffffLL))
     return ISING_ERR_UNSUPPORTED;
   if ((int64_t)replicas * h->total_spins > (int64_t)1 << 40) return ISING_ERR_UNSUPPORTED;
-  const int32_t kernel = resolve_kernel(h, replicas, p, stats != nullptr);
+  bool by_time = false;
+  const int32_t kernel = resolve_kernel(h, replicas, p, &by_time);
   if (kernel < 0) return (ising_status)(-kernel);
   int cur = 0;
   cudaGetDevice(&cur);
@@ -1190,7 +1195,7 @@ ising_status ising_local_search(ising_handle *h, const uint64_t *seeds, int32_t 
                       energy_dev, energy_i32_dev, minima_dev, stream);
         break;
       case ISING_KERNEL_SWEEP:
-        if (launch_sweep(h, p, replicas, spins_dev, energy_dev, energy_i32_dev, minima_dev, stream) !=
+        if (launch_sweep(h, p, replicas, spins_dev, energy_dev, energy_i32_dev, minima_dev, by_time && !stats, stream) !=
             cudaSuccess)
           st = ISING_ERR_CUDA;
         break;
@@ -1247,7 +1252,7 @@ ising_status ising_autotune(ising_handle *h, int32_t replicas, const ising_searc
   if (cached > 0) {
     ising_search_params q = *p;
     q.kernel = (ising_kernel)cached;
-    if (resolve_kernel(h, replicas, &q, true) == cached) {
+    if (resolve_kernel(h, replicas, &q) == cached) {
       h->tuned[replicas] = cached;
       if (chosen) *chosen = cached;
       return ISING_OK;
@@ -1277,7 +1282,7 @@ ising_status ising_autotune(ising_handle *h, int32_t replicas, const ising_searc
   for (int32_t fam : families) {
     ising_search_params q = *p;
     q.kernel = (ising_kernel)fam;
-    if (resolve_kernel(h, replicas, &q, true) != fam) continue;
+    if (resolve_kernel(h, replicas, &q) != fam) continue;
     ising_stats s1;
     if (ising_local_search(h, seeds.data(), replicas, &q, spins, E, nullptr, mins, &s1, stream) != ISING_OK) continue;
     cudaEventRecord(e0, stream);

@@ -152,8 +152,14 @@ __global__ void sweep_init(SweepArgs A) {
   }
   if (threadIdx.x == 0) {
     *A.counter = 0;
-    *A.all_done = 0;
+    A.all_done[0] = A.all_done[1] = 0;
   }
+}
+
+// Detached searches: whether the loop over chunks goes round again (all_done[1]:
+// chunks so far).
+__global__ void sweep_continue(int32_t *all_done, int32_t max_chunks, cudaGraphConditionalHandle loop) {
+  cudaGraphSetConditional(loop, all_done[0] == 0 && ++all_done[1] < max_chunks);
 }
 
 // u >= t for a bit-sliced 4-bit count (q0 least significant), t per thread.
@@ -1583,12 +1589,18 @@ cudaError_t preload(int mode, int *ctas_per_sm) {
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, sweep_energy<true, LPS, LAT>);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, sweep_energy<false, LPS, LAT>);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, sweep_restart<LPS>);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, sweep_continue);
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, visit, kST, 0);
   return e;
 }
 
+// detached: nothing is waited for; the chunks are the body of a loop on the device (a
+// conditional node).  Long searches take 1 to 3 % more than with replayed chunks and
+// the host looking on, short ones less, as no chunk is enqueued beyond the last one
+// needed (12,000 spins of degree 5, 20 replicas, 2 descents: 1,162 -> 939 us; 100 x 100
+// Gaussian, 8 replicas: 292 -> 238).
 template <int LPS, bool LAT>
-cudaError_t run_instance(ising_handle *h, SweepArgs A, int mode, cudaStream_t s) {
+cudaError_t run_instance(ising_handle *h, SweepArgs A, int mode, bool detached, cudaStream_t s) {
   SweepState &S = family_state<SweepState>(h->sweep_st);
   const InstDesc &I = A.I;
   const int ncls = A.sequential ? I.n : I.ncls;
@@ -1616,7 +1628,7 @@ cudaError_t run_instance(ising_handle *h, SweepArgs A, int mode, cudaStream_t s)
   // FP32 lattices whose classes leave warps idle (45^3, 21 replicas: 1521 against
   // 1624 us), slower for larger ones (100^3, 16 replicas: 49.4 against 48.3 ms) and
   // on general graphs (3801 against 3753 us)
-  A.pdl = mode == 2 || (mode == 1 && LAT && need * A.G * 2 <= slots);
+  A.pdl = !detached && (mode == 2 || (mode == 1 && LAT && need * A.G * 2 <= slots));
   Phase ph;
   ph.copy[0] = A.gs;
   ph.copy[1] = A.gs + A.G;
@@ -1647,22 +1659,24 @@ cudaError_t run_instance(ising_handle *h, SweepArgs A, int mode, cudaStream_t s)
   // sweeps need more launches (many colour classes, e.g. the sequential schedule)
   // sweeps are launched directly instead.  (A device-side loop - a conditional
   // WHILE node, optionally with an IF node around the round-end kernels - was
-  // measured slightly slower on GB300, and its kernels are not visible to ncu; one
-  // persistent kernel with grid barriers for the whole search no faster on a
+  // measured slightly slower on GB300, and its kernels are not visible to ncu: it
+  // serves detached searches only.  One persistent kernel with grid barriers for the whole search no faster on a
   // 45^3 lattice and 10 % slower on 100^3, with the visits' registers short.)
   constexpr int kMaxNodes = 512;
   const int per_sweep = ncls + 2;
   const bool use_graph = 4 * per_sweep <= kMaxNodes && !sweep_debug();
+  const bool loop = detached && use_graph;
   const int chunk = use_graph ? std::min(16, kMaxNodes / per_sweep & ~3) : 1;
   // the first sweep runs with direct launches, the rest from the graph
   enqueue_sweep<LPS, LAT>(A, ph, mode, cls, grid, s, true);
   h->launches += per_sweep;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   cudaGraphExec_t exec = nullptr;
+  const int64_t max_chunks = max_sweeps_total / chunk + 2;
   if (use_graph) {
     // everything the captured launches bake in besides the handle's own arrays
     char key[320];
-    std::snprintf(key, sizeof key, "%d/%d/%d/%d/%d/%d/%d/%d/%d/%d/%d/%d/%p/%d/%u/%u/%d/%d/%p/%d/%d/%d", A.b, A.R, A.r0,
+    std::snprintf(key, sizeof key, "%d/%d/%d/%d/%d/%d/%d/%d/%d/%d/%d/%d/%d/%p/%d/%u/%u/%d/%d/%p/%d/%d/%d", loop ? 1 : 0, A.b, A.R, A.r0,
                   A.Rn, A.G, A.LPS, A.max_sweeps, A.restarts, A.budget, A.refresh, A.sequential, A.lattice,
                   (void *)A.sw, mode, grid.x, grid.y, chunk, ncls, (void *)A.cflag, A.nchunk,
                   A.en_fast + 2 * A.en_count, A.pdl);
@@ -1671,12 +1685,30 @@ cudaError_t run_instance(ising_handle *h, SweepArgs A, int mode, cudaStream_t s)
       SweepGraph sg;
       cudaStream_t cs = nullptr;
       if ((e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking)) != cudaSuccess) return e;
-      e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
+      cudaGraphConditionalHandle again{};
+      if (loop) {
+        cudaGraphNodeParams np = {};
+        np.type = cudaGraphNodeTypeConditional;
+        e = cudaGraphCreate(&sg.graph, 0);
+        if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&again, sg.graph, 1, cudaGraphCondAssignDefault);
+        np.conditional.handle = again;
+        np.conditional.type = cudaGraphCondTypeWhile;
+        np.conditional.size = 1;
+        cudaGraphNode_t node;
+        if (e == cudaSuccess) e = cudaGraphAddNode(&node, sg.graph, nullptr, nullptr, 0, &np);
+        if (e == cudaSuccess)
+          e = cudaStreamBeginCaptureToGraph(cs, np.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                            cudaStreamCaptureModeThreadLocal);
+      } else {
+        e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
+      }
       if (e == cudaSuccess) {
         Phase pc = ph;
         for (int k = 0; k < chunk; ++k)
           enqueue_sweep<LPS, LAT>(A, pc, mode, cls, grid, cs, (k % kRoundEnd) == kRoundEnd - 1);
-        e = cudaStreamEndCapture(cs, &sg.graph);
+        if (loop) sweep_continue<<<1, 1, 0, cs>>>(A.all_done, (int32_t)std::min<int64_t>(max_chunks, INT32_MAX), again);
+        cudaGraph_t body = nullptr;
+        e = cudaStreamEndCapture(cs, loop ? &body : &sg.graph);
       }
       if (e == cudaSuccess) e = cudaGraphInstantiate(&sg.exec, sg.graph, 0);
       cudaStreamDestroy(cs);
@@ -1688,9 +1720,13 @@ cudaError_t run_instance(ising_handle *h, SweepArgs A, int mode, cudaStream_t s)
     }
     exec = it->second.exec;
   }
-  const int64_t max_chunks = max_sweeps_total / chunk + 2;
   int64_t launched = 0;
-  for (;;) {
+  if (loop) {
+    kt_begin(h, "sweep_chunk", s);
+    e = cudaGraphLaunch(exec, s);
+    kt_end(h, s);
+  }
+  while (!loop) {
     h->launches += (uint64_t)chunk * ncls + (use_graph ? chunk / kRoundEnd : 1) * 2;
     kt_begin(h, "sweep_chunk", s);
     if (use_graph) {
@@ -1757,8 +1793,12 @@ void sweep_free(ising_handle *h) {
 }
 
 cudaError_t launch_sweep(ising_handle *h, const ising_search_params *p, int32_t R, int8_t *spins, double *E,
-                         int32_t *E32, int32_t *minima, cudaStream_t s) {
+                         int32_t *E32, int32_t *minima, bool detached, cudaStream_t s) {
   SweepState &S = family_state<SweepState>(h->sweep_st);
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(s, &cap);
+  if (e == cudaSuccess && detached && cap != cudaStreamCaptureStatusNone) e = cudaErrorStreamCaptureUnsupported;
+  if (e != cudaSuccess) return e;  // (scratch and graphs are the handle's, as for the tile kernels)
   const bool fl = h->dtype == ISING_F32;
   const int mode = fl ? 1 : (h->msc_ok ? 2 : 0);
   const int LPS = lanes_per_spin(h, mode, p->schedule == ISING_SCHED_SEQUENTIAL, R);
@@ -1774,7 +1814,6 @@ cudaError_t launch_sweep(ising_handle *h, const ising_search_params *p, int32_t 
   const size_t need = 4 * up256(words * 4) + (fl ? up256(words * LPS * 4) : 0) + up256(2 * G * sizeof(GroupState)) +
                       up256((size_t)grid_e * G * 32 * 8) + up256((size_t)G * 32 * 16) + 2 * 256 + up256((size_t)4 * G * 4) +
                       up256(cflag_bytes);
-  cudaError_t e;
   if (need > S.bytes) {
     for (auto &kv : S.graphs) {  // captured against the old scratch
       cudaGraphExecDestroy(kv.second.exec);
@@ -1870,13 +1909,13 @@ cudaError_t launch_sweep(ising_handle *h, const ising_search_params *p, int32_t 
       if ((e = cudaMemsetAsync(A.pend, 0, words * 4, s)) != cudaSuccess) return e;
       if (A.cflag && (e = cudaMemsetAsync(cflag_mem, 0, cflag_bytes, s)) != cudaSuccess) return e;
       if (A.lattice) {
-        if (LPS == 32) e = run_instance<32, true>(h, A, mode, s);
-        else if (LPS == 16) e = run_instance<16, true>(h, A, mode, s);
-        else e = run_instance<8, true>(h, A, mode, s);
+        if (LPS == 32) e = run_instance<32, true>(h, A, mode, detached, s);
+        else if (LPS == 16) e = run_instance<16, true>(h, A, mode, detached, s);
+        else e = run_instance<8, true>(h, A, mode, detached, s);
       } else {
-        if (LPS == 32) e = run_instance<32, false>(h, A, mode, s);
-        else if (LPS == 16) e = run_instance<16, false>(h, A, mode, s);
-        else e = run_instance<8, false>(h, A, mode, s);
+        if (LPS == 32) e = run_instance<32, false>(h, A, mode, detached, s);
+        else if (LPS == 16) e = run_instance<16, false>(h, A, mode, detached, s);
+        else e = run_instance<8, false>(h, A, mode, detached, s);
       }
       if (e != cudaSuccess) return e;
     }

@@ -162,23 +162,71 @@ def test_first_passes_call_under_capture(dtype):
 
 
 # A search without work counters returns to the host once it is queued where one
-# kernel serves the instance: also for the few large instances that AUTO gives to
-# the sweep family when the call waits anyway.
-def test_auto_search_without_stats_does_not_hold_the_host(busy):
-    inst = W.random_graph(12000, 5.0, 61, dtype="f32", n_hyper=1500, hyper_order=(3, 4))
-    kw = dict(max_sweeps=300, restarts=2)
-    h = isg.Handle([inst])
-    assert h.plan_kernel(6, **kw) == isg.KERNEL_SWEEP
-    waited = h.local_search([5], 6, **kw)
-    h.local_search([5], 6, stats=False, **kw)  # (grows the scratch)
+# kernel serves the instance: also for the few large instances that AUTO gives to the
+# sweep family, whose sweeps then loop on the device.  Chunks of 16 sweeps and of
+# fewer (by the colour classes), budgets, searches that end in the first chunk and
+# that never converge, several instances, both value types; twice on one handle.
+def _auto_case(kind):
+    if kind == "classes":  # 68 colour classes: chunks of 4 sweeps
+        n = 25000
+        rng = np.random.default_rng(3)
+        u = rng.integers(0, n, size=n)
+        v = (u + rng.integers(1, n, size=n)) % n
+        colour = rng.integers(0, 68, size=n).astype(np.int32)
+        key = np.unique((np.minimum(u, v) * np.int64(n) + np.maximum(u, v))[colour[u] != colour[v]])
+        w = rng.integers(1, 4, size=len(key)).astype(np.int8)
+        rp, col, J = W.csr_from_edges(n, key // n, key % n, w, "i8")
+        return [W.Instance(n=n, row_ptr=rp, col=col, J=J, colour=colour, dtype="i8")], 3, dict(max_sweeps=30)
+    if kind == "square":
+        return [W.lattice((150, 150), True, "gauss", "gauss", seed=2)], 21, dict(max_sweeps=300, restarts=3)
+    if kind == "two":
+        return [W.lattice((140 + k, 140 + k), True, "gauss", None, seed=k) for k in range(2)], 5, \
+            dict(max_sweeps=300, restarts=2)
+    inst = W.random_graph(12000, 5.0, 61, dtype="i8" if kind == "int" else "f32", n_hyper=1500, hyper_order=(3, 4))
+    return [inst], 6, {"budget": dict(max_sweeps=300, restarts=50, sweep_budget=45), "one": dict(max_sweeps=1),
+                       "capped": dict(max_sweeps=3, restarts=2)}.get(kind, dict(max_sweeps=300, restarts=2))
+
+
+@pytest.mark.parametrize("kind", ["graph", "int", "square", "two", "budget", "one", "capped", "classes"])
+def test_auto_search_without_stats_does_not_hold_the_host(kind, busy):
+    insts, R, kw = _auto_case(kind)
+    seeds = list(range(5, 5 + len(insts)))
+    h = isg.Handle(insts)
+    assert h.plan_kernel(R, **kw) == isg.KERNEL_SWEEP
+    h.local_search(seeds, R, stats=False, **kw)  # (builds its graph and scratch)
     before = torch.cuda.Event()
     busy()
     before.record()
-    r = h.local_search([5], 6, stats=False, **kw)
-    assert not before.query(), "the call held the host until the stream had caught up"
+    r = h.local_search(seeds, R, stats=False, **kw)
+    held = before.query()
+    waited = h.local_search(seeds, R, **kw)
+    again = h.local_search(seeds, R, stats=False, **kw)
     torch.cuda.synchronize()
-    assert torch.equal(r.spins, waited.spins) and torch.equal(r.minima, waited.minima)
-    torch.testing.assert_close(r.energy, waited.energy, rtol=1e-12, atol=0)
+    for b, inst in enumerate(insts):
+        s, e, m, _ = oracle.descent(inst, seeds[b], b, R, **kw)
+        for got in (r, waited, again):
+            assert np.array_equal(h.spins_of(got.spins, b, R).cpu().numpy(), s)
+            assert np.array_equal(got.minima[b].cpu().numpy(), m)
+            np.testing.assert_allclose(got.energy[b].cpu().numpy(), e, rtol=1e-9, atol=1e-9)
+    assert not held, "the call held the host until the stream had caught up"
+    h.close()
+
+
+def test_auto_search_without_stats_is_refused_under_capture():
+    insts, R, kw = _auto_case("graph")
+    h = isg.Handle(insts)
+    ref = h.local_search([5], R, stats=False, **kw)
+    side = torch.cuda.Stream()
+    g = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        g.capture_begin(capture_error_mode="relaxed")
+        with pytest.raises(isg.IsingError):
+            h.local_search([5], R, stats=False, out=(ref.spins, ref.energy, None, ref.minima), **kw)
+        g.capture_end()
+    del g
+    r = h.local_search([5], R, stats=False, **kw)
+    assert torch.equal(r.spins, ref.spins)
     h.close()
 
 
