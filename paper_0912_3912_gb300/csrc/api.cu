@@ -575,9 +575,9 @@ const ClusterPlan &cluster_plan(ising_handle *h, int32_t R, const ising_search_p
 // descents of 64 replicas 323 / 230 / 218, of 1,024 447 / 561 / 553.  +/-J: 31^3, 1,024
 // replicas, 10 descents 2499 / 1572 / 1279; 16 x 16, 64 replicas, 10 descents 52 / 42 /
 // 44 (125 in one segment).
-// In the index order a CTA of any size decides a spin at a time; multi-spin coded, its
-// barrier per spin takes longer the more warps wait at it (64 x 64, 64 replicas 9.1 /
-// 9.3 / 10.1 ms).
+// The index order, a spin at a time in any CTA, runs at 256 threads only: multi-spin
+// coded, its barrier per spin takes longer the more warps wait at it (64 x 64, 64
+// replicas 6.4 ms; in a kernel for both orders 9.1 / 9.3 / 10.1).
 const TilePlan *tile_plan(ising_handle *h, int mode, int32_t R, const ising_search_params *p) {
   TilePlan &T = h->tile_plan_cache;
   const int32_t parallel = p->sweep_budget > 0 ? 1 : p->restarts;
@@ -599,6 +599,7 @@ const TilePlan *tile_plan(ising_handle *h, int mode, int32_t R, const ising_sear
   weight *= (double)((R + 31) / 32) * parallel;
   double best = 0.0;
   for (int threads : {256, 512, 1024}) {
+    if (sequential && threads != 256) break;
     // FP32 lanes: fields in shared memory for every instance that fits, within a
     // budget that lets four CTAs share an SM (one CTA of 1024 threads with four
     // times as much, and so less L1, was 5 % slower)
@@ -606,13 +607,13 @@ const TilePlan *tile_plan(ising_handle *h, int mode, int32_t R, const ising_sear
     if (nmin > fsm_cap) fsm_cap = 0;
     size_t smem = tile_smem_bytes(mode, h->nmax);
     if (fsm_cap > 0) smem = (smem + 15) / 16 * 16 + (size_t)fsm_cap * 128;
-    const int64_t slots = (int64_t)tile_max_ctas_per_sm(mode, threads, smem) * h->sm_count;
+    const int64_t slots = (int64_t)tile_max_ctas_per_sm(mode, threads, smem, sequential) * h->sm_count;
     if (slots < 1) continue;
     const double per_step = mode >= 2 ? 2.0 * threads : (double)ncls * threads / 32;
     const double fixed = mode >= 2 ? 30.0 : (mode == 0 ? 6.0 : (threads == 1024 ? 15.0 : 10.0));
-    const double unit = sequential ? 1.0 + (mode >= 2 ? 1e-4 * threads : 0.0) : fixed + std::ceil(h->nmax / per_step);
+    const double unit = fixed + std::ceil(h->nmax / per_step);
     double waves = weight / (double)slots;
-    if (mode != 1 || sequential) {
+    if (mode != 1) {
       waves = std::max(1.0, waves);
       if (nmin == h->nmax && waves < 2.0) waves = std::ceil(waves);
     } else if (waves < 1.0) {
@@ -741,7 +742,7 @@ ising_status run_tile(ising_handle *h, int mode, int32_t R, const ising_search_p
   if (cap != cudaStreamCaptureStatusNone) return ISING_ERR_CUDA;  // (scratch and work queue are the handle's)
   CUDA_OK(cudaMemsetAsync(h->d_queue, 0, sizeof(int32_t) * (4 + (size_t)counters), s));
   kt_begin(h, "tile_kernel", s);
-  CUDA_OK(launch_tile(a, mode, threads, segs > 1 || a.sequential, grid, smem, s));
+  CUDA_OK(launch_tile(a, mode, threads, segs > 1, grid, smem, s));
   kt_end(h, s);
   h->launches += 1;
   return ISING_OK;

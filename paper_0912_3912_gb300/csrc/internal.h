@@ -254,7 +254,7 @@ cudaError_t launch_tile(const TileArgs &a, int mode, int threads, bool seg, int 
 size_t tile_smem_bytes(int mode, int nmax);
 size_t tile_smem_limit();  // dynamic shared memory of a tile CTA at most
 int tile_fsm_cap(int nmax, size_t budget);
-int tile_max_ctas_per_sm(int mode, int threads, size_t smem);
+int tile_max_ctas_per_sm(int mode, int threads, size_t smem, bool seq);
 cudaError_t launch_energy(ising_handle *h, const int8_t *spins, int32_t R, double *E,
                           int32_t *E32, cudaStream_t s);
 void energy_plan_free(ising_handle *h);

@@ -493,9 +493,9 @@ __device__ __forceinline__ uint32_t own_visit(const DevGraph &G, const uint32_t 
 
 // SEG: tiles in segments of descents.  (A separate instantiation: the segments'
 // few values in the whole-tile kernel spill at 64 registers and cost full batches
-// 8 %.  For the same reason only the segments' instantiations know the index order:
-// one segment of them where there is one.)
-template <int MODE, int THREADS, bool SEG>
+// 8 %.)  SEQ: the index order, at 256 threads and with segments (one where there are
+// none); its tests in the colour order's loops cost small instances 4 %.
+template <int MODE, int THREADS, bool SEG, bool SEQ = false>
 __global__ void __launch_bounds__(THREADS, (MODE == 3 ? 512 : 1024) / THREADS < 1 ? 1 : (MODE == 3 ? 512 : 1024) / THREADS)
 tile_kernel(const __grid_constant__ TileArgs A) {
   // (a parameter, so that its pointers stay in constant memory: read through a pointer
@@ -543,12 +543,11 @@ tile_kernel(const __grid_constant__ TileArgs A) {
     const int rem = A.R - 32 * g;
     const uint32_t lane_valid = rem >= 32 ? 0xffffffffu : ((1u << rem) - 1u);
     const uint64_t seed = A.seeds[b];
-    const bool index_order = SEG && A.sequential;  // (launched with SEG alone)
     // On lanes, warp 0 takes the spins of the index order one after another and the
     // others wait for the sweep's end; multi-spin coded, a thread takes one and the
     // CTA waits for it.
-    const bool seq = MODE <= 1 && index_order;
-    const int ncls = seq ? 1 : (index_order ? n : I.ncls);
+    constexpr bool seq = MODE <= 1 && SEQ;
+    const int ncls = seq ? 1 : (SEQ ? n : I.ncls);
     float *Fc = (MODE == 1 && n <= A.fsm_cap) ? Fs : F;
     if (tid < 32) {
       s_total[tid] = 0;
@@ -599,7 +598,7 @@ tile_kernel(const __grid_constant__ TileArgs A) {
         uint32_t anyf = 0;
         for (int c = 0; c < ncls; ++c) {
           int c0, c1;
-          if (index_order) {
+          if (SEQ) {
             c0 = c;
             c1 = seq ? n : c + 1;
           } else {
@@ -658,7 +657,7 @@ tile_kernel(const __grid_constant__ TileArgs A) {
             const int8_t *Ji = reinterpret_cast<const int8_t *>(G.J);
             const int8_t *hi = reinterpret_cast<const int8_t *>(G.h);
             for (int v = c0 + tid; v < c1; v += THREADS) {
-              const int j = index_order ? v : __ldg(G.order + I.spin_off + v);
+              const int j = SEQ ? v : __ldg(G.order + I.spin_off + v);
               if (!pending(j)) continue;
               clear_pending(j);
               my_eval += __popc(active);
@@ -1074,17 +1073,18 @@ template <int MODE>
 TileKernel tile_kernel_of(int threads, bool seg) {
   return seg ? tile_kernel_of<MODE, true>(threads) : tile_kernel_of<MODE, false>(threads);
 }
-TileKernel tile_kernel_for(int mode, int threads, bool seg) {
+TileKernel tile_kernel_for(int mode, int threads, bool seg, bool seq) {
+  if (seq) return mode == 0 ? tile_kernel<0, 256, true, true> : (mode == 1 ? tile_kernel<1, 256, true, true> : tile_kernel<2, 256, true, true>);
   return mode == 0 ? tile_kernel_of<0>(threads, seg)
                    : (mode == 1 ? tile_kernel_of<1>(threads, seg)
                                 : (mode == 2 ? tile_kernel_of<2>(threads, seg) : tile_kernel_of<3>(threads, seg)));
 }
 }  // namespace
 
-int tile_max_ctas_per_sm(int mode, int threads, size_t smem) {
+int tile_max_ctas_per_sm(int mode, int threads, size_t smem, bool seq) {
   int blocks = 0, least = 0;
   for (int seg = 0; seg < 2; ++seg) {
-    const TileKernel k = tile_kernel_for(mode, threads, seg != 0);
+    const TileKernel k = tile_kernel_for(mode, threads, seg != 0, seq);
     // (the same limit for every size: the attribute is the process's, and another
     // thread's handle may launch the same kernel at a larger size)
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tile_smem_limit());
@@ -1097,7 +1097,7 @@ int tile_max_ctas_per_sm(int mode, int threads, size_t smem) {
 
 // Launch only: the shared-memory attribute was set by tile_max_ctas_per_sm.
 cudaError_t launch_tile(const TileArgs &a, int mode, int threads, bool seg, int grid, size_t smem, cudaStream_t s) {
-  tile_kernel_for(mode, threads, seg)<<<grid, threads, smem, s>>>(a);
+  tile_kernel_for(mode, threads, seg, a.sequential != 0)<<<grid, threads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
