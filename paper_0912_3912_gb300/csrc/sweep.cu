@@ -1781,11 +1781,11 @@ int lanes_per_spin(const ising_handle *h, int mode, bool sequential, int32_t R) 
 void sweep_free(ising_handle *h) {
   if (!h->sweep_st) return;
   SweepState &S = static_cast<SweepState &>(*h->sweep_st);
+  cudaFree(S.mem);  // (waits for a detached search that may still run)
   for (auto &kv : S.graphs) {
     cudaGraphExecDestroy(kv.second.exec);
     cudaGraphDestroy(kv.second.graph);
   }
-  cudaFree(S.mem);
   if (S.h_done) cudaFreeHost(S.h_done);
   for (auto &e : S.ev)
     if (e) cudaEventDestroy(e);
@@ -1815,12 +1815,12 @@ cudaError_t launch_sweep(ising_handle *h, const ising_search_params *p, int32_t 
                       up256((size_t)grid_e * G * 32 * 8) + up256((size_t)G * 32 * 16) + 2 * 256 + up256((size_t)4 * G * 4) +
                       up256(cflag_bytes);
   if (need > S.bytes) {
+    cudaFree(S.mem);  // (waits for a detached search that may still run)
     for (auto &kv : S.graphs) {  // captured against the old scratch
       cudaGraphExecDestroy(kv.second.exec);
       cudaGraphDestroy(kv.second.graph);
     }
     S.graphs.clear();
-    cudaFree(S.mem);
     S.mem = nullptr;
     S.bytes = 0;
     if ((e = cudaMalloc(&S.mem, need)) != cudaSuccess) return e;

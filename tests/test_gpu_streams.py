@@ -230,6 +230,28 @@ def test_auto_search_without_stats_is_refused_under_capture():
     h.close()
 
 
+# A handle closed, and one whose scratch grows, while such a search still runs.
+def test_auto_search_without_stats_outlives_nothing_it_needs(busy):
+    insts, R, kw = _auto_case("graph")
+    s, _, m, _ = oracle.descent(insts[0], 5, 0, R, **kw)
+    s40, _, _, _ = oracle.descent(insts[0], 6, 0, 40, **kw)
+    for close in (True, False):
+        h = isg.Handle(insts)
+        h.local_search([5], R, stats=False, **kw)
+        busy()
+        r = h.local_search([5], R, stats=False, **kw)
+        if close:
+            h.close()
+        else:
+            wider = h.local_search([6], 40, stats=False, **kw)
+        torch.cuda.synchronize()
+        assert np.array_equal(r.spins.cpu().numpy().reshape(R, -1), s)
+        assert np.array_equal(r.minima[0].cpu().numpy(), m)
+        if not close:
+            assert np.array_equal(wider.spins.cpu().numpy().reshape(40, -1), s40)
+            h.close()
+
+
 # Two handles of one kernel and different sizes, from two host threads: neither
 # changes what the other may launch.
 def test_cluster_launches_of_two_sizes_from_two_threads():
